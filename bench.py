@@ -141,9 +141,9 @@ def ring_bytes_allreduce(S, R):
 
 
 def direct_bytes_allreduce(S, R):
-    """Stage-decomposed schedule: moves 2 S (R-1) into the owners' inbox slots, one chain sum per rank (R reads and one write per
-    output byte: S (R+1)), all-gather moves 2 S (R-1)."""
-    return 4.0 * S * (R - 1) + S * (R + 1)
+    """Stage-decomposed schedule on the copy route: one chain sum per rank that reads the R contributions where they lie and writes
+    each output byte once (S (R+1)), all-gather moves 2 S (R-1)."""
+    return 2.0 * S * (R - 1) + S * (R + 1)
 
 
 def reference_arm(args, world):
@@ -385,8 +385,8 @@ def main():
             "stream": "%d buckets of %d MiB and one of %d MiB per rank (%.1f GiB); every bucket is the same work, %d are timed" %
                       (len(sizes) - 1, S >> 20, sizes[-1] * 2 >> 20, sum(sizes) * 2 / 2 ** 30, steps),
             "step": "one hoccl_allreduce call on one bucket", "path": "CE (driver copy route)", "sum_ctas": 8,
-            "schedule": ("stage-decomposed reduce-scatter and all-gather, one chain sum per rank in the ring's order (chosen automatically: "
-                         "the attached scratch holds its R-1 inbox slots per rank)") if direct else "ring, step by step",
+            "schedule": ("stage-decomposed reduce-scatter and all-gather, one chain sum per rank in the ring's order that reads the contributions "
+                         "where they lie (chosen automatically: the attached scratch holds R-1 inbox slots per rank)") if direct else "ring, step by step",
             "executor": "cuda graph replay", "pieces_per_chunk": st["n_pieces"],
             "l2": "inputs larger than L2: %d bucket sets of %d MiB in rotation" % (B.nsets, 2 * R * S >> 20),
             "gemm_probe": "not running during the timed steps; gemm_loss_matched times the same stream beside it",

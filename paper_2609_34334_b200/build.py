@@ -12,7 +12,7 @@ SOURCES = ["api.cu", "exec.cu", "p2p.cu", "kernels.cu", "plan.cpp", "static_scra
 HEADERS = ["comm.h", "kernels.cuh", "device_common.cuh", "plan.h", "proxy.h", "sched.h", "options.h", os.path.join("..", "..", "include", "hoccl.h"), os.path.join("..", "..", "include", "hoccl_diag.h")]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "-Xcompiler", "-fPIC,-Wall,-Wno-unused-function", "-shared", "-cudart", "static",
+    "-Xcompiler", "-fPIC,-Wall,-Wno-unused-function", "-shared", "-cudart", "static", "--threads", "0",
 ]
 
 

@@ -733,11 +733,19 @@ hoccl_result_t hoccl_chain_launch(const void* first, size_t stride_bytes, int ns
       ((uintptr_t)first % e) || ((uintptr_t)local % e) || ((uintptr_t)out % e))
     return HOCCL_ERR_INVALID_ARG;
   if (count == 0) return HOCCL_OK;
-  ChainBatch b;
-  b.nseg = 1;
-  b.dtype = (int)dtype;
-  b.seg[0] = ChainSeg{first, local, out, (unsigned long long)count, (unsigned long long)stride_bytes, nsrc, 0};
-  return launch_chain(b, ctas, (cudaStream_t)stream) == cudaSuccess ? HOCCL_OK : HOCCL_ERR_CUDA;
+  const void* ops[kMaxChainSrcs + 1];
+  const size_t e_step = kMaxChainSegBytes / e;
+  for (size_t at = 0; at < count; at += e_step) {
+    for (int j = 0; j < nsrc; j++) ops[j] = (const char*)first + (size_t)j * stride_bytes + at * e;
+    ops[nsrc] = (const char*)local + at * e;
+    void* dst = (char*)out + at * e;
+    ChainBatch b;
+    b.nseg = b.nptr = 0;
+    b.dtype = (int)dtype;
+    add_chain_seg(&b, ops, nsrc + 1, &dst, 1, (unsigned long long)std::min(e_step, count - at));
+    if (launch_chain(b, ctas, (cudaStream_t)stream) != cudaSuccess) return HOCCL_ERR_CUDA;
+  }
+  return HOCCL_OK;
 }
 
 hoccl_result_t hoccl_selftest_bf16_add(unsigned long long* counts, hoccl_stream_t stream) {

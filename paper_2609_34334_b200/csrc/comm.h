@@ -38,6 +38,10 @@ struct Seg {
   uint64_t host_off = 0;  // HOCCL_PATH_CE_HOST: where this move bounces in the pinned host staging
   int nsrc = 1;           // OP_CHAIN: inbox operands at src + j * src_stride
   uint64_t src_stride = 0;
+  // OP_CHAIN that reads the contributions where they lie (see read_in_place): all operands in the order of addition, the owner's
+  // last; and, if the sum stores the result for every rank, all destinations (otherwise `dst`)
+  std::vector<const void*> ops;
+  std::vector<void*> dsts;
   bool host_first = true; // HOCCL_PATH_CE_HOST: this move issues the outbound copy into host_off (false: another move of the group did)
 };
 
@@ -64,6 +68,15 @@ struct HostCopy {
   char* dev;
   char* host;
   size_t pitch, width, rows;
+};
+
+// One kernel launch of a schedule: the batch is its only parameter, by value.
+struct KernelLaunch {
+  const void* fn = nullptr;
+  int grid = 0, threads = 0;
+  std::vector<char> args;
+  double bytes = 0;   // algorithmic bytes
+  long moves = 0;     // MOVE operations it carries (0: a sum)
 };
 
 struct GraphEntry {
@@ -187,9 +200,10 @@ struct Tally {
 };
 
 // exec.cu
-void fill_sum_batch(const RGroup& g, size_t first, size_t n, int dtype, size_t elem, SumBatch* b);
+// The kernel launches that carry out one group: its sums, or (SM route) its moves.
+std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, const RGroup& g);
+cudaError_t launch_kernel(const KernelLaunch& k, cudaStream_t stream);
 void fill_copy_batch(const RGroup& g, size_t first, size_t n, CopyBatch* b);
-void fill_chain_batch(const RGroup& g, size_t first, size_t n, int dtype, size_t elem, ChainBatch* b);
 // Moves of a group that read the same bytes (same source and length; the direct all-gather on the SM path) become fan-out
 // segments: one read, one store per destination.  Returns false (and leaves *out empty) if no source repeats: the plain
 // copy batches are used then.  bytes_out[i] = HBM bytes of batch i (reads + writes), moves_out[i] = moves it carries.

@@ -76,8 +76,45 @@ static void share_host_legs(std::vector<RGroup>* groups, size_t* host_need) {
   }
 }
 
+constexpr size_t kStoreAllBytesPerCta = 384 << 10;
+constexpr size_t kGradeInPlace = 4 << 20;   // ring chunk from which pieces are graded on the SM path when contributions are read in place
+
+// How the direct reduce-scatter's contributions reach the owner's sum.
+enum Contributions {
+  STAGED = 0,      // moved into the owner's inbox slots first (the plan as it is)
+  READ_IN_PLACE,   // the sum reads them where they lie: the plan's moves into the inbox fall away
+  READ_AND_STORE   // ... and it stores the result for every rank: the all-gather's moves fall away too
+};
+
+// All ranks live in one device's memory, so a sum can read the other ranks' contributions without a copy of them.  Staging
+// them costs 2 (R - 1) bytes of traffic per output byte and buys nothing for the sum, which reads R operands either way.
+// Only the automatic schedule does this: "rs_direct" = 1 keeps the staged form that a rank-local owner needs.
+//   * The send buffers have to share their 16-byte phase.  (Inbox slots are placed so that the operands always do; contributions
+//     that do not would be summed element by element.)
+//   * The host-bounce path keeps its moves: that no SM takes part in them is what it is chosen for.  So does the pipelined host
+//     entry, which PCIe bounds (25 MiB per rank 5.41 ms with them, 5.50 without).
+// The sum stores for all ranks on the SM route (on the copy route the all-gather's moves are the driver's) when its grid is the
+// whole GPU, or when the message is so short that the second launch and not the stores decide: a CTA stores ~60 GB/s, so R S
+// bytes over n CTAs take R S / (60 n) ns against ~2.5 us for a launch of its own and the wider copy grid.  Measured, one kernel
+// against two, 8-CTA sums and 148 copy CTAs: R = 8 bf16 4 KiB per rank 3.0 / 6.2 us, 384 KiB 10.3 / 12.3, 512 KiB 14.4 / 12.4;
+// R = 4 fp32 512 KiB 8.2 / 10.3, 1 MiB 14.4 / 12.4; R = 2 bf16 1 MiB 8.3 / 9.0, 2 MiB 14.4 / 12.4: the line lies at R S = 3 MiB.
+static Contributions contributions(const hoccl_comm* c, const Call& call, const OptionsOut& opt, size_t S) {
+  if (!(opt.plan_kind & PLAN_FLAG_RS_DIRECT) || c->rs_direct != 2 || c->R < 2 || c->path == HOCCL_PATH_CE_HOST || call.h_send) return STAGED;
+  if (opt.executor != EXEC_GRAPH && opt.executor != EXEC_STREAMS && opt.executor != EXEC_PROXY) return STAGED;
+  const uintptr_t phase = (uintptr_t)call.send[0] & 15;
+  bool recv_too = true;
+  for (int r = 0; r < c->R; r++) {
+    if (((uintptr_t)call.send[r] & 15) != phase) return STAGED;
+    recv_too = recv_too && ((uintptr_t)call.recv[r] & 15) == phase;
+  }
+  if (call.kind == PLAN_ALLREDUCE && c->path == HOCCL_PATH_SM && (opt.plan_kind & PLAN_FLAG_AG_DIRECT) && recv_too &&
+      (c->sum_ctas >= 128 || (size_t)c->R * S <= (size_t)c->sum_ctas * kStoreAllBytesPerCta))
+    return READ_AND_STORE;
+  return READ_IN_PLACE;
+}
+
 // Turns plan offsets into addresses (the plan already places pieces inside the scratch slots).
-void resolve(hoccl_comm* c, const Plan& P, const Call& call, std::vector<RGroup>* out, size_t* host_need) {
+void resolve(hoccl_comm* c, const Plan& P, const Call& call, Contributions how, std::vector<RGroup>* out, size_t* host_need) {
   *host_need = 0;
   const int R = P.R;
   char* inbox0 = (char*)c->scratch;
@@ -116,13 +153,48 @@ void resolve(hoccl_comm* c, const Plan& P, const Call& call, std::vector<RGroup>
         s.dst = addr(op.dst_buf, op.dst_rank, op.chunk, op.dst_off);  // dst_rank == rank except in the forward variant
         s.nsrc = op.nsrc;
         s.src_stride = op.src_stride;
+        if (op.kind == OP_CHAIN && how != STAGED) {
+          for (int j = 1; j <= R; j++) s.ops.push_back((const char*)call.send[(op.rank + j) % R] + op.local_off);
+          if (how == READ_AND_STORE)
+            for (int r = 0; r < R; r++) s.dsts.push_back((char*)call.recv[r] + op.dst_off);
+        }
       }
       if (op.kind == OP_MOVE && c->path == HOCCL_PATH_CE_HOST) {
         s.host_off = *host_need;
         *host_need += (s.bytes + 255) / 256 * 256;
       }
       rg.segs.push_back(s);
+      if (op.kind == OP_CHAIN) {   // the chain kernels use 32-bit offsets inside a segment
+        while (rg.segs.back().bytes > kMaxChainSegBytes) {
+          Seg& head = rg.segs.back();
+          Seg rest = head;
+          head.bytes = kMaxChainSegBytes;
+          rest.bytes -= kMaxChainSegBytes;
+          rest.src += kMaxChainSegBytes;
+          rest.local += kMaxChainSegBytes;
+          rest.dst += kMaxChainSegBytes;
+          for (const void*& p : rest.ops) p = (const char*)p + kMaxChainSegBytes;
+          for (void*& p : rest.dsts) p = (char*)p + kMaxChainSegBytes;
+          rg.segs.push_back(rest);
+        }
+      }
     }
+  }
+  if (how != STAGED) {   // the moves the sums do themselves
+    std::vector<RGroup> kept;
+    std::vector<int> remap(out->size(), -1);
+    for (size_t g = 0; g < out->size(); g++) {
+      RGroup& cur = (*out)[g];
+      if (cur.kind == OP_MOVE && (how == READ_AND_STORE || cur.phase == PHASE_RS)) continue;
+      std::vector<int> deps;
+      for (int d : cur.deps)
+        if (remap[d] >= 0) deps.push_back(remap[d]);
+      cur.deps.swap(deps);
+      if (cur.chain_dep >= 0) cur.chain_dep = remap[cur.chain_dep];
+      remap[g] = (int)kept.size();
+      kept.push_back(std::move(cur));
+    }
+    out->swap(kept);
   }
   // SM path: the stages of an all-to-all are independent (disjoint blocks, no dependencies), so their moves go into as few
   // batched launches as the segment table allows instead of one launch per stage
@@ -151,9 +223,9 @@ void resolve(hoccl_comm* c, const Plan& P, const Call& call, std::vector<RGroup>
       RGroup& cur = (*out)[g];
       for (int& d : cur.deps) d = remap[d];
       if (cur.chain_dep >= 0) cur.chain_dep = remap[cur.chain_dep];
-      const bool tail_move = cur.kind == OP_MOVE && !has_user[g] && P.groups[g].phase != PHASE_RS;
+      const bool tail_move = cur.kind == OP_MOVE && !has_user[g] && cur.phase != PHASE_RS;
       if (tail_move && !merged.empty() && g > 0 && remap[g - 1] == (int)merged.size() - 1 && merged.back().kind == OP_MOVE &&
-          !has_user[g - 1] && P.groups[g - 1].phase != PHASE_RS && merged.back().piece == cur.piece && merged.back().deps == cur.deps) {
+          !has_user[g - 1] && merged.back().phase != PHASE_RS && merged.back().piece == cur.piece && merged.back().deps == cur.deps) {
         merged.back().segs.insert(merged.back().segs.end(), cur.segs.begin(), cur.segs.end());
         remap[g] = (int)merged.size() - 1;
       } else {
@@ -163,31 +235,6 @@ void resolve(hoccl_comm* c, const Plan& P, const Call& call, std::vector<RGroup>
     }
     out->swap(merged);
     if (c->path == HOCCL_PATH_CE_HOST) share_host_legs(out, host_need);
-  }
-}
-
-void fill_sum_batch(const RGroup& g, size_t first, size_t n, int dtype, size_t elem, SumBatch* b) {
-  b->nseg = (int)n;
-  b->dtype = dtype;
-  for (size_t i = 0; i < n; i++) {
-    const Seg& s = g.segs[first + i];
-    b->seg[i] = SumSeg{s.src, s.local, s.dst, (unsigned long long)(s.bytes / elem)};
-  }
-}
-void fill_chain_batch(const RGroup& g, size_t first, size_t n, int dtype, size_t elem, ChainBatch* b) {
-  b->nseg = (int)n;
-  b->dtype = dtype;
-  for (size_t i = 0; i < n; i++) {
-    const Seg& s = g.segs[first + i];
-    b->seg[i] = ChainSeg{s.src, s.local, s.dst, (unsigned long long)(s.bytes / elem), (unsigned long long)s.src_stride, s.nsrc, 0};
-  }
-}
-void fill_copy_batch(const RGroup& g, size_t first, size_t n, CopyBatch* b) {
-  b->nseg = (int)n;
-  b->pad = 0;
-  for (size_t i = 0; i < n; i++) {
-    const Seg& s = g.segs[first + i];
-    b->seg[i] = CopySeg{s.src, s.dst, (unsigned long long)s.bytes};
   }
 }
 
@@ -249,6 +296,112 @@ bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<
   return true;
 }
 
+void fill_copy_batch(const RGroup& g, size_t first, size_t n, CopyBatch* b) {
+  b->nseg = (int)n;
+  b->pad = 0;
+  for (size_t i = 0; i < n; i++) {
+    const Seg& s = g.segs[first + i];
+    b->seg[i] = CopySeg{s.src, s.dst, (unsigned long long)s.bytes};
+  }
+}
+
+// Fills *b with chain segments of g from `first` on; returns how many fitted.
+static size_t fill_chain_batch(const RGroup& g, size_t first, int dtype, size_t elem, ChainBatch* b) {
+  b->nseg = 0;
+  b->nptr = 0;
+  b->dtype = dtype;
+  size_t i = first;
+  for (; i < g.segs.size(); i++) {
+    const Seg& s = g.segs[i];
+    const void* ops[kMaxRanks];
+    int nops = 0;
+    if (!s.ops.empty()) {
+      for (const void* p : s.ops) ops[nops++] = p;
+    } else {
+      for (int j = 0; j < s.nsrc; j++) ops[nops++] = s.src + (size_t)j * s.src_stride;
+      ops[nops++] = s.local;
+    }
+    void* one = s.dst;
+    void* const* dsts = s.dsts.empty() ? &one : s.dsts.data();
+    const int ndst = s.dsts.empty() ? 1 : (int)s.dsts.size();
+    if (!add_chain_seg(b, ops, nops, dsts, ndst, (unsigned long long)(s.bytes / elem))) break;
+  }
+  return i - first;
+}
+
+template <class Batch>
+static KernelLaunch make_launch(const Batch& b, const void* fn, long grid, int threads, double bytes, long moves) {
+  KernelLaunch k;
+  k.fn = fn;
+  k.grid = (int)grid;
+  k.threads = threads;
+  k.args.assign(reinterpret_cast<const char*>(&b), reinterpret_cast<const char*>(&b) + sizeof(b));
+  k.bytes = bytes;
+  k.moves = moves;
+  return k;
+}
+
+std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, const RGroup& g) {
+  std::vector<KernelLaunch> out;
+  int threads = 0;
+  if (g.kind == OP_CHAIN) {
+    for (size_t first = 0; first < g.segs.size();) {
+      ChainBatch b;
+      const size_t n = fill_chain_batch(g, first, P.dtype, P.elem, &b);
+      prepare_chain_batch(&b, (int)c->sum_ctas);
+      double bytes = 0;
+      for (int i = 0; i < b.nseg; i++) bytes += (double)(b.seg[i].nops + b.seg[i].ndst) * (double)b.seg[i].n * (double)P.elem;
+      const void* fn = chain_kernel_entry(b, (int)c->sum_ctas, &threads);
+      out.push_back(make_launch(b, fn, c->sum_ctas, threads, bytes, 0));
+      first += n;
+    }
+    return out;
+  }
+  if (g.kind == OP_SUM) {
+    for (size_t first = 0; first < g.segs.size(); first += kMaxSegs) {
+      SumBatch b;
+      b.nseg = (int)std::min<size_t>(kMaxSegs, g.segs.size() - first);
+      b.dtype = P.dtype;
+      double bytes = 0;
+      for (int i = 0; i < b.nseg; i++) {
+        const Seg& s = g.segs[first + i];
+        b.seg[i] = SumSeg{s.src, s.local, s.dst, (unsigned long long)(s.bytes / P.elem)};
+        bytes += 3.0 * (double)s.bytes;
+      }
+      prepare_sum_batch(&b, (int)c->sum_ctas);
+      const void* fn = sum_kernel_entry(P.dtype, (int)c->sum_ctas, &threads);
+      out.push_back(make_launch(b, fn, c->sum_ctas, threads, bytes, 0));
+    }
+    return out;
+  }
+  std::vector<FanBatch> fans;
+  std::vector<double> fan_bytes;
+  std::vector<long> fan_moves;
+  if (P.ag_direct && build_fan_batches(g, &fans, &fan_bytes, &fan_moves)) {
+    const void* fn = fan_kernel_entry((int)c->copy_ctas, &threads);
+    for (size_t i = 0; i < fans.size(); i++) {
+      prepare_fan_batch(&fans[i], (int)c->copy_ctas);
+      out.push_back(make_launch(fans[i], fn, c->copy_ctas, threads, fan_bytes[i], fan_moves[i]));
+    }
+    return out;
+  }
+  const void* fn = copy_kernel_entry((int)c->copy_ctas, &threads);
+  for (size_t first = 0; first < g.segs.size(); first += kMaxSegs) {
+    CopyBatch b;
+    fill_copy_batch(g, first, std::min<size_t>(kMaxSegs, g.segs.size() - first), &b);
+    double bytes = 0;
+    for (int i = 0; i < b.nseg; i++) bytes += 2.0 * (double)b.seg[i].bytes;
+    prepare_copy_batch(&b, (int)c->copy_ctas);
+    out.push_back(make_launch(b, fn, c->copy_ctas, threads, bytes, b.nseg));
+  }
+  return out;
+}
+
+cudaError_t launch_kernel(const KernelLaunch& k, cudaStream_t stream) {
+  void* args[1] = {const_cast<char*>(k.args.data())};
+  return cudaLaunchKernel(k.fn, dim3((unsigned)k.grid), dim3((unsigned)k.threads), args, 0, stream);
+}
+
 // ------------------------------------------------------------------ stream executor -------------
 hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, cudaStream_t user, Tally* tally) {
   const int lanes = (int)std::max<long>(1, std::min<long>(c->lanes, kMaxLanes));
@@ -283,19 +436,8 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
     for (int d : rg.deps)
       if (where[d] != s) CU_TRY(c, cudaStreamWaitEvent(s, done[d], 0));
     // chain_dep needs no event here: every SUM is on the one sum stream
-    if (rg.kind == OP_CHAIN) {
-      for (size_t first = 0; first < rg.segs.size(); first += kMaxSegs) {
-        size_t n = std::min<size_t>(kMaxSegs, rg.segs.size() - first);
-        ChainBatch b;
-        fill_chain_batch(rg, first, n, P.dtype, P.elem, &b);
-        CU_TRY(c, launch_chain(b, (int)c->sum_ctas, s));
-        tally->sum_launches++;
-      }
-    } else if (rg.kind == OP_SUM) {
-      for (size_t first = 0; first < rg.segs.size(); first += kMaxSegs) {
-        size_t n = std::min<size_t>(kMaxSegs, rg.segs.size() - first);
-        SumBatch b;
-        fill_sum_batch(rg, first, n, P.dtype, P.elem, &b);
+    if (rg.kind != OP_MOVE) {
+      for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
         std::pair<cudaEvent_t, cudaEvent_t> pe{nullptr, nullptr};
         if (c->profile) {
           if (c->prof_pool.empty()) {
@@ -309,12 +451,10 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
           }
           CU_TRY(c, cudaEventRecord(pe.first, s));
         }
-        CU_TRY(c, launch_sum(b, (int)c->sum_ctas, s));
+        CU_TRY(c, launch_kernel(k, s));
         if (c->profile) {
           CU_TRY(c, cudaEventRecord(pe.second, s));
-          double bytes = 0;
-          for (size_t i = 0; i < n; i++) bytes += 3.0 * (double)rg.segs[first + i].bytes;
-          c->prof_open.push_back({pe, bytes});
+          c->prof_open.push_back({pe, k.bytes});
         }
         tally->sum_launches++;
       }
@@ -332,24 +472,10 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
         tally->moves++;
       }
     } else {
-      std::vector<FanBatch> fans;
-      std::vector<double> fan_bytes;
-      std::vector<long> fan_moves;
-      if (P.ag_direct && build_fan_batches(rg, &fans, &fan_bytes, &fan_moves)) {
-        for (size_t i = 0; i < fans.size(); i++) {
-          CU_TRY(c, launch_fan(fans[i], (int)c->copy_ctas, s));
-          tally->moves += fan_moves[i];
-          tally->move_launches++;
-        }
-      } else {
-        for (size_t first = 0; first < rg.segs.size(); first += kMaxSegs) {
-          size_t n = std::min<size_t>(kMaxSegs, rg.segs.size() - first);
-          CopyBatch b;
-          fill_copy_batch(rg, first, n, &b);
-          CU_TRY(c, launch_copy(b, (int)c->copy_ctas, s));
-          tally->moves += (long)n;
-          tally->move_launches++;
-        }
+      for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
+        CU_TRY(c, launch_kernel(k, s));
+        tally->moves += k.moves;
+        tally->move_launches++;
       }
     }
     cudaEvent_t ev = next_event(c);
@@ -683,6 +809,8 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   int max_pieces = (int)c->max_pieces;
   const bool reduction = call->kind == PLAN_ALLREDUCE || call->kind == PLAN_REDUCE_SCATTER;
   const size_t ring_chunk = (call->kind == PLAN_ALLREDUCE ? (call->count + c->R - 1) / c->R : call->count) * dtype_size(call->dtype);
+  const Contributions how = contributions(c, *call, opt, call->count * dtype_size(call->dtype));
+  const bool sum_only = how == READ_AND_STORE || (how == READ_IN_PLACE && call->kind == PLAN_REDUCE_SCATTER);   // no moves at all
   // Copy route with overlap ("ce_overlap"): the direct schedule cut into pieces whose three parts run on three internal
   // streams (see launch_entry).  Automatic (-1): 2 pieces from 2 MiB per ring chunk, from 4 MiB on pieces of about 4 MiB, at
   // least 4 and at most 32 of them; below that the ~30 us of host time per call and the extra copies cost more than the overlap
@@ -694,10 +822,22 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
     const size_t most = c->sum_ctas >= 64 ? 8 : 32;
     overlap_pieces = ring_chunk >= ((size_t)4 << 20) ? (long)std::min<size_t>(most, std::max<size_t>(4, ring_chunk >> 22))
                                                      : ring_chunk >= ((size_t)2 << 20) ? 2 : 0;
+    // With the contributions read in place only the all-gather's copies are left to hide behind the sums, so fewer and larger
+    // pieces are best, and below 4 MiB per chunk (8 MiB with whole-GPU sums) one graph is (R = 8, bf16, 8-CTA sums: 25 MiB per rank
+    // 0.221 ms whole and 0.221 in 2 pieces, 32 MiB 0.286 / 0.281, 40 MiB 0.364 / 0.344 and 0.348 in 4, 64 MiB 0.600 whole and 0.536 in
+    // 3, 128 MiB 1.058 in 6, 256 MiB 2.088 in 12, 2.138 in 24; 148-CTA sums: 16 MiB 0.056 / 0.076, 64 MiB 0.244 / 0.225, 0.262 in 6)
+    if (how == READ_IN_PLACE) {
+      if (c->sum_ctas >= 64) overlap_pieces = (long)std::min<size_t>(8, ring_chunk >> 22);
+      else overlap_pieces = ring_chunk >= ((size_t)5 << 20) ? (long)std::min<size_t>(32, std::max<size_t>(4, ring_chunk * 3 >> 23))
+                                                            : ring_chunk >= ((size_t)4 << 20) ? 2 : 0;
+    }
   }
   const bool overlap = overlap_pieces > 1 && c->path == HOCCL_PATH_CE && opt.executor == EXEC_GRAPH && !call->h_send &&
-                       (plan_kind & PLAN_FLAG_RS_DIRECT) && c->R > 1 && !c->piece_bytes_set;
-  if (overlap) {
+                       (plan_kind & PLAN_FLAG_RS_DIRECT) && c->R > 1 && !c->piece_bytes_set && !sum_only;
+  if (sum_only && !c->piece_bytes_set && !call->h_send) {   // nothing to overlap
+    piece_bytes = (size_t)1 << 60;
+    max_pieces = 1;
+  } else if (overlap) {
     max_pieces = (int)overlap_pieces;
     piece_bytes = std::max<size_t>((size_t)64 << 10, ((ring_chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
   } else if (!c->piece_bytes_set && c->path == HOCCL_PATH_SM && opt.executor == EXEC_GRAPH && !call->h_send && reduction &&
@@ -706,7 +846,12 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
     // software pipeline (see build_graph): a piece's copies run beside another piece's chain sum (measured, 8-CTA sums and
     // 40 copy CTAs: 40 MiB per rank 0.46 ms with 2 pieces, 0.41 with 4, 0.38 with 8, 0.45 with 10; 25 MiB 0.30 / 0.26 / 0.245 /
     // 0.29 ms with 2 / 4 / 5 / 7 pieces; 256 MiB 2.92 / 2.57 / 2.40 / 2.32 ms with 2 / 4 / 8 / 16 pieces)
-    piece_bytes = std::min<size_t>((size_t)2 << 20, std::max<size_t>((size_t)640 << 10, (ring_chunk / 8 + 1023) / 1024 * 1024));
+    // With the contributions read in place: a sixth of a chunk, between 1 and 3.25 MiB, from 4 MiB per chunk on (32 MiB per rank
+    // 0.271 ms, 40 MiB 0.329, 64 MiB 0.508, 128 MiB 1.010, 256 MiB 1.978; an eighth: 0.282 / 0.336 / 0.519 / 1.016 / 1.986).
+    if (how == READ_IN_PLACE && ring_chunk >= kGradeInPlace)
+      piece_bytes = std::min<size_t>((size_t)3328 << 10, std::max<size_t>((size_t)1 << 20, (ring_chunk / 6 + 1023) / 1024 * 1024));
+    else
+      piece_bytes = std::min<size_t>((size_t)2 << 20, std::max<size_t>((size_t)640 << 10, (ring_chunk / 8 + 1023) / 1024 * 1024));
     max_pieces = 64;
   } else if (call->h_send) {   // pipelined host all-reduce: host_pieces pieces per chunk, whatever the chunk size
     const size_t q = (call->count + c->R - 1) / c->R;
@@ -736,8 +881,10 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   // buckets: copy route 0.423 -> 0.444 ms, SM path 0.380 -> 0.431: the small outer pieces cost more in fixed time per piece than
   // their shorter fill saves), so automatic means: from 8 MiB per ring chunk, under a SUM budget (with whole-GPU sums the outer
   // pieces' moves are no longer what is exposed: 256 MiB per rank, copy route, 148-CTA sums 1.51 -> 1.53 ms)
+  // (with the contributions read in place the SM path gains from 4 MiB per ring chunk on: 40 MiB per rank in 5 pieces 0.340 -> 0.329)
+  const size_t grade_from = how == READ_IN_PLACE && c->path == HOCCL_PATH_SM ? kGradeInPlace : (size_t)8 << 20;
   const bool graded = reduction && !call->h_send && !fused && (plan_kind & PLAN_FLAG_RS_DIRECT) &&
-                      (c->piece_grade == 1 || (c->piece_grade < 0 && ring_chunk >= ((size_t)8 << 20) && c->sum_ctas < 64));
+                      (c->piece_grade == 1 || (c->piece_grade < 0 && ring_chunk >= grade_from && c->sum_ctas < 64));
   if (!build_plan(&P, plan_kind | (graded ? PLAN_FLAG_GRADED : 0), c->R, call->count, call->dtype, call->in_place, piece_bytes, max_pieces, align))
     return HOCCL_ERR_INVALID_ARG;
   if (P.slot_bytes) {
@@ -753,7 +900,7 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   c->stats.max_sum_ctas = 0;
   std::vector<RGroup> groups;
   size_t host_need = 0;
-  resolve(c, P, *call, &groups, &host_need);
+  resolve(c, P, *call, how, &groups, &host_need);
   if (c->path == HOCCL_PATH_CE_HOST && (!c->host_staging || host_need > c->host_staging_bytes)) return HOCCL_ERR_SCRATCH;
   if (graphs) {
     if (c->handshake) {

@@ -60,6 +60,17 @@ cudaError_t enqueue_host_copy(const HostCopy& hc, bool to_device, cudaStream_t s
   return cudaMemcpy2DAsync(dst, hc.pitch, src, hc.pitch, hc.width, hc.rows, kind, s);
 }
 
+// The parameters are copied into the node when it is added; `args` only has to live until then.
+static cudaKernelNodeParams node_params(const KernelLaunch& k, void** args) {
+  args[0] = const_cast<char*>(k.args.data());
+  cudaKernelNodeParams kp = {};
+  kp.func = const_cast<void*>(k.fn);
+  kp.gridDim = dim3((unsigned)k.grid);
+  kp.blockDim = dim3((unsigned)k.threads);
+  kp.kernelParams = args;
+  return kp;
+}
+
 // only_piece >= 0 builds the graph of that piece alone (dependencies never cross pieces) and stores it in *out_exec.
 hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry, int only_piece,
                            cudaGraphExec_t* out_exec, int part) {
@@ -153,6 +164,7 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
     if (rg.chain_dep >= 0 && std::find(rg.deps.begin(), rg.deps.end(), rg.chain_dep) == rg.deps.end())
       deps.insert(deps.end(), tail[rg.chain_dep].begin(), tail[rg.chain_dep].end());
     std::vector<cudaGraphNode_t> nodes;
+    void* args[1];
     cudaError_t e = cudaSuccess;
     if (deps.empty() && many_root_copies && rg.kind == OP_MOVE) {
       if (!root) {
@@ -171,30 +183,8 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
       deps.push_back(root);
     }
     if (rg.kind == OP_SUM || rg.kind == OP_CHAIN) {
-      for (size_t first = 0; first < rg.segs.size() && e == cudaSuccess; first += kMaxSegs) {
-        size_t n = std::min<size_t>(kMaxSegs, rg.segs.size() - first);
-        SumBatch b;
-        ChainBatch cb;
-        void* args[1];
-        cudaKernelNodeParams kp = {};
-        int sum_threads = 0;
-        double bytes = 0;
-        if (rg.kind == OP_SUM) {
-          fill_sum_batch(rg, first, n, P.dtype, P.elem, &b);
-          prepare_sum_batch(&b, (int)c->sum_ctas);
-          args[0] = &b;
-          kp.func = const_cast<void*>(sum_kernel_entry(P.dtype, (int)c->sum_ctas, &sum_threads));
-          for (size_t i = 0; i < n; i++) bytes += 3.0 * (double)rg.segs[first + i].bytes;
-        } else {
-          fill_chain_batch(rg, first, n, P.dtype, P.elem, &cb);
-          prepare_chain_batch(&cb, (int)c->sum_ctas);
-          args[0] = &cb;
-          kp.func = const_cast<void*>(chain_kernel_entry(cb, (int)c->sum_ctas, &sum_threads));
-          for (size_t i = 0; i < n; i++) bytes += (2.0 + (double)rg.segs[first + i].nsrc) * (double)rg.segs[first + i].bytes;
-        }
-        kp.gridDim = dim3((unsigned)c->sum_ctas);
-        kp.blockDim = dim3((unsigned)sum_threads);
-        kp.kernelParams = args;
+      for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
+        const cudaKernelNodeParams kp = node_params(k, args);
         // launches of one group are chained too (they share the SM budget)
         std::vector<cudaGraphNode_t> d2 = nodes.empty() ? deps : std::vector<cudaGraphNode_t>{nodes.back()};
         cudaGraphNode_t start_rec = nullptr;
@@ -203,7 +193,7 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
           if ((e = cudaEventCreate(&pe.first)) != cudaSuccess) break;
           if ((e = cudaEventCreate(&pe.second)) != cudaSuccess) break;
           entry->prof_events.push_back(pe);
-          entry->prof_bytes.push_back(bytes);
+          entry->prof_bytes.push_back(k.bytes);
           if ((e = cudaGraphAddEventRecordNode(&start_rec, g, d2.data(), d2.size(), pe.first)) != cudaSuccess) break;
           d2.assign(1, start_rec);
         }
@@ -256,62 +246,32 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
         entry->n_moves++;
       }
     } else {
-      // one kernel node per batch; `batch` is copied into the node when it is added
-      auto add_move_node = [&](void* batch, const void* func, int threads, double hbm_bytes, long n_moves) -> cudaError_t {
-        void* args[] = {batch};
-        cudaKernelNodeParams kp = {};
-        kp.func = const_cast<void*>(func);
-        kp.gridDim = dim3((unsigned)c->copy_ctas);
-        kp.blockDim = dim3((unsigned)threads);
-        kp.kernelParams = args;
+      for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
+        const cudaKernelNodeParams kp = node_params(k, args);
         // copy launches are chained as well: the CTA budget for copies is global, two never run at the same time
         std::vector<cudaGraphNode_t> d2 = deps;
         if (last_copy_node && std::find(d2.begin(), d2.end(), last_copy_node) == d2.end()) d2.push_back(last_copy_node);
         std::pair<cudaEvent_t, cudaEvent_t> pe{nullptr, nullptr};
-        cudaError_t err;
         if (c->profile) {
-          if ((err = cudaEventCreate(&pe.first)) != cudaSuccess) return err;
-          if ((err = cudaEventCreate(&pe.second)) != cudaSuccess) return err;
+          if ((e = cudaEventCreate(&pe.first)) != cudaSuccess) break;
+          if ((e = cudaEventCreate(&pe.second)) != cudaSuccess) break;
           entry->prof_events.push_back(pe);
-          entry->prof_bytes.push_back(-hbm_bytes);   // negative: a copy launch (reads + writes), kept apart from the sums
+          entry->prof_bytes.push_back(-k.bytes);   // negative: a copy launch (reads + writes), kept apart from the sums
           cudaGraphNode_t start_rec;
-          if ((err = cudaGraphAddEventRecordNode(&start_rec, g, d2.data(), d2.size(), pe.first)) != cudaSuccess) return err;
+          if ((e = cudaGraphAddEventRecordNode(&start_rec, g, d2.data(), d2.size(), pe.first)) != cudaSuccess) break;
           d2.assign(1, start_rec);
         }
         cudaGraphNode_t kn;
-        if ((err = cudaGraphAddKernelNode(&kn, g, d2.data(), d2.size(), &kp)) != cudaSuccess) return err;
+        if ((e = cudaGraphAddKernelNode(&kn, g, d2.data(), d2.size(), &kp)) != cudaSuccess) break;
         if (c->profile) {
           cudaGraphNode_t end_rec;
-          if ((err = cudaGraphAddEventRecordNode(&end_rec, g, &kn, 1, pe.second)) != cudaSuccess) return err;
+          if ((e = cudaGraphAddEventRecordNode(&end_rec, g, &kn, 1, pe.second)) != cudaSuccess) break;
           kn = end_rec;
         }
         last_copy_node = kn;
         nodes.push_back(kn);
-        entry->n_moves += n_moves;
+        entry->n_moves += k.moves;
         entry->n_move_launches++;
-        return cudaSuccess;
-      };
-      std::vector<FanBatch> fans;
-      std::vector<double> fan_bytes;
-      std::vector<long> fan_moves;
-      int move_threads = 0;
-      if (P.ag_direct && build_fan_batches(rg, &fans, &fan_bytes, &fan_moves)) {
-        const void* fn = fan_kernel_entry((int)c->copy_ctas, &move_threads);
-        for (size_t i = 0; i < fans.size() && e == cudaSuccess; i++) {
-          prepare_fan_batch(&fans[i], (int)c->copy_ctas);
-          e = add_move_node(&fans[i], fn, move_threads, fan_bytes[i], fan_moves[i]);
-        }
-      } else {
-        const void* fn = copy_kernel_entry((int)c->copy_ctas, &move_threads);
-        for (size_t first = 0; first < rg.segs.size() && e == cudaSuccess; first += kMaxSegs) {
-          size_t n = std::min<size_t>(kMaxSegs, rg.segs.size() - first);
-          CopyBatch b;
-          fill_copy_batch(rg, first, n, &b);
-          prepare_copy_batch(&b, (int)c->copy_ctas);
-          double bytes = 0;
-          for (size_t i = 0; i < n; i++) bytes += 2.0 * (double)rg.segs[first + i].bytes;
-          e = add_move_node(&b, fn, move_threads, bytes, (long)n);
-        }
       }
     }
     if (e != cudaSuccess) {

@@ -146,86 +146,88 @@ __global__ void __launch_bounds__(THREADS, 1) copy_kernel(const __grid_constant_
   }
 }
 
-// One element of a chain segment, element-wise: the same adds in the same order as the vector body.
+// One element of a chain segment, element-wise: the same adds in the same order as the vector bodies.
 template <int DT>
-__device__ __forceinline__ void chain_scalar(const ChainSeg& sg, unsigned long long i) {
+__device__ __forceinline__ void chain_scalar(const ChainBatch& b, const ChainSeg& sg, unsigned long long i) {
+  void* const* op = b.ptr + sg.first_ptr;
   if (DT == 0) {
-    float acc = static_cast<const float*>(sg.first)[i];
-    for (int q = 1; q < sg.nsrc; q++)
-      acc = __fadd_rn(acc, reinterpret_cast<const float*>(static_cast<const char*>(sg.first) + (size_t)q * sg.stride)[i]);
-    static_cast<float*>(sg.out)[i] = __fadd_rn(acc, static_cast<const float*>(sg.local)[i]);
+    float acc = static_cast<const float*>(op[0])[i];
+    for (int q = 1; q < sg.nops; q++) acc = __fadd_rn(acc, static_cast<const float*>(op[q])[i]);
+    for (int d = 0; d < sg.ndst; d++) static_cast<float*>(op[sg.nops + d])[i] = acc;
   } else {
-    unsigned short acc = static_cast<const unsigned short*>(sg.first)[i];
-    for (int q = 1; q <= sg.nsrc; q++) {
-      const unsigned short b = q < sg.nsrc ? reinterpret_cast<const unsigned short*>(static_cast<const char*>(sg.first) + (size_t)q * sg.stride)[i]
-                                           : static_cast<const unsigned short*>(sg.local)[i];
-      const float s2 = __fadd_rn(__uint_as_float((uint32_t)acc << 16), __uint_as_float((uint32_t)b << 16));
+    unsigned short acc = static_cast<const unsigned short*>(op[0])[i];
+    for (int q = 1; q < sg.nops; q++) {
+      const float s2 = __fadd_rn(__uint_as_float((uint32_t)acc << 16), __uint_as_float((uint32_t) static_cast<const unsigned short*>(op[q])[i] << 16));
       acc = __bfloat16_as_ushort(__float2bfloat16_rn(s2));
     }
-    static_cast<unsigned short*>(sg.out)[i] = acc;
+    for (int d = 0; d < sg.ndst; d++) static_cast<unsigned short*>(op[sg.nops + d])[i] = acc;
   }
 }
 
-// Chain sum of the direct reduce-scatter: per element nsrc inbox operands and the local one, added in the ring's order with a
-// rounding into the I/O dtype after every add.  One 16-byte vector per thread and tile; the operands are loaded in batches of
-// up to 8 before they are added, so up to 8 x 16 KiB are in flight per CTA.  Store bound under a CTA budget like every kernel
-// here, but it writes each output byte once instead of R-1 times, which is the point of the direct form.
-template <int DT, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant__ ChainBatch batch) {
+// Element-wise items of a launch: heads, tails and segments without a common 16-byte phase.
+template <int DT>
+__device__ __forceinline__ void chain_scalar_items(const ChainBatch& batch) {
   using T = Traits<DT>;
   const Flat& f = batch.flat;
-  const int nseg = batch.nseg;
+  const unsigned long long total = (unsigned long long)gridDim.x * blockDim.x;
+  const unsigned long long S = f.spre[batch.nseg];
+  int k = 0;
+  for (unsigned long long j = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; j < S; j += total) {
+    while (j >= f.spre[k + 1]) k++;
+    unsigned long long i = j - f.spre[k];
+    if (i >= f.head[k]) i += f.nvec[k] * T::VE;
+    chain_scalar<DT>(batch, batch.seg[k], i);
+  }
+}
+
+template <int DT>
+__device__ __forceinline__ uint4 chain_add(uint4 a, uint4 b) {
+  return DT == 1 ? add_vec_bf16_native(a, b) : Traits<DT>::add_vec(a, b);
+}
+
+template <class Batch>
+__device__ __forceinline__ void report_sm(const Batch& batch) {
   if (batch.smid_out != nullptr && threadIdx.x == 0) {
     unsigned id;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
     batch.smid_out[blockIdx.x] = id;
   }
-  const unsigned long long total = (unsigned long long)gridDim.x * blockDim.x;
-  const unsigned long long gt = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-  {
-    const unsigned long long T_all = f.tpre[nseg];
-    int k = 0;
-    for (unsigned long long t = blockIdx.x; t < T_all; t += gridDim.x) {
-      while (t >= f.tpre[k + 1]) k++;
-      const unsigned long long v = (t - f.tpre[k]) * blockDim.x + threadIdx.x;   // vector of segment k
-      if (v >= f.nvec[k]) continue;
-      const ChainSeg& sg = batch.seg[k];
-      const size_t off = (size_t)f.head[k] * T::E + (size_t)v * 16;
-      const char* src = static_cast<const char*>(sg.first) + off;
-      const int n_ops = sg.nsrc + 1;   // operand j < nsrc: inbox slot j; operand nsrc: the local contribution
-      uint4 acc;
-      for (int j0 = 0; j0 < n_ops; j0 += 8) {
-        uint4 buf[8];
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-          const int q = j0 + j;
-          if (q < sg.nsrc) buf[j] = __ldcs(reinterpret_cast<const uint4*>(src + (size_t)q * sg.stride));
-          else if (q == sg.nsrc) buf[j] = __ldcs(reinterpret_cast<const uint4*>(static_cast<const char*>(sg.local) + off));
-        }
-#pragma unroll
-        for (int j = 0; j < 8; j++) {
-          const int q = j0 + j;
-          if (q < n_ops) acc = (q == 0) ? buf[j] : (DT == 1 ? add_vec_bf16_native(acc, buf[j]) : T::add_vec(acc, buf[j]));
-        }
-      }
-      *reinterpret_cast<uint4*>(static_cast<char*>(sg.out) + off) = acc;
-    }
-  }
-  // element-wise items: heads, tails and segments without a common 16-byte phase
-  {
-    const unsigned long long S = f.spre[nseg];
-    int k = 0;
-    for (unsigned long long j = gt; j < S; j += total) {
-      while (j >= f.spre[k + 1]) k++;
-      unsigned long long i = j - f.spre[k];
-      if (i >= f.head[k]) i += f.nvec[k] * T::VE;
-      chain_scalar<DT>(batch.seg[k], i);
-    }
-  }
 }
 
-// Software-pipelined form of the chain sum for a compile-time operand count NOPS (inbox operands + the local one) that all
-// segments of the launch share.  Under a CTA budget the chain sum is bound by the bytes one SM keeps in flight: a load takes
+// Chain sum for any number of operands and destinations: one 16-byte vector per thread and tile; the operands are loaded in
+// batches of up to 8 before they are added, so up to 8 x 16 KiB are in flight per CTA.  Serves more than 8 operands (the forms
+// below are compiled for 2 to 8).
+template <int DT, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant__ ChainBatch batch) {
+  using T = Traits<DT>;
+  const Flat& f = batch.flat;
+  report_sm(batch);
+  const unsigned long long T_all = f.tpre[batch.nseg];
+  int k = 0;
+  for (unsigned long long t = blockIdx.x; t < T_all; t += gridDim.x) {
+    while (t >= f.tpre[k + 1]) k++;
+    const unsigned long long v = (t - f.tpre[k]) * blockDim.x + threadIdx.x;   // vector of segment k
+    if (v >= f.nvec[k]) continue;
+    const ChainSeg& sg = batch.seg[k];
+    void* const* op = batch.ptr + sg.first_ptr;
+    const size_t off = (size_t)f.head[k] * T::E + (size_t)v * 16;
+    uint4 acc;
+    for (int j0 = 0; j0 < sg.nops; j0 += 8) {
+      uint4 buf[8];
+#pragma unroll
+      for (int j = 0; j < 8; j++)
+        if (j0 + j < sg.nops) buf[j] = __ldcs(reinterpret_cast<const uint4*>(static_cast<const char*>(op[j0 + j]) + off));
+#pragma unroll
+      for (int j = 0; j < 8; j++)
+        if (j0 + j < sg.nops) acc = (j0 + j == 0) ? buf[j] : chain_add<DT>(acc, buf[j]);
+    }
+    for (int d = 0; d < sg.ndst; d++) *reinterpret_cast<uint4*>(static_cast<char*>(op[sg.nops + d]) + off) = acc;
+  }
+  chain_scalar_items<DT>(batch);
+}
+
+// Software-pipelined form of the chain sum for a compile-time operand count NOPS that all segments of the launch share, one
+// destination each.  Under a CTA budget the chain sum is bound by the bytes one SM keeps in flight: a load takes
 // the better part of a microsecond to come back, so a thread that loads a tile, adds it, stores it and only then loads the
 // next one leaves the memory port idle most of the time.  Here every thread keeps P tiles in registers: the loads of tile
 // t + P - 1 are issued before the adds and the store of tile t, so P - 1 to P tiles of NOPS x 16 bytes per thread are in
@@ -235,17 +237,14 @@ __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant
 // by segment, and inside a segment the full tiles run through a loop whose body has no branch: unconditional loads, adds,
 // store (measured: 163 GB/s per SM for 8 operands with P = 3 and 512 threads, against 111 for chain_kernel).  The ragged
 // last tile of a segment and ranges shorter than P tiles take a plain guarded path.  The order of the adds and their
-// rounding are those of chain_kernel (operand 0 first, the local contribution last).  Tiles are THREADS vectors.
+// rounding are those of chain_kernel.  Tiles are THREADS vectors.  The operand pointers are the same for all threads and a
+// thread's offset fits 32 bits (kMaxChainSegBytes), which keeps the NOPS + 1 addresses out of the per-thread registers.
 template <int DT, int NOPS, int P, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_pipe_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
   const Flat& f = batch.flat;
   const int nseg = batch.nseg;
-  if (batch.smid_out != nullptr && threadIdx.x == 0) {
-    unsigned id;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
-    batch.smid_out[blockIdx.x] = id;
-  }
+  report_sm(batch);
   {
     const unsigned long long T_all = f.tpre[nseg];
     // this CTA's share of the flattened tile space: [A, B)
@@ -254,31 +253,29 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe_kernel(const __grid_con
     int k = 0;
     while (k < nseg && f.tpre[k + 1] <= A) k++;
     for (; k < nseg && f.tpre[k] < B; k++) {
-      const unsigned long long a = (A > f.tpre[k] ? A : f.tpre[k]) - f.tpre[k];                 // tiles [a, b) of segment k
-      const unsigned long long b = (B < f.tpre[k + 1] ? B : f.tpre[k + 1]) - f.tpre[k];
-      const unsigned long long nvec = f.nvec[k];
-      const unsigned long long bf = b < nvec / THREADS ? b : nvec / THREADS;                    // full tiles end here
-      const ChainSeg& sg = batch.seg[k];
-      const size_t off0 = (size_t)f.head[k] * T::E + (size_t)threadIdx.x * 16;
-      const char* src = static_cast<const char*>(sg.first) + off0;
-      const char* loc = static_cast<const char*>(sg.local) + off0;
-      char* out = static_cast<char*>(sg.out) + off0;
-      const size_t stride = sg.stride;
-      uint4 buf[P][NOPS];
-      auto load = [&](uint4(&bb)[NOPS], unsigned long long t) {
-        const size_t o = (size_t)t * THREADS * 16;
+      const unsigned a = (unsigned)((A > f.tpre[k] ? A : f.tpre[k]) - f.tpre[k]);                 // tiles [a, b) of segment k
+      const unsigned b = (unsigned)((B < f.tpre[k + 1] ? B : f.tpre[k + 1]) - f.tpre[k]);
+      const unsigned nvec = (unsigned)f.nvec[k];
+      const unsigned bf = b < nvec / THREADS ? b : nvec / THREADS;                                // full tiles end here
+      const char* src[NOPS];
 #pragma unroll
-        for (int q = 0; q < NOPS - 1; q++) bb[q] = __ldcs(reinterpret_cast<const uint4*>(src + (size_t)q * stride + o));
-        bb[NOPS - 1] = __ldcs(reinterpret_cast<const uint4*>(loc + o));
+      for (int q = 0; q < NOPS; q++) src[q] = static_cast<const char*>(batch.ptr[batch.seg[k].first_ptr + q]);
+      char* out = static_cast<char*>(batch.ptr[batch.seg[k].first_ptr + NOPS]);
+      const unsigned off0 = f.head[k] * T::E + threadIdx.x * 16;
+      uint4 buf[P][NOPS];
+      auto load = [&](uint4(&bb)[NOPS], unsigned t) {
+        const unsigned o = off0 + t * (THREADS * 16);
+#pragma unroll
+        for (int q = 0; q < NOPS; q++) bb[q] = __ldcs(reinterpret_cast<const uint4*>(src[q] + o));
       };
-      auto finish = [&](const uint4(&bb)[NOPS], unsigned long long t) {
+      auto finish = [&](const uint4(&bb)[NOPS], unsigned t) {
         uint4 acc = bb[0];
 #pragma unroll
-        for (int q = 1; q < NOPS; q++) acc = DT == 1 ? add_vec_bf16_native(acc, bb[q]) : T::add_vec(acc, bb[q]);
-        *reinterpret_cast<uint4*>(out + (size_t)t * THREADS * 16) = acc;
+        for (int q = 1; q < NOPS; q++) acc = chain_add<DT>(acc, bb[q]);
+        *reinterpret_cast<uint4*>(out + (off0 + t * (THREADS * 16))) = acc;
       };
-      unsigned long long i = a;
-      if (bf > a && bf - a >= (unsigned long long)P) {
+      unsigned i = a;
+      if (bf > a && bf - a >= (unsigned)P) {
 #pragma unroll
         for (int p = 0; p < P - 1; p++) load(buf[p], i + p);
         for (; i + 2 * P - 1 <= bf; i += P) {   // steady state: no branch between a tile's loads and the adds of an older tile
@@ -302,18 +299,51 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe_kernel(const __grid_con
       }
     }
   }
-  // element-wise items: heads, tails and segments without a common 16-byte phase (as in chain_kernel)
-  {
-    const unsigned long long total = (unsigned long long)gridDim.x * blockDim.x;
-    const unsigned long long S = f.spre[nseg];
-    int k = 0;
-    for (unsigned long long j = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; j < S; j += total) {
-      while (j >= f.spre[k + 1]) k++;
-      unsigned long long i = j - f.spre[k];
-      if (i >= f.head[k]) i += f.nvec[k] * T::VE;
-      chain_scalar<DT>(batch.seg[k], i);
+  chain_scalar_items<DT>(batch);
+}
+
+// The sum that carries the all-gather too: NOPS operands are read once, the result is stored to NOPS destinations (one per
+// rank).  NOPS reads and NOPS writes per element are what the collective cannot do without; bound by HBM with a whole-GPU grid.
+// A tile is U x THREADS vectors, so U x NOPS loads are in flight per thread before the first add.
+template <int DT, int NOPS, int U, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_constant__ ChainBatch batch) {
+  using T = Traits<DT>;
+  const Flat& f = batch.flat;
+  report_sm(batch);
+  const unsigned long long T_all = f.tpre[batch.nseg];
+  int k = 0;
+  for (unsigned long long t = blockIdx.x; t < T_all; t += gridDim.x) {
+    while (t >= f.tpre[k + 1]) k++;
+    void* const* ptr = batch.ptr + batch.seg[k].first_ptr;
+    const unsigned v0 = (unsigned)(t - f.tpre[k]) * (U * THREADS) + threadIdx.x;   // first vector of this thread in segment k
+    const unsigned off = f.head[k] * T::E + v0 * 16;
+    const unsigned nvec = (unsigned)f.nvec[k];
+    auto finish = [&](const uint4(&bb)[NOPS], int u) {
+      uint4 acc = bb[0];
+#pragma unroll
+      for (int q = 1; q < NOPS; q++) acc = chain_add<DT>(acc, bb[q]);
+#pragma unroll
+      for (int d = 0; d < NOPS; d++) *reinterpret_cast<uint4*>(static_cast<char*>(ptr[NOPS + d]) + (off + u * (THREADS * 16))) = acc;
+    };
+    uint4 buf[U][NOPS];
+    if (v0 + (U - 1) * THREADS < nvec) {
+#pragma unroll
+      for (int u = 0; u < U; u++)
+#pragma unroll
+        for (int q = 0; q < NOPS; q++) buf[u][q] = __ldcs(reinterpret_cast<const uint4*>(static_cast<const char*>(ptr[q]) + (off + u * (THREADS * 16))));
+#pragma unroll
+      for (int u = 0; u < U; u++) finish(buf[u], u);
+    } else {
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        if (v0 + u * THREADS >= nvec) break;
+#pragma unroll
+        for (int q = 0; q < NOPS; q++) buf[u][q] = __ldcs(reinterpret_cast<const uint4*>(static_cast<const char*>(ptr[q]) + (off + u * (THREADS * 16))));
+        finish(buf[u], u);
+      }
     }
   }
+  chain_scalar_items<DT>(batch);
 }
 
 // Fan-out copy: the tile walk of copy_kernel, but a tile that was loaded once is stored to every destination of its segment.
@@ -589,8 +619,8 @@ void prepare_copy_batch(CopyBatch* b, int ctas) {
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
 }
 
-// Which chain kernel serves a batch.  The software-pipelined form needs one operand count for the whole launch (the usual
-// case: every rank's chain has R - 1 inbox operands and the local one) and is compiled for 2 to 8 operands.  Measured on
+// Which chain kernel serves a batch.  The compiled forms need one operand count for the whole launch (the usual case: R) from
+// 2 to 8, and one destination (chain_pipe_kernel) or as many as operands (chain_fan_kernel).  Measured on
 // B200 (8 operands, 25 MiB each, bf16): 163 against 111 GB/s per SM with 8 CTAs, 158 / 107 with 16, 138 / 99 with 32,
 // 113 / 89 with 48, 88 / 80 with 64, 59 / 58 with 96; with 148 CTAs both are HBM bound (5.7 TB/s).  Variants with the same
 // or more bytes in flight (P = 2 with 640 threads, P = 4 with 384, P = 4 and 6 with 256) end at the same 159-163 GB/s per
@@ -598,42 +628,78 @@ void prepare_copy_batch(CopyBatch* b, int ctas) {
 struct ChainVariant {
   const void* fn;
   int threads;
+  int tile;      // vectors of a tile
 };
+template <int DT, int NOPS, int P, int THREADS>
+static ChainVariant pipe_of() {
+  return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, NOPS, P, THREADS>), THREADS, THREADS};
+}
+template <int DT, int NOPS, int U, int THREADS>
+static ChainVariant fan_of() {
+  return {reinterpret_cast<const void*>(&chain_fan_kernel<DT, NOPS, U, THREADS>), THREADS, U * THREADS};
+}
 template <int DT>
 static ChainVariant chain_pipe_variant(int nops) {
   // P x NOPS vectors per thread: 16 to 24, i.e. 128 to 192 KiB per SM with 512 threads
   switch (nops) {
-    case 2: return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, 2, 8, 512>), 512};
-    case 3: return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, 3, 6, 512>), 512};
-    case 4: return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, 4, 5, 512>), 512};
-    case 5: return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, 5, 4, 512>), 512};
-    case 6: return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, 6, 3, 512>), 512};
-    case 7: return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, 7, 3, 512>), 512};
-    case 8: return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, 8, 3, 512>), 512};
-    default: return {nullptr, 0};
+    case 2: return pipe_of<DT, 2, 8, 512>();
+    case 3: return pipe_of<DT, 3, 6, 512>();
+    case 4: return pipe_of<DT, 4, 5, 512>();
+    case 5: return pipe_of<DT, 5, 4, 512>();
+    case 6: return pipe_of<DT, 6, 3, 512>();
+    case 7: return pipe_of<DT, 7, 3, 512>();
+    case 8: return pipe_of<DT, 8, 3, 512>();
+    default: return {nullptr, 0, 0};
+  }
+}
+template <int DT>
+static ChainVariant chain_fan_variant(int nops) {
+  // U x NOPS loads per thread: 8 to 16
+  switch (nops) {
+    case 2: return fan_of<DT, 2, 4, 512>();
+    case 3: return fan_of<DT, 3, 4, 512>();
+    case 4: return fan_of<DT, 4, 2, 512>();
+    case 5: return fan_of<DT, 5, 2, 512>();
+    case 6: return fan_of<DT, 6, 2, 512>();
+    case 7: return fan_of<DT, 7, 2, 512>();
+    case 8: return fan_of<DT, 8, 2, 512>();
+    default: return {nullptr, 0, 0};
   }
 }
 static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
-  ChainVariant plain{b.dtype == 0 ? reinterpret_cast<const void*>(&chain_kernel<0, 1024>) : reinterpret_cast<const void*>(&chain_kernel<1, 1024>), 1024};
-  if (ctas >= 128 || b.nseg <= 0) return plain;
-  const int nops = b.seg[0].nsrc + 1;
+  ChainVariant plain{b.dtype == 0 ? reinterpret_cast<const void*>(&chain_kernel<0, 1024>) : reinterpret_cast<const void*>(&chain_kernel<1, 1024>), 1024, 1024};
+  if (b.nseg <= 0) return plain;
+  const int nops = b.seg[0].nops, ndst = b.seg[0].ndst;
   for (int k = 1; k < b.nseg; k++)
-    if (b.seg[k].nsrc + 1 != nops) return plain;
-  ChainVariant pv = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
-  return pv.fn ? pv : plain;
+    if (b.seg[k].nops != nops || b.seg[k].ndst != ndst) return plain;
+  ChainVariant v = plain;
+  if (ndst == 1 && ctas < 128) v = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
+  else if (ndst == nops) v = b.dtype == 0 ? chain_fan_variant<0>(nops) : chain_fan_variant<1>(nops);
+  return v.fn ? v : plain;
 }
 
 void prepare_chain_batch(ChainBatch* b, int ctas) {
   const int E = b->dtype == 0 ? 4 : 2, VE = 16 / E;
-  const unsigned long long tile_v = (unsigned long long)chain_variant(*b, ctas).threads;   // one vector per thread and tile
+  const unsigned long long tile_v = (unsigned long long)chain_variant(*b, ctas).tile;
   unsigned head[kMaxSegs];
   unsigned long long nvec[kMaxSegs], nscalar[kMaxSegs];
   for (int k = 0; k < b->nseg; k++) {
     const ChainSeg& s = b->seg[k];
-    const unsigned ma = (unsigned)((uintptr_t)s.first & 15), mb = (unsigned)((uintptr_t)s.local & 15), mo = (unsigned)((uintptr_t)s.out & 15);
-    split_segment(s.n, ma, ma == mb && mb == mo && (s.stride & 15) == 0, E, VE, &head[k], &nvec[k], &nscalar[k]);
+    const unsigned phase = (unsigned)((uintptr_t)b->ptr[s.first_ptr] & 15);
+    bool same = true;
+    for (int q = 1; q < s.nops + s.ndst; q++) same = same && ((unsigned)((uintptr_t)b->ptr[s.first_ptr + q] & 15) == phase);
+    split_segment(s.n, phase, same, E, VE, &head[k], &nvec[k], &nscalar[k]);
   }
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
+}
+
+bool add_chain_seg(ChainBatch* b, const void* const* ops, int nops, void* const* dsts, int ndst, unsigned long long n) {
+  if (b->nseg == kMaxSegs || b->nptr + nops + ndst > kMaxChainPtrs) return false;
+  ChainSeg& s = b->seg[b->nseg++];
+  s = ChainSeg{n, b->nptr, nops, ndst, 0};
+  for (int q = 0; q < nops; q++) b->ptr[b->nptr++] = const_cast<void*>(ops[q]);
+  for (int d = 0; d < ndst; d++) b->ptr[b->nptr++] = dsts[d];
+  return true;
 }
 
 cudaError_t launch_chain(const ChainBatch& batch, int ctas, cudaStream_t stream) {
@@ -752,7 +818,7 @@ cudaError_t preload_kernels() {
     if (e != cudaSuccess) return e;
   }
   for (int nops = 2; nops <= 8; nops++)
-    for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn}) {
+    for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn, chain_fan_variant<0>(nops).fn, chain_fan_variant<1>(nops).fn}) {
       cudaFuncAttributes a;
       cudaError_t e = cudaFuncGetAttributes(&a, f);
       if (e != cudaSuccess) return e;

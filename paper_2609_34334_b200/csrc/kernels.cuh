@@ -35,23 +35,25 @@ struct SumBatch {
   unsigned int* smid_out = nullptr;  // diagnostics: if set, CTA b stores the id of the SM it runs on to smid_out[b]
 };
 
-// One chain segment (direct reduce-scatter): out[i] = (((s_0[i] + s_1[i]) + ...) + s_{nsrc-1}[i]) + local[i], every add one
-// binary32 add rounded into the I/O dtype: the ring's order and rounding for one chunk, done by its owner in one pass.
-// s_j = first + j * stride bytes: the owner's inbox slots, filled by the R-1 direct moves.
+// One chain segment (direct reduce-scatter): out[i] = (((s_0[i] + s_1[i]) + ...) + s_{nops-1}[i]), every add one binary32 add
+// rounded into the I/O dtype: the ring's order and rounding for one chunk in one pass (the last operand is the owner's own
+// contribution).  The result is stored to `ndst` places: one (the owner's buffer) or, when the sum carries the all-gather too,
+// every rank's buffer.  The pointers sit in the batch's pool: operands ptr[first_ptr + q], q < nops, then the ndst destinations.
 struct ChainSeg {
-  const void* first;
-  const void* local;
-  void* out;
-  unsigned long long n;       // elements
-  unsigned long long stride;  // bytes, a multiple of 16
-  int nsrc;                   // 1..kMaxChainSrcs
+  unsigned long long n;       // elements; at most kMaxChainSegBytes, so that the kernels can use 32-bit offsets
+  int first_ptr, nops, ndst;  // nops 2..64, ndst 1..64
   int pad;
 };
-constexpr int kMaxChainSrcs = 63;
+constexpr int kMaxChainSrcs = 63;     // inbox operands of hoccl_chain_launch
+constexpr int kMaxChainPtrs = 512;
+constexpr unsigned long long kMaxChainSegBytes = 1ull << 30;
 struct ChainBatch {
   int nseg;
   int dtype;
+  int nptr;
+  int pad;
   ChainSeg seg[kMaxSegs];
+  void* ptr[kMaxChainPtrs];
   Flat flat;  // filled by prepare_chain_batch (launch_chain does it itself)
   unsigned int* smid_out = nullptr;
 };
@@ -154,6 +156,8 @@ cudaError_t launch_sum(const SumBatch& batch, int ctas, cudaStream_t stream);
 cudaError_t launch_copy(const CopyBatch& batch, int ctas, cudaStream_t stream);
 cudaError_t launch_chain(const ChainBatch& batch, int ctas, cudaStream_t stream);
 void prepare_chain_batch(ChainBatch* batch, int ctas);
+// Appends a segment (operands in the order they are added); false if the batch has no room for it.
+bool add_chain_seg(ChainBatch* batch, const void* const* ops, int nops, void* const* dsts, int ndst, unsigned long long n);
 // kernel and thread count that serve `batch` with `ctas` CTAs (the batch must have been prepared for the same `ctas`)
 const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads);
 // counts: two device words, zeroed by the caller; see bf16_add_selftest_kernel

@@ -187,6 +187,14 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                "fused" nor "onepass" is set (it was measured faster than the ring at every size and on every path), the ring
  *                otherwise.  So a communicator with hoccl_scratch_bytes of scratch runs the ring, one with
  *                hoccl_scratch_bytes_direct runs the direct form; the bits are the same.
+ *                The automatic direct form makes use of all ranks living in one memory: when the send buffers share their address
+ *                modulo 16 the chain sum reads the other ranks' contributions where they lie and the R (R-1) moves into the
+ *                inbox slots fall away (S (R+1) instead of 2 S (R-1) + S (R+1) bytes); an all-reduce on the route of HOCCL_PATH_SM
+ *                that is short (R * S up to 384 KiB per SUM CTA) or has 128 or more SUM CTAs stores the result for every rank from
+ *                the same kernel (2 S R bytes in all, one launch, no moves).  hoccl_last_stats counts the moves that remain.
+ *                "rs_direct" = 1 keeps the rank-local form, as do HOCCL_PATH_CE_HOST, "roles" and hoccl_host_allreduce.  Measured
+ *                on B200 (R = 8, bf16, default settings): 25 MiB reduce-scatter + all-gather 0.291 -> 0.226 ms, 40 MiB all-reduce
+ *                0.417 -> 0.348 ms; HOCCL_PATH_SM with 148 + 148 CTAs, 64 MiB fp32 0.355 -> 0.183 ms.
  *  "ce_small_bytes" on HOCCL_PATH_CE a call whose per-rank message (S in the convention of each collective: all-reduce
  *                count, reduce-scatter / all-gather / all-to-all R * count elements) is at most this many bytes issues its
  *                moves as batched launches of the SM copy kernel with "ce_small_ctas" CTAs instead of driver copies, i.e.
@@ -201,7 +209,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                run on three internal streams, ordered by events, so that one piece's driver copies run beside another
  *                piece's sum (inside ONE graph, and on plain streams, they were never seen to overlap).  Sums still run one
  *                at a time.  Costs ~8 us of host time per piece and call.  -1 (default) = automatic: 2 pieces from 2 MiB per
- *                ring chunk, from 4 MiB on pieces of about 4 MiB (at least 4, at most 32 of them), off below; 0 = off;
+ *                ring chunk, from 4 MiB per ring chunk on pieces of about 4 MiB (at least 4, at most 32 of them), off below; with contributions read
+ *                in place ("rs_direct" = 2) 2 pieces from 4 MiB, from 5 MiB on pieces of about 2.7 MiB (4 to 32); 0 = off;
  *                2..64 = that many pieces.  Ignored when "piece_bytes" is set.
  *  "ce_small_ctas" CTAs of those launches, 1..1024 (default 148: like the driver's own copies they may use the whole GPU,
  *                for tens of microseconds)
@@ -241,7 +250,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *  "piece_grade" all-reduce and reduce-scatter on the stage-decomposed schedule: 1 = the pieces of a ring chunk are graded, the
  *                first and the last ones smaller (a third, two thirds of a middle piece; pieces of 256 KiB or more only), so that
  *                less of the moves in front of the first sum and behind the last one is exposed; 0 = equal pieces; -1 (default)
- *                = automatic: graded from 8 MiB per ring chunk on under a SUM budget (sum_ctas < 64), where it was measured to
+ *                = automatic: graded from 8 MiB per ring chunk on (4 MiB on HOCCL_PATH_SM with contributions read in place) under a
+ *                SUM budget (sum_ctas < 64), where it was measured to
  *                gain 1-5 %, equal otherwise (below that size the small outer pieces cost more than they save).  Same
  *                operations, same bits.
  *  "host_pieces" pieces per ring chunk of the pipelined hoccl_host_allreduce (1..64, default 8; 1 = not pipelined)

@@ -1,5 +1,6 @@
-"""Thin ctypes binding of libhoccl.so: same names as include/hoccl.h, argument marshalling only (the diagnostics of
-include/hoccl_diag.h are bound in diag.py).
+"""Thin binding of libhoccl.so: same names as include/hoccl.h, argument marshalling only (the diagnostics of
+include/hoccl_diag.h are bound in diag.py).  The calls of a program's inner loop (collectives, send/recv) are marshalled in C
+(csrc/calls.c), everything else with ctypes; both use the one library that lib() loads.
 
 Buffers are given as objects with a `data_ptr()` method (torch tensors) or as integer device
 addresses; streams as `torch.cuda.Stream`, raw integer handles or None (the current torch stream).
@@ -62,6 +63,7 @@ class HocclError(RuntimeError):
 
 
 _lib = None
+_calls = None   # the module built from csrc/calls.c
 
 
 def library_path() -> str:
@@ -71,7 +73,7 @@ def library_path() -> str:
 
 def lib() -> ctypes.CDLL:
     """Builds (if stale) and loads libhoccl.so.  Raises if that is not possible."""
-    global _lib
+    global _lib, _calls
     if _lib is not None:
         return _lib
     path = _build.build()
@@ -121,8 +123,15 @@ def lib() -> ctypes.CDLL:
         fn = getattr(L, name)
         fn.restype = res
         fn.argtypes = args
-    _lib = L
+    from . import _calls as calls
+
+    calls.bind(*[ctypes.cast(getattr(L, "hoccl_" + name), vp).value for name in _INNER_LOOP])
+    _lib, _calls = L, calls
     return L
+
+
+# functions called through csrc/calls.c, in the order its bind() takes them
+_INNER_LOOP = ["allreduce", "reduce_scatter", "host_allreduce", "allgather", "alltoall", "alltoallv", "send", "recv", "allreduce_static"]
 
 
 def error_string(code: int) -> str:
@@ -228,25 +237,22 @@ class Comm:
 
     # -- collectives (raise on error; the *_rc variants return the code)
     def allreduce_rc(self, send, recv, count, dtype, stream=None, op=SUM) -> int:
-        return lib().hoccl_allreduce(_ptr_array(send), _ptr_array(recv), count, _dtype(dtype), op, self._h, _stream(stream))
+        return _calls.allreduce(self._h.value, send, recv, count, dtype, op, stream)
 
     def reduce_scatter_rc(self, send, recv, count, dtype, stream=None, op=SUM) -> int:
-        return lib().hoccl_reduce_scatter(_ptr_array(send), _ptr_array(recv), count, _dtype(dtype), op, self._h, _stream(stream))
+        return _calls.reduce_scatter(self._h.value, send, recv, count, dtype, op, stream)
 
     def allgather_rc(self, send, recv, count, dtype, stream=None) -> int:
-        return lib().hoccl_allgather(_ptr_array(send), _ptr_array(recv), count, _dtype(dtype), self._h, _stream(stream))
+        return _calls.allgather(self._h.value, send, recv, count, dtype, stream)
 
     def alltoall_rc(self, send, recv, count, dtype, stream=None) -> int:
-        return lib().hoccl_alltoall(_ptr_array(send), _ptr_array(recv), count, _dtype(dtype), self._h, _stream(stream))
+        return _calls.alltoall(self._h.value, send, recv, count, dtype, stream)
 
     def alltoall(self, send, recv, count, dtype, stream=None):
         self._check(self.alltoall_rc(send, recv, count, dtype, stream), "hoccl_alltoall")
 
     def alltoallv_rc(self, send, sendcounts, sdispls, recv, rdispls, dtype, stream=None) -> int:
-        R = self.R
-        arr = lambda xs: (ctypes.c_size_t * (R * R))(*[int(x) for x in xs])
-        return lib().hoccl_alltoallv(_ptr_array(send), arr(sendcounts), arr(sdispls), _ptr_array(recv), arr(rdispls), _dtype(dtype),
-                                     self._h, _stream(stream))
+        return _calls.alltoallv(self._h.value, self.R, send, sendcounts, sdispls, recv, rdispls, dtype, stream)
 
     def alltoallv(self, send, sendcounts, sdispls, recv, rdispls, dtype, stream=None):
         self._check(self.alltoallv_rc(send, sendcounts, sdispls, recv, rdispls, dtype, stream), "hoccl_alltoallv")
@@ -261,15 +267,14 @@ class Comm:
         self._check(self.allgather_rc(send, recv, count, dtype, stream), "hoccl_allgather")
 
     def host_allreduce(self, h_send, h_recv, count, dtype, stream=None, op=SUM):
-        self._check(lib().hoccl_host_allreduce(_ptr_array(h_send), _ptr_array(h_recv), count, _dtype(dtype), op, self._h,
-                                               _stream(stream)), "hoccl_host_allreduce")
+        self._check(_calls.host_allreduce(self._h.value, h_send, h_recv, count, dtype, op, stream), "hoccl_host_allreduce")
 
     # -- point to point
     def send_rc(self, buf, count, dtype, src, dst, stream=None) -> int:
-        return lib().hoccl_send(_ptr(buf), count, _dtype(dtype), src, dst, self._h, _stream(stream))
+        return _calls.send(self._h.value, buf, count, dtype, src, dst, stream)
 
     def recv_rc(self, buf, count, dtype, src, dst, stream=None) -> int:
-        return lib().hoccl_recv(_ptr(buf), count, _dtype(dtype), src, dst, self._h, _stream(stream))
+        return _calls.recv(self._h.value, buf, count, dtype, src, dst, stream)
 
     def send(self, buf, count, dtype, src, dst, stream=None):
         self._check(self.send_rc(buf, count, dtype, src, dst, stream), "hoccl_send")
@@ -307,7 +312,8 @@ STATIC_SCRATCH_BYTES = 32 << 20
 def allreduce_static(send, recv, count, dtype, R, stream=None, op=SUM) -> int:
     """hoccl_allreduce_static: all-reduce that allocates nothing and uses the library's fixed scratch array.
     Returns the result code (OK, or ERR_SCRATCH when the buffers are too large for the fixed array)."""
-    return lib().hoccl_allreduce_static(_ptr_array(send), _ptr_array(recv), count, _dtype(dtype), op, R, _stream(stream))
+    lib()
+    return _calls.allreduce_static(send, recv, count, dtype, op, R, stream)
 
 
 def scratch_bytes(R: int, max_count: int, dtype) -> int:

@@ -1,13 +1,16 @@
-"""Builds libhoccl.so (sm_100a) in-tree from csrc/ with nvcc.  No JIT cache: the .so sits next to this file."""
+"""Builds libhoccl.so (sm_100a, nvcc) and the Python call entry points _calls.so (gcc) in-tree from csrc/.  No JIT cache: both sit
+next to this file."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhoccl.so")
+CALLS, CALLS_SOURCE = os.path.join(HERE, "_calls.so"), os.path.join(CSRC, "calls.c")
 SOURCES = ["api.cu", "exec.cu", "p2p.cu", "kernels.cu", "plan.cpp", "static_scratch.cu", "proxy.cu", "sched.cpp", "probe.cu", "ring.cu", "graph.cu", "ring_host.cu", "options.cpp", "roles.cu"]
 HEADERS = ["comm.h", "kernels.cuh", "device_common.cuh", "plan.h", "proxy.h", "sched.h", "options.h", os.path.join("..", "..", "include", "hoccl.h"), os.path.join("..", "..", "include", "hoccl_diag.h")]
 NVCC_FLAGS = [
@@ -23,16 +26,33 @@ def _nvcc() -> str:
     return "nvcc"
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB):
+def _older(target: str, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [os.path.abspath(__file__)]
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def is_stale() -> bool:
+    return _older(LIB, [os.path.join(CSRC, s) for s in SOURCES + HEADERS] + [os.path.abspath(__file__)])
+
+
+def build_calls(force: bool = False) -> str:
+    """The CPython module that marshals the arguments of the inner-loop calls (csrc/calls.c)."""
+    if force or _older(CALLS, [CALLS_SOURCE, os.path.abspath(__file__)]):
+        tmp = CALLS + ".tmp.%d" % os.getpid()
+        cmd = [os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I" + sysconfig.get_paths()["include"], CALLS_SOURCE, "-o", tmp]
+        res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        if res.returncode != 0:
+            sys.stderr.write(res.stdout)
+            raise RuntimeError("gcc failed building _calls.so")
+        os.replace(tmp, CALLS)
+    return CALLS
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile if the library is missing or older than its sources.  Returns the library path."""
+    """Compile whatever is missing or older than its sources.  Returns the path of the library."""
+    build_calls(force)
     if not force and not is_stale():
         return LIB
     tmp = LIB + ".tmp.%d" % os.getpid()

@@ -204,6 +204,11 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                4 KiB 34 -> 10 us, 1 MiB 48 -> 25 us, 4 MiB 88 -> 54 us, 8 MiB 107 -> 97 us, equal from 16 MiB on; R = 4 fp32
  *                all-reduce of 4 MiB 37 -> 33 us.  Default 8 MiB; 0 = driver copies at every size.  "HOCCL_PATH_CE" therefore
  *                means: the copy route above this size.  Not applied to hoccl_host_allreduce, send/recv or hoccl_alltoallv.
+ *                Unless it is 0, copies the driver does badly do not go to it at any size (it takes 4 us more for a copy of 1 MiB or
+ *                more that does not start on a 128-byte line and end after whole 4 KiB, and runs at half rate or less when the two
+ *                ends differ modulo 4): an all-gather or all-to-all of such blocks runs on the copy kernel like a small one, and an
+ *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of its all-gather's copies to one
+ *                launch of the copy kernel ("copy_ctas" CTAs) per piece.
  *  "ce_overlap"  HOCCL_PATH_CE, direct reduce-scatter: the ring chunks are cut into this many pieces and every piece's three
  *                parts (the reduce-scatter's moves, the chain sum, the all-gather's moves) become graphs of their own that
  *                run on three internal streams, ordered by events, so that one piece's driver copies run beside another

@@ -52,6 +52,7 @@ struct RGroup {
   std::vector<Seg> segs;
   std::vector<int> deps;
   int chain_dep;
+  bool edges = false;   // copy route: the ends of driver copies, carried by a copy-kernel launch (see trim_driver_copies)
 };
 
 struct Post {

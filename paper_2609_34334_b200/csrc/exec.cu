@@ -11,6 +11,7 @@
 //   * stream executor: internal move lanes plus one sum stream, ordered with CUDA events
 //     (fork from the caller's stream, join back into it).
 // SUM launches are chained (one at a time) so that the SM budget for sums is global, not per piece.
+#include <climits>
 #include <tuple>
 
 #include "comm.h"
@@ -113,6 +114,45 @@ static Contributions contributions(const hoccl_comm* c, const Call& call, const 
   return READ_IN_PLACE;
 }
 
+// What a driver copy inside one device does at once, as timed on B200: a copy of 1 MiB or more whose destination does not start on a
+// 128-byte line or whose length is not a multiple of 4 KiB takes 4 us more than a whole one (8 MiB 8.3 against 4.3 us, 64 MiB 28.7
+// against 24.6), one whose ends differ modulo 4 runs at half the rate.
+constexpr size_t kDriverLine = 128, kDriverPage = 4096, kDriverWhole = 1 << 20;
+
+// Copy route, contributions read in place: the all-gather's copies keep what the driver does at once and their ends (less than 128 bytes
+// in front, less than 4 KiB behind) go to one launch of the copy kernel per piece, "copy_ctas" CTAs, instead of a second pass per copy.
+static void trim_driver_copies(std::vector<RGroup>* groups) {
+  const size_t n = groups->size();
+  for (size_t g = 0; g < n; g++) {
+    if ((*groups)[g].kind != OP_MOVE) continue;
+    RGroup ends = (*groups)[g];
+    ends.segs.clear();
+    ends.edges = true;
+    for (Seg& s : (*groups)[g].segs) {
+      if (s.bytes < kDriverWhole) continue;
+      const uint64_t head = (kDriverLine - (uintptr_t)s.dst % kDriverLine) % kDriverLine;
+      const uint64_t body = (s.bytes - head) / kDriverPage * kDriverPage, tail = s.bytes - head - body;
+      if (head == 0 && tail == 0) continue;
+      Seg e = s;
+      e.bytes = head;
+      if (head) ends.segs.push_back(e);
+      e.src += head + body;
+      e.dst += head + body;
+      e.bytes = tail;
+      if (tail) ends.segs.push_back(e);
+      s.src += head;
+      s.dst += head;
+      s.bytes = body;
+    }
+    if (ends.segs.empty()) continue;
+    // the ends of a piece's stages wait for the same sum: one group
+    if (groups->size() > n && groups->back().piece == ends.piece && groups->back().deps == ends.deps)
+      groups->back().segs.insert(groups->back().segs.end(), ends.segs.begin(), ends.segs.end());
+    else
+      groups->push_back(std::move(ends));
+  }
+}
+
 // Turns plan offsets into addresses (the plan already places pieces inside the scratch slots).
 void resolve(hoccl_comm* c, const Plan& P, const Call& call, Contributions how, std::vector<RGroup>* out, size_t* host_need) {
   *host_need = 0;
@@ -195,6 +235,7 @@ void resolve(hoccl_comm* c, const Plan& P, const Call& call, Contributions how, 
       kept.push_back(std::move(cur));
     }
     out->swap(kept);
+    if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0) trim_driver_copies(out);
   }
   // SM path: the stages of an all-to-all are independent (disjoint blocks, no dependencies), so their moves go into as few
   // batched launches as the segment table allows instead of one launch per stage
@@ -238,32 +279,41 @@ void resolve(hoccl_comm* c, const Plan& P, const Call& call, Contributions how, 
   }
 }
 
-bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<double>* bytes_out, std::vector<long>* moves_out) {
-  out->clear();
-  bytes_out->clear();
-  moves_out->clear();
-  if (g.kind != OP_MOVE) return false;
-  // classes: same source, same length, same 16-byte phase of the destination (so that a class is all-vector or all-element-wise)
-  struct Class {
-    const char* src;
-    size_t bytes;
-    unsigned phase;
-    std::vector<void*> dsts;
-  };
-  std::vector<Class> classes;
+namespace {
+// Moves of a group with the same source, the same length and the same 16-byte phase of the destination.
+struct MoveClass {
+  const char* src;
+  size_t bytes;
+  std::vector<void*> dsts;
+};
+}  // namespace
+
+// *repeats: whether some source goes to more than one destination of a class.
+static std::vector<MoveClass> move_classes(const RGroup& g, bool* repeats) {
+  std::vector<MoveClass> classes;
   std::map<std::tuple<const char*, size_t, unsigned>, size_t> index;
-  bool repeats = false;
+  *repeats = false;
   for (const Seg& s : g.segs) {
     auto key = std::make_tuple((const char*)s.src, (size_t)s.bytes, (unsigned)((uintptr_t)s.dst & 15));
     auto it = index.find(key);
     if (it == index.end()) {
       index.emplace(key, classes.size());
-      classes.push_back(Class{s.src, s.bytes, std::get<2>(key), {s.dst}});
+      classes.push_back(MoveClass{s.src, s.bytes, {s.dst}});
     } else {
       classes[it->second].dsts.push_back(s.dst);
-      repeats = true;
+      *repeats = true;
     }
   }
+  return classes;
+}
+
+bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<double>* bytes_out, std::vector<long>* moves_out) {
+  out->clear();
+  bytes_out->clear();
+  moves_out->clear();
+  if (g.kind != OP_MOVE) return false;
+  bool repeats = false;
+  const std::vector<MoveClass> classes = move_classes(g, &repeats);
   if (!repeats) return false;
   FanBatch cur;
   cur.nseg = 0;
@@ -280,7 +330,7 @@ bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<
     cur_bytes = 0;
     cur_moves = 0;
   };
-  for (const Class& cl : classes) {
+  for (const MoveClass& cl : classes) {
     size_t done = 0;
     while (done < cl.dsts.size()) {   // a class with more destinations than a batch holds is cut
       if (cur.nseg == kMaxSegs || cur.ndst_total == kMaxFanDsts) flush();
@@ -341,6 +391,51 @@ static KernelLaunch make_launch(const Batch& b, const void* fn, long grid, int t
   return k;
 }
 
+// move_kernel serves a group whose copies it can do wide and copy_kernel cannot (some source and destination differ modulo 16
+// and are long enough to have a body), long copies to destinations off the 128-byte lines (it aligns its stores to them: in-place
+// all-gather of 8 ragged chunks of 5 MiB 78 -> 67 us), and a group of more copies than one batch of copy_kernel holds (an
+// all-to-all of 8 ranks: one launch instead of two).
+static bool wants_move_kernel(const RGroup& g) {
+  for (const Seg& s : g.segs)
+    if (((((uintptr_t)s.src ^ (uintptr_t)s.dst) & 15) && s.bytes >= 64) || (((uintptr_t)s.dst & 127) && s.bytes >= kMoveLineBytes)) return true;
+  bool repeats = false;
+  return g.segs.size() > (size_t)kMaxSegs && move_classes(g, &repeats).size() > (size_t)kMaxSegs;
+}
+
+static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup& g) {
+  std::vector<KernelLaunch> out;
+  int threads = 0;
+  const void* fn = move_kernel_entry((int)c->copy_ctas, &threads);
+  MoveBatch b;
+  b.nseg = b.ndst_total = 0;
+  double bytes = 0;
+  auto flush = [&]() {
+    if (b.nseg == 0) return;
+    prepare_move_batch(&b, (int)c->copy_ctas);
+    out.push_back(make_launch(b, fn, c->copy_ctas, threads, bytes, b.ndst_total));
+    b.nseg = b.ndst_total = 0;
+    bytes = 0;
+  };
+  bool repeats = false;
+  for (const MoveClass& cl : move_classes(g, &repeats))
+    for (size_t done = 0; done < cl.dsts.size();) {
+      const size_t n = std::min<size_t>(cl.dsts.size() - done, (size_t)kMaxRanks);
+      for (size_t at = 0; at < cl.bytes; at += kMaxMoveSegBytes) {
+        const size_t len = std::min<size_t>(kMaxMoveSegBytes, cl.bytes - at);
+        std::vector<void*> dsts(cl.dsts.begin() + done, cl.dsts.begin() + done + n);
+        for (void*& d : dsts) d = (char*)d + at;
+        if (!add_move_seg(&b, cl.src + at, dsts.data(), (int)n, len)) {
+          flush();
+          add_move_seg(&b, cl.src + at, dsts.data(), (int)n, len);
+        }
+        bytes += (1.0 + (double)n) * (double)len;
+      }
+      done += n;
+    }
+  flush();
+  return out;
+}
+
 std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, const RGroup& g) {
   std::vector<KernelLaunch> out;
   int threads = 0;
@@ -374,6 +469,7 @@ std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, co
     }
     return out;
   }
+  if (wants_move_kernel(g)) return move_launches(c, g);
   std::vector<FanBatch> fans;
   std::vector<double> fan_bytes;
   std::vector<long> fan_moves;
@@ -458,7 +554,7 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
         }
         tally->sum_launches++;
       }
-    } else if (c->path == HOCCL_PATH_CE) {
+    } else if (c->path == HOCCL_PATH_CE && !rg.edges) {
       for (const Seg& sg : rg.segs) {
         CU_TRY(c, cudaMemcpyAsync(sg.dst, sg.src, sg.bytes, cudaMemcpyDeviceToDevice, s));
         tally->moves++;
@@ -474,7 +570,7 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
     } else {
       for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
         CU_TRY(c, launch_kernel(k, s));
-        tally->moves += k.moves;
+        if (!rg.edges) tally->moves += k.moves;
         tally->move_launches++;
       }
     }
@@ -718,13 +814,32 @@ hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype) {
   return resolve_options(options_of(c, kind, count, dtype, false), &o);
 }
 
+// Whether some block of an all-gather or all-to-all is a copy the driver does badly (see kDriverLine).  Such a call runs on the copy
+// kernel at any size, like a small one: of the blocks of 64 MiB per rank, 16 bytes short of whole, an all-gather of 8 ranks took
+// 0.372 ms in driver copies and takes 0.112 (0.174 for whole blocks in driver copies), an all-to-all 0.384 and 0.185 (0.174); two
+// bytes out of phase 0.818 and 0.113, 0.838 and 0.190.
+static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
+  const size_t block = call.count * dtype_size(call.dtype);
+  if (block < kDriverWhole) return false;
+  if (block % kDriverPage) return true;
+  for (int u = 0; u < c->R; u++)
+    for (int v = 0; v < c->R; v++) {
+      const size_t s = (size_t)(uintptr_t)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0);
+      const size_t d = (size_t)(uintptr_t)call.recv[v] + (size_t)u * block;
+      if ((d % kDriverLine) || ((s ^ d) & 15)) return true;
+    }
+  return false;
+}
+
 hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   const double t0 = now_us();
   if (!c) return HOCCL_ERR_INVALID_ARG;
   if (dtype_size(call->dtype) == 0) return HOCCL_ERR_UNSUPPORTED;
   if (!call->send || !call->recv) return HOCCL_ERR_INVALID_ARG;
   // One place decides how the settings combine for this call (options.h); a contradictory combination is refused here.
-  const OptionsIn oin = options_of(c, call->kind, call->count, call->dtype, call->h_send != nullptr);
+  OptionsIn oin = options_of(c, call->kind, call->count, call->dtype, call->h_send != nullptr);
+  if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && (call->kind == PLAN_ALLGATHER || call->kind == PLAN_ALLTOALL) && blocks_bad_for_driver(c, *call))
+    oin.ce_small_bytes = LONG_MAX;
   OptionsOut opt;
   {
     hoccl_result_t orc = resolve_options(oin, &opt);

@@ -109,7 +109,7 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
   if (c->order_kernels && (c->path == HOCCL_PATH_CE || c->path == HOCCL_PATH_CE_HOST)) {
     size_t n_root = 0;
     for (size_t gi = 0; gi < groups.size(); gi++)
-      if (included(gi) && groups[gi].kind == OP_MOVE && inner_deps(gi) == 0) n_root += groups[gi].segs.size();
+      if (included(gi) && groups[gi].kind == OP_MOVE && !groups[gi].edges && inner_deps(gi) == 0) n_root += groups[gi].segs.size();
     many_root_copies = n_root >= 2;
   }
   // The same holds behind a group of copies: copy nodes (or the end of the graph) that wait for several copy nodes start
@@ -212,7 +212,7 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
         nodes.assign(1, kn);
         entry->n_sum_launches++;
       }
-    } else if (c->path == HOCCL_PATH_CE) {
+    } else if (c->path == HOCCL_PATH_CE && !rg.edges) {
       for (const Seg& sg : rg.segs) {
         // optional sub-copies: driver copies of 4-8 MiB pay a ~4 us serialised start-up that smaller ones do not
         size_t sub = sg.bytes;
@@ -270,7 +270,7 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
         }
         last_copy_node = kn;
         nodes.push_back(kn);
-        entry->n_moves += k.moves;
+        if (!rg.edges) entry->n_moves += k.moves;   // (the ends belong to the driver copies' moves)
         entry->n_move_launches++;
       }
     }

@@ -146,26 +146,38 @@ __global__ void __launch_bounds__(THREADS, 1) copy_kernel(const __grid_constant_
   }
 }
 
-// One element of a chain segment, element-wise: the same adds in the same order as the vector bodies.
-template <int DT>
+// One element of a chain segment, element-wise: the same adds in the same order as the vector bodies.  NOPS > 0: the operand count,
+// so that an element's loads are in flight together (one after the other they cost ~0.7 us each).
+template <int DT, int NOPS>
 __device__ __forceinline__ void chain_scalar(const ChainBatch& b, const ChainSeg& sg, unsigned long long i) {
   void* const* op = b.ptr + sg.first_ptr;
+  const int nops = NOPS ? NOPS : sg.nops;
   if (DT == 0) {
-    float acc = static_cast<const float*>(op[0])[i];
-    for (int q = 1; q < sg.nops; q++) acc = __fadd_rn(acc, static_cast<const float*>(op[q])[i]);
-    for (int d = 0; d < sg.ndst; d++) static_cast<float*>(op[sg.nops + d])[i] = acc;
+    float x[NOPS ? NOPS : 1];
+#pragma unroll
+    for (int q = 0; q < NOPS; q++) x[q] = static_cast<const float*>(op[q])[i];
+    float acc = NOPS ? x[0] : static_cast<const float*>(op[0])[i];
+#pragma unroll
+    for (int q = 1; q < NOPS; q++) acc = __fadd_rn(acc, x[q]);
+    for (int q = 1; q < nops && !NOPS; q++) acc = __fadd_rn(acc, static_cast<const float*>(op[q])[i]);
+    for (int d = 0; d < sg.ndst; d++) static_cast<float*>(op[nops + d])[i] = acc;
   } else {
-    unsigned short acc = static_cast<const unsigned short*>(op[0])[i];
-    for (int q = 1; q < sg.nops; q++) {
-      const float s2 = __fadd_rn(__uint_as_float((uint32_t)acc << 16), __uint_as_float((uint32_t) static_cast<const unsigned short*>(op[q])[i] << 16));
-      acc = __bfloat16_as_ushort(__float2bfloat16_rn(s2));
-    }
-    for (int d = 0; d < sg.ndst; d++) static_cast<unsigned short*>(op[sg.nops + d])[i] = acc;
+    auto add = [](unsigned short a, unsigned short c) {
+      return __bfloat16_as_ushort(__float2bfloat16_rn(__fadd_rn(__uint_as_float((uint32_t)a << 16), __uint_as_float((uint32_t)c << 16))));
+    };
+    unsigned short x[NOPS ? NOPS : 1];
+#pragma unroll
+    for (int q = 0; q < NOPS; q++) x[q] = static_cast<const unsigned short*>(op[q])[i];
+    unsigned short acc = NOPS ? x[0] : static_cast<const unsigned short*>(op[0])[i];
+#pragma unroll
+    for (int q = 1; q < NOPS; q++) acc = add(acc, x[q]);
+    for (int q = 1; q < nops && !NOPS; q++) acc = add(acc, static_cast<const unsigned short*>(op[q])[i]);
+    for (int d = 0; d < sg.ndst; d++) static_cast<unsigned short*>(op[nops + d])[i] = acc;
   }
 }
 
 // Element-wise items of a launch: heads, tails and segments without a common 16-byte phase.
-template <int DT>
+template <int DT, int NOPS>
 __device__ __forceinline__ void chain_scalar_items(const ChainBatch& batch) {
   using T = Traits<DT>;
   const Flat& f = batch.flat;
@@ -176,7 +188,7 @@ __device__ __forceinline__ void chain_scalar_items(const ChainBatch& batch) {
     while (j >= f.spre[k + 1]) k++;
     unsigned long long i = j - f.spre[k];
     if (i >= f.head[k]) i += f.nvec[k] * T::VE;
-    chain_scalar<DT>(batch, batch.seg[k], i);
+    chain_scalar<DT, NOPS>(batch, batch.seg[k], i);
   }
 }
 
@@ -223,7 +235,7 @@ __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant
     }
     for (int d = 0; d < sg.ndst; d++) *reinterpret_cast<uint4*>(static_cast<char*>(op[sg.nops + d]) + off) = acc;
   }
-  chain_scalar_items<DT>(batch);
+  chain_scalar_items<DT, 0>(batch);
 }
 
 // Software-pipelined form of the chain sum for a compile-time operand count NOPS that all segments of the launch share, one
@@ -299,7 +311,7 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe_kernel(const __grid_con
       }
     }
   }
-  chain_scalar_items<DT>(batch);
+  chain_scalar_items<DT, NOPS>(batch);
 }
 
 // The sum that carries the all-gather too: NOPS operands are read once, the result is stored to NOPS destinations (one per
@@ -343,7 +355,7 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
       }
     }
   }
-  chain_scalar_items<DT>(batch);
+  chain_scalar_items<DT, NOPS>(batch);
 }
 
 // Fan-out copy: the tile walk of copy_kernel, but a tile that was loaded once is stored to every destination of its segment.
@@ -406,6 +418,97 @@ __global__ void __launch_bounds__(THREADS, 1) fan_kernel(const __grid_constant__
       const unsigned char v = static_cast<const unsigned char*>(batch.seg[k].src)[i];
       void* const* dsts = batch.dst + batch.seg[k].first_dst;
       for (int d = 0; d < batch.seg[k].ndst; d++) static_cast<unsigned char*>(dsts[d])[i] = v;
+    }
+  }
+}
+
+// The 16 bytes that start `sh` bytes into the 32 bytes lo, hi; sh (0..15) is the same for all threads.
+__device__ __forceinline__ uint4 bytes_at(uint4 lo, uint4 hi, unsigned sh) {
+  uint32_t w0 = lo.x, w1 = lo.y, w2 = lo.z, w3 = lo.w, w4 = hi.x, w5 = hi.y, w6 = hi.z, w7 = hi.w;
+  if (sh & 8) {
+    w0 = w2;
+    w1 = w3;
+    w2 = w4;
+    w3 = w5;
+    w4 = w6;
+    w5 = w7;
+  }
+  if (sh & 4) {
+    w0 = w1;
+    w1 = w2;
+    w2 = w3;
+    w3 = w4;
+    w4 = w5;
+  }
+  const unsigned b = (sh & 3) * 8;
+  return make_uint4(__funnelshift_r(w0, w1, b), __funnelshift_r(w1, w2, b), __funnelshift_r(w2, w3, b), __funnelshift_r(w3, w4, b));
+}
+
+// Segment of item t: the largest k with pre[k] <= t (pre is non-decreasing, pre[n] > t).
+__device__ __forceinline__ int find_segment(const unsigned* pre, int n, unsigned t) {
+  int lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (pre[mid] <= t) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// Moves whose source and destination lie differently modulo 16, or too many for the batches above.  Byte by byte such moves ran
+// at a tenth of the copy rate (8 chunks of 500,014 bytes to 8 ranks each: 37 us of a 38 us all-gather).  Here a thread
+// loads the two aligned vectors that hold its 16 bytes (the second is its neighbour's first, an L1 hit), shifts them into place
+// and stores aligned vectors to every destination.
+template <int U, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant__ MoveBatch batch) {
+  const int nseg = batch.nseg;
+  const unsigned T_all = batch.tpre[nseg];
+  if (blockIdx.x < T_all) {
+    int k = find_segment(batch.tpre, nseg, blockIdx.x);
+    for (unsigned t = blockIdx.x; t < T_all; t += gridDim.x) {
+      while (t >= batch.tpre[k + 1]) k++;
+      const MoveSeg& sg = batch.seg[k];
+      const unsigned first = (t - batch.tpre[k]) * (U * THREADS) + threadIdx.x;
+      const char* s = static_cast<const char*>(sg.src) + sg.head;
+      const unsigned sh = (unsigned)(uintptr_t)s & 15;
+      const uint4* a = reinterpret_cast<const uint4*>(s - sh) + first;
+      uint4 v[U];
+      if (sh == 0) {
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          if (first + u * THREADS < sg.nvec) v[u] = __ldcs(a + u * THREADS);
+      } else {
+#pragma unroll
+        for (int h = 0; h < U; h += 4) {   // 4 pairs in flight
+          uint4 hi[4];
+#pragma unroll
+          for (int u = 0; u < 4; u++)
+            if (first + (h + u) * THREADS < sg.nvec) {
+              v[h + u] = a[(h + u) * THREADS];
+              hi[u] = a[(h + u) * THREADS + 1];
+            }
+#pragma unroll
+          for (int u = 0; u < 4; u++) v[h + u] = bytes_at(v[h + u], hi[u], sh);
+        }
+      }
+      for (int d = 0; d < sg.ndst; d++) {
+        uint4* o = reinterpret_cast<uint4*>(static_cast<char*>(batch.dst[sg.first_dst + d]) + sg.head) + first;
+#pragma unroll
+        for (int u = 0; u < U; u++)
+          if (first + u * THREADS < sg.nvec) o[u * THREADS] = v[u];
+      }
+    }
+  }
+  const unsigned S = batch.spre[nseg], j0 = blockIdx.x * THREADS + threadIdx.x;
+  if (j0 < S) {
+    int k = find_segment(batch.spre, nseg, j0);
+    for (unsigned j = j0; j < S; j += gridDim.x * THREADS) {
+      while (j >= batch.spre[k + 1]) k++;
+      const MoveSeg& sg = batch.seg[k];
+      unsigned long long i = j - batch.spre[k];
+      if (i >= sg.head) i += (unsigned long long)sg.nvec * 16;
+      const unsigned char v = static_cast<const unsigned char*>(sg.src)[i];
+      for (int d = 0; d < sg.ndst; d++) static_cast<unsigned char*>(batch.dst[sg.first_dst + d])[i] = v;
     }
   }
 }
@@ -689,6 +792,16 @@ void prepare_chain_batch(ChainBatch* b, int ctas) {
     bool same = true;
     for (int q = 1; q < s.nops + s.ndst; q++) same = same && ((unsigned)((uintptr_t)b->ptr[s.first_ptr + q] & 15) == phase);
     split_segment(s.n, phase, same, E, VE, &head[k], &nvec[k], &nscalar[k]);
+    // Start the body of a long segment on a 128-byte line where all operands have one together: a warp's 512 bytes then touch four
+    // lines of each operand, not five (40 MiB per rank over 8 ranks in ragged chunks: 406 -> 351 us with the loads of an element-wise
+    // item in flight together).
+    const unsigned line = (unsigned)((uintptr_t)b->ptr[s.first_ptr] & 127);
+    for (int q = 1; q < s.nops; q++) same = same && ((unsigned)((uintptr_t)b->ptr[s.first_ptr + q] & 127) == line);
+    if (same && nvec[k] >= 4096 && line % E == 0) {
+      head[k] = ((128 - line) & 127) / E;
+      nvec[k] = (s.n - head[k]) / VE;
+      nscalar[k] = s.n - nvec[k] * VE;
+    }
   }
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
 }
@@ -732,6 +845,44 @@ cudaError_t launch_fan(const FanBatch& batch, int ctas, cudaStream_t stream) {
   if (wide_copy_grid(ctas)) fan_kernel<4, 512><<<ctas, 512, 0, stream>>>(b);
   else fan_kernel<8, 1024><<<ctas, 1024, 0, stream>>>(b);
   return cudaGetLastError();
+}
+
+bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, unsigned long long bytes) {
+  if (b->nseg == kMaxMoveSegs || b->ndst_total + ndst > kMaxMoveDsts) return false;
+  MoveSeg& s = b->seg[b->nseg++];
+  s.src = src;
+  s.bytes = bytes;
+  s.first_dst = b->ndst_total;
+  s.ndst = ndst;
+  for (int d = 0; d < ndst; d++) b->dst[b->ndst_total++] = dsts[d];
+  return true;
+}
+
+void prepare_move_batch(MoveBatch* b, int ctas) {
+  const unsigned tile_v = wide_copy_grid(ctas) ? 4u * 512 : 8u * 1024;
+  b->tpre[0] = b->spre[0] = 0;
+  for (int k = 0; k < b->nseg; k++) {
+    MoveSeg& s = b->seg[k];
+    const unsigned long long at = (uintptr_t)s.src & 15;
+    // destination on a 128-byte line if the segment is long (a warp's 512 bytes then touch four lines, not five), on a vector if not
+    const unsigned long long grid = s.bytes >= kMoveLineBytes ? 128 : 16;
+    unsigned long long head = (grid - ((uintptr_t)b->dst[s.first_dst] & (grid - 1))) & (grid - 1);
+    const unsigned long long sh = (at + head) & 15;                                // where a vector starts inside the source's
+    if (head < sh) head += 16;                 // the first aligned vector of the source must not start in front of it
+    const unsigned long long reach = sh ? 32 - sh : 16;   // source bytes from the start of a vector to the end of what it loads
+    unsigned long long nvec = 0;
+    if (s.bytes >= head + reach) nvec = (s.bytes - head - reach) / 16 + 1;
+    else head = 0;
+    s.head = (unsigned)head;
+    s.nvec = (unsigned)nvec;
+    b->tpre[k + 1] = b->tpre[k] + (unsigned)((nvec + tile_v - 1) / tile_v);
+    b->spre[k + 1] = b->spre[k] + (unsigned)(s.bytes - nvec * 16);
+  }
+}
+
+const void* move_kernel_entry(int ctas, int* threads) {
+  *threads = wide_copy_grid(ctas) ? 512 : 1024;
+  return wide_copy_grid(ctas) ? reinterpret_cast<const void*>(&move_kernel<4, 512>) : reinterpret_cast<const void*>(&move_kernel<8, 1024>);
 }
 
 cudaError_t launch_sum(const SumBatch& batch, int ctas, cudaStream_t stream) {
@@ -811,6 +962,7 @@ cudaError_t preload_kernels() {
                        reinterpret_cast<const void*>(&onepass_kernel<1, 512>),  reinterpret_cast<const void*>(&onepass_kernel<0, 1024>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 1024>), reinterpret_cast<const void*>(&fan_kernel<4, 512>),
                        reinterpret_cast<const void*>(&fan_kernel<8, 1024>), reinterpret_cast<const void*>(&graph_root_kernel),
+                       reinterpret_cast<const void*>(&move_kernel<4, 512>), reinterpret_cast<const void*>(&move_kernel<8, 1024>),
                        reinterpret_cast<const void*>(&chain_kernel<0, 1024>), reinterpret_cast<const void*>(&chain_kernel<1, 1024>)};
   for (const void* f : fns) {
     cudaFuncAttributes a;

@@ -90,6 +90,35 @@ struct FanBatch {
   unsigned int* smid_out = nullptr;  // diagnostics, as in SumBatch
 };
 
+// Moves of one launch that copy_kernel and fan_kernel do not serve well: sources and destinations out of phase (their addresses
+// differ modulo 16), or more segments than those batches hold.  A segment is stored to ndst destinations of one phase; its body
+// is cut at the destination's 16-byte boundaries and, if the source lies differently, kept away from both ends of the source
+// far enough that the aligned vectors that hold its bytes lie inside the source.  Tiles and vectors fit 32 bits (a segment has
+// at most kMaxMoveSegBytes bytes).
+constexpr int kMaxMoveSegs = 128, kMaxMoveDsts = 512;
+constexpr unsigned long long kMaxMoveSegBytes = 8ull << 30;
+constexpr unsigned long long kMoveLineBytes = 64 << 10;   // segments from this length on are cut at the destination's 128-byte lines
+struct MoveSeg {
+  const void* src;
+  unsigned int nvec;          // 16-byte vectors in the body
+  unsigned int head;          // bytes before the body
+  unsigned long long bytes;
+  int first_dst, ndst;
+};
+struct MoveBatch {
+  int nseg;
+  int ndst_total;
+  MoveSeg seg[kMaxMoveSegs];
+  void* dst[kMaxMoveDsts];
+  unsigned int tpre[kMaxMoveSegs + 1];   // prefix sums of vector tiles
+  unsigned int spre[kMaxMoveSegs + 1];   // prefix sums of byte-wise items
+};
+// Appends a segment (all destinations in one phase); false if the batch has no room for it.  Batches are prepared with the CTA
+// count they are launched with.
+bool add_move_seg(MoveBatch* batch, const void* src, void* const* dsts, int ndst, unsigned long long bytes);
+void prepare_move_batch(MoveBatch* batch, int ctas);
+const void* move_kernel_entry(int ctas, int* threads);
+
 // One-pass variant of the ring reduction (comparison point, not rank local): every element is reduced in registers in
 // the ring's order, chunk c as ((x_{c+1} + x_{c+2}) + ... ) + x_c with a rounding to the I/O dtype after every add, and
 // written to its destinations directly.  Same bits as the ring, R reads + R (or 1) writes per element instead of 7(R-1).

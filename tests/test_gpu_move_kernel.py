@@ -1,0 +1,93 @@
+"""Moves between buffers that lie differently modulo 16, and groups of more copies than one batch of the plain copy kernel holds."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_34334_b200 import binding as hb
+from gpu_util import DevBuf
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _need_gpu():
+    assert torch.cuda.is_available(), "these tests need a CUDA device"
+    torch.cuda.set_device(0)
+    yield
+    torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("ctas", [3, 40, 148])
+@pytest.mark.parametrize("R,count", [(8, 1), (3, 7), (8, 33), (2, 2048 * 8 + 1), (5, 8 * 1024 * 8 + 11), (8, 70_001), (16, 4099)])
+def test_ragged_blocks(R, count, ctas):
+    """Odd counts: the blocks of a rank lie at every phase of 2 bytes; heads, bodies and tails of each, source against destination."""
+    rng = np.random.default_rng(R * 1000 + count)
+    x = rng.integers(0, 1 << 16, (R, R * count), dtype=np.uint16)
+    comm = hb.Comm(R, 0)
+    comm.set_path(hb.PATH_SM)
+    comm.set_param("copy_ctas", ctas)
+    for shift in (0, 1, 5):
+        send = [DevBuf(R * count * 2, 2 * ((r * shift) % 8)).put(x[r]) for r in range(R)]
+        recv = [DevBuf(R * count * 2, 2 * ((r + shift) % 8)) for r in range(R)]
+        comm.alltoall(send, recv, count, "bf16")
+        torch.cuda.synchronize()
+        for r in range(R):
+            want = np.concatenate([x[u][r * count:(r + 1) * count] for u in range(R)])
+            assert (recv[r].get(np.uint16) == want).all() and recv[r].guards_intact() and (send[r].get(np.uint16) == x[r]).all(), (shift, r)
+        assert comm.last_stats()["n_moves"] == R * R
+        # all-gather: every block goes to R destinations of differing phases
+        src = [DevBuf(count * 2, 2 * (r % 8)).put(x[r][:count]) for r in range(R)]
+        for b in recv:
+            b.view.fill_(0)
+        comm.allgather(src, recv, count, "bf16")
+        torch.cuda.synchronize()
+        want = np.concatenate([x[u][:count] for u in range(R)])
+        assert all((recv[r].get(np.uint16) == want).all() and recv[r].guards_intact() for r in range(R)), shift
+    comm.destroy()
+
+
+def test_an_all_to_all_of_eight_ranks_is_one_launch():
+    R, count = 8, 4096
+    send = [DevBuf(R * count * 4) for _ in range(R)]
+    recv = [DevBuf(R * count * 4) for _ in range(R)]
+    comm = hb.Comm(R, 0)
+    comm.set_path(hb.PATH_SM)
+    comm.alltoall(send, recv, count, "fp32")
+    torch.cuda.synchronize()
+    assert (comm.last_stats()["n_move_launches"], comm.last_stats()["n_moves"]) == (1, 64)
+    comm.destroy()
+
+
+@pytest.mark.parametrize("op", ["allgather", "alltoall", "allreduce"])
+@pytest.mark.parametrize("count", [(1 << 20) - 8, (1 << 20) + 1, 600_064, 1 << 20])
+def test_copies_the_driver_does_badly(op, count):
+    """Copy route above the small-message size: blocks of 1 to 2 MiB that end inside a page or start off a 128-byte line run on the
+    copy kernel (all-gather, all-to-all) or leave their ends to it (all-reduce); whole blocks stay with the driver."""
+    R = 8
+    comm = hb.Comm(R, 0)
+    n = R * count
+    nb = hb.scratch_bytes_direct(R, n, "bf16")
+    scratch = torch.empty(nb, dtype=torch.uint8, device="cuda")
+    comm.set_scratch(scratch, nb)
+    g = torch.Generator(device="cuda").manual_seed(count)
+    ints = lambda k: torch.randint(-8, 9, (k,), generator=g, device="cuda").to(torch.bfloat16)     # sums of 8 are exact
+    for pad in (0, 3):
+        make = lambda k: torch.zeros(k + pad, dtype=torch.bfloat16, device="cuda")[pad:]
+        recv = [make(n) for _ in range(R)]
+        if op == "allgather":
+            send = [make(count).copy_(ints(count)) for _ in range(R)]
+            comm.allgather(send, recv, count, "bf16")
+            want = [torch.cat(send)] * R
+        else:
+            send = [make(n).copy_(ints(n)) for _ in range(R)]
+            if op == "alltoall":
+                comm.alltoall(send, recv, count, "bf16")
+                want = [torch.cat([s[r * count:(r + 1) * count] for s in send]) for r in range(R)]
+            else:
+                comm.allreduce(send, recv, n, "bf16")
+                want = [torch.stack([s.float() for s in send]).sum(0).to(torch.bfloat16)] * R
+        torch.cuda.synchronize()
+        assert all(torch.equal(recv[r], want[r]) for r in range(R)), (op, count, pad)
+        whole = count * 2 % 4096 == 0 and pad == 0
+        assert (comm.last_stats()["n_move_launches"] == 0) == whole, (op, count, pad, comm.last_stats())
+    comm.destroy()

@@ -203,10 +203,10 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                kernel is a pure gain: measured on B200 with the default schedule and 8-CTA sums, R = 8 bf16 all-reduce of
  *                4 KiB 34 -> 10 us, 1 MiB 48 -> 25 us, 4 MiB 88 -> 54 us, 8 MiB 107 -> 97 us, equal from 16 MiB on; R = 4 fp32
  *                all-reduce of 4 MiB 37 -> 33 us.  Default 8 MiB; 0 = driver copies at every size.  "HOCCL_PATH_CE" therefore
- *                means: the copy route above this size.  Not applied to hoccl_host_allreduce, send/recv or hoccl_alltoallv.
+ *                means: the copy route above this size.  Not applied to hoccl_host_allreduce and send/recv.
  *                Unless it is 0, copies the driver does badly do not go to it at any size (it takes 4 us more for a copy of 1 MiB or
  *                more that does not start on a 128-byte line and end after whole 4 KiB, and runs at half rate or less when the two
- *                ends differ modulo 4): an all-gather or all-to-all of such blocks runs on the copy kernel like a small one, and an
+ *                ends differ modulo 4): an all-gather or all-to-all of such blocks, or of blocks below 2 MiB, runs on the copy kernel like a small one, and an
  *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of its all-gather's copies to one
  *                launch of the copy kernel ("copy_ctas" CTAs) per piece.
  *  "ce_overlap"  HOCCL_PATH_CE, direct reduce-scatter: the ring chunks are cut into this many pieces and every piece's three
@@ -361,15 +361,16 @@ hoccl_result_t hoccl_alltoall(const void* const* send, void* const* recv, size_t
  * traffic matrix).  MPI-style all-to-allv over the R logical ranks: rank u sends sendcounts[u*R+v] elements, taken
  * from send[u] + sdispls[u*R+v], to rank v, which stores them at recv[v] + rdispls[v*R+u] (counts and
  * displacements are HOST arrays of R*R entries, in elements).  u == v is a local copy.
- * The flows form the origin traffic matrix C; the collective scheduler (hoccl_sched_*) cuts it into stages by
- * peeling matchings (Algorithm 1 with an empty RDMA domain: T = C) and, inside a stage, serves every source rank's
- * flows from one serial queue in a size-weighted chunk interleaving (chunk = the "piece_bytes" parameter, at least
- * 64 KiB; chunks that follow one another in a queue and continue the same flow are issued as one operation).  Stages
- * run one after the other.  With "use_graph" = 1 (default) the schedule becomes a CUDA graph that is cached under the
+ * The flows form the origin traffic matrix C.  In one memory they share no link and wait for nothing, so all of them are issued
+ * at once, each as one move; the collective scheduler (hoccl_sched_*) with its stages and chunks serves the modelled topologies
+ * below.  On HOCCL_PATH_CE ("ce_small_bytes" not 0) a pattern of at most "ce_small_bytes" per rank, one with flows the driver
+ * copies badly (see "ce_small_bytes") and one whose flows are 3 MiB or shorter on average run as one launch of the copy kernel.
+ * With "use_graph" = 1 (default) the pattern becomes a CUDA graph that is cached under the
  * call's full signature (every pointer, count and displacement), so a pattern that repeats on the same buffers replays
  * it; otherwise, and with "use_graph" = 0, it is issued with streams and events.  No scratch.
  * Modelled topology ("model_gpus_per_node" = g with 0 < g < R): the R logical ranks are treated as GPUs of R / g nodes (rank r
- * sits on node r / g, the last node may be smaller) and the scheduler runs the paper's full expansion (Eq. 2-4, Algorithm 1):
+ * sits on node r / g, the last node may be smaller) and the scheduler runs the paper's full expansion (Eq. 2-4, Algorithm 1;
+ * chunk = the "piece_bytes" parameter, at least 64 KiB; stages run one after the other):
  * a flow between two nodes is carried, portion by portion as Algorithm 1 stages it, by a forwarding copy to the sender's
  * symmetric peer, the "RDMA" leg to the receiver's symmetric peer and a forwarding copy to the receiver, all as real copies
  * through the memory attached with hoccl_comm_set_staging, while native flows fill the NVLink slack of the stages.  The

@@ -354,6 +354,30 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
       C[(size_t)u * R + v] = (uint64_t)sendcounts[(size_t)u * R + v] * e;
       total += C[(size_t)u * R + v];
     }
+  // The move route, as for the other collectives: on the copy route a short pattern, and one with copies the driver does badly,
+  // runs on the copy kernel, and so does one of mostly short flows (every driver copy costs a microsecond, and the short ones of
+  // an uneven pattern leave the GPU part empty).  R = 8, driver copies against the kernel: 1 MiB per rank 20.8 / 5.5 us, 12 MiB (flows
+  // of 1.5 MiB on average) 49 / 39, 32 MiB (4 MiB) 93 / 95, 128 MiB 334 / 366; in rows of 666 bytes 32 MiB 447 / 98; R = 4, 12 MiB (3 MiB)
+  // 20.7 / 15.2; R = 16, 12 MiB (0.75 MiB) 147 / 79, 32 MiB (2 MiB) 239 / 192.
+  hoccl_path_t route = c->path;
+  if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && !modelled) {
+    constexpr uint64_t kShortFlow = 3 << 20;
+    uint64_t most = 0, flows = 0;
+    bool bad = false;
+    for (int u = 0; u < R; u++) {
+      uint64_t out = 0, in = 0;
+      for (int v = 0; v < R; v++) {
+        const size_t i = (size_t)u * R + v;
+        out += C[i];
+        flows += C[i] != 0;
+        in += C[(size_t)v * R + u];
+        bad = bad || bad_for_driver((const char*)send[u] + sdispls[i] * e, (const char*)recv[v] + rdispls[(size_t)v * R + u] * e, C[i]);
+      }
+      most = std::max(most, std::max(out, in));
+    }
+    if (bad || most <= (uint64_t)c->ce_small_bytes || total <= flows * kShortFlow) route = HOCCL_PATH_SM;
+  }
+  RouteGuard guard(c, route, route == c->path ? c->copy_ctas : c->ce_small_ctas);
   // A pattern that was issued before with the same buffers (same counts, displacements, pointers and settings) replays
   // its cached graph: validation, Algorithm 1 and the per-operation host cost were paid when it was built.
   std::vector<uint64_t> key;
@@ -406,16 +430,45 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
     }
   c->stats = hoccl_stats_t{};
   if (total == 0) return HOCCL_OK;
-  Schedule S;
-  const uint64_t chunk_bytes = (uint64_t)std::max<long>(c->piece_bytes, 65536);
-  if (!build_schedule(topo, C, chunk_bytes, &S)) return HOCCL_ERR_INTERNAL;
   CU_TRY(c, cudaSetDevice(c->device));
   cudaStream_t user = (cudaStream_t)stream;
+  // One memory: the flows have no link to share and wait for nothing, so all of them are issued at once, each as one move (on the
+  // copy route grouped by source rank, for the lanes of the stream executor).  The scheduler's stages and chunks exist to keep
+  // flows that share a link apart; they serve the modelled topologies.  (In stages and 4 MiB chunks an expert-parallel exchange of
+  // 32 MiB per rank over 8 ranks took 0.315 ms, at once 0.096; one of 1 MiB 0.082 ms, now 0.006.)
+  Plan P;
+  P.R = R;
+  P.kind = PLAN_ALLTOALL;
+  P.dtype = (int)dtype;
+  P.elem = e;
+  std::vector<RGroup> groups;
+  for (int u = 0; u < R && !modelled; u++) {
+    if (groups.empty() || c->path == HOCCL_PATH_CE) {
+      groups.emplace_back();
+      groups.back().kind = OP_MOVE;
+      groups.back().piece = 0;
+      groups.back().phase = PHASE_A2A;
+      groups.back().chain_dep = -1;
+    }
+    for (int k = 0; k < R; k++) {
+      const int v = (u + k) % R;
+      const size_t i = (size_t)u * R + v;
+      if (!C[i]) continue;
+      Seg s = {};
+      s.src = (const char*)send[u] + sdispls[i] * e;
+      s.dst = (char*)recv[v] + rdispls[(size_t)v * R + u] * e;
+      s.bytes = C[i];
+      groups.back().segs.push_back(s);
+    }
+  }
   if (c->use_graph) {
     GraphEntry entry;
     entry.key = key;
     hoccl_result_t grc;
     if (modelled) {
+      Schedule S;
+      const uint64_t chunk_bytes = (uint64_t)std::max<long>(c->piece_bytes, 65536);
+      if (!build_schedule(topo, C, chunk_bytes, &S)) return HOCCL_ERR_INTERNAL;
       // staging for the flows between modelled nodes: what has left the sender's side and what has arrived at the receiver's
       std::vector<uint64_t> off((size_t)R * R, 0);
       uint64_t need = 0;
@@ -432,7 +485,8 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
       grc = build_pattern_graph_modelled(c, S, send, sdispls, recv, rdispls, e, (char*)c->staging, (char*)c->staging + need, off,
                                          (size_t)chunk_bytes, (size_t)c->model_rdma_sub_bytes, &entry);
     } else {
-      grc = build_pattern_graph(c, S, send, sdispls, recv, rdispls, e, &entry);
+      entry.n_pieces = 1;
+      grc = build_graph(c, P, groups, &entry, -1, &entry.exec);
     }
     if (grc != HOCCL_OK) return grc;
     GraphEntry* en = cache_put(c, std::move(entry));
@@ -445,96 +499,13 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
     c->stats.host_launch_us = now_us() - t0;
     return HOCCL_OK;
   }
-  const int lanes = c->path == HOCCL_PATH_SM ? 1 : (int)std::max<long>(1, std::min<long>(c->lanes, kMaxLanes));
-  c->ev_next = 0;
-  cudaEvent_t fork = next_event(c);
-  if (!fork) return cuda_fail(c, cudaErrorMemoryAllocation, "event pool");
-  CU_TRY(c, cudaEventRecord(fork, user));
-  for (int l = 0; l < lanes; l++) CU_TRY(c, cudaStreamWaitEvent(c->lane[l], fork, 0));
-  long moves = 0, launches = 0;
-  for (size_t si = 0; si < S.stages.size(); si++) {
-    const Stage& st = S.stages[si];
-    auto endpoints = [&](const ChunkItem& it, const char** src, char** dst) {
-      const StageFlow& f = st.flows[it.flow];
-      const size_t so = sdispls[(size_t)f.origin_src * R + f.origin_dst] * e + f.origin_offset + it.offset;
-      const size_t dofs = rdispls[(size_t)f.origin_dst * R + f.origin_src] * e + f.origin_offset + it.offset;
-      *src = (const char*)send[f.origin_src] + so;
-      *dst = (char*)recv[f.origin_dst] + dofs;
-    };
-    // Service order is the scheduler's; chunks that follow one another in a queue and continue the same flow are
-    // issued as one operation (a queue that serves a single flow, the uniform case, becomes one copy per flow).
-    std::vector<std::vector<ChunkItem>> queues(R);
-    for (int g = 0; g < R; g++)
-      for (const ChunkItem& it : st.queues[g]) {
-        if (!queues[g].empty() && queues[g].back().flow == it.flow && queues[g].back().offset + queues[g].back().bytes == it.offset)
-          queues[g].back().bytes += it.bytes;
-        else
-          queues[g].push_back(it);
-      }
-    if (c->path == HOCCL_PATH_CE) {
-      // every DMA queue (one per source rank) is a serial chain on its lane, in the interleaved chunk order
-      for (int g = 0; g < R; g++) {
-        cudaStream_t lane = c->lane[g % lanes];
-        for (const ChunkItem& it : queues[g]) {
-          const char* src;
-          char* dst;
-          endpoints(it, &src, &dst);
-          CU_TRY(c, cudaMemcpyAsync(dst, src, it.bytes, cudaMemcpyDeviceToDevice, lane));
-          moves++;
-        }
-      }
-    } else {
-      // SM path: the k-th chunk of every queue goes into one batched copy launch (the queues advance in lock step,
-      // which is what R engines of equal speed would do), so a stage costs as many launches as its longest queue
-      size_t depth = 0;
-      for (int g = 0; g < R; g++) depth = std::max(depth, queues[g].size());
-      for (size_t k = 0; k < depth; k++) {
-        CopyBatch b;
-        b.nseg = 0;
-        b.pad = 0;
-        for (int g = 0; g < R; g++) {
-          if (k >= queues[g].size()) continue;
-          const ChunkItem& it = queues[g][k];
-          const char* src;
-          char* dst;
-          endpoints(it, &src, &dst);
-          b.seg[b.nseg++] = CopySeg{src, dst, (unsigned long long)it.bytes};
-          moves++;
-          if (b.nseg == kMaxSegs) {
-            CU_TRY(c, launch_copy(b, (int)c->copy_ctas, c->lane[0]));
-            launches++;
-            b.nseg = 0;
-          }
-        }
-        if (b.nseg > 0) {
-          CU_TRY(c, launch_copy(b, (int)c->copy_ctas, c->lane[0]));
-          launches++;
-        }
-      }
-    }
-    // stages run one after the other (the paper's serial stages): barrier over the lanes
-    if (si + 1 < S.stages.size() && lanes > 1) {
-      std::vector<cudaEvent_t> evs(lanes);
-      for (int l = 0; l < lanes; l++) {
-        evs[l] = next_event(c);
-        if (!evs[l]) return cuda_fail(c, cudaErrorMemoryAllocation, "event pool");
-        CU_TRY(c, cudaEventRecord(evs[l], c->lane[l]));
-      }
-      for (int l = 0; l < lanes; l++)
-        for (int m = 0; m < lanes; m++)
-          if (m != l) CU_TRY(c, cudaStreamWaitEvent(c->lane[l], evs[m], 0));
-    }
-  }
-  for (int l = 0; l < lanes; l++) {
-    cudaEvent_t ev = next_event(c);
-    if (!ev) return cuda_fail(c, cudaErrorMemoryAllocation, "event pool");
-    CU_TRY(c, cudaEventRecord(ev, c->lane[l]));
-    CU_TRY(c, cudaStreamWaitEvent(user, ev, 0));
-  }
-  c->stats.n_moves = moves;
-  c->stats.n_move_launches = launches;
-  c->stats.max_copy_ctas = launches ? c->copy_ctas : 0;
-  c->stats.n_pieces = (long)S.stages.size();
+  Tally tally;
+  hoccl_result_t src = run_streams(c, P, groups, user, &tally);
+  if (src != HOCCL_OK) return src;
+  c->stats.n_moves = tally.moves;
+  c->stats.n_move_launches = tally.move_launches;
+  c->stats.max_copy_ctas = tally.move_launches ? c->copy_ctas : 0;
+  c->stats.n_pieces = 1;
   c->stats.host_launch_us = now_us() - t0;
   return HOCCL_OK;
 }

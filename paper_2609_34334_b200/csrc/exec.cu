@@ -114,11 +114,6 @@ static Contributions contributions(const hoccl_comm* c, const Call& call, const 
   return READ_IN_PLACE;
 }
 
-// What a driver copy inside one device does at once, as timed on B200: a copy of 1 MiB or more whose destination does not start on a
-// 128-byte line or whose length is not a multiple of 4 KiB takes 4 us more than a whole one (8 MiB 8.3 against 4.3 us, 64 MiB 28.7
-// against 24.6), one whose ends differ modulo 4 runs at half the rate.
-constexpr size_t kDriverLine = 128, kDriverPage = 4096, kDriverWhole = 1 << 20;
-
 // Copy route, contributions read in place: the all-gather's copies keep what the driver does at once and their ends (less than 128 bytes
 // in front, less than 4 KiB behind) go to one launch of the copy kernel per piece, "copy_ctas" CTAs, instead of a second pass per copy.
 static void trim_driver_copies(std::vector<RGroup>* groups) {
@@ -814,20 +809,18 @@ hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype) {
   return resolve_options(options_of(c, kind, count, dtype, false), &o);
 }
 
-// Whether some block of an all-gather or all-to-all is a copy the driver does badly (see kDriverLine).  Such a call runs on the copy
+// Whether some block of an all-gather or all-to-all is a copy the driver does badly (see kDriverLine), or short (all-gather of 9 MiB
+// per rank over 8 ranks 24.7 us in driver copies, 14.4 on the kernel; all-to-all of 9 MiB 32.7 / 28.9, of 16 MiB equal).  Such a call runs on the copy
 // kernel at any size, like a small one: of the blocks of 64 MiB per rank, 16 bytes short of whole, an all-gather of 8 ranks took
 // 0.372 ms in driver copies and takes 0.112 (0.174 for whole blocks in driver copies), an all-to-all 0.384 and 0.185 (0.174); two
 // bytes out of phase 0.818 and 0.113, 0.838 and 0.190.
 static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t block = call.count * dtype_size(call.dtype);
-  if (block < kDriverWhole) return false;
-  if (block % kDriverPage) return true;
+  if (block < kDriverShort) return true;
   for (int u = 0; u < c->R; u++)
-    for (int v = 0; v < c->R; v++) {
-      const size_t s = (size_t)(uintptr_t)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0);
-      const size_t d = (size_t)(uintptr_t)call.recv[v] + (size_t)u * block;
-      if ((d % kDriverLine) || ((s ^ d) & 15)) return true;
-    }
+    for (int v = 0; v < c->R; v++)
+      if (bad_for_driver((const char*)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0), (const char*)call.recv[v] + (size_t)u * block, block))
+        return true;
   return false;
 }
 
@@ -846,17 +839,7 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
     if (orc != HOCCL_OK) return orc;
   }
   // a small message on the copy route runs on the copy kernel's route: the communicator shows that route for this call only
-  struct RouteGuard {
-    hoccl_comm* c;
-    hoccl_path_t path;
-    long ctas;
-    ~RouteGuard() {
-      c->path = path;
-      c->copy_ctas = ctas;
-    }
-  } guard{c, c->path, c->copy_ctas};
-  c->path = (hoccl_path_t)opt.path;
-  c->copy_ctas = opt.copy_ctas;
+  RouteGuard guard(c, (hoccl_path_t)opt.path, opt.copy_ctas);
   const bool onepass_case = opt.executor == EXEC_ONEPASS;
   const bool fused = opt.executor == EXEC_ONE_KERNEL;
   const bool roles = opt.executor == EXEC_ROLES;

@@ -336,125 +336,8 @@ GraphEntry* cache_put(hoccl_comm* c, GraphEntry&& entry) {
   return &c->cache.back();
 }
 
-// The schedule of a user-defined pattern (paper Sec. 3.4) as a CUDA graph: stages one after the other (a join node between
-// them), inside a stage every source rank's queue is a serial chain in the scheduler's service order (copy route), or the
-// k-th operations of all queues share one batched copy launch and the launches form one chain (SM path).
-hoccl_result_t build_pattern_graph(hoccl_comm* c, const Schedule& S, const void* const* send, const size_t* sdispls, void* const* recv,
-                                   const size_t* rdispls, size_t e, GraphEntry* entry) {
-  const int R = c->R;
-  cudaGraph_t g = nullptr;
-  CU_TRY(c, cudaGraphCreate(&g, 0));
-  cudaError_t err = cudaSuccess;
-  cudaGraphNode_t stage_dep = nullptr;
-  if (c->path == HOCCL_PATH_CE && c->order_kernels) {   // one empty kernel in front of the first stage's copy chains (see build_graph)
-    cudaKernelNodeParams kp = {};
-    kp.func = const_cast<void*>(graph_root_kernel_entry());
-    kp.gridDim = dim3(1);
-    kp.blockDim = dim3(32);
-    kp.kernelParams = nullptr;
-    err = cudaGraphAddKernelNode(&stage_dep, g, nullptr, 0, &kp);
-    if (err == cudaSuccess) entry->n_order_launches++;
-  }
-  for (size_t si = 0; si < S.stages.size() && err == cudaSuccess; si++) {
-    const Stage& st = S.stages[si];
-    auto endpoints = [&](const ChunkItem& it, const char** src, char** dst) {
-      const StageFlow& f = st.flows[it.flow];
-      *src = (const char*)send[f.origin_src] + sdispls[(size_t)f.origin_src * R + f.origin_dst] * e + f.origin_offset + it.offset;
-      *dst = (char*)recv[f.origin_dst] + rdispls[(size_t)f.origin_dst * R + f.origin_src] * e + f.origin_offset + it.offset;
-    };
-    // chunks that follow one another in a queue and continue the same flow are one operation
-    std::vector<std::vector<ChunkItem>> queues(R);
-    for (int q = 0; q < R; q++)
-      for (const ChunkItem& it : st.queues[q]) {
-        if (!queues[q].empty() && queues[q].back().flow == it.flow && queues[q].back().offset + queues[q].back().bytes == it.offset)
-          queues[q].back().bytes += it.bytes;
-        else
-          queues[q].push_back(it);
-      }
-    std::vector<cudaGraphNode_t> tails;
-    if (c->path == HOCCL_PATH_CE) {
-      for (int q = 0; q < R && err == cudaSuccess; q++) {
-        cudaGraphNode_t prev = stage_dep;
-        for (const ChunkItem& it : queues[q]) {
-          const char* src;
-          char* dst;
-          endpoints(it, &src, &dst);
-          cudaGraphNode_t n;
-          err = cudaGraphAddMemcpyNode1D(&n, g, prev ? &prev : nullptr, prev ? 1 : 0, dst, src, it.bytes, cudaMemcpyDeviceToDevice);
-          if (err != cudaSuccess) break;
-          prev = n;
-          entry->n_moves++;
-        }
-        if (prev && prev != stage_dep) tails.push_back(prev);
-      }
-    } else {
-      size_t depth = 0;
-      for (int q = 0; q < R; q++) depth = std::max(depth, queues[q].size());
-      cudaGraphNode_t prev = stage_dep;
-      auto add_launch = [&](CopyBatch& b) {
-        prepare_copy_batch(&b, (int)c->copy_ctas);
-        void* args[] = {&b};
-        cudaKernelNodeParams kp = {};
-        int threads = 0;
-        kp.func = const_cast<void*>(copy_kernel_entry((int)c->copy_ctas, &threads));
-        kp.gridDim = dim3((unsigned)c->copy_ctas);
-        kp.blockDim = dim3((unsigned)threads);
-        kp.kernelParams = args;
-        cudaGraphNode_t n;
-        err = cudaGraphAddKernelNode(&n, g, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
-        if (err == cudaSuccess) {
-          prev = n;
-          entry->n_move_launches++;
-        }
-        b.nseg = 0;
-      };
-      for (size_t k = 0; k < depth && err == cudaSuccess; k++) {
-        CopyBatch b;
-        b.nseg = 0;
-        b.pad = 0;
-        for (int q = 0; q < R && err == cudaSuccess; q++) {
-          if (k >= queues[q].size()) continue;
-          const char* src;
-          char* dst;
-          endpoints(queues[q][k], &src, &dst);
-          b.seg[b.nseg++] = CopySeg{src, dst, (unsigned long long)queues[q][k].bytes};
-          entry->n_moves++;
-          if (b.nseg == kMaxSegs) add_launch(b);
-        }
-        if (b.nseg > 0 && err == cudaSuccess) add_launch(b);
-      }
-      if (prev && prev != stage_dep) tails.push_back(prev);
-    }
-    if (err != cudaSuccess) break;
-    if (tails.size() == 1) {
-      stage_dep = tails[0];
-    } else if (tails.size() > 1) {
-      cudaGraphNode_t join;
-      if (c->path == HOCCL_PATH_CE && c->order_kernels) {   // copy chains wait for copy chains: an empty kernel as the join (see build_graph)
-        cudaKernelNodeParams kp = {};
-        kp.func = const_cast<void*>(graph_root_kernel_entry());
-        kp.gridDim = dim3(1);
-        kp.blockDim = dim3(32);
-        kp.kernelParams = nullptr;
-        err = cudaGraphAddKernelNode(&join, g, tails.data(), tails.size(), &kp);
-        if (err == cudaSuccess) entry->n_order_launches++;
-      } else {
-        err = cudaGraphAddEmptyNode(&join, g, tails.data(), tails.size());
-      }
-      if (err == cudaSuccess) stage_dep = join;
-    }
-  }
-  hoccl_result_t rc = HOCCL_OK;
-  if (err == cudaSuccess) err = cudaGraphInstantiate(&entry->exec, g, 0);
-  if (err != cudaSuccess) rc = cuda_fail(c, err, "pattern graph");
-  cudaGraphDestroy(g);
-  entry->n_pieces = (long)S.stages.size();
-  if (rc != HOCCL_OK) destroy_entry(entry);
-  return rc;
-}
-
-// The same for a MODELLED topology with more than one node (paper Sec. 3.4, Eq. 2-4 and Algorithm 1 run as real copies on one
-// device).  A logical flow u -> v between two nodes is carried, portion by portion as Algorithm 1 stages it, by three copies
+// The schedule of a user-defined pattern over a MODELLED topology with more than one node as a CUDA graph (paper Sec. 3.4, Eq. 2-4
+// and Algorithm 1 run as real copies on one device).  A logical flow u -> v between two nodes is carried, portion by portion as Algorithm 1 stages it, by three copies
 // per chunk: the sender-side forwarding copy f' from u's send buffer into a staging slot at u's symmetric peer, the "RDMA"
 // leg f from that slot into a staging slot at v's symmetric peer (optionally cut into serial sub-copies of `rdma_sub` bytes, a
 // crude stand-in for the slower domain), and the receiver-side forwarding copy f'' from there into v's receive buffer.

@@ -59,7 +59,7 @@ def test_an_all_to_all_of_eight_ranks_is_one_launch():
 
 
 @pytest.mark.parametrize("op", ["allgather", "alltoall", "allreduce"])
-@pytest.mark.parametrize("count", [(1 << 20) - 8, (1 << 20) + 1, 600_064, 1 << 20])
+@pytest.mark.parametrize("count", [(1 << 20) - 8, (1 << 20) + 1, 1_100_032, 600_064, 1 << 20])
 def test_copies_the_driver_does_badly(op, count):
     """Copy route above the small-message size: blocks of 1 to 2 MiB that end inside a page or start off a 128-byte line run on the
     copy kernel (all-gather, all-to-all) or leave their ends to it (all-reduce); whole blocks stay with the driver."""
@@ -88,6 +88,35 @@ def test_copies_the_driver_does_badly(op, count):
                 want = [torch.stack([s.float() for s in send]).sum(0).to(torch.bfloat16)] * R
         torch.cuda.synchronize()
         assert all(torch.equal(recv[r], want[r]) for r in range(R)), (op, count, pad)
-        whole = count * 2 % 4096 == 0 and pad == 0
+        whole = count * 2 % 4096 == 0 and pad == 0 and (op == "allreduce" or count >= 1 << 20)
         assert (comm.last_stats()["n_move_launches"] == 0) == whole, (op, count, pad, comm.last_stats())
+    comm.destroy()
+
+
+@pytest.mark.parametrize("R,mib,width,kernel", [(8, 1, 1024, True), (8, 16, 1024, True), (8, 40, 1024, False), (8, 40, 333, True), (20, 8, 1024, True)])
+def test_route_of_a_user_defined_pattern(R, mib, width, kernel):
+    """Copy route: short patterns, short flows and rows the driver copies badly go to the copy kernel in one launch; the rest is one
+    driver copy per flow.  Uneven flows, one of them empty, displacements with gaps."""
+    rng = np.random.default_rng(mib + width)
+    counts = rng.integers(1, 8, (R, R)) * max(1, (mib << 20) // (2 * width * 32)) * width
+    counts[2, 5] = 0
+    sd = np.cumsum(counts, 1) - counts
+    rd = (np.cumsum(counts, 0) - counts).T + 8 * np.arange(R)[None, :]        # [receiver, sender]
+    if width % 64 == 0:
+        rd = rd + 56 * np.arange(R)[None, :]                                  # gaps of whole 128-byte lines
+    send = [torch.randint(-30000, 30000, (int(counts[u].sum()),), dtype=torch.int16, device="cuda") for u in range(R)]
+    recv = [torch.zeros(int(counts[:, v].sum()) + 64 * R, dtype=torch.int16, device="cuda") for v in range(R)]
+    comm = hb.Comm(R, 0)
+    for rep in range(2):
+        comm.alltoallv(send, counts.ravel(), sd.ravel(), recv, rd.ravel(), "bf16")
+        torch.cuda.synchronize()
+        for v in range(R):
+            want = torch.zeros_like(recv[v])
+            for u in range(R):
+                n = int(counts[u, v])
+                want[int(rd[v, u]):int(rd[v, u]) + n] = send[u][int(sd[u, v]):int(sd[u, v]) + n]
+            assert torch.equal(recv[v], want), (rep, v)
+            recv[v].zero_()
+        st = comm.last_stats()
+        assert (st["n_move_launches"], st["n_moves"], st["graph_hit"]) == (int(kernel) * -(-(R * R - 1) // 128), R * R - 1, rep), st
     comm.destroy()

@@ -810,33 +810,25 @@ hoccl_result_t hoccl_fanout_launch(const void* src, void* const* dsts, int ndst,
       if (ranges_overlap((const char*)dsts[k], bytes, (const char*)dsts[d], bytes)) return HOCCL_ERR_INVALID_ARG;
   }
   if (bytes == 0) return HOCCL_OK;
-  // the same grouping as the collectives use: one segment per 16-byte phase of the destinations
-  RGroup g;
-  g.kind = OP_MOVE;
-  g.piece = 0;
-  g.chain_dep = -1;
-  for (int d = 0; d < ndst; d++) {
-    Seg s = {};
-    s.src = (const char*)src;
-    s.dst = (char*)dsts[d];
-    s.bytes = bytes;
-    g.segs.push_back(s);
-  }
-  std::vector<FanBatch> fans;
-  std::vector<double> hbm;
-  std::vector<long> moves;
-  if (!build_fan_batches(g, &fans, &hbm, &moves)) {   // no two destinations share a phase (or there is only one): plain copies
-    for (size_t first = 0; first < g.segs.size(); first += kMaxSegs) {
-      const size_t n = std::min<size_t>(kMaxSegs, g.segs.size() - first);
-      CopyBatch b;
-      fill_copy_batch(g, first, n, &b);
-      if (launch_copy(b, ctas, (cudaStream_t)stream) != cudaSuccess) return HOCCL_ERR_CUDA;
+  // as the collectives do: one segment per 16-byte phase of the destinations
+  MoveBatch b;
+  b.nseg = b.ndst_total = 0;
+  for (unsigned phase = 0; phase < 16; phase++) {
+    std::vector<void*> mine;
+    for (int d = 0; d < ndst; d++)
+      if (((uintptr_t)dsts[d] & 15) == phase) mine.push_back(dsts[d]);
+    for (size_t at = 0; at < bytes && !mine.empty(); at += kMaxMoveSegBytes) {
+      std::vector<void*> here = mine;
+      for (void*& d : here) d = (char*)d + at;
+      const size_t len = std::min<size_t>(kMaxMoveSegBytes, bytes - at);
+      if (!add_move_seg(&b, (const char*)src + at, here.data(), (int)here.size(), len)) {
+        if (launch_moves(&b, ctas, (cudaStream_t)stream) != cudaSuccess) return HOCCL_ERR_CUDA;
+        b.nseg = b.ndst_total = 0;
+        add_move_seg(&b, (const char*)src + at, here.data(), (int)here.size(), len);
+      }
     }
-    return HOCCL_OK;
   }
-  for (const FanBatch& f : fans)
-    if (launch_fan(f, ctas, (cudaStream_t)stream) != cudaSuccess) return HOCCL_ERR_CUDA;
-  return HOCCL_OK;
+  return launch_moves(&b, ctas, (cudaStream_t)stream) == cudaSuccess ? HOCCL_OK : HOCCL_ERR_CUDA;
 }
 
 // ---------------------------------------------------------------- plan inspection ----------------

@@ -227,7 +227,6 @@ struct Tally {
 // The kernel launches that carry out one group: its sums, or (SM route) its moves.
 std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, const RGroup& g);
 cudaError_t launch_kernel(const KernelLaunch& k, cudaStream_t stream);
-void fill_copy_batch(const RGroup& g, size_t first, size_t n, CopyBatch* b);
 // Moves of a group that read the same bytes (same source and length; the direct all-gather on the SM path) become fan-out
 // segments: one read, one store per destination.  Returns false (and leaves *out empty) if no source repeats: the plain
 // copy batches are used then.  bytes_out[i] = HBM bytes of batch i (reads + writes), moves_out[i] = moves it carries.

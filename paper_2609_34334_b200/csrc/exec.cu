@@ -77,7 +77,6 @@ static void share_host_legs(std::vector<RGroup>* groups, size_t* host_need) {
   }
 }
 
-constexpr size_t kStoreAllBytesPerCta = 384 << 10;
 constexpr size_t kGradeInPlace = 4 << 20;   // ring chunk from which pieces are graded on the SM path when contributions are read in place
 
 // How the direct reduce-scatter's contributions reach the owner's sum.
@@ -341,15 +340,6 @@ bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<
   return true;
 }
 
-void fill_copy_batch(const RGroup& g, size_t first, size_t n, CopyBatch* b) {
-  b->nseg = (int)n;
-  b->pad = 0;
-  for (size_t i = 0; i < n; i++) {
-    const Seg& s = g.segs[first + i];
-    b->seg[i] = CopySeg{s.src, s.dst, (unsigned long long)s.bytes};
-  }
-}
-
 // Fills *b with chain segments of g from `first` on; returns how many fitted.
 static size_t fill_chain_batch(const RGroup& g, size_t first, int dtype, size_t elem, ChainBatch* b) {
   b->nseg = 0;
@@ -386,28 +376,19 @@ static KernelLaunch make_launch(const Batch& b, const void* fn, long grid, int t
   return k;
 }
 
-// move_kernel serves a group whose copies it can do wide and copy_kernel cannot (some source and destination differ modulo 16
-// and are long enough to have a body), long copies to destinations off the 128-byte lines (it aligns its stores to them: in-place
-// all-gather of 8 ragged chunks of 5 MiB 78 -> 67 us), and a group of more copies than one batch of copy_kernel holds (an
-// all-to-all of 8 ranks: one launch instead of two).
-static bool wants_move_kernel(const RGroup& g) {
-  for (const Seg& s : g.segs)
-    if (((((uintptr_t)s.src ^ (uintptr_t)s.dst) & 15) && s.bytes >= 64) || (((uintptr_t)s.dst & 127) && s.bytes >= kMoveLineBytes)) return true;
-  bool repeats = false;
-  return g.segs.size() > (size_t)kMaxSegs && move_classes(g, &repeats).size() > (size_t)kMaxSegs;
-}
-
 static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup& g) {
   std::vector<KernelLaunch> out;
   int threads = 0;
-  const void* fn = move_kernel_entry((int)c->copy_ctas, &threads);
   MoveBatch b;
   b.nseg = b.ndst_total = 0;
   double bytes = 0;
   auto flush = [&]() {
     if (b.nseg == 0) return;
     prepare_move_batch(&b, (int)c->copy_ctas);
-    out.push_back(make_launch(b, fn, c->copy_ctas, threads, bytes, b.ndst_total));
+    MoveBatchSmall small;
+    const bool fits = shrink_move_batch(b, &small);
+    const void* fn = move_kernel_entry((int)c->copy_ctas, fits, &threads);
+    out.push_back(fits ? make_launch(small, fn, c->copy_ctas, threads, bytes, b.ndst_total) : make_launch(b, fn, c->copy_ctas, threads, bytes, b.ndst_total));
     b.nseg = b.ndst_total = 0;
     bytes = 0;
   };
@@ -464,28 +445,7 @@ std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, co
     }
     return out;
   }
-  if (wants_move_kernel(g)) return move_launches(c, g);
-  std::vector<FanBatch> fans;
-  std::vector<double> fan_bytes;
-  std::vector<long> fan_moves;
-  if (P.ag_direct && build_fan_batches(g, &fans, &fan_bytes, &fan_moves)) {
-    const void* fn = fan_kernel_entry((int)c->copy_ctas, &threads);
-    for (size_t i = 0; i < fans.size(); i++) {
-      prepare_fan_batch(&fans[i], (int)c->copy_ctas);
-      out.push_back(make_launch(fans[i], fn, c->copy_ctas, threads, fan_bytes[i], fan_moves[i]));
-    }
-    return out;
-  }
-  const void* fn = copy_kernel_entry((int)c->copy_ctas, &threads);
-  for (size_t first = 0; first < g.segs.size(); first += kMaxSegs) {
-    CopyBatch b;
-    fill_copy_batch(g, first, std::min<size_t>(kMaxSegs, g.segs.size() - first), &b);
-    double bytes = 0;
-    for (int i = 0; i < b.nseg; i++) bytes += 2.0 * (double)b.seg[i].bytes;
-    prepare_copy_batch(&b, (int)c->copy_ctas);
-    out.push_back(make_launch(b, fn, c->copy_ctas, threads, bytes, b.nseg));
-  }
-  return out;
+  return move_launches(c, g);
 }
 
 cudaError_t launch_kernel(const KernelLaunch& k, cudaStream_t stream) {

@@ -19,6 +19,8 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "device_common.cuh"
 
 namespace hoccl {
@@ -358,70 +360,6 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
   chain_scalar_items<DT, NOPS>(batch);
 }
 
-// Fan-out copy: the tile walk of copy_kernel, but a tile that was loaded once is stored to every destination of its segment.
-template <int U, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1) fan_kernel(const __grid_constant__ FanBatch batch) {
-  const Flat& f = batch.flat;
-  const int nseg = batch.nseg;
-  if (batch.smid_out != nullptr && threadIdx.x == 0) {
-    unsigned id;
-    asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
-    batch.smid_out[blockIdx.x] = id;
-  }
-  const unsigned long long total = (unsigned long long)gridDim.x * blockDim.x;
-  const unsigned long long gt = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-  {
-    const unsigned long long T_all = f.tpre[nseg];
-    const unsigned tile_v = U * blockDim.x;
-    int k = 0;
-    for (unsigned long long t = blockIdx.x; t < T_all; t += gridDim.x) {
-      while (t >= f.tpre[k + 1]) k++;
-      const unsigned long long first = (t - f.tpre[k]) * tile_v;
-      const unsigned long long left = f.nvec[k] - first;
-      const unsigned n_here = left < tile_v ? (unsigned)left : tile_v;
-      const uint4* a = reinterpret_cast<const uint4*>(static_cast<const char*>(batch.seg[k].src) + f.head[k]) + first;
-      void* const* dsts = batch.dst + batch.seg[k].first_dst;
-      const int nd = batch.seg[k].ndst;
-      uint4 va[U];
-      if (n_here == tile_v) {
-#pragma unroll
-        for (int u = 0; u < U; u++) va[u] = __ldcs(a + threadIdx.x + u * blockDim.x);
-        for (int d = 0; d < nd; d++) {
-          uint4* o = reinterpret_cast<uint4*>(static_cast<char*>(dsts[d]) + f.head[k]) + first;
-#pragma unroll
-          for (int u = 0; u < U; u++) o[threadIdx.x + u * blockDim.x] = va[u];
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-          const unsigned i = threadIdx.x + u * blockDim.x;
-          if (i < n_here) va[u] = __ldcs(a + i);
-        }
-        for (int d = 0; d < nd; d++) {
-          uint4* o = reinterpret_cast<uint4*>(static_cast<char*>(dsts[d]) + f.head[k]) + first;
-#pragma unroll
-          for (int u = 0; u < U; u++) {
-            const unsigned i = threadIdx.x + u * blockDim.x;
-            if (i < n_here) o[i] = va[u];
-          }
-        }
-      }
-    }
-  }
-  {
-    const unsigned long long S = f.spre[nseg];
-    int k = 0;
-    for (unsigned long long j = gt; j < S; j += total) {
-      while (j >= f.spre[k + 1]) k++;
-      unsigned long long i = j - f.spre[k];
-      if (i >= f.head[k]) i += f.nvec[k] * 16;
-      const unsigned char v = static_cast<const unsigned char*>(batch.seg[k].src)[i];
-      void* const* dsts = batch.dst + batch.seg[k].first_dst;
-      for (int d = 0; d < batch.seg[k].ndst; d++) static_cast<unsigned char*>(dsts[d])[i] = v;
-    }
-  }
-}
-
 // The 16 bytes that start `sh` bytes into the 32 bytes lo, hi; sh (0..15) is the same for all threads.
 __device__ __forceinline__ uint4 bytes_at(uint4 lo, uint4 hi, unsigned sh) {
   uint32_t w0 = lo.x, w1 = lo.y, w2 = lo.z, w3 = lo.w, w4 = hi.x, w5 = hi.y, w6 = hi.z, w7 = hi.w;
@@ -455,20 +393,22 @@ __device__ __forceinline__ int find_segment(const unsigned* pre, int n, unsigned
   return lo;
 }
 
-// Moves whose source and destination lie differently modulo 16, or too many for the batches above.  Byte by byte such moves ran
-// at a tenth of the copy rate (8 chunks of 500,014 bytes to 8 ranks each: 37 us of a 38 us all-gather).  Here a thread
-// loads the two aligned vectors that hold its 16 bytes (the second is its neighbour's first, an L1 hit), shifts them into place
-// and stores aligned vectors to every destination.
-template <int U, int THREADS>
-__global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant__ MoveBatch batch) {
+// The moves of a launch: copies and fan-outs (one read, ndst stores) of any phase and length, the tile walk of copy_kernel with the
+// tile chosen for the launch.  In phase it is HBM bound with a whole-GPU grid and bound by the SM's stores (62 GB/s) under a CTA
+// budget.  Out of phase a byte-wise copy ran at a tenth of that (8 chunks of 500,014 bytes to 8 ranks each: 37 us of a 38 us
+// all-gather, now 10); here a thread loads the two aligned vectors that hold its 16 bytes (the second is its neighbour's first, an
+// L1 hit), shifts them into place and stores aligned vectors.
+template <int U, int THREADS, class Batch>
+__global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant__ Batch batch) {
   const int nseg = batch.nseg;
-  const unsigned T_all = batch.tpre[nseg];
+  const unsigned T_all = batch.tpre[nseg], tile_u = batch.tile_u;
   if (blockIdx.x < T_all) {
     int k = find_segment(batch.tpre, nseg, blockIdx.x);
     for (unsigned t = blockIdx.x; t < T_all; t += gridDim.x) {
       while (t >= batch.tpre[k + 1]) k++;
       const MoveSeg& sg = batch.seg[k];
-      const unsigned first = (t - batch.tpre[k]) * (U * THREADS) + threadIdx.x;
+      const unsigned first = (t - batch.tpre[k]) * (tile_u * THREADS) + threadIdx.x;
+      const unsigned tile_end = (t - batch.tpre[k] + 1) * (tile_u * THREADS), end = tile_end < sg.nvec ? tile_end : sg.nvec;
       const char* s = static_cast<const char*>(sg.src) + sg.head;
       const unsigned sh = (unsigned)(uintptr_t)s & 15;
       const uint4* a = reinterpret_cast<const uint4*>(s - sh) + first;
@@ -476,14 +416,14 @@ __global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant_
       if (sh == 0) {
 #pragma unroll
         for (int u = 0; u < U; u++)
-          if (first + u * THREADS < sg.nvec) v[u] = __ldcs(a + u * THREADS);
+          if (first + u * THREADS < end) v[u] = __ldcs(a + u * THREADS);
       } else {
 #pragma unroll
         for (int h = 0; h < U; h += 4) {   // 4 pairs in flight
           uint4 hi[4];
 #pragma unroll
           for (int u = 0; u < 4; u++)
-            if (first + (h + u) * THREADS < sg.nvec) {
+            if (first + (h + u) * THREADS < end) {
               v[h + u] = a[(h + u) * THREADS];
               hi[u] = a[(h + u) * THREADS + 1];
             }
@@ -495,7 +435,7 @@ __global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant_
         uint4* o = reinterpret_cast<uint4*>(static_cast<char*>(batch.dst[sg.first_dst + d]) + sg.head) + first;
 #pragma unroll
         for (int u = 0; u < U; u++)
-          if (first + u * THREADS < sg.nvec) o[u * THREADS] = v[u];
+          if (first + u * THREADS < end) o[u * THREADS] = v[u];
       }
     }
   }
@@ -838,17 +778,8 @@ void prepare_fan_batch(FanBatch* b, int ctas) {
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
 }
 
-cudaError_t launch_fan(const FanBatch& batch, int ctas, cudaStream_t stream) {
-  if (batch.nseg <= 0) return cudaSuccess;
-  FanBatch b = batch;
-  prepare_fan_batch(&b, ctas);
-  if (wide_copy_grid(ctas)) fan_kernel<4, 512><<<ctas, 512, 0, stream>>>(b);
-  else fan_kernel<8, 1024><<<ctas, 1024, 0, stream>>>(b);
-  return cudaGetLastError();
-}
-
 bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, unsigned long long bytes) {
-  if (b->nseg == kMaxMoveSegs || b->ndst_total + ndst > kMaxMoveDsts) return false;
+  if (b->nseg == MoveBatch::kSegs || b->ndst_total + ndst > MoveBatch::kDsts) return false;
   MoveSeg& s = b->seg[b->nseg++];
   s.src = src;
   s.bytes = bytes;
@@ -859,8 +790,8 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
 }
 
 void prepare_move_batch(MoveBatch* b, int ctas) {
-  const unsigned tile_v = wide_copy_grid(ctas) ? 4u * 512 : 8u * 1024;
-  b->tpre[0] = b->spre[0] = 0;
+  const unsigned threads = wide_copy_grid(ctas) ? 512 : 1024, most_u = wide_copy_grid(ctas) ? 4 : 8;
+  b->spre[0] = 0;
   for (int k = 0; k < b->nseg; k++) {
     MoveSeg& s = b->seg[k];
     const unsigned long long at = (uintptr_t)s.src & 15;
@@ -875,14 +806,65 @@ void prepare_move_batch(MoveBatch* b, int ctas) {
     else head = 0;
     s.head = (unsigned)head;
     s.nvec = (unsigned)nvec;
-    b->tpre[k + 1] = b->tpre[k] + (unsigned)((nvec + tile_v - 1) / tile_v);
     b->spre[k + 1] = b->spre[k] + (unsigned)(s.bytes - nvec * 16);
   }
+  // Tiles: as large as a thread's registers hold (a tile's loads are in flight together), smaller where that would leave CTAs
+  // without a tile or with one more than others.  In units of one vector per thread stored once, a tile costs its stores and ~3 for
+  // the loads to come back; the grid runs ceil(tiles / ctas) of them one after another.
+  double best = 0;
+  for (unsigned u = most_u; u >= 1; u /= 2) {
+    unsigned long long tiles = 0;
+    for (int k = 0; k < b->nseg; k++) tiles += (b->seg[k].nvec + u * threads - 1) / (u * threads);
+    const double per_tile = 3.0 + (double)u * b->ndst_total / (b->nseg > 0 ? b->nseg : 1);
+    const double cost = (double)((tiles + ctas - 1) / ctas) * per_tile;
+    if (u == most_u || cost < best) {
+      best = cost;
+      b->tile_u = u;
+    }
+  }
+  b->tpre[0] = 0;
+  for (int k = 0; k < b->nseg; k++) b->tpre[k + 1] = b->tpre[k] + (b->seg[k].nvec + b->tile_u * threads - 1) / (b->tile_u * threads);
 }
 
-const void* move_kernel_entry(int ctas, int* threads) {
-  *threads = wide_copy_grid(ctas) ? 512 : 1024;
-  return wide_copy_grid(ctas) ? reinterpret_cast<const void*>(&move_kernel<4, 512>) : reinterpret_cast<const void*>(&move_kernel<8, 1024>);
+bool shrink_move_batch(const MoveBatch& b, MoveBatchSmall* o) {
+  if (b.nseg > MoveBatchSmall::kSegs || b.ndst_total > MoveBatchSmall::kDsts) return false;
+  o->nseg = b.nseg;
+  o->ndst_total = b.ndst_total;
+  o->tile_u = b.tile_u;
+  std::copy(b.seg, b.seg + b.nseg, o->seg);
+  std::copy(b.dst, b.dst + b.ndst_total, o->dst);
+  std::copy(b.tpre, b.tpre + b.nseg + 1, o->tpre);
+  std::copy(b.spre, b.spre + b.nseg + 1, o->spre);
+  return true;
+}
+
+const void* move_kernel_entry(int ctas, bool small, int* threads) {
+  const bool wide = wide_copy_grid(ctas);
+  *threads = wide ? 512 : 1024;
+  if (small)
+    return wide ? reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatchSmall>) : reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatchSmall>);
+  return wide ? reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatch>) : reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatch>);
+}
+
+cudaError_t launch_moves(MoveBatch* b, int ctas, cudaStream_t stream) {
+  if (b->nseg <= 0) return cudaSuccess;
+  prepare_move_batch(b, ctas);
+  MoveBatchSmall small;
+  const bool fits = shrink_move_batch(*b, &small);
+  int threads = 0;
+  const void* fn = move_kernel_entry(ctas, fits, &threads);
+  void* args[1] = {fits ? static_cast<void*>(&small) : static_cast<void*>(b)};
+  return cudaLaunchKernel(fn, dim3((unsigned)ctas), dim3((unsigned)threads), args, 0, stream);
+}
+
+cudaError_t launch_move(const void* src, void* dst, unsigned long long bytes, int ctas, cudaStream_t stream) {
+  MoveBatch b;
+  b.nseg = b.ndst_total = 0;
+  for (unsigned long long at = 0; at < bytes; at += kMaxMoveSegBytes) {
+    void* d = static_cast<char*>(dst) + at;
+    add_move_seg(&b, static_cast<const char*>(src) + at, &d, 1, std::min(kMaxMoveSegBytes, bytes - at));
+  }
+  return launch_moves(&b, ctas, stream);
 }
 
 cudaError_t launch_sum(const SumBatch& batch, int ctas, cudaStream_t stream) {
@@ -947,11 +929,6 @@ const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads) 
   return v.fn;
 }
 const void* graph_root_kernel_entry() { return reinterpret_cast<const void*>(&graph_root_kernel); }
-const void* fan_kernel_entry(int ctas, int* threads) {
-  *threads = wide_copy_grid(ctas) ? 512 : 1024;
-  return wide_copy_grid(ctas) ? reinterpret_cast<const void*>(&fan_kernel<4, 512>) : reinterpret_cast<const void*>(&fan_kernel<8, 1024>);
-}
-
 // Forces the module that holds these kernels to be loaded now.  Loading a kernel on first launch can synchronise the
 // device; that must never happen while a stream is parked in a hand-over that only the launching thread can finish.
 cudaError_t preload_kernels() {
@@ -960,9 +937,9 @@ cudaError_t preload_kernels() {
                        reinterpret_cast<const void*>(&copy_kernel<4, 512>),     reinterpret_cast<const void*>(&copy_kernel<8, 1024>),
                        reinterpret_cast<const void*>(&occupy_kernel),           reinterpret_cast<const void*>(&onepass_kernel<0, 512>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 512>),  reinterpret_cast<const void*>(&onepass_kernel<0, 1024>),
-                       reinterpret_cast<const void*>(&onepass_kernel<1, 1024>), reinterpret_cast<const void*>(&fan_kernel<4, 512>),
-                       reinterpret_cast<const void*>(&fan_kernel<8, 1024>), reinterpret_cast<const void*>(&graph_root_kernel),
-                       reinterpret_cast<const void*>(&move_kernel<4, 512>), reinterpret_cast<const void*>(&move_kernel<8, 1024>),
+                       reinterpret_cast<const void*>(&onepass_kernel<1, 1024>), reinterpret_cast<const void*>(&graph_root_kernel),
+                       reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatch>), reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatch>),
+                       reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatchSmall>), reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatchSmall>),
                        reinterpret_cast<const void*>(&chain_kernel<0, 1024>), reinterpret_cast<const void*>(&chain_kernel<1, 1024>)};
   for (const void* f : fns) {
     cudaFuncAttributes a;

@@ -46,6 +46,9 @@ struct ChainSeg {
 };
 constexpr int kMaxChainSrcs = 63;     // inbox operands of hoccl_chain_launch
 constexpr int kMaxChainPtrs = 512;
+// A sum stores the result for every rank itself instead of leaving it to a launch of copies when R * S bytes are at most this
+// many per summing CTA: see contributions() for the measurement.
+constexpr size_t kStoreAllBytesPerCta = 384 << 10;
 constexpr unsigned long long kMaxChainSegBytes = 1ull << 30;
 struct ChainBatch {
   int nseg;
@@ -72,7 +75,7 @@ struct CopyBatch {
   unsigned int* smid_out = nullptr;  // diagnostics, as in SumBatch
 };
 
-// One fan-out segment: every dst[first_dst + d][0..bytes), d < ndst, <- src[0..bytes).  The source is read once and stored ndst
+// Fan-out segments as the roles kernel and the host-only inspection pack them: every dst[first_dst + d][0..bytes), d < ndst, <- src[0..bytes).  The source is read once and stored ndst
 // times (the direct all-gather on the SM path: a rank's chunk goes to all its peers, 1 + ndst instead of 2 ndst bytes of
 // traffic per chunk byte).  All addresses of a segment share their 16-byte phase or the segment runs element-wise.
 constexpr int kMaxFanDsts = 256;
@@ -86,16 +89,14 @@ struct FanBatch {
   int ndst_total;
   FanSeg seg[kMaxSegs];
   void* dst[kMaxFanDsts];
-  Flat flat;  // filled by prepare_fan_batch (launch_fan does it itself)
+  Flat flat;  // filled by prepare_fan_batch
   unsigned int* smid_out = nullptr;  // diagnostics, as in SumBatch
 };
 
-// Moves of one launch that copy_kernel and fan_kernel do not serve well: sources and destinations out of phase (their addresses
-// differ modulo 16), or more segments than those batches hold.  A segment is stored to ndst destinations of one phase; its body
-// is cut at the destination's 16-byte boundaries and, if the source lies differently, kept away from both ends of the source
-// far enough that the aligned vectors that hold its bytes lie inside the source.  Tiles and vectors fit 32 bits (a segment has
-// at most kMaxMoveSegBytes bytes).
-constexpr int kMaxMoveSegs = 128, kMaxMoveDsts = 512;
+// The moves of one launch (move_kernel).  A segment is read once and stored to ndst destinations of one 16-byte phase (the direct
+// all-gather: a chunk goes to all peers); its body is cut at the destination's 16-byte vectors, or 128-byte lines if it is long,
+// and, if the source lies differently modulo 16, kept away from both ends of the source far enough that the aligned vectors that
+// hold its bytes lie inside the source.  Tiles and vectors fit 32 bits (a segment has at most kMaxMoveSegBytes bytes).
 constexpr unsigned long long kMaxMoveSegBytes = 8ull << 30;
 constexpr unsigned long long kMoveLineBytes = 64 << 10;   // segments from this length on are cut at the destination's 128-byte lines
 struct MoveSeg {
@@ -105,19 +106,28 @@ struct MoveSeg {
   unsigned long long bytes;
   int first_dst, ndst;
 };
-struct MoveBatch {
+template <int NSEG, int NDST>
+struct MoveBatchT {
+  static constexpr int kSegs = NSEG, kDsts = NDST;
   int nseg;
   int ndst_total;
-  MoveSeg seg[kMaxMoveSegs];
-  void* dst[kMaxMoveDsts];
-  unsigned int tpre[kMaxMoveSegs + 1];   // prefix sums of vector tiles
-  unsigned int spre[kMaxMoveSegs + 1];   // prefix sums of byte-wise items
+  unsigned int tile_u;            // vectors per thread of a tile, chosen by prepare_move_batch
+  MoveSeg seg[NSEG];
+  void* dst[NDST];
+  unsigned int tpre[NSEG + 1];    // prefix sums of vector tiles
+  unsigned int spre[NSEG + 1];    // prefix sums of byte-wise items
 };
-// Appends a segment (all destinations in one phase); false if the batch has no room for it.  Batches are prepared with the CTA
-// count they are launched with.
+// Batches are built large; what fits is launched small (a launch outside a graph copies 1.3 KB of parameters instead of 9).
+using MoveBatch = MoveBatchT<128, 512>;
+using MoveBatchSmall = MoveBatchT<16, 64>;
+// Appends a segment (all destinations in one phase); false if the batch has no room for it.
 bool add_move_seg(MoveBatch* batch, const void* src, void* const* dsts, int ndst, unsigned long long bytes);
+// Batches are prepared with the CTA count they are launched with.
 void prepare_move_batch(MoveBatch* batch, int ctas);
-const void* move_kernel_entry(int ctas, int* threads);
+bool shrink_move_batch(const MoveBatch& batch, MoveBatchSmall* out);   // false if it does not fit
+const void* move_kernel_entry(int ctas, bool small, int* threads);
+cudaError_t launch_moves(MoveBatch* batch, int ctas, cudaStream_t stream);   // prepares and launches; nothing for an empty batch
+cudaError_t launch_move(const void* src, void* dst, unsigned long long bytes, int ctas, cudaStream_t stream);   // one copy
 
 // One-pass variant of the ring reduction (comparison point, not rank local): every element is reduced in registers in
 // the ring's order, chunk c as ((x_{c+1} + x_{c+2}) + ... ) + x_c with a rounding to the I/O dtype after every add, and
@@ -191,9 +201,7 @@ bool add_chain_seg(ChainBatch* batch, const void* const* ops, int nops, void* co
 const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads);
 // counts: two device words, zeroed by the caller; see bf16_add_selftest_kernel
 cudaError_t launch_bf16_add_selftest(unsigned long long* counts, cudaStream_t stream);
-cudaError_t launch_fan(const FanBatch& batch, int ctas, cudaStream_t stream);
 void prepare_fan_batch(FanBatch* batch, int ctas);
-const void* fan_kernel_entry(int ctas, int* threads);
 // Fill batch->flat for the kernel variant that `ctas` CTAs select (needed before a batch is handed to a graph kernel node).
 void prepare_sum_batch(SumBatch* batch, int ctas);
 void prepare_copy_batch(CopyBatch* batch, int ctas);

@@ -129,11 +129,7 @@ hoccl_result_t p2p_post(hoccl_comm* c, bool is_send, void* buf, size_t count, in
     if (c->path == HOCCL_PATH_CE) {
       CU_TRY(c, cudaMemcpyAsync(dbuf, sbuf, bytes, cudaMemcpyDeviceToDevice, stream));
     } else {
-      CopyBatch b;
-      b.nseg = 1;
-      b.pad = 0;
-      b.seg[0] = CopySeg{sbuf, dbuf, (unsigned long long)bytes};
-      CU_TRY(c, launch_copy(b, (int)c->copy_ctas, stream));
+      CU_TRY(c, launch_move(sbuf, dbuf, bytes, (int)c->copy_ctas, stream));
       c->stats.n_move_launches = 1;
       c->stats.max_copy_ctas = c->copy_ctas;
     }
@@ -157,11 +153,7 @@ hoccl_result_t p2p_post(hoccl_comm* c, bool is_send, void* buf, size_t count, in
       if (c->path == HOCCL_PATH_CE) {
         CU_TRY(c, cudaMemcpyAsync((char*)dbuf + off, (const char*)sbuf + off, len, cudaMemcpyDeviceToDevice, run));
       } else {
-        CopyBatch b;
-        b.nseg = 1;
-        b.pad = 0;
-        b.seg[0] = CopySeg{(const char*)sbuf + off, (char*)dbuf + off, (unsigned long long)len};
-        CU_TRY(c, launch_copy(b, (int)c->copy_ctas, run));
+        CU_TRY(c, launch_move((const char*)sbuf + off, (char*)dbuf + off, len, (int)c->copy_ctas, run));
         c->stats.n_move_launches++;
         c->stats.max_copy_ctas = c->copy_ctas;
       }

@@ -84,11 +84,7 @@ cudaError_t Proxy::init() {
   e = cudaMemsetAsync(warm_, 0, 512, stream_);
   if (e == cudaSuccess) e = cudaMemcpyAsync(static_cast<char*>(warm_) + 256, warm_, 256, cudaMemcpyDeviceToDevice, stream_);
   if (e == cudaSuccess) {
-    CopyBatch b;
-    b.nseg = 1;
-    b.pad = 0;
-    b.seg[0] = CopySeg{warm_, static_cast<char*>(warm_) + 256, 256};
-    e = launch_copy(b, 1, stream_);
+    e = launch_move(warm_, static_cast<char*>(warm_) + 256, 256, 1, stream_);
   }
   cudaGraph_t g = nullptr;
   cudaGraphExec_t ge = nullptr;
@@ -344,11 +340,7 @@ void Proxy::loop() {
             if (s.task.path == 0) {
               e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, stream_);
             } else {
-              CopyBatch b;
-              b.nseg = 1;
-              b.pad = 0;
-              b.seg[0] = CopySeg{src, dst, (unsigned long long)bytes};
-              e = launch_copy(b, s.task.copy_ctas, stream_);
+              e = launch_move(src, dst, bytes, s.task.copy_ctas, stream_);
             }
           }
           if (e == cudaSuccess) e = cudaEventRecord(s.done, stream_);

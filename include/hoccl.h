@@ -454,6 +454,9 @@ hoccl_result_t hoccl_host_allreduce(const void* const* h_send, void* const* h_re
  * in-place and no-overlap rules as hoccl_allreduce).  R: number of logical ranks, 1..64.  `stream` must
  * belong to the device that is current when the call is made.
  *
+ * Buffers that share their address modulo 16 do without the array: the chain sum (8 CTAs) reads the contributions where they lie
+ * and one launch of moves (32 CTAs), or for short vectors the sum itself, brings the result to every rank.
+ *
  * Limits and sharing.  The scratch need is 2 * R * roundup256(ceil(count/R) * sizeof(dtype) + 16) bytes;
  * a call that would need more than HOCCL_STATIC_SCRATCH_BYTES is rejected with HOCCL_ERR_SCRATCH and
  * enqueues nothing (with R = 8 this allows a little under 16 MiB per rank buffer).  All calls on a device

@@ -9,6 +9,10 @@
 //
 // Nothing here calls cudaMalloc, cudaFree, or creates streams, events or graphs: the whole schedule is
 // issued as kernel launches on the caller's stream in the planner's (topological) order.
+//
+// Buffers that share their address modulo 16 (the usual case) do not need the scratch at all: the chain sum reads every rank's
+// contribution where it lies, as the communicator's automatic schedule does, and one launch of moves, or the sum itself, brings
+// the result to every rank (6 ranks of 500,009 fp32: 123 us as a ring of 15 launches, 26 us as two).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -45,6 +49,45 @@ cudaError_t scratch_base(int device, void** out) {
   return cudaSuccess;
 }
 
+// The all-reduce in one or two launches for buffers of one 16-byte phase.  q: elements of a full ring chunk.
+cudaError_t read_in_place(const void* const* send, void* const* recv, size_t count, size_t q, int dtype, size_t e, int R, cudaStream_t st) {
+  const bool store_all = (size_t)R * count * e <= (size_t)kStaticSumCtas * kStoreAllBytesPerCta;
+  ChainBatch b;
+  MoveBatch m;
+  b.dtype = dtype;
+  b.nseg = b.nptr = 0;
+  m.nseg = m.ndst_total = 0;
+  cudaError_t err = cudaSuccess;
+  // all sums first: a chunk is final before any move of it is issued
+  for (int c = 0; c < R && err == cudaSuccess; c++) {
+    const size_t lo = std::min((size_t)c * q, count), n = std::min(lo + q, count) - lo;
+    if (!n) continue;
+    const void* ops[64];
+    void* dsts[64];
+    for (int j = 1; j <= R; j++) ops[j - 1] = (const char*)send[(c + j) % R] + lo * e;
+    for (int r = 0; r < R; r++) dsts[r] = (char*)recv[(c + r) % R] + lo * e;   // the owner's first
+    const int ndst = store_all ? R : 1;
+    if (!add_chain_seg(&b, ops, R, dsts, ndst, (unsigned long long)n)) {
+      err = launch_chain(b, kStaticSumCtas, st);
+      b.nseg = b.nptr = 0;
+      add_chain_seg(&b, ops, R, dsts, ndst, (unsigned long long)n);
+    }
+  }
+  if (err == cudaSuccess) err = launch_chain(b, kStaticSumCtas, st);
+  for (int c = 0; c < R && !store_all && err == cudaSuccess; c++) {
+    const size_t lo = std::min((size_t)c * q, count), n = std::min(lo + q, count) - lo;
+    if (!n) continue;
+    void* dsts[64];
+    for (int k = 1; k < R; k++) dsts[k - 1] = (char*)recv[(c + k) % R] + lo * e;
+    if (!add_move_seg(&m, (const char*)recv[c] + lo * e, dsts, R - 1, (unsigned long long)(n * e))) {
+      err = launch_moves(&m, kStaticCopyCtas, st);
+      m.nseg = m.ndst_total = 0;
+      add_move_seg(&m, (const char*)recv[c] + lo * e, dsts, R - 1, (unsigned long long)(n * e));
+    }
+  }
+  return err == cudaSuccess ? launch_moves(&m, kStaticCopyCtas, st) : err;
+}
+
 bool overlap(const char* a, size_t an, const char* b, size_t bn) { return an && bn && a < b + bn && b < a + an; }
 
 }  // namespace
@@ -71,6 +114,15 @@ extern "C" hoccl_result_t hoccl_allreduce_static(const void* const* send, void* 
         return HOCCL_ERR_INVALID_ARG;
     }
   if (count == 0) return HOCCL_OK;
+
+  if (R > 1) {
+    const size_t q = (count + R - 1) / R;
+    if (2 * (size_t)R * ((q * e + 16 + 255) / 256 * 256) > (size_t)HOCCL_STATIC_SCRATCH_BYTES) return HOCCL_ERR_SCRATCH;
+    bool one_phase = true;
+    for (int r = 0; r < R; r++) one_phase = one_phase && !((((uintptr_t)send[r] ^ (uintptr_t)send[0]) | ((uintptr_t)recv[r] ^ (uintptr_t)send[0])) & 15);
+    if (one_phase)
+      return read_in_place(send, recv, count, q, (int)dtype, e, R, (cudaStream_t)stream) == cudaSuccess ? HOCCL_OK : HOCCL_ERR_CUDA;
+  }
 
   // one piece per ring chunk: the schedule runs on one stream, so pieces would buy nothing
   Plan P;

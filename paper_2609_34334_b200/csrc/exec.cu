@@ -387,7 +387,7 @@ static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup
     prepare_move_batch(&b, (int)c->copy_ctas);
     MoveBatchSmall small;
     const bool fits = shrink_move_batch(b, &small);
-    const void* fn = move_kernel_entry((int)c->copy_ctas, fits, &threads);
+    const void* fn = move_kernel_entry(b, (int)c->copy_ctas, fits, &threads);
     out.push_back(fits ? make_launch(small, fn, c->copy_ctas, threads, bytes, b.ndst_total) : make_launch(b, fn, c->copy_ctas, threads, bytes, b.ndst_total));
     b.nseg = b.ndst_total = 0;
     bytes = 0;

@@ -324,38 +324,51 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
   using T = Traits<DT>;
   const Flat& f = batch.flat;
   report_sm(batch);
+  // tile t of the flattened space belongs to CTA t mod grid; walked segment by segment, so that the 2 NOPS pointers are loaded
+  // once per segment and not once per tile (R = 8, 64 MiB fp32, tiles of 384 vectors: 194 us with a look-up per tile, 171 without)
   const unsigned long long T_all = f.tpre[batch.nseg];
   int k = 0;
-  for (unsigned long long t = blockIdx.x; t < T_all; t += gridDim.x) {
-    while (t >= f.tpre[k + 1]) k++;
-    void* const* ptr = batch.ptr + batch.seg[k].first_ptr;
-    const unsigned v0 = (unsigned)(t - f.tpre[k]) * (U * THREADS) + threadIdx.x;   // first vector of this thread in segment k
-    const unsigned off = f.head[k] * T::E + v0 * 16;
-    const unsigned nvec = (unsigned)f.nvec[k];
-    auto finish = [&](const uint4(&bb)[NOPS], int u) {
-      uint4 acc = bb[0];
+  for (unsigned long long at = blockIdx.x; at < T_all;) {
+    while (at >= f.tpre[k + 1]) k++;
+    const unsigned tiles = (unsigned)(f.tpre[k + 1] - f.tpre[k]);
+    const char* src[NOPS];
+    char* dst[NOPS];
 #pragma unroll
-      for (int q = 1; q < NOPS; q++) acc = chain_add<DT>(acc, bb[q]);
+    for (int q = 0; q < NOPS; q++) {
+      src[q] = static_cast<const char*>(batch.ptr[batch.seg[k].first_ptr + q]);
+      dst[q] = static_cast<char*>(batch.ptr[batch.seg[k].first_ptr + NOPS + q]);
+    }
+    const unsigned nvec = (unsigned)f.nvec[k], head = f.head[k] * T::E;
+    unsigned t = (unsigned)(at - f.tpre[k]);
+    for (; t < tiles; t += gridDim.x) {
+      const unsigned v0 = t * (U * THREADS) + threadIdx.x;   // first vector of this thread
+      const unsigned off = head + v0 * 16;
+      auto finish = [&](const uint4(&bb)[NOPS], int u) {
+        uint4 acc = bb[0];
 #pragma unroll
-      for (int d = 0; d < NOPS; d++) *reinterpret_cast<uint4*>(static_cast<char*>(ptr[NOPS + d]) + (off + u * (THREADS * 16))) = acc;
-    };
-    uint4 buf[U][NOPS];
-    if (v0 + (U - 1) * THREADS < nvec) {
+        for (int q = 1; q < NOPS; q++) acc = chain_add<DT>(acc, bb[q]);
 #pragma unroll
-      for (int u = 0; u < U; u++)
+        for (int d = 0; d < NOPS; d++) *reinterpret_cast<uint4*>(dst[d] + (off + u * (THREADS * 16))) = acc;
+      };
+      uint4 buf[U][NOPS];
+      if (v0 + (U - 1) * THREADS < nvec) {
 #pragma unroll
-        for (int q = 0; q < NOPS; q++) buf[u][q] = __ldcs(reinterpret_cast<const uint4*>(static_cast<const char*>(ptr[q]) + (off + u * (THREADS * 16))));
+        for (int u = 0; u < U; u++)
 #pragma unroll
-      for (int u = 0; u < U; u++) finish(buf[u], u);
-    } else {
+          for (int q = 0; q < NOPS; q++) buf[u][q] = __ldcs(reinterpret_cast<const uint4*>(src[q] + (off + u * (THREADS * 16))));
 #pragma unroll
-      for (int u = 0; u < U; u++) {
-        if (v0 + u * THREADS >= nvec) break;
+        for (int u = 0; u < U; u++) finish(buf[u], u);
+      } else {
 #pragma unroll
-        for (int q = 0; q < NOPS; q++) buf[u][q] = __ldcs(reinterpret_cast<const uint4*>(static_cast<const char*>(ptr[q]) + (off + u * (THREADS * 16))));
-        finish(buf[u], u);
+        for (int u = 0; u < U; u++) {
+          if (v0 + u * THREADS >= nvec) break;
+#pragma unroll
+          for (int q = 0; q < NOPS; q++) buf[u][q] = __ldcs(reinterpret_cast<const uint4*>(src[q] + (off + u * (THREADS * 16))));
+          finish(buf[u], u);
+        }
       }
     }
+    at = f.tpre[k] + t;
   }
   chain_scalar_items<DT, NOPS>(batch);
 }
@@ -400,6 +413,7 @@ __device__ __forceinline__ int find_segment(const unsigned* pre, int n, unsigned
 // L1 hit), shifts them into place and stores aligned vectors.
 template <int U, int THREADS, class Batch>
 __global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant__ Batch batch) {
+  constexpr int H = U < 4 ? U : 4;
   const int nseg = batch.nseg;
   const unsigned T_all = batch.tpre[nseg], tile_u = batch.tile_u;
   if (blockIdx.x < T_all) {
@@ -419,16 +433,16 @@ __global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant_
           if (first + u * THREADS < end) v[u] = __ldcs(a + u * THREADS);
       } else {
 #pragma unroll
-        for (int h = 0; h < U; h += 4) {   // 4 pairs in flight
-          uint4 hi[4];
+        for (int h = 0; h < U; h += H) {   // H pairs in flight
+          uint4 hi[H];
 #pragma unroll
-          for (int u = 0; u < 4; u++)
+          for (int u = 0; u < H; u++)
             if (first + (h + u) * THREADS < end) {
               v[h + u] = a[(h + u) * THREADS];
               hi[u] = a[(h + u) * THREADS + 1];
             }
 #pragma unroll
-          for (int u = 0; u < 4; u++) v[h + u] = bytes_at(v[h + u], hi[u], sh);
+          for (int u = 0; u < H; u++) v[h + u] = bytes_at(v[h + u], hi[u], sh);
         }
       }
       for (int d = 0; d < sg.ndst; d++) {
@@ -696,8 +710,23 @@ static ChainVariant chain_pipe_variant(int nops) {
   }
 }
 template <int DT>
-static ChainVariant chain_fan_variant(int nops) {
-  // U x NOPS loads per thread: 8 to 16
+static ChainVariant chain_fan_variant(int nops, int ctas) {
+  // Whole-GPU grids: 42 to 50 KiB of loads in flight per SM.  More of them make it slower (the reads then come in longer bursts
+  // between the writes): 8 operands of 64 MiB to 8 destinations 5.85 TB/s with 128 KiB, 6.02 with 64, 6.26 with 48, 6.11 with 40; 4
+  // and 4 5.90 with 64, 6.13 with 48; 2 and 2 of 256 MiB 5.85 with 64, 6.27 with 48.
+  if (wide_grid(ctas)) {
+    switch (nops) {
+      case 2: return fan_of<DT, 2, 4, 384>();
+      case 3: return fan_of<DT, 3, 2, 448>();
+      case 4: return fan_of<DT, 4, 2, 384>();
+      case 5: return fan_of<DT, 5, 2, 320>();
+      case 6: return fan_of<DT, 6, 1, 448>();
+      case 7: return fan_of<DT, 7, 1, 416>();
+      case 8: return fan_of<DT, 8, 1, 384>();
+      default: return {nullptr, 0, 0};
+    }
+  }
+  // Few CTAs serve short messages only: U x NOPS loads per thread, 8 to 16
   switch (nops) {
     case 2: return fan_of<DT, 2, 4, 512>();
     case 3: return fan_of<DT, 3, 4, 512>();
@@ -717,7 +746,7 @@ static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
     if (b.seg[k].nops != nops || b.seg[k].ndst != ndst) return plain;
   ChainVariant v = plain;
   if (ndst == 1 && ctas < 128) v = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
-  else if (ndst == nops) v = b.dtype == 0 ? chain_fan_variant<0>(nops) : chain_fan_variant<1>(nops);
+  else if (ndst == nops) v = b.dtype == 0 ? chain_fan_variant<0>(nops, ctas) : chain_fan_variant<1>(nops, ctas);
   return v.fn ? v : plain;
 }
 
@@ -789,8 +818,21 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
   return true;
 }
 
+// Launch shape: a thread keeps up to u vectors.  Under a CTA budget 8 x 1024 (the bytes in flight per SM decide).  Whole-GPU grids
+// are bound by HBM and want less in flight: copies of 64 MiB 5.26 TB/s with 4 x 512, 6.46 with 4 x 640 (256 MiB: 5.9 and 6.2; 8 x 1024: 4.2); one read stored 7 times 5.4 with 4 x 512, 5.9 with 2 x 256.
+struct MoveShape {
+  int u, threads;
+};
+static MoveShape move_shape(const MoveBatch& b, int ctas) {
+  if (!wide_copy_grid(ctas)) return {8, 1024};
+  bool in_phase = true;
+  for (int k = 0; k < b.nseg; k++) in_phase = in_phase && ((((uintptr_t)b.seg[k].src ^ (uintptr_t)b.dst[b.seg[k].first_dst]) & 15) == 0);
+  return in_phase && b.ndst_total >= 2 * b.nseg ? MoveShape{2, 256} : MoveShape{4, 640};
+}
+
 void prepare_move_batch(MoveBatch* b, int ctas) {
-  const unsigned threads = wide_copy_grid(ctas) ? 512 : 1024, most_u = wide_copy_grid(ctas) ? 4 : 8;
+  const MoveShape shape = move_shape(*b, ctas);
+  const unsigned threads = (unsigned)shape.threads, most_u = (unsigned)shape.u;
   b->spre[0] = 0;
   for (int k = 0; k < b->nseg; k++) {
     MoveSeg& s = b->seg[k];
@@ -838,12 +880,18 @@ bool shrink_move_batch(const MoveBatch& b, MoveBatchSmall* o) {
   return true;
 }
 
-const void* move_kernel_entry(int ctas, bool small, int* threads) {
-  const bool wide = wide_copy_grid(ctas);
-  *threads = wide ? 512 : 1024;
-  if (small)
-    return wide ? reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatchSmall>) : reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatchSmall>);
-  return wide ? reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatch>) : reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatch>);
+template <class Batch>
+static const void* move_entry(MoveShape shape) {
+  switch (shape.u * 10000 + shape.threads) {
+    case 40640: return reinterpret_cast<const void*>(&move_kernel<4, 640, Batch>);
+    case 20256: return reinterpret_cast<const void*>(&move_kernel<2, 256, Batch>);
+    default: return reinterpret_cast<const void*>(&move_kernel<8, 1024, Batch>);
+  }
+}
+const void* move_kernel_entry(const MoveBatch& b, int ctas, bool small, int* threads) {
+  const MoveShape s = move_shape(b, ctas);
+  *threads = s.threads;
+  return small ? move_entry<MoveBatchSmall>(s) : move_entry<MoveBatch>(s);
 }
 
 cudaError_t launch_moves(MoveBatch* b, int ctas, cudaStream_t stream) {
@@ -852,7 +900,7 @@ cudaError_t launch_moves(MoveBatch* b, int ctas, cudaStream_t stream) {
   MoveBatchSmall small;
   const bool fits = shrink_move_batch(*b, &small);
   int threads = 0;
-  const void* fn = move_kernel_entry(ctas, fits, &threads);
+  const void* fn = move_kernel_entry(*b, ctas, fits, &threads);
   void* args[1] = {fits ? static_cast<void*>(&small) : static_cast<void*>(b)};
   return cudaLaunchKernel(fn, dim3((unsigned)ctas), dim3((unsigned)threads), args, 0, stream);
 }
@@ -938,8 +986,8 @@ cudaError_t preload_kernels() {
                        reinterpret_cast<const void*>(&occupy_kernel),           reinterpret_cast<const void*>(&onepass_kernel<0, 512>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 512>),  reinterpret_cast<const void*>(&onepass_kernel<0, 1024>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 1024>), reinterpret_cast<const void*>(&graph_root_kernel),
-                       reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatch>), reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatch>),
-                       reinterpret_cast<const void*>(&move_kernel<4, 512, MoveBatchSmall>), reinterpret_cast<const void*>(&move_kernel<8, 1024, MoveBatchSmall>),
+                       move_entry<MoveBatch>({4, 640}), move_entry<MoveBatch>({2, 256}), move_entry<MoveBatch>({8, 1024}),
+                       move_entry<MoveBatchSmall>({4, 640}), move_entry<MoveBatchSmall>({2, 256}), move_entry<MoveBatchSmall>({8, 1024}),
                        reinterpret_cast<const void*>(&chain_kernel<0, 1024>), reinterpret_cast<const void*>(&chain_kernel<1, 1024>)};
   for (const void* f : fns) {
     cudaFuncAttributes a;
@@ -947,7 +995,8 @@ cudaError_t preload_kernels() {
     if (e != cudaSuccess) return e;
   }
   for (int nops = 2; nops <= 8; nops++)
-    for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn, chain_fan_variant<0>(nops).fn, chain_fan_variant<1>(nops).fn}) {
+    for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn, chain_fan_variant<0>(nops, 8).fn, chain_fan_variant<1>(nops, 8).fn,
+                          chain_fan_variant<0>(nops, 148).fn, chain_fan_variant<1>(nops, 148).fn}) {
       cudaFuncAttributes a;
       cudaError_t e = cudaFuncGetAttributes(&a, f);
       if (e != cudaSuccess) return e;

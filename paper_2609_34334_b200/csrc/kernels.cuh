@@ -125,7 +125,7 @@ bool add_move_seg(MoveBatch* batch, const void* src, void* const* dsts, int ndst
 // Batches are prepared with the CTA count they are launched with.
 void prepare_move_batch(MoveBatch* batch, int ctas);
 bool shrink_move_batch(const MoveBatch& batch, MoveBatchSmall* out);   // false if it does not fit
-const void* move_kernel_entry(int ctas, bool small, int* threads);
+const void* move_kernel_entry(const MoveBatch& batch, int ctas, bool small, int* threads);
 cudaError_t launch_moves(MoveBatch* batch, int ctas, cudaStream_t stream);   // prepares and launches; nothing for an empty batch
 cudaError_t launch_move(const void* src, void* dst, unsigned long long bytes, int ctas, cudaStream_t stream);   // one copy
 

@@ -203,10 +203,11 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                kernel is a pure gain: measured on B200 with the default schedule and 8-CTA sums, R = 8 bf16 all-reduce of
  *                4 KiB 34 -> 10 us, 1 MiB 48 -> 25 us, 4 MiB 88 -> 54 us, 8 MiB 107 -> 97 us, equal from 16 MiB on; R = 4 fp32
  *                all-reduce of 4 MiB 37 -> 33 us.  Default 8 MiB; 0 = driver copies at every size.  "HOCCL_PATH_CE" therefore
- *                means: the copy route above this size.  Not applied to hoccl_host_allreduce and send/recv.
+ *                means: the copy route above this size.  Not applied to hoccl_host_allreduce; a send/recv message counts
+ *                by its own size.
  *                Unless it is 0, copies the driver does badly do not go to it at any size (it takes 4 us more for a copy of 1 MiB or
  *                more that does not start on a 128-byte line and end after whole 4 KiB, and runs at half rate or less when the two
- *                ends differ modulo 4): an all-gather or all-to-all of such blocks, or of blocks below 2 MiB, runs on the copy kernel like a small one, and an
+ *                ends differ modulo 4): a send/recv message, an all-gather or all-to-all of such blocks, or of blocks below 2 MiB, runs on the copy kernel like a small one, and an
  *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of its all-gather's copies to one
  *                launch of the copy kernel ("copy_ctas" CTAs) per piece.
  *  "ce_overlap"  HOCCL_PATH_CE, direct reduce-scatter: the ring chunks are cut into this many pieces and every piece's three
@@ -390,7 +391,8 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
  * happens once both sides are known).  Posts are matched per (src, dst) pair in FIFO order; either
  * side may come first.  The first post parks {buffer, count, dtype, stream} on the host and marks its place in its
  * stream with an event; nothing else is enqueued.  The second post enqueues ONE device-to-device move of count
- * elements that runs after both streams have reached their posts and that both streams then wait for.
+ * elements that runs after both streams have reached their posts and that both streams then wait for (on HOCCL_PATH_CE it is
+ * enqueued on the second poster's stream itself).
  * What this cannot give: work that the FIRST poster enqueues on its stream between its own post and the partner's is
  * not ordered against the transfer (a stream cannot be made to wait, after the fact, for something that is enqueued
  * later): a consumer of the receive buffer, or a writer of the send buffer, must be enqueued after the partner has

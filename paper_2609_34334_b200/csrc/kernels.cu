@@ -819,7 +819,9 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
 }
 
 // Launch shape: a thread keeps up to u vectors.  Under a CTA budget 8 x 1024 (the bytes in flight per SM decide).  Whole-GPU grids
-// are bound by HBM and want less in flight: copies of 64 MiB 5.26 TB/s with 4 x 512, 6.46 with 4 x 640 (256 MiB: 5.9 and 6.2; 8 x 1024: 4.2); one read stored 7 times 5.4 with 4 x 512, 5.9 with 2 x 256.
+// are bound by HBM and want some 40 KiB in flight per SM: all-to-all of 64 MiB over 8 ranks 186 us with 4 x 512, 177 with 4 x 576, 173
+// with 4 x 640 and 4 x 704 (the latter 2 % ahead out of phase and where part of the source is in L2), copies with 8 x 1024 4.2 TB/s;
+// one read stored 7 times 5.4 TB/s with 4 x 512, 5.9 with 2 x 256.
 struct MoveShape {
   int u, threads;
 };
@@ -827,7 +829,7 @@ static MoveShape move_shape(const MoveBatch& b, int ctas) {
   if (!wide_copy_grid(ctas)) return {8, 1024};
   bool in_phase = true;
   for (int k = 0; k < b.nseg; k++) in_phase = in_phase && ((((uintptr_t)b.seg[k].src ^ (uintptr_t)b.dst[b.seg[k].first_dst]) & 15) == 0);
-  return in_phase && b.ndst_total >= 2 * b.nseg ? MoveShape{2, 256} : MoveShape{4, 640};
+  return in_phase && b.ndst_total >= 2 * b.nseg ? MoveShape{2, 256} : MoveShape{4, 704};
 }
 
 void prepare_move_batch(MoveBatch* b, int ctas) {
@@ -883,7 +885,7 @@ bool shrink_move_batch(const MoveBatch& b, MoveBatchSmall* o) {
 template <class Batch>
 static const void* move_entry(MoveShape shape) {
   switch (shape.u * 10000 + shape.threads) {
-    case 40640: return reinterpret_cast<const void*>(&move_kernel<4, 640, Batch>);
+    case 40704: return reinterpret_cast<const void*>(&move_kernel<4, 704, Batch>);
     case 20256: return reinterpret_cast<const void*>(&move_kernel<2, 256, Batch>);
     default: return reinterpret_cast<const void*>(&move_kernel<8, 1024, Batch>);
   }
@@ -986,8 +988,8 @@ cudaError_t preload_kernels() {
                        reinterpret_cast<const void*>(&occupy_kernel),           reinterpret_cast<const void*>(&onepass_kernel<0, 512>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 512>),  reinterpret_cast<const void*>(&onepass_kernel<0, 1024>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 1024>), reinterpret_cast<const void*>(&graph_root_kernel),
-                       move_entry<MoveBatch>({4, 640}), move_entry<MoveBatch>({2, 256}), move_entry<MoveBatch>({8, 1024}),
-                       move_entry<MoveBatchSmall>({4, 640}), move_entry<MoveBatchSmall>({2, 256}), move_entry<MoveBatchSmall>({8, 1024}),
+                       move_entry<MoveBatch>({4, 704}), move_entry<MoveBatch>({2, 256}), move_entry<MoveBatch>({8, 1024}),
+                       move_entry<MoveBatchSmall>({4, 704}), move_entry<MoveBatchSmall>({2, 256}), move_entry<MoveBatchSmall>({8, 1024}),
                        reinterpret_cast<const void*>(&chain_kernel<0, 1024>), reinterpret_cast<const void*>(&chain_kernel<1, 1024>)};
   for (const void* f : fns) {
     cudaFuncAttributes a;

@@ -123,15 +123,28 @@ hoccl_result_t p2p_post(hoccl_comm* c, bool is_send, void* buf, size_t count, in
     nsplit = (int)std::min<size_t>((size_t)c->p2p_split, bytes / ((size_t)16 << 20));
     nsplit = std::max(1, std::min<int>(nsplit, kMaxLanes));
   }
+  // Short messages, and those the driver copies badly, go to the move kernel as in the collectives ("ce_small_bytes").
+  const bool by_kernel = c->path == HOCCL_PATH_SM || (c->ce_small_bytes > 0 && (bytes <= (size_t)c->ce_small_bytes || bad_for_driver((const char*)sbuf, (const char*)dbuf, bytes)));
+  const int ctas = (int)(c->path == HOCCL_PATH_SM ? c->copy_ctas : c->ce_small_ctas);
+  auto move = [&](const char* from, char* to, size_t n, cudaStream_t on) {
+    if (!by_kernel) return cudaMemcpyAsync(to, from, n, cudaMemcpyDeviceToDevice, on);
+    c->stats.n_move_launches++;
+    c->stats.max_copy_ctas = ctas;
+    return launch_move(from, to, n, ctas, on);
+  };
   long n_moves = 0;
-  if (!two_streams && nsplit == 1) {
-    // both posts came from the same stream: its own order is the whole dependency
-    if (c->path == HOCCL_PATH_CE) {
-      CU_TRY(c, cudaMemcpyAsync(dbuf, sbuf, bytes, cudaMemcpyDeviceToDevice, stream));
-    } else {
-      CU_TRY(c, launch_move(sbuf, dbuf, bytes, (int)c->copy_ctas, stream));
-      c->stats.n_move_launches = 1;
-      c->stats.max_copy_ctas = c->copy_ctas;
+  if ((c->path == HOCCL_PATH_CE || !two_streams) && (nsplit == 1 || by_kernel)) {
+    // The move runs on the second poster's stream, behind the first poster's place in its own; the first poster's stream then
+    // waits for it.  (On an internal lane it would wait for, and be waited for by, both streams: three more event operations, which
+    // bound a chain of short messages on the host, and one more hop between streams.)
+    if (two_streams) CU_TRY(c, cudaStreamWaitEvent(stream, peer.at_post, 0));
+    CU_TRY(c, move((const char*)sbuf, (char*)dbuf, bytes, stream));
+    if (two_streams) {
+      c->ev_next = 0;
+      cudaEvent_t ed = next_event(c);
+      if (!ed) return cuda_fail(c, cudaErrorMemoryAllocation, "event pool");
+      CU_TRY(c, cudaEventRecord(ed, stream));
+      CU_TRY(c, cudaStreamWaitEvent(peer.stream, ed, 0));
     }
     n_moves = 1;
   } else {
@@ -150,13 +163,7 @@ hoccl_result_t p2p_post(hoccl_comm* c, bool is_send, void* buf, size_t count, in
       cudaStream_t run = c->path == HOCCL_PATH_CE ? c->lane[(c->p2p_rr++) % kMaxLanes] : c->lane[0];
       if (two_streams) CU_TRY(c, cudaStreamWaitEvent(run, ea, 0));
       CU_TRY(c, cudaStreamWaitEvent(run, eb, 0));
-      if (c->path == HOCCL_PATH_CE) {
-        CU_TRY(c, cudaMemcpyAsync((char*)dbuf + off, (const char*)sbuf + off, len, cudaMemcpyDeviceToDevice, run));
-      } else {
-        CU_TRY(c, launch_move((const char*)sbuf + off, (char*)dbuf + off, len, (int)c->copy_ctas, run));
-        c->stats.n_move_launches++;
-        c->stats.max_copy_ctas = c->copy_ctas;
-      }
+      CU_TRY(c, move((const char*)sbuf + off, (char*)dbuf + off, len, run));
       n_moves++;
       cudaEvent_t ed = next_event(c);
       if (!ed) return cuda_fail(c, cudaErrorMemoryAllocation, "event pool");

@@ -120,3 +120,29 @@ def test_route_of_a_user_defined_pattern(R, mib, width, kernel):
         st = comm.last_stats()
         assert (st["n_move_launches"], st["n_moves"], st["graph_hit"]) == (int(kernel) * -(-(R * R - 1) // 128), R * R - 1, rep), st
     comm.destroy()
+
+
+@pytest.mark.parametrize("two_streams", [False, True])
+@pytest.mark.parametrize("nbytes,kernel", [(2, True), (8 << 20, True), ((8 << 20) + 4096, False), ((8 << 20) + 2, True)])
+def test_route_of_a_message(nbytes, kernel, two_streams):
+    """Copy route: messages up to ce_small_bytes and those the driver copies badly on the kernel, the rest as driver copies; a chain of
+    hops over one or several streams delivers, whichever side posts first."""
+    comm = hb.Comm(4, 0)
+    n = nbytes // 2
+    streams = [torch.cuda.Stream() if two_streams else torch.cuda.current_stream() for _ in range(4)]
+    for k in (0, 1):
+        bufs = [torch.zeros(n, dtype=torch.int16, device="cuda") for _ in range(4)]
+        data = torch.randint(-30000, 30000, (n,), dtype=torch.int16, device="cuda")
+        torch.cuda.synchronize()
+        with torch.cuda.stream(streams[0]):
+            bufs[0].copy_(data)
+        for s in range(3):
+            posts = [lambda: comm.send(bufs[s], n, "bf16", s, s + 1, streams[s]), lambda: comm.recv(bufs[s + 1], n, "bf16", s, s + 1, streams[s + 1])]
+            for post in posts if k == 0 else reversed(posts):
+                post()
+        with torch.cuda.stream(streams[0]):
+            bufs[0].zero_()                              # the sender's stream goes on only after its message has left
+        torch.cuda.synchronize()
+        assert torch.equal(bufs[3], data) and torch.equal(bufs[1], data) and int(bufs[0].abs().sum()) == 0
+        assert (comm.last_stats()["n_move_launches"], comm.last_stats()["n_moves"]) == (int(kernel), 1)
+    assert comm.destroy() == hb.OK

@@ -208,9 +208,8 @@ __device__ __forceinline__ void report_sm(const Batch& batch) {
   }
 }
 
-// Chain sum for any number of operands and destinations: one 16-byte vector per thread and tile; the operands are loaded in
-// batches of up to 8 before they are added, so up to 8 x 16 KiB are in flight per CTA.  Serves more than 8 operands (the forms
-// below are compiled for 2 to 8).
+// Chain sum for any number of operands and destinations (the forms below are compiled for 2 to 16): one 16-byte vector per thread and tile; the operands are loaded in
+// batches of up to 8 before they are added, so up to 8 x 16 KiB are in flight per CTA.
 template <int DT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
@@ -316,15 +315,93 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe_kernel(const __grid_con
   chain_scalar_items<DT, NOPS>(batch);
 }
 
-// The sum that carries the all-gather too: NOPS operands are read once, the result is stored to NOPS destinations (one per
-// rank).  NOPS reads and NOPS writes per element are what the collective cannot do without; bound by HBM with a whole-GPU grid.
+// The same for 9 to 16 operands, which do not fit a thread's registers P at a time: a tile is two steps of NA and NOPS - NA operands,
+// the accumulator is carried from the first to the second, and P steps of loads are in flight.  chain_kernel, which loads 8
+// operands, waits, adds and only then loads the rest, ran at 75 (9 operands) to 133 GB/s per SM (16) with 8 CTAs (64 MiB per
+// rank: 910 and 1051 us, now 526 and 838).
+template <int DT, int NOPS, int P, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) chain_pipe2_kernel(const __grid_constant__ ChainBatch batch) {
+  using T = Traits<DT>;
+  constexpr int NA = (NOPS + 1) / 2, NB = NOPS - NA;
+  constexpr int STEPS = P % 2 ? 2 * P : P;             // steps of one round: whole tiles, and every buffer back in its place
+  constexpr int AHEAD = (P - 2) / 2 + 1;               // tiles the prologue touches
+  const Flat& f = batch.flat;
+  const int nseg = batch.nseg;
+  report_sm(batch);
+  {
+    const unsigned long long T_all = f.tpre[nseg];
+    const unsigned long long A = T_all / gridDim.x * blockIdx.x + min((unsigned long long)blockIdx.x, T_all % gridDim.x);
+    const unsigned long long B = A + T_all / gridDim.x + (blockIdx.x < T_all % gridDim.x ? 1 : 0);
+    int k = 0;
+    while (k < nseg && f.tpre[k + 1] <= A) k++;
+    for (; k < nseg && f.tpre[k] < B; k++) {
+      const unsigned a = (unsigned)((A > f.tpre[k] ? A : f.tpre[k]) - f.tpre[k]);   // tiles [a, b) of segment k
+      const unsigned b = (unsigned)((B < f.tpre[k + 1] ? B : f.tpre[k + 1]) - f.tpre[k]);
+      const unsigned nvec = (unsigned)f.nvec[k];
+      const unsigned bf = b < nvec / THREADS ? b : nvec / THREADS;                  // full tiles end here
+      const char* src[NOPS];
+#pragma unroll
+      for (int q = 0; q < NOPS; q++) src[q] = static_cast<const char*>(batch.ptr[batch.seg[k].first_ptr + q]);
+      char* out = static_cast<char*>(batch.ptr[batch.seg[k].first_ptr + NOPS]);
+      const unsigned off0 = f.head[k] * T::E + threadIdx.x * 16;
+      uint4 buf[P][NA], acc;
+      auto load = [&](uint4(&bb)[NA], unsigned t, int h) {   // step h of tile t
+        const unsigned o = off0 + t * (THREADS * 16);
+#pragma unroll
+        for (int q = 0; q < NA; q++)
+          if (h == 0 || q < NB) bb[q] = __ldcs(reinterpret_cast<const uint4*>(src[(h ? NA : 0) + (h && q >= NB ? 0 : q)] + o));
+      };
+      auto consume = [&](const uint4(&bb)[NA], unsigned t, int h) {
+        if (h == 0) {
+          acc = bb[0];
+#pragma unroll
+          for (int q = 1; q < NA; q++) acc = chain_add<DT>(acc, bb[q]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < NB; q++) acc = chain_add<DT>(acc, bb[q]);
+          *reinterpret_cast<uint4*>(out + (off0 + t * (THREADS * 16))) = acc;
+        }
+      };
+      unsigned i = a;
+      if (bf > a && bf - a >= (unsigned)AHEAD) {
+#pragma unroll
+        for (int s = 0; s < P - 1; s++) load(buf[s], i + s / 2, s % 2);
+        for (; i + (STEPS + P - 2) / 2 < bf; i += STEPS / 2) {   // steady state: straight-line code, as above
+#pragma unroll
+          for (int s = 0; s < STEPS; s++) {
+            load(buf[(s + P - 1) % P], i + (s + P - 1) / 2, (s + P - 1) % 2);
+            consume(buf[s % P], i + s / 2, s % 2);
+          }
+        }
+#pragma unroll
+        for (int s = 0; s < P - 1; s++) consume(buf[s], i + s / 2, s % 2);
+        if ((P - 1) % 2) {   // the last tile the prologue touched has its first step only
+          load(buf[P - 1], i + (P - 2) / 2, 1);
+          consume(buf[P - 1], i + (P - 2) / 2, 1);
+        }
+        i += AHEAD;
+      }
+      for (; i < b; i++) {   // what is left: full tiles and the ragged last one
+        if (i * THREADS + threadIdx.x >= nvec) break;
+        load(buf[0], i, 0);
+        load(buf[1], i, 1);
+        consume(buf[0], i, 0);
+        consume(buf[1], i, 1);
+      }
+    }
+  }
+  chain_scalar_items<DT, NOPS>(batch);
+}
+
+// Whole-GPU sums, and the sum that carries the all-gather too: NOPS operands are read once, the result is stored to NDST
+// destinations (1, or NOPS: one per rank).  That is what the collective cannot do without; bound by HBM with a whole-GPU grid.
 // A tile is U x THREADS vectors, so U x NOPS loads are in flight per thread before the first add.
-template <int DT, int NOPS, int U, int THREADS>
+template <int DT, int NOPS, int NDST, int U, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
   const Flat& f = batch.flat;
   report_sm(batch);
-  // tile t of the flattened space belongs to CTA t mod grid; walked segment by segment, so that the 2 NOPS pointers are loaded
+  // tile t of the flattened space belongs to CTA t mod grid; walked segment by segment, so that the NOPS + NDST pointers are loaded
   // once per segment and not once per tile (R = 8, 64 MiB fp32, tiles of 384 vectors: 194 us with a look-up per tile, 171 without)
   const unsigned long long T_all = f.tpre[batch.nseg];
   int k = 0;
@@ -332,12 +409,11 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
     while (at >= f.tpre[k + 1]) k++;
     const unsigned tiles = (unsigned)(f.tpre[k + 1] - f.tpre[k]);
     const char* src[NOPS];
-    char* dst[NOPS];
+    char* dst[NDST];
 #pragma unroll
-    for (int q = 0; q < NOPS; q++) {
-      src[q] = static_cast<const char*>(batch.ptr[batch.seg[k].first_ptr + q]);
-      dst[q] = static_cast<char*>(batch.ptr[batch.seg[k].first_ptr + NOPS + q]);
-    }
+    for (int q = 0; q < NOPS; q++) src[q] = static_cast<const char*>(batch.ptr[batch.seg[k].first_ptr + q]);
+#pragma unroll
+    for (int d = 0; d < NDST; d++) dst[d] = static_cast<char*>(batch.ptr[batch.seg[k].first_ptr + NOPS + d]);
     const unsigned nvec = (unsigned)f.nvec[k], head = f.head[k] * T::E;
     unsigned t = (unsigned)(at - f.tpre[k]);
     for (; t < tiles; t += gridDim.x) {
@@ -348,7 +424,7 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
 #pragma unroll
         for (int q = 1; q < NOPS; q++) acc = chain_add<DT>(acc, bb[q]);
 #pragma unroll
-        for (int d = 0; d < NOPS; d++) *reinterpret_cast<uint4*>(dst[d] + (off + u * (THREADS * 16))) = acc;
+        for (int d = 0; d < NDST; d++) *reinterpret_cast<uint4*>(dst[d] + (off + u * (THREADS * 16))) = acc;
       };
       uint4 buf[U][NOPS];
       if (v0 + (U - 1) * THREADS < nvec) {
@@ -676,8 +752,8 @@ void prepare_copy_batch(CopyBatch* b, int ctas) {
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
 }
 
-// Which chain kernel serves a batch.  The compiled forms need one operand count for the whole launch (the usual case: R) from
-// 2 to 8, and one destination (chain_pipe_kernel) or as many as operands (chain_fan_kernel).  Measured on
+// Which chain kernel serves a batch.  The compiled forms need one operand count for the whole launch (the usual case: R), from 2 to
+// 8 or 9 to 16, and one destination (chain_pipe_kernel, chain_pipe2_kernel) or, up to 8, as many as operands (chain_fan_kernel).  Measured on
 // B200 (8 operands, 25 MiB each, bf16): 163 against 111 GB/s per SM with 8 CTAs, 158 / 107 with 16, 138 / 99 with 32,
 // 113 / 89 with 48, 88 / 80 with 64, 59 / 58 with 96; with 148 CTAs both are HBM bound (5.7 TB/s).  Variants with the same
 // or more bytes in flight (P = 2 with 640 threads, P = 4 with 384, P = 4 and 6 with 256) end at the same 159-163 GB/s per
@@ -691,9 +767,17 @@ template <int DT, int NOPS, int P, int THREADS>
 static ChainVariant pipe_of() {
   return {reinterpret_cast<const void*>(&chain_pipe_kernel<DT, NOPS, P, THREADS>), THREADS, THREADS};
 }
+template <int DT, int NOPS, int P, int THREADS>
+static ChainVariant pipe2_of() {
+  return {reinterpret_cast<const void*>(&chain_pipe2_kernel<DT, NOPS, P, THREADS>), THREADS, THREADS};
+}
 template <int DT, int NOPS, int U, int THREADS>
 static ChainVariant fan_of() {
-  return {reinterpret_cast<const void*>(&chain_fan_kernel<DT, NOPS, U, THREADS>), THREADS, U * THREADS};
+  return {reinterpret_cast<const void*>(&chain_fan_kernel<DT, NOPS, NOPS, U, THREADS>), THREADS, U * THREADS};
+}
+template <int DT, int NOPS, int U, int THREADS>
+static ChainVariant wide_of() {
+  return {reinterpret_cast<const void*>(&chain_fan_kernel<DT, NOPS, 1, U, THREADS>), THREADS, U * THREADS};
 }
 template <int DT>
 static ChainVariant chain_pipe_variant(int nops) {
@@ -706,6 +790,29 @@ static ChainVariant chain_pipe_variant(int nops) {
     case 6: return pipe_of<DT, 6, 3, 512>();
     case 7: return pipe_of<DT, 7, 3, 512>();
     case 8: return pipe_of<DT, 8, 3, 512>();
+    case 9: return pipe2_of<DT, 9, 4, 512>();
+    case 10: return pipe2_of<DT, 10, 4, 512>();
+    case 11: return pipe2_of<DT, 11, 4, 512>();
+    case 12: return pipe2_of<DT, 12, 4, 512>();
+    case 13: return pipe2_of<DT, 13, 3, 512>();
+    case 14: return pipe2_of<DT, 14, 3, 512>();
+    case 15: return pipe2_of<DT, 15, 3, 512>();
+    case 16: return pipe2_of<DT, 16, 3, 512>();
+    default: return {nullptr, 0, 0};
+  }
+}
+template <int DT>
+static ChainVariant chain_wide_variant(int nops) {
+  // One destination, whole-GPU grids.  The mix is read heavy and takes 60 to 80 KiB of loads in flight per SM; what chain_kernel
+  // lost with few operands was the look-up per tile (R = 2, 256 MiB per rank: 152 us, now 126).
+  switch (nops) {
+    case 2: return wide_of<DT, 2, 4, 512>();
+    case 3: return wide_of<DT, 3, 2, 768>();
+    case 4: return wide_of<DT, 4, 2, 640>();
+    case 5: return wide_of<DT, 5, 2, 448>();
+    case 6: return wide_of<DT, 6, 2, 384>();
+    case 7: return wide_of<DT, 7, 1, 640>();
+    case 8: return wide_of<DT, 8, 1, 640>();
     default: return {nullptr, 0, 0};
   }
 }
@@ -745,7 +852,8 @@ static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
   for (int k = 1; k < b.nseg; k++)
     if (b.seg[k].nops != nops || b.seg[k].ndst != ndst) return plain;
   ChainVariant v = plain;
-  if (ndst == 1 && ctas < 128) v = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
+  if (ndst == 1 && !wide_grid(ctas)) v = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
+  else if (ndst == 1) v = b.dtype == 0 ? chain_wide_variant<0>(nops) : chain_wide_variant<1>(nops);
   else if (ndst == nops) v = b.dtype == 0 ? chain_fan_variant<0>(nops, ctas) : chain_fan_variant<1>(nops, ctas);
   return v.fn ? v : plain;
 }
@@ -996,9 +1104,16 @@ cudaError_t preload_kernels() {
     cudaError_t e = cudaFuncGetAttributes(&a, f);
     if (e != cudaSuccess) return e;
   }
+  for (int nops = 9; nops <= 16; nops++)
+    for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn}) {
+      cudaFuncAttributes a;
+      cudaError_t e = cudaFuncGetAttributes(&a, f);
+      if (e != cudaSuccess) return e;
+    }
   for (int nops = 2; nops <= 8; nops++)
     for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn, chain_fan_variant<0>(nops, 8).fn, chain_fan_variant<1>(nops, 8).fn,
-                          chain_fan_variant<0>(nops, 148).fn, chain_fan_variant<1>(nops, 148).fn}) {
+                          chain_fan_variant<0>(nops, 148).fn, chain_fan_variant<1>(nops, 148).fn, chain_wide_variant<0>(nops).fn,
+                          chain_wide_variant<1>(nops).fn}) {
       cudaFuncAttributes a;
       cudaError_t e = cudaFuncGetAttributes(&a, f);
       if (e != cudaSuccess) return e;

@@ -503,6 +503,16 @@ __global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant_
       const unsigned sh = (unsigned)(uintptr_t)s & 15;
       const uint4* a = reinterpret_cast<const uint4*>(s - sh) + first;
       uint4 v[U];
+      if (sh == 0 && tile_u == U && tile_end <= sg.nvec) {   // a whole tile: no bounds between its loads
+#pragma unroll
+        for (int u = 0; u < U; u++) v[u] = __ldcs(a + u * THREADS);
+        for (int d = 0; d < sg.ndst; d++) {
+          uint4* o = reinterpret_cast<uint4*>(static_cast<char*>(batch.dst[sg.first_dst + d]) + sg.head) + first;
+#pragma unroll
+          for (int u = 0; u < U; u++) o[u * THREADS] = v[u];
+        }
+        continue;
+      }
       if (sh == 0) {
 #pragma unroll
         for (int u = 0; u < U; u++)
@@ -927,21 +937,35 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
 }
 
 // Launch shape: a thread keeps up to u vectors.  Under a CTA budget 8 x 1024 (the bytes in flight per SM decide).  Whole-GPU grids
-// are bound by HBM and want some 40 KiB in flight per SM: all-to-all of 64 MiB over 8 ranks 186 us with 4 x 512, 177 with 4 x 576, 173
-// with 4 x 640 and 4 x 704 (the latter 2 % ahead out of phase and where part of the source is in L2), copies with 8 x 1024 4.2 TB/s;
-// one read stored 7 times 5.4 TB/s with 4 x 512, 5.9 with 2 x 256.
+// are bound by HBM and want little in flight per SM, the less the more often a vector is stored (the reads otherwise come in bursts
+// between the writes): 44 KiB for copies, 7 for one read stored 7 times.  Measured in TB/s at 256 MiB per stream: copies 4 x 704 6.2
+// (4 x 512 5.8, 8 x 1024 4.2), 1:2 2 x 704 6.0 (2 x 256 4.0), 1:3 4 x 384 6.0 (2 x 256 4.5), 1:4 and 1:5 2 x 384 5.8 (2 x 256 4.8 and 5.1), 1:7
+// 1 x 448 5.8 (4 x 512 3.9).  Out of phase every vector is loaded twice, from L1 the second time: 4 x 704.
 struct MoveShape {
   int u, threads;
 };
-static MoveShape move_shape(const MoveBatch& b, int ctas) {
-  if (!wide_copy_grid(ctas)) return {8, 1024};
-  bool in_phase = true;
-  for (int k = 0; k < b.nseg; k++) in_phase = in_phase && ((((uintptr_t)b.seg[k].src ^ (uintptr_t)b.dst[b.seg[k].first_dst]) & 15) == 0);
-  return in_phase && b.ndst_total >= 2 * b.nseg ? MoveShape{2, 256} : MoveShape{4, 704};
+static constexpr MoveShape kMoveShapes[] = {{8, 1024}, {4, 704}, {2, 704}, {4, 384}, {2, 384}, {1, 448}};
+static int move_shape(const MoveBatch& b, int ctas) {
+  if (!wide_copy_grid(ctas)) return 0;
+  for (int k = 0; k < b.nseg; k++)
+    if (((uintptr_t)b.seg[k].src ^ (uintptr_t)b.dst[b.seg[k].first_dst]) & 15) return 1;
+  const int per_seg = b.nseg > 0 ? (b.ndst_total + b.nseg / 2) / b.nseg : 1;   // stores per load, rounded
+  return per_seg <= 1 ? 1 : per_seg == 2 ? 2 : per_seg == 3 ? 3 : per_seg <= 5 ? 4 : 5;
+}
+template <class Batch>
+static const void* move_entry(int shape) {
+  switch (shape) {
+    case 1: return reinterpret_cast<const void*>(&move_kernel<4, 704, Batch>);
+    case 2: return reinterpret_cast<const void*>(&move_kernel<2, 704, Batch>);
+    case 3: return reinterpret_cast<const void*>(&move_kernel<4, 384, Batch>);
+    case 4: return reinterpret_cast<const void*>(&move_kernel<2, 384, Batch>);
+    case 5: return reinterpret_cast<const void*>(&move_kernel<1, 448, Batch>);
+    default: return reinterpret_cast<const void*>(&move_kernel<8, 1024, Batch>);
+  }
 }
 
 void prepare_move_batch(MoveBatch* b, int ctas) {
-  const MoveShape shape = move_shape(*b, ctas);
+  const MoveShape shape = kMoveShapes[move_shape(*b, ctas)];
   const unsigned threads = (unsigned)shape.threads, most_u = (unsigned)shape.u;
   b->spre[0] = 0;
   for (int k = 0; k < b->nseg; k++) {
@@ -990,18 +1014,10 @@ bool shrink_move_batch(const MoveBatch& b, MoveBatchSmall* o) {
   return true;
 }
 
-template <class Batch>
-static const void* move_entry(MoveShape shape) {
-  switch (shape.u * 10000 + shape.threads) {
-    case 40704: return reinterpret_cast<const void*>(&move_kernel<4, 704, Batch>);
-    case 20256: return reinterpret_cast<const void*>(&move_kernel<2, 256, Batch>);
-    default: return reinterpret_cast<const void*>(&move_kernel<8, 1024, Batch>);
-  }
-}
 const void* move_kernel_entry(const MoveBatch& b, int ctas, bool small, int* threads) {
-  const MoveShape s = move_shape(b, ctas);
-  *threads = s.threads;
-  return small ? move_entry<MoveBatchSmall>(s) : move_entry<MoveBatch>(s);
+  const int shape = move_shape(b, ctas);
+  *threads = kMoveShapes[shape].threads;
+  return small ? move_entry<MoveBatchSmall>(shape) : move_entry<MoveBatch>(shape);
 }
 
 cudaError_t launch_moves(MoveBatch* b, int ctas, cudaStream_t stream) {
@@ -1096,14 +1112,18 @@ cudaError_t preload_kernels() {
                        reinterpret_cast<const void*>(&occupy_kernel),           reinterpret_cast<const void*>(&onepass_kernel<0, 512>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 512>),  reinterpret_cast<const void*>(&onepass_kernel<0, 1024>),
                        reinterpret_cast<const void*>(&onepass_kernel<1, 1024>), reinterpret_cast<const void*>(&graph_root_kernel),
-                       move_entry<MoveBatch>({4, 704}), move_entry<MoveBatch>({2, 256}), move_entry<MoveBatch>({8, 1024}),
-                       move_entry<MoveBatchSmall>({4, 704}), move_entry<MoveBatchSmall>({2, 256}), move_entry<MoveBatchSmall>({8, 1024}),
                        reinterpret_cast<const void*>(&chain_kernel<0, 1024>), reinterpret_cast<const void*>(&chain_kernel<1, 1024>)};
   for (const void* f : fns) {
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, f);
     if (e != cudaSuccess) return e;
   }
+  for (int shape = 0; shape < (int)(sizeof(kMoveShapes) / sizeof(kMoveShapes[0])); shape++)
+    for (const void* f : {move_entry<MoveBatch>(shape), move_entry<MoveBatchSmall>(shape)}) {
+      cudaFuncAttributes a;
+      cudaError_t e = cudaFuncGetAttributes(&a, f);
+      if (e != cudaSuccess) return e;
+    }
   for (int nops = 9; nops <= 16; nops++)
     for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn}) {
       cudaFuncAttributes a;

@@ -207,7 +207,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                by its own size.
  *                Unless it is 0, copies the driver does badly do not go to it at any size (it takes 4 us more for a copy of 1 MiB or
  *                more that does not start on a 128-byte line and end after whole 4 KiB, and runs at half rate or less when the two
- *                ends differ modulo 4): a send/recv message, an all-gather or all-to-all of such blocks, or of blocks below 2 MiB, runs on the copy kernel like a small one, and an
+ *                ends differ modulo 4): a send/recv message, an all-gather or all-to-all of such blocks, an all-to-all of blocks below 4 MiB and an
+ *                all-gather of 3 ranks or more (the kernel reads a block once, driver copies once per destination) runs on the copy kernel like a small one, and an
  *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of its all-gather's copies to one
  *                launch of the copy kernel ("copy_ctas" CTAs) per piece.
  *  "ce_overlap"  HOCCL_PATH_CE, direct reduce-scatter: the ring chunks are cut into this many pieces and every piece's three

@@ -199,7 +199,7 @@ struct Call {
 // What a driver copy inside one device does at once, as timed on B200: a copy of 1 MiB or more whose destination does not start on a
 // 128-byte line or whose length is not a multiple of 4 KiB takes 4 us more than a whole one (8 MiB 8.3 against 4.3 us, 64 MiB 28.7
 // against 24.6), one whose ends differ modulo 4 runs at half the rate.
-constexpr size_t kDriverLine = 128, kDriverPage = 4096, kDriverWhole = 1 << 20, kDriverShort = 2 << 20;
+constexpr size_t kDriverLine = 128, kDriverPage = 4096, kDriverWhole = 1 << 20, kDriverShort = 4 << 20;
 inline bool bad_for_driver(const char* src, const char* dst, size_t bytes) {
   return bytes >= kDriverWhole && (bytes % kDriverPage || (uintptr_t)dst % kDriverLine || (((uintptr_t)src ^ (uintptr_t)dst) & 15));
 }

@@ -769,14 +769,16 @@ hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype) {
   return resolve_options(options_of(c, kind, count, dtype, false), &o);
 }
 
-// Whether some block of an all-gather or all-to-all is a copy the driver does badly (see kDriverLine), or short (all-gather of 9 MiB
-// per rank over 8 ranks 24.7 us in driver copies, 14.4 on the kernel; all-to-all of 9 MiB 32.7 / 28.9, of 16 MiB equal).  Such a call runs on the copy
-// kernel at any size, like a small one: of the blocks of 64 MiB per rank, 16 bytes short of whole, an all-gather of 8 ranks took
-// 0.372 ms in driver copies and takes 0.112 (0.174 for whole blocks in driver copies), an all-to-all 0.384 and 0.185 (0.174); two
-// bytes out of phase 0.818 and 0.113, 0.838 and 0.190.
+// Whether an all-gather or all-to-all is better not left to driver copies.  Such a call runs on the move kernel at any size, like a
+// small one.
+//   * Some block is a copy the driver does badly (see kDriverLine): 64 MiB per rank over 8 ranks, blocks 16 bytes short of whole: all-gather
+//     372 us in driver copies, 96 on the kernel, all-to-all 384 and 173; two bytes out of phase 818 and 114, 838 and 175.
+//   * The blocks of an all-to-all are short: 16 MiB per rank 51 and 47 us, 40 MiB 112 and 110, 64 MiB 175 and 173, 256 MiB 660 and 690.
+//   * An all-gather of 3 ranks or more: the kernel reads a block once, driver copies once per destination (9 MiB per rank over 8 ranks
+//     24.7 and 14.4 us, 40 MiB 84 and 62, 64 MiB 150 and 96, 256 MiB 572 and 367; over 3 ranks 64 MiB 45 and 38).
 static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t block = call.count * dtype_size(call.dtype);
-  if (block < kDriverShort) return true;
+  if (block < kDriverShort || (call.kind == PLAN_ALLGATHER && c->R >= 3)) return true;
   for (int u = 0; u < c->R; u++)
     for (int v = 0; v < c->R; v++)
       if (bad_for_driver((const char*)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0), (const char*)call.recv[v] + (size_t)u * block, block))

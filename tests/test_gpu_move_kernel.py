@@ -59,10 +59,11 @@ def test_an_all_to_all_of_eight_ranks_is_one_launch():
 
 
 @pytest.mark.parametrize("op", ["allgather", "alltoall", "allreduce"])
-@pytest.mark.parametrize("count", [(1 << 20) - 8, (1 << 20) + 1, 1_100_032, 600_064, 1 << 20])
+@pytest.mark.parametrize("count", [(1 << 20) - 8, (1 << 20) + 1, 1_100_032, 600_064, 1 << 20, 2 << 20])
 def test_copies_the_driver_does_badly(op, count):
     """Copy route above the small-message size: blocks of 1 to 2 MiB that end inside a page or start off a 128-byte line run on the
-    copy kernel (all-gather, all-to-all) or leave their ends to it (all-reduce); whole blocks stay with the driver."""
+    copy kernel (all-to-all; all-gathers of several ranks always) or leave their ends to it (all-reduce); whole blocks stay with the
+    driver, in an all-to-all from 4 MiB on."""
     R = 8
     comm = hb.Comm(R, 0)
     n = R * count
@@ -88,7 +89,7 @@ def test_copies_the_driver_does_badly(op, count):
                 want = [torch.stack([s.float() for s in send]).sum(0).to(torch.bfloat16)] * R
         torch.cuda.synchronize()
         assert all(torch.equal(recv[r], want[r]) for r in range(R)), (op, count, pad)
-        whole = count * 2 % 4096 == 0 and pad == 0 and (op == "allreduce" or count >= 1 << 20)
+        whole = count * 2 % 4096 == 0 and pad == 0 and (op == "allreduce" or op == "alltoall" and count >= 2 << 20)
         assert (comm.last_stats()["n_move_launches"] == 0) == whole, (op, count, pad, comm.last_stats())
     comm.destroy()
 

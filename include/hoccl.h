@@ -261,7 +261,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                SUM budget (sum_ctas < 64), where it was measured to
  *                gain 1-5 %, equal otherwise (below that size the small outer pieces cost more than they save).  Same
  *                operations, same bits.
- *  "host_pieces" pieces per ring chunk of the pipelined hoccl_host_allreduce (1..64, default 8; 1 = not pipelined)
+ *  "host_pieces" pieces per ring chunk of the pipelined hoccl_host_allreduce (1..64, default 8; 1 = not pipelined).  If the key is not
+ *                set and the direct schedule runs: by size (see hoccl_host_allreduce)
  *  "use_graph"   1 = run a cached CUDA graph built from the plan (default), 0 = streams and events
  *  "handshake"   1 = the paper's stream manager (Sec. 3.2): instead of launching into the caller's stream, the call
  *                enqueues three stream memory operations (write "hand-over n has arrived", wait for "hand-over n is
@@ -431,7 +432,11 @@ hoccl_result_t hoccl_comm_proxy_stats(hoccl_comm_t comm, double* busy_us, double
  * piece (its own cached graph) runs on `stream` as soon as the piece has arrived, and the device-to-host copies follow on
  * a second internal stream, so that the inbound copies, the ring and the outbound copies of different pieces overlap
  * (chunk pipelining, Sec. 3.3.1, applied across the PCIe link); `stream` waits for the last outbound copy.  Chunk boundaries, and therefore every bit of
- * the result, are those of hoccl_allreduce on the whole buffer.  Host buffers of different ranks must not overlap
+ * the result, are those of hoccl_allreduce on the whole buffer.  When the sums can read contributions in place ("rs_direct" = 2, see
+ * there) and the ranks' vectors are at most 72 MB together, a piece is a contiguous range of the vector instead, one copy per rank
+ * and direction, summed once and copied out to every rank from one buffer; the number of pieces then follows the size (1 up to
+ * 1 MiB per rank, 3 at 4 MiB) unless "host_pieces" was set, as it does for longer vectors on the direct schedule (5 at 25 MiB).
+ * Host buffers of different ranks must not overlap
  * partially (INVALID_ARG); h_recv[r] == h_send[r] is legal.  With host_pieces = 1, use_graph = 0, handshake, onepass,
  * fused or HOCCL_PATH_CE_HOST the three stages run one after the other.
  * Errors: as hoccl_allreduce, SCRATCH if staging is missing or too small.

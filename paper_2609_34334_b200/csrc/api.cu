@@ -173,6 +173,9 @@ hoccl_result_t hoccl_comm_set_param(hoccl_comm_t c, const char* key, long value)
     value = (value + 1023) / 1024 * 1024;
     c->piece_bytes_set = true;
   }
+  if (std::strcmp(key, "host_pieces") == 0) {
+    c->host_pieces_set = true;
+  }
   *p = value;
   return HOCCL_OK;
 }

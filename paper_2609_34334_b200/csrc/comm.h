@@ -117,6 +117,7 @@ struct hoccl_comm {
        ce_small_bytes = 8 << 20, ce_small_ctas = 148, p2p_strict = 0, ce_overlap = -1, model_gpus_per_node = 0, model_rdma_sub_bytes = 0, roles = 0, piece_grade = -1,
        roles_missing = 0 /* self-test only: summing CTAs wait for this many movers that do not exist */;
   bool piece_bytes_set = false;  // the caller chose a piece size: no automatic choice
+  bool host_pieces_set = false;  // the same for "host_pieces"
   hoccl::Proxy* proxy = nullptr;
   cudaStream_t lane[hoccl::kMaxLanes] = {};
   cudaStream_t sum_stream = nullptr;

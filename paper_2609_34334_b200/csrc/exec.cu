@@ -12,6 +12,7 @@
 //     (fork from the caller's stream, join back into it).
 // SUM launches are chained (one at a time) so that the SM budget for sums is global, not per piece.
 #include <climits>
+#include <cmath>
 #include <tuple>
 
 #include "comm.h"
@@ -77,6 +78,7 @@ static void share_host_legs(std::vector<RGroup>* groups, size_t* host_need) {
   }
 }
 
+constexpr size_t kHostInPlaceBytes = 72000000;   // R * S up to which the host entry reads in place
 constexpr size_t kGradeInPlace = 4 << 20;   // ring chunk from which pieces are graded on the SM path when contributions are read in place
 
 // How the direct reduce-scatter's contributions reach the owner's sum.
@@ -91,15 +93,17 @@ enum Contributions {
 // Only the automatic schedule does this: "rs_direct" = 1 keeps the staged form that a rank-local owner needs.
 //   * The send buffers have to share their 16-byte phase.  (Inbox slots are placed so that the operands always do; contributions
 //     that do not would be summed element by element.)
-//   * The host-bounce path keeps its moves: that no SM takes part in them is what it is chosen for.  So does the pipelined host
-//     entry, which PCIe bounds (25 MiB per rank 5.41 ms with them, 5.50 without).
+//   * The host-bounce path keeps its moves: that no SM takes part in them is what it is chosen for.  The host entry keeps them for
+//     long vectors (see run_host_in_place).
 // The sum stores for all ranks on the SM route (on the copy route the all-gather's moves are the driver's) when its grid is the
 // whole GPU, or when the message is so short that the second launch and not the stores decide: a CTA stores ~60 GB/s, so R S
 // bytes over n CTAs take R S / (60 n) ns against ~2.5 us for a launch of its own and the wider copy grid.  Measured, one kernel
 // against two, 8-CTA sums and 148 copy CTAs: R = 8 bf16 4 KiB per rank 3.0 / 6.2 us, 384 KiB 10.3 / 12.3, 512 KiB 14.4 / 12.4;
 // R = 4 fp32 512 KiB 8.2 / 10.3, 1 MiB 14.4 / 12.4; R = 2 bf16 1 MiB 8.3 / 9.0, 2 MiB 14.4 / 12.4: the line lies at R S = 3 MiB.
 static Contributions contributions(const hoccl_comm* c, const Call& call, const OptionsOut& opt, size_t S) {
-  if (!(opt.plan_kind & PLAN_FLAG_RS_DIRECT) || c->rs_direct != 2 || c->R < 2 || c->path == HOCCL_PATH_CE_HOST || call.h_send) return STAGED;
+  if (!(opt.plan_kind & PLAN_FLAG_RS_DIRECT) || c->rs_direct != 2 || c->R < 2 || c->path == HOCCL_PATH_CE_HOST ||
+      (call.h_send && (size_t)c->R * S > kHostInPlaceBytes))
+    return STAGED;
   if (opt.executor != EXEC_GRAPH && opt.executor != EXEC_STREAMS && opt.executor != EXEC_PROXY) return STAGED;
   const uintptr_t phase = (uintptr_t)call.send[0] & 15;
   bool recv_too = true;
@@ -582,7 +586,7 @@ std::vector<uint64_t> make_key(hoccl_comm* c, const Call& call) {
     k.push_back((uint64_t)(uintptr_t)call.send[r]);
     k.push_back((uint64_t)(uintptr_t)call.recv[r]);
   }
-  k.push_back(call.h_send ? (uint64_t)c->host_pieces : 0);
+  k.push_back(call.h_send ? (uint64_t)c->host_pieces * 2 + (c->host_pieces_set ? 1 : 0) : 0);
   if (call.h_send)
     for (int r = 0; r < c->R; r++) {
       k.push_back((uint64_t)(uintptr_t)call.h_send[r]);
@@ -786,6 +790,68 @@ static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   return false;
 }
 
+// Host all-reduce whose sums read the ranks' staging buffers in place: no schedule over ring chunks is left, so a piece is one
+// contiguous range of the vector (one plain copy per rank and direction instead of a 2-D copy and one for the shorter last chunk),
+// the sum writes it once, and every rank's result is copied out of that one buffer.
+// Pieces: with np equal pieces the two directions overlap in all but one piece each, (1 + 1 / np) S R / 50 GB/s, and every copy costs
+// 6 to 9 us beside one of the other direction, np R of them; so the best np grows with the root of S (1 up to 1 MiB per rank, 3 at 4 MiB,
+// 5 at 16 MiB).  Measured over 8 ranks against 8 pieces of every ring chunk: 64 KiB per rank 122 -> 89 us, 1 MiB 403 -> 380, 4 MiB 1372 ->
+// 1087, 8 MiB 2120 -> 2060; over 3 ranks 64 KiB 74 -> 38, 1 MiB 243 -> 150, 16 MiB 1541 -> 1460.  Beyond ~64 MiB for all ranks together the 2-D
+// copies of the staged form are the faster ones (8 ranks of 16 MiB 3.58 against 3.68 ms, of 25 MiB 5.23 against 5.45).
+static size_t host_pieces(const hoccl_comm* c, size_t S, double unit) {
+  if (c->host_pieces_set) return (size_t)c->host_pieces;
+  return std::min<size_t>(32, std::max<size_t>(1, (size_t)(std::sqrt((double)S / unit) + 0.5)));
+}
+static hoccl_result_t run_host_in_place(hoccl_comm* c, const Call& call, std::vector<uint64_t>&& key, cudaStream_t user, double t0) {
+  const int R = c->R;
+  Plan P;
+  P.kind = PLAN_ALLREDUCE;
+  P.R = R;
+  P.dtype = call.dtype;
+  P.elem = dtype_size(call.dtype);
+  const size_t S = call.count * P.elem, chunk = (call.count + R - 1) / R * P.elem;
+  const size_t np = host_pieces(c, S, 600e3);
+  const size_t piece = ((S + np - 1) / np + 4095) & ~(size_t)4095;
+  GraphEntry entry;
+  entry.key = std::move(key);
+  std::vector<RGroup> groups;
+  char* result = (char*)call.recv[0];
+  for (size_t a = 0; a < S; a += piece) {
+    const size_t b = std::min(S, a + piece);
+    RGroup g;
+    g.kind = OP_CHAIN;
+    g.piece = (int)groups.size();
+    g.phase = PHASE_RS;
+    g.chain_dep = -1;
+    for (size_t at = a; at < b;) {   // one segment per ring chunk the range touches: the order of the adds is the chunk's
+      const int owner = (int)(at / chunk);
+      Seg s = {};
+      s.bytes = std::min<size_t>(std::min(b, (size_t)(owner + 1) * chunk) - at, kMaxChainSegBytes);
+      for (int j = 1; j <= R; j++) s.ops.push_back((const char*)call.send[(owner + j) % R] + at);
+      s.dst = result + at;
+      g.segs.push_back(s);
+      at += s.bytes;
+    }
+    groups.push_back(std::move(g));
+    entry.h2d.emplace_back();
+    entry.d2h.emplace_back();
+    for (int r = 0; r < R; r++) {
+      entry.h2d.back().push_back(HostCopy{(char*)call.send[r] + a, (char*)call.h_send[r] + a, b - a, b - a, 1});
+      entry.d2h.back().push_back(HostCopy{result + a, (char*)call.h_recv[r] + a, b - a, b - a, 1});
+    }
+  }
+  entry.n_pieces = (long)groups.size();
+  entry.piece_exec.assign(groups.size(), nullptr);
+  for (size_t p = 0; p < groups.size(); p++) {
+    const hoccl_result_t rc = build_graph(c, P, groups, &entry, (int)p, &entry.piece_exec[p]);
+    if (rc != HOCCL_OK) {
+      destroy_entry(&entry);
+      return rc;
+    }
+  }
+  return launch_entry(c, cache_put(c, std::move(entry)), user, t0);
+}
+
 hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   const double t0 = now_us();
   if (!c) return HOCCL_ERR_INVALID_ARG;
@@ -870,6 +936,9 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   const bool reduction = call->kind == PLAN_ALLREDUCE || call->kind == PLAN_REDUCE_SCATTER;
   const size_t ring_chunk = (call->kind == PLAN_ALLREDUCE ? (call->count + c->R - 1) / c->R : call->count) * dtype_size(call->dtype);
   const Contributions how = contributions(c, *call, opt, call->count * dtype_size(call->dtype));
+  if (call->h_send && how != STAGED) return run_host_in_place(c, *call, std::move(key), user, t0);
+  // the staged form of the direct schedule: 5 pieces at 25 MiB per rank (8 ranks 5.23 ms; 8 pieces 5.27), 4 at 16 MiB (3.58; 3.81)
+  const size_t host_np = call->h_send && (opt.plan_kind & PLAN_FLAG_RS_DIRECT) ? host_pieces(c, call->count * dtype_size(call->dtype), 1e6) : (size_t)c->host_pieces;
   const bool sum_only = how == READ_AND_STORE || (how == READ_IN_PLACE && call->kind == PLAN_REDUCE_SCATTER);   // no moves at all
   // Copy route with overlap ("ce_overlap"): the direct schedule cut into pieces whose three parts run on three internal
   // streams (see launch_entry).  Automatic (-1): 2 pieces from 2 MiB per ring chunk, from 4 MiB on pieces of about 4 MiB, at
@@ -916,7 +985,7 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   } else if (call->h_send) {   // pipelined host all-reduce: host_pieces pieces per chunk, whatever the chunk size
     const size_t q = (call->count + c->R - 1) / c->R;
     const size_t chunk = q * dtype_size(call->dtype);
-    max_pieces = (int)c->host_pieces;
+    max_pieces = (int)host_np;
     piece_bytes = std::max<size_t>((size_t)64 << 10, ((chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
   } else if (roles) {
     // the piece rule of the graph form of the same schedule (above): both forms measured best with the same pieces

@@ -1032,6 +1032,15 @@ cudaError_t launch_moves(MoveBatch* b, int ctas, cudaStream_t stream) {
 }
 
 cudaError_t launch_move(const void* src, void* dst, unsigned long long bytes, int ctas, cudaStream_t stream) {
+  // One long copy in phase leaves nothing to choose: copy_kernel's plain tile walk is 0.5 to 0.8 % faster there (waves of 42.8 MB
+  // messages on 40 CTAs, three communicators at once: 98.7 -> 98.0 us).  Below 16 MB its tiles leave CTAs without work.
+  if (bytes >= (16ull << 20) && (((uintptr_t)src ^ (uintptr_t)dst) & 15) == 0 && ((uintptr_t)dst & 127) == 0) {
+    CopyBatch cb;
+    cb.nseg = 1;
+    cb.pad = 0;
+    cb.seg[0] = CopySeg{src, dst, bytes};
+    return launch_copy(cb, ctas, stream);
+  }
   MoveBatch b;
   b.nseg = b.ndst_total = 0;
   for (unsigned long long at = 0; at < bytes; at += kMaxMoveSegBytes) {

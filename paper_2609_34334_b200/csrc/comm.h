@@ -45,6 +45,15 @@ struct Seg {
   bool host_first = true; // HOCCL_PATH_CE_HOST: this move issues the outbound copy into host_off (false: another move of the group did)
 };
 
+// One kernel launch of a schedule: the batch is its only parameter, by value.
+struct KernelLaunch {
+  const void* fn = nullptr;
+  int grid = 0, threads = 0;
+  std::vector<char> args;
+  double bytes = 0;   // algorithmic bytes
+  long moves = 0;     // MOVE operations it carries (0: a sum)
+};
+
 struct RGroup {
   int kind;
   int piece;
@@ -52,6 +61,7 @@ struct RGroup {
   std::vector<Seg> segs;
   std::vector<int> deps;
   int chain_dep;
+  std::vector<KernelLaunch> ready;   // if not empty, the launches that carry out the group (instead of batches built from segs)
   bool edges = false;   // copy route: the ends of driver copies, carried by a copy-kernel launch (see trim_driver_copies)
 };
 
@@ -69,15 +79,6 @@ struct HostCopy {
   char* dev;
   char* host;
   size_t pitch, width, rows;
-};
-
-// One kernel launch of a schedule: the batch is its only parameter, by value.
-struct KernelLaunch {
-  const void* fn = nullptr;
-  int grid = 0, threads = 0;
-  std::vector<char> args;
-  double bytes = 0;   // algorithmic bytes
-  long moves = 0;     // MOVE operations it carries (0: a sum)
 };
 
 struct GraphEntry {

@@ -151,6 +151,18 @@ static void trim_driver_copies(std::vector<RGroup>* groups) {
   }
 }
 
+template <class Batch>
+static KernelLaunch make_launch(const Batch& b, const void* fn, long grid, int threads, double bytes, long moves) {
+  KernelLaunch k;
+  k.fn = fn;
+  k.grid = (int)grid;
+  k.threads = threads;
+  k.args.assign(reinterpret_cast<const char*>(&b), reinterpret_cast<const char*>(&b) + sizeof(b));
+  k.bytes = bytes;
+  k.moves = moves;
+  return k;
+}
+
 // Turns plan offsets into addresses (the plan already places pieces inside the scratch slots).
 void resolve(hoccl_comm* c, const Plan& P, const Call& call, Contributions how, std::vector<RGroup>* out, size_t* host_need) {
   *host_need = 0;
@@ -233,6 +245,19 @@ void resolve(hoccl_comm* c, const Plan& P, const Call& call, Contributions how, 
       kept.push_back(std::move(cur));
     }
     out->swap(kept);
+    if (how == READ_AND_STORE && out->size() == 1 && c->sum_ctas < 128) {   // a short message: the kernel without tables
+      StoreAllArgs a;
+      int grid = 0, threads = 0;
+      const void* fn = store_all_entry(R, P.dtype, (int)c->sum_ctas, call.count, &a, &grid, &threads);
+      if (fn) {
+        a.phase = (unsigned)((uintptr_t)call.send[0] & 15);
+        for (int r = 0; r < R; r++) {
+          a.x[r] = call.send[r];
+          a.y[r] = call.recv[r];
+        }
+        out->front().ready.push_back(make_launch(a, fn, grid, threads, 2.0 * R * (double)call.count * (double)P.elem, 0));
+      }
+    }
     if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0) trim_driver_copies(out);
   }
   // SM path: the stages of an all-to-all are independent (disjoint blocks, no dependencies), so their moves go into as few
@@ -368,18 +393,6 @@ static size_t fill_chain_batch(const RGroup& g, size_t first, int dtype, size_t 
   return i - first;
 }
 
-template <class Batch>
-static KernelLaunch make_launch(const Batch& b, const void* fn, long grid, int threads, double bytes, long moves) {
-  KernelLaunch k;
-  k.fn = fn;
-  k.grid = (int)grid;
-  k.threads = threads;
-  k.args.assign(reinterpret_cast<const char*>(&b), reinterpret_cast<const char*>(&b) + sizeof(b));
-  k.bytes = bytes;
-  k.moves = moves;
-  return k;
-}
-
 static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup& g) {
   std::vector<KernelLaunch> out;
   int threads = 0;
@@ -417,6 +430,7 @@ static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup
 }
 
 std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, const RGroup& g) {
+  if (!g.ready.empty()) return g.ready;
   std::vector<KernelLaunch> out;
   int threads = 0;
   if (g.kind == OP_CHAIN) {

@@ -449,6 +449,62 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
   chain_scalar_items<DT, NOPS>(batch);
 }
 
+// See StoreAllArgs.
+template <int DT, int NOPS, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) store_all_kernel(const __grid_constant__ StoreAllArgs a) {
+  using T = Traits<DT>;
+  const unsigned c = blockIdx.x / a.parts, part = blockIdx.x - c * a.parts;
+  const char* src[NOPS];
+#pragma unroll
+  for (int j = 0; j < NOPS; j++) src[j] = static_cast<const char*>(a.x[(c + 1 + j) % NOPS]);
+  const unsigned lo = min(c * a.q, a.count), n = min(a.q, a.count - lo);      // elements [lo, lo + n)
+  const unsigned at = lo * T::E;                                              // byte offset of the chunk
+  const unsigned head = min(((16u - ((a.phase + at) & 15u)) & 15u) / T::E, n), nvec = (n - head) / T::VE;
+  const unsigned per = (nvec + a.parts - 1) / a.parts, v1 = min(nvec, (part + 1) * per);
+  constexpr int U = NOPS <= 4 ? 4 : 2;   // vectors of a thread in flight
+  for (unsigned v = part * per + threadIdx.x; v < v1; v += U * THREADS) {
+    uint4 buf[U][NOPS];
+#pragma unroll
+    for (int u = 0; u < U; u++)
+      if (v + u * THREADS < v1) {
+#pragma unroll
+        for (int j = 0; j < NOPS; j++) buf[u][j] = __ldcs(reinterpret_cast<const uint4*>(src[j] + (at + head * T::E + (v + u * THREADS) * 16)));
+      }
+#pragma unroll
+    for (int u = 0; u < U; u++)
+      if (v + u * THREADS < v1) {
+        uint4 acc = buf[u][0];
+#pragma unroll
+        for (int j = 1; j < NOPS; j++) acc = chain_add<DT>(acc, buf[u][j]);
+#pragma unroll
+        for (int r = 0; r < NOPS; r++) *reinterpret_cast<uint4*>(static_cast<char*>(a.y[r]) + (at + head * T::E + (v + u * THREADS) * 16)) = acc;
+      }
+  }
+  // head and tail, element by element
+  const unsigned ns = n - nvec * T::VE;
+  if (part == a.parts - 1 && threadIdx.x < ns) {
+    const unsigned i = lo + (threadIdx.x < head ? threadIdx.x : threadIdx.x + nvec * T::VE);
+    if (DT == 0) {
+      float x[NOPS];
+#pragma unroll
+      for (int j = 0; j < NOPS; j++) x[j] = reinterpret_cast<const float*>(src[j])[i];
+#pragma unroll
+      for (int j = 1; j < NOPS; j++) x[0] = __fadd_rn(x[0], x[j]);
+#pragma unroll
+      for (int r = 0; r < NOPS; r++) static_cast<float*>(a.y[r])[i] = x[0];
+    } else {
+      unsigned short x[NOPS];
+#pragma unroll
+      for (int j = 0; j < NOPS; j++) x[j] = reinterpret_cast<const unsigned short*>(src[j])[i];
+#pragma unroll
+      for (int j = 1; j < NOPS; j++)
+        x[0] = __bfloat16_as_ushort(__float2bfloat16_rn(__fadd_rn(__uint_as_float((uint32_t)x[0] << 16), __uint_as_float((uint32_t)x[j] << 16))));
+#pragma unroll
+      for (int r = 0; r < NOPS; r++) static_cast<unsigned short*>(a.y[r])[i] = x[0];
+    }
+  }
+}
+
 // The 16 bytes that start `sh` bytes into the 32 bytes lo, hi; sh (0..15) is the same for all threads.
 __device__ __forceinline__ uint4 bytes_at(uint4 lo, uint4 hi, unsigned sh) {
   uint32_t w0 = lo.x, w1 = lo.y, w2 = lo.z, w3 = lo.w, w4 = hi.x, w5 = hi.y, w6 = hi.z, w7 = hi.w;
@@ -893,6 +949,34 @@ void prepare_chain_batch(ChainBatch* b, int ctas) {
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
 }
 
+template <int DT>
+static const void* store_all_of(int R) {
+  switch (R) {
+    case 2: return reinterpret_cast<const void*>(&store_all_kernel<DT, 2, 512>);
+    case 3: return reinterpret_cast<const void*>(&store_all_kernel<DT, 3, 512>);
+    case 4: return reinterpret_cast<const void*>(&store_all_kernel<DT, 4, 512>);
+    case 5: return reinterpret_cast<const void*>(&store_all_kernel<DT, 5, 512>);
+    case 6: return reinterpret_cast<const void*>(&store_all_kernel<DT, 6, 512>);
+    case 7: return reinterpret_cast<const void*>(&store_all_kernel<DT, 7, 512>);
+    case 8: return reinterpret_cast<const void*>(&store_all_kernel<DT, 8, 512>);
+    default: return nullptr;
+  }
+}
+const void* store_all_entry(int R, int dtype, int ctas, unsigned long long count, StoreAllArgs* a, int* grid, int* threads) {
+  const void* fn = dtype == 0 ? store_all_of<0>(R) : store_all_of<1>(R);
+  if (!fn || ctas < R || count > (1ull << 28)) return nullptr;   // 32-bit byte offsets
+  a->count = (unsigned)count;
+  a->q = (unsigned)((count + R - 1) / R);
+  // no more CTAs than have a round of vectors each
+  const unsigned vecs = a->q / (dtype == 0 ? 4 : 8), useful = (vecs + 511) / 512;
+  a->parts = std::max(1u, std::min((unsigned)(ctas / R), useful));
+  // CTAs that the chunks do not divide among themselves stay idle: fine while latency decides, not when the stores do
+  if (R * a->parts < (unsigned)ctas && vecs > a->parts * 1024u) return nullptr;
+  *grid = R * (int)a->parts;
+  *threads = 512;
+  return fn;
+}
+
 bool add_chain_seg(ChainBatch* b, const void* const* ops, int nops, void* const* dsts, int ndst, unsigned long long n) {
   if (b->nseg == kMaxSegs || b->nptr + nops + ndst > kMaxChainPtrs) return false;
   ChainSeg& s = b->seg[b->nseg++];
@@ -1127,6 +1211,12 @@ cudaError_t preload_kernels() {
     cudaError_t e = cudaFuncGetAttributes(&a, f);
     if (e != cudaSuccess) return e;
   }
+  for (int R = 2; R <= kMaxStoreAllRanks; R++)
+    for (const void* f : {store_all_of<0>(R), store_all_of<1>(R)}) {
+      cudaFuncAttributes a;
+      cudaError_t e = cudaFuncGetAttributes(&a, f);
+      if (e != cudaSuccess) return e;
+    }
   for (int shape = 0; shape < (int)(sizeof(kMoveShapes) / sizeof(kMoveShapes[0])); shape++)
     for (const void* f : {move_entry<MoveBatch>(shape), move_entry<MoveBatchSmall>(shape)}) {
       cudaFuncAttributes a;

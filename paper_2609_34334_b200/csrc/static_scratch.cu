@@ -52,6 +52,20 @@ cudaError_t scratch_base(int device, void** out) {
 // The all-reduce in one or two launches for buffers of one 16-byte phase.  q: elements of a full ring chunk.
 cudaError_t read_in_place(const void* const* send, void* const* recv, size_t count, size_t q, int dtype, size_t e, int R, cudaStream_t st) {
   const bool store_all = (size_t)R * count * e <= (size_t)kStaticSumCtas * kStoreAllBytesPerCta;
+  if (store_all) {
+    StoreAllArgs a;
+    int grid = 0, threads = 0;
+    const void* fn = store_all_entry(R, dtype, kStaticSumCtas, count, &a, &grid, &threads);
+    if (fn) {
+      a.phase = (unsigned)((uintptr_t)send[0] & 15);
+      for (int r = 0; r < R; r++) {
+        a.x[r] = send[r];
+        a.y[r] = recv[r];
+      }
+      void* args[1] = {&a};
+      return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, 0, st);
+    }
+  }
   ChainBatch b;
   MoveBatch m;
   b.dtype = dtype;

@@ -408,7 +408,7 @@ def main():
                      "ordering_kernel": "empty, 1 CTA of 32 threads, ~2 us each (orders copy nodes inside the graph)"},
         "e2e": {"value": units / t_e2e_slowest / 1e9, "unit": "GB/s", "h2d_bytes_per_step": R * S, "d2h_bytes_per_step": R * S,
                 "ms_per_step": t_e2e_slowest * 1e3, "steps": k_e2e, "matches_oracle": None,
-                "call": "hoccl_host_allreduce (pinned host buffers; inbound copies, the collective and outbound copies pipelined over 8 pieces per chunk)"},
+                "call": "hoccl_host_allreduce (pinned host buffers; inbound copies, the collective and outbound copies pipelined piece by piece)"},
         "gpu_launches": int(launches_per_step * steps),
         "clocks": clocks,
         "host_launch_us_per_call": st["host_launch_us"],

@@ -190,6 +190,41 @@ hoccl_result_t hoccl_plan_get_op(hoccl_plan_t plan, int index, hoccl_plan_op_t* 
 /* Dependencies are between groups: writes up to `cap` predecessor group ids of `group` into deps, returns their number. */
 int hoccl_plan_group_deps(hoccl_plan_t plan, int group, int* deps, int cap);
 
+/* ---------------------------------------------------------------- layout inspection (host only) - */
+
+/*
+ * What a call would run: the plan's groups over the call's addresses, after everything that depends on the addresses (sums
+ * that read the contributions in place, ends of driver copies, merged groups), from the function every collective runs
+ * through.  A group starts when the groups it depends on are done; its segments run side by side, in no order.  So two
+ * accesses of different groups that touch the same byte, one of them a write, need a path of dependencies between them.
+ * Nothing is enqueued and no address is read or written.  kind: 0 all-reduce, 1 reduce-scatter, 2 all-gather, 3 all-to-all.
+ * Returns what the call itself would return for such arguments; HOCCL_ERR_UNSUPPORTED for "onepass", which has no plan.
+ */
+typedef struct hoccl_layout* hoccl_layout_t;
+typedef struct {
+  int group, segment; /* segments are numbered inside their group */
+  int kind;           /* hoccl_plan_op_kind_t of the group */
+  int piece;
+  int edges;          /* 1: the ends of driver copies, carried by a launch of the copy kernel */
+  int write;
+  uint64_t addr, bytes;
+} hoccl_access_t;
+/* A communicator for these calls alone, without a device: parameters, path and scratch are set as usual, a call that would
+ * enqueue anything returns HOCCL_ERR_CUDA.  Free with hoccl_comm_destroy. */
+hoccl_result_t hoccl_comm_init_host_only(hoccl_comm_t* comm, int R);
+hoccl_result_t hoccl_layout_build(hoccl_layout_t* layout, hoccl_comm_t comm, int kind, const void* const* sendbufs, void* const* recvbufs,
+                                  size_t count, hoccl_dtype_t dtype);
+void hoccl_layout_destroy(hoccl_layout_t layout);
+int hoccl_layout_num_groups(hoccl_layout_t layout);
+int hoccl_layout_num_pieces(hoccl_layout_t layout);
+int hoccl_layout_num_accesses(hoccl_layout_t layout);
+hoccl_result_t hoccl_layout_get_access(hoccl_layout_t layout, int index, hoccl_access_t* out);
+/* Writes up to `cap` group ids that `group` waits for into deps, returns their number (-1: no such group). */
+int hoccl_layout_group_deps(hoccl_layout_t layout, int group, int* deps, int cap);
+/* The words under which the call's graph is cached: calls with the same words replay the same graph.  Writes up to `cap`, returns
+ * their number. */
+int hoccl_layout_signature(hoccl_layout_t layout, uint64_t* words, int cap);
+
 /* ---------------------------------------------------------------- option rules (host only) ---- */
 
 /*

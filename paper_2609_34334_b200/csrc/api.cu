@@ -40,8 +40,20 @@ hoccl_result_t hoccl_comm_init(hoccl_comm_t* comm, int R, int device) {
   return HOCCL_OK;
 }
 
+hoccl_result_t hoccl_comm_init_host_only(hoccl_comm_t* comm, int R) {
+  if (!comm || R < 1 || R > kMaxRanks) return HOCCL_ERR_INVALID_ARG;
+  *comm = new hoccl_comm();
+  (*comm)->R = R;
+  (*comm)->device = -1;   // every call that would enqueue something fails at its cudaSetDevice
+  return HOCCL_OK;
+}
+
 hoccl_result_t hoccl_comm_destroy(hoccl_comm_t c) {
   if (!c) return HOCCL_ERR_INVALID_ARG;
+  if (c->device < 0) {   // hoccl_comm_init_host_only: nothing of the device to give back
+    delete c;
+    return HOCCL_OK;
+  }
   if (c->n_pending > 0) return HOCCL_ERR_PENDING;
   bool forced = false;
   if (c->proxy) {
@@ -899,6 +911,75 @@ int hoccl_plan_group_deps(hoccl_plan_t plan, int group, int* deps, int cap) {
   return n;
 }
 
+
+// ---------------------------------------------------------------- layout inspection --------------
+struct hoccl_layout {
+  Layout lay;
+  std::vector<hoccl_access_t> access;
+  std::vector<uint64_t> key;
+};
+
+hoccl_result_t hoccl_layout_build(hoccl_layout_t* layout, hoccl_comm_t c, int kind, const void* const* send, void* const* recv, size_t count,
+                                  hoccl_dtype_t dtype) {
+  if (!layout) return HOCCL_ERR_INVALID_ARG;
+  *layout = nullptr;
+  const size_t e = dtype_size((int)dtype);
+  if (!c || !send || !recv || kind < PLAN_ALLREDUCE || kind > PLAN_ALLTOALL) return HOCCL_ERR_INVALID_ARG;
+  if (e == 0) return HOCCL_ERR_UNSUPPORTED;
+  const size_t one = count * e, all = (size_t)c->R * one;
+  Call call{kind, count, (int)dtype, false, kind == PLAN_REDUCE_SCATTER || kind == PLAN_ALLTOALL ? all : one,
+            kind == PLAN_ALLGATHER || kind == PLAN_ALLTOALL ? all : one, send, recv};
+  hoccl_layout* h = new hoccl_layout();
+  const hoccl_result_t rc = inspect_call(c, &call, &h->lay, &h->key);
+  if (rc != HOCCL_OK) {
+    delete h;
+    return rc;
+  }
+  for (size_t g = 0; g < h->lay.groups.size(); g++) {
+    const RGroup& rg = h->lay.groups[g];
+    for (size_t k = 0; k < rg.segs.size(); k++) {
+      const Seg& s = rg.segs[k];
+      auto add = [&](bool write, const void* p) {
+        h->access.push_back(hoccl_access_t{(int)g, (int)k, rg.kind, rg.piece, rg.edges ? 1 : 0, write ? 1 : 0, (uint64_t)(uintptr_t)p, s.bytes});
+      };
+      if (s.ops.empty()) {
+        for (int j = 0; j < s.nsrc; j++) add(false, s.src + (size_t)j * s.src_stride);
+        if (rg.kind != OP_MOVE) add(false, s.local);
+      }
+      for (const void* p : s.ops) add(false, p);
+      if (s.dsts.empty()) add(true, s.dst);
+      for (void* p : s.dsts) add(true, p);
+    }
+  }
+  *layout = h;
+  return HOCCL_OK;
+}
+
+void hoccl_layout_destroy(hoccl_layout_t l) { delete l; }
+int hoccl_layout_num_groups(hoccl_layout_t l) { return l ? (int)l->lay.groups.size() : 0; }
+int hoccl_layout_num_pieces(hoccl_layout_t l) { return l ? l->lay.plan.pieces : 0; }
+int hoccl_layout_num_accesses(hoccl_layout_t l) { return l ? (int)l->access.size() : 0; }
+
+hoccl_result_t hoccl_layout_get_access(hoccl_layout_t l, int index, hoccl_access_t* out) {
+  if (!l || !out || index < 0 || index >= (int)l->access.size()) return HOCCL_ERR_INVALID_ARG;
+  *out = l->access[(size_t)index];
+  return HOCCL_OK;
+}
+
+int hoccl_layout_group_deps(hoccl_layout_t l, int group, int* deps, int cap) {
+  if (!l || group < 0 || group >= (int)l->lay.groups.size()) return -1;
+  const RGroup& g = l->lay.groups[(size_t)group];
+  std::vector<int> all = g.deps;
+  if (g.chain_dep >= 0) all.push_back(g.chain_dep);
+  for (int i = 0; i < (int)all.size() && deps && i < cap; i++) deps[i] = all[(size_t)i];
+  return (int)all.size();
+}
+
+int hoccl_layout_signature(hoccl_layout_t l, uint64_t* words, int cap) {
+  if (!l) return 0;
+  for (int i = 0; i < (int)l->key.size() && words && i < cap; i++) words[i] = l->key[(size_t)i];
+  return (int)l->key.size();
+}
 
 }  // extern "C"
 

@@ -38,7 +38,7 @@ struct Seg {
   uint64_t host_off = 0;  // HOCCL_PATH_CE_HOST: where this move bounces in the pinned host staging
   int nsrc = 1;           // OP_CHAIN: inbox operands at src + j * src_stride
   uint64_t src_stride = 0;
-  // OP_CHAIN that reads the contributions where they lie (see read_in_place): all operands in the order of addition, the owner's
+  // OP_CHAIN that reads the contributions where they lie (see contributions() in exec.cu): all operands in the order of addition, the owner's
   // last; and, if the sum stores the result for every rank, all destinations (otherwise `dst`)
   std::vector<const void*> ops;
   std::vector<void*> dsts;
@@ -197,6 +197,13 @@ struct Call {
   void* const* h_recv = nullptr;
 };
 
+// A call laid out: its plan, and the plan's groups over the call's addresses.
+struct Layout {
+  Plan plan;
+  std::vector<RGroup> groups;
+  size_t host_need = 0;   // bytes of pinned host staging the moves bounce through (HOCCL_PATH_CE_HOST)
+  bool overlap = false;   // copy route: the pieces' parts run on three internal streams
+};
 
 // What a driver copy inside one device does at once, as timed on B200: a copy of 1 MiB or more whose destination does not start on a
 // 128-byte line or whose length is not a multiple of 4 KiB takes 4 us more than a whole one (8 MiB 8.3 against 4.3 us, 64 MiB 28.7
@@ -248,6 +255,8 @@ hoccl_result_t build_roles(hoccl_comm* c, const Plan& P, const std::vector<RGrou
 hoccl_result_t launch_roles(hoccl_comm* c, GraphEntry* entry, cudaStream_t stream);
 // exec.cu
 hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user);
+// What run_collective would run for this call, and the signature its graph would be cached under; nothing is enqueued.
+hoccl_result_t inspect_call(hoccl_comm* c, Call* call, Layout* out, std::vector<uint64_t>* key);
 hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, cudaStream_t user, Tally* tally);
 // HOCCL_OK if the communicator's settings fit together for such a call (see options.h); nothing is enqueued
 hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype);

@@ -119,8 +119,13 @@ static Contributions contributions(const hoccl_comm* c, const Call& call, const 
 
 // Copy route, contributions read in place: the all-gather's copies keep what the driver does at once and their ends (less than 128 bytes
 // in front, less than 4 KiB behind) go to one launch of the copy kernel per piece, "copy_ctas" CTAs, instead of a second pass per copy.
+// The ends take over what their copy waited for.  That is all they need only while no copy waits for another copy: in a ring
+// all-gather a step forwards what the step before it has written, ends included, so its copies stay whole.
 static void trim_driver_copies(std::vector<RGroup>* groups) {
   const size_t n = groups->size();
+  for (const RGroup& g : *groups)
+    for (int d : g.deps)
+      if (g.kind == OP_MOVE && (*groups)[(size_t)d].kind == OP_MOVE) return;
   for (size_t g = 0; g < n; g++) {
     if ((*groups)[g].kind != OP_MOVE) continue;
     RGroup ends = (*groups)[g];
@@ -866,18 +871,145 @@ static hoccl_result_t run_host_in_place(hoccl_comm* c, const Call& call, std::ve
   return launch_entry(c, cache_put(c, std::move(entry)), user, t0);
 }
 
+// How the communicator's settings combine for this call (options.h); a contradictory combination is refused here.
+static hoccl_result_t call_options(hoccl_comm* c, const Call& call, OptionsOut* opt) {
+  OptionsIn oin = options_of(c, call.kind, call.count, call.dtype, call.h_send != nullptr);
+  if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && (call.kind == PLAN_ALLGATHER || call.kind == PLAN_ALLTOALL) && blocks_bad_for_driver(c, call))
+    oin.ce_small_bytes = LONG_MAX;
+  return resolve_options(oin, opt);
+}
+
+// Pure host work, nothing is enqueued.  The communicator shows the call's route (RouteGuard).
+static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut& opt, Contributions how, Layout* out) {
+  const bool fused = opt.executor == EXEC_ONE_KERNEL, roles = opt.executor == EXEC_ROLES;
+  Plan& P = out->plan;
+  unsigned char align[kMaxRanks];
+  for (int r = 0; r < c->R; r++) align[r] = (unsigned char)((uintptr_t)call.send[r] & 15);
+  const int plan_kind = opt.plan_kind;
+  // Piece size: the caller's if set.  Otherwise: on the SM path under CTA budgets a reduction is cut into at least two
+  // pieces (the copy kernel of one piece then overlaps the sum kernel of the other: measured 1.6x on a 3 MiB chunk with
+  // 8 + 8 CTAs) of at most 4 MiB.  That does not pay with driver copies (they take the whole GPU and never overlap a sum:
+  // every extra copy only adds its start-up) nor with whole-GPU grids (two kernels then share the same SMs), so the
+  // copy route and the SM path with 128 CTAs or more for both kernels keep whole chunks up to 256 MiB (measured, R = 8,
+  // bf16, 64 MiB to 1 GiB per rank: 7-15 % faster than 4 MiB pieces on the copy route with 8-CTA sums, 19-33 % with
+  // 148-CTA sums, 3-14 % on the whole-GPU SM path).
+  size_t piece_bytes = (size_t)c->piece_bytes;
+  int max_pieces = (int)c->max_pieces;
+  const bool reduction = call.kind == PLAN_ALLREDUCE || call.kind == PLAN_REDUCE_SCATTER;
+  const size_t ring_chunk = (call.kind == PLAN_ALLREDUCE ? (call.count + c->R - 1) / c->R : call.count) * dtype_size(call.dtype);
+  // the staged form of the direct schedule: 5 pieces at 25 MiB per rank (8 ranks 5.23 ms; 8 pieces 5.27), 4 at 16 MiB (3.58; 3.81)
+  const size_t host_np = call.h_send && (opt.plan_kind & PLAN_FLAG_RS_DIRECT) ? host_pieces(c, call.count * dtype_size(call.dtype), 1e6) : (size_t)c->host_pieces;
+  const bool sum_only = how == READ_AND_STORE || (how == READ_IN_PLACE && call.kind == PLAN_REDUCE_SCATTER);   // no moves at all
+  // Copy route with overlap ("ce_overlap"): the direct schedule cut into pieces whose three parts run on three internal
+  // streams (see launch_entry).  Automatic (-1): 2 pieces from 2 MiB per ring chunk, from 4 MiB on pieces of about 4 MiB, at
+  // least 4 and at most 32 of them; below that the ~30 us of host time per call and the extra copies cost more than the overlap
+  // gives (measured on B200, R = 8, bf16, 8-CTA sums: 25 MiB per rank 0.290 -> 0.280 ms with 2 pieces; 40 MiB 0.468 -> 0.421 with
+  // 4; 256 MiB 2.97 -> 2.44 with 8; 1 GiB 11.8 -> 9.72 with 8, 9.52 with 32).
+  long overlap_pieces = c->ce_overlap;
+  if (overlap_pieces < 0) {
+    // (whole-GPU sums are short: beside them more than 8 pieces only add copies; 1 GiB per rank 6.34 ms with 8, 6.80 with 32)
+    const size_t most = c->sum_ctas >= 64 ? 8 : 32;
+    overlap_pieces = ring_chunk >= ((size_t)4 << 20) ? (long)std::min<size_t>(most, std::max<size_t>(4, ring_chunk >> 22))
+                                                     : ring_chunk >= ((size_t)2 << 20) ? 2 : 0;
+    // With the contributions read in place only the all-gather's copies are left to hide behind the sums, so fewer and larger
+    // pieces are best, and below 4 MiB per chunk (8 MiB with whole-GPU sums) one graph is (R = 8, bf16, 8-CTA sums: 25 MiB per rank
+    // 0.221 ms whole and 0.221 in 2 pieces, 32 MiB 0.286 / 0.281, 40 MiB 0.364 / 0.344 and 0.348 in 4, 64 MiB 0.600 whole and 0.536 in
+    // 3, 128 MiB 1.058 in 6, 256 MiB 2.088 in 12, 2.138 in 24; 148-CTA sums: 16 MiB 0.056 / 0.076, 64 MiB 0.244 / 0.225, 0.262 in 6)
+    if (how == READ_IN_PLACE) {
+      if (c->sum_ctas >= 64) overlap_pieces = (long)std::min<size_t>(8, ring_chunk >> 22);
+      else overlap_pieces = ring_chunk >= ((size_t)5 << 20) ? (long)std::min<size_t>(32, std::max<size_t>(4, ring_chunk * 3 >> 23))
+                                                            : ring_chunk >= ((size_t)4 << 20) ? 2 : 0;
+    }
+  }
+  const bool overlap = overlap_pieces > 1 && c->path == HOCCL_PATH_CE && opt.executor == EXEC_GRAPH && !call.h_send &&
+                       (plan_kind & PLAN_FLAG_RS_DIRECT) && c->R > 1 && !c->piece_bytes_set && !sum_only;
+  if (sum_only && !c->piece_bytes_set && !call.h_send) {   // nothing to overlap
+    piece_bytes = (size_t)1 << 60;
+    max_pieces = 1;
+  } else if (overlap) {
+    max_pieces = (int)overlap_pieces;
+    piece_bytes = std::max<size_t>((size_t)64 << 10, ((ring_chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
+  } else if (!c->piece_bytes_set && c->path == HOCCL_PATH_SM && opt.executor == EXEC_GRAPH && !call.h_send && reduction &&
+             (plan_kind & PLAN_FLAG_RS_DIRECT) && c->sum_ctas < 64 && c->copy_ctas < 128 && ring_chunk >= ((size_t)1 << 20)) {
+    // SM path, direct schedule under CTA budgets: pieces of an eighth of a ring chunk, between 640 KiB and 2 MiB, issued as a
+    // software pipeline (see build_graph): a piece's copies run beside another piece's chain sum (measured, 8-CTA sums and
+    // 40 copy CTAs: 40 MiB per rank 0.46 ms with 2 pieces, 0.41 with 4, 0.38 with 8, 0.45 with 10; 25 MiB 0.30 / 0.26 / 0.245 /
+    // 0.29 ms with 2 / 4 / 5 / 7 pieces; 256 MiB 2.92 / 2.57 / 2.40 / 2.32 ms with 2 / 4 / 8 / 16 pieces)
+    // With the contributions read in place: a sixth of a chunk, between 1 and 3.25 MiB, from 4 MiB per chunk on (32 MiB per rank
+    // 0.271 ms, 40 MiB 0.329, 64 MiB 0.508, 128 MiB 1.010, 256 MiB 1.978; an eighth: 0.282 / 0.336 / 0.519 / 1.016 / 1.986).
+    if (how == READ_IN_PLACE && ring_chunk >= kGradeInPlace)
+      piece_bytes = std::min<size_t>((size_t)3328 << 10, std::max<size_t>((size_t)1 << 20, (ring_chunk / 6 + 1023) / 1024 * 1024));
+    else
+      piece_bytes = std::min<size_t>((size_t)2 << 20, std::max<size_t>((size_t)640 << 10, (ring_chunk / 8 + 1023) / 1024 * 1024));
+    max_pieces = 64;
+  } else if (call.h_send) {   // pipelined host all-reduce: host_pieces pieces per chunk, whatever the chunk size
+    const size_t q = (call.count + c->R - 1) / c->R;
+    const size_t chunk = q * dtype_size(call.dtype);
+    max_pieces = (int)host_np;
+    piece_bytes = std::max<size_t>((size_t)64 << 10, ((chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
+  } else if (roles) {
+    // the piece rule of the graph form of the same schedule (above): both forms measured best with the same pieces
+    if (!c->piece_bytes_set)
+      piece_bytes = std::min<size_t>((size_t)2 << 20, std::max<size_t>((size_t)640 << 10, (ring_chunk / 8 + 1023) / 1024 * 1024));
+    max_pieces = 64;   // (when the tables of that many pieces do not fit into shared memory the graph form runs the plan)
+  } else if (fused) {   // one kernel walks the steps in order; whole chunks measured faster than pieces (fewer barriers and tails)
+    piece_bytes = (size_t)1 << 60;
+    max_pieces = 1;
+  } else if (!c->piece_bytes_set && reduction &&
+             (c->path == HOCCL_PATH_CE || (c->path == HOCCL_PATH_SM && std::min(c->sum_ctas, c->copy_ctas) >= 128))) {
+    // "whole" stops at 256 MiB: several concurrent driver copies of 512 MiB each ran at half speed (R = 2, 1 GiB per rank)
+    piece_bytes = (size_t)256 << 20;
+  } else if (!c->piece_bytes_set && c->path == HOCCL_PATH_SM && std::max(c->sum_ctas, c->copy_ctas) < 64 &&
+      (call.kind == PLAN_ALLREDUCE || call.kind == PLAN_REDUCE_SCATTER)) {
+    const size_t q = call.kind == PLAN_ALLREDUCE ? (call.count + c->R - 1) / c->R : call.count;
+    const size_t chunk = q * dtype_size(call.dtype);
+    if (chunk >= ((size_t)1 << 20)) piece_bytes = std::min(piece_bytes, (chunk / 2 + 1023) / 1024 * 1024);
+  }
+  // graded pieces ("piece_grade"; -1 = automatic): measured on B200 (R = 8, bf16, 8-CTA sums) they gain 1-5 % from 64 MiB per rank
+  // on (256 MiB: copy route 2.46 -> 2.44 ms, SM path 8 + 40 CTAs 2.32 -> 2.27, roles kernel 2.32 -> 2.25) and lose below (40 MiB
+  // buckets: copy route 0.423 -> 0.444 ms, SM path 0.380 -> 0.431: the small outer pieces cost more in fixed time per piece than
+  // their shorter fill saves), so automatic means: from 8 MiB per ring chunk, under a SUM budget (with whole-GPU sums the outer
+  // pieces' moves are no longer what is exposed: 256 MiB per rank, copy route, 148-CTA sums 1.51 -> 1.53 ms)
+  // (with the contributions read in place the SM path gains from 4 MiB per ring chunk on: 40 MiB per rank in 5 pieces 0.340 -> 0.329)
+  const size_t grade_from = how == READ_IN_PLACE && c->path == HOCCL_PATH_SM ? kGradeInPlace : (size_t)8 << 20;
+  const bool graded = reduction && !call.h_send && !fused && (plan_kind & PLAN_FLAG_RS_DIRECT) &&
+                      (c->piece_grade == 1 || (c->piece_grade < 0 && ring_chunk >= grade_from && c->sum_ctas < 64));
+  if (!build_plan(&P, plan_kind | (graded ? PLAN_FLAG_GRADED : 0), c->R, call.count, call.dtype, call.in_place, piece_bytes, max_pieces, align))
+    return HOCCL_ERR_INVALID_ARG;
+  if (P.slot_bytes) {
+    size_t need = P.scratch_need();
+    if (!c->scratch || c->scratch_bytes < need) return HOCCL_ERR_SCRATCH;
+    // scratch must not overlap any rank buffer
+    for (int r = 0; r < c->R; r++)
+      if (ranges_overlap((const char*)c->scratch, need, (const char*)call.send[r], call.send_bytes) ||
+          ranges_overlap((const char*)c->scratch, need, (const char*)call.recv[r], call.recv_bytes))
+        return HOCCL_ERR_INVALID_ARG;
+  }
+  out->overlap = overlap && P.pieces > 1;   // with one piece there is nothing to overlap
+  resolve(c, P, call, how, &out->groups, &out->host_need);
+  return HOCCL_OK;
+}
+
+hoccl_result_t inspect_call(hoccl_comm* c, Call* call, Layout* out, std::vector<uint64_t>* key) {
+  OptionsOut opt;
+  hoccl_result_t rc = call_options(c, *call, &opt);
+  if (rc != HOCCL_OK) return rc;
+  if (opt.executor == EXEC_ONEPASS || call->h_send) return HOCCL_ERR_UNSUPPORTED;
+  RouteGuard guard(c, (hoccl_path_t)opt.path, opt.copy_ctas);
+  *key = make_key(c, *call);
+  rc = validate(c, call);
+  if (rc != HOCCL_OK || call->count == 0) return rc;
+  return lay_out(c, *call, opt, contributions(c, *call, opt, call->count * dtype_size(call->dtype)), out);
+}
+
 hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   const double t0 = now_us();
   if (!c) return HOCCL_ERR_INVALID_ARG;
   if (dtype_size(call->dtype) == 0) return HOCCL_ERR_UNSUPPORTED;
   if (!call->send || !call->recv) return HOCCL_ERR_INVALID_ARG;
-  // One place decides how the settings combine for this call (options.h); a contradictory combination is refused here.
-  OptionsIn oin = options_of(c, call->kind, call->count, call->dtype, call->h_send != nullptr);
-  if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && (call->kind == PLAN_ALLGATHER || call->kind == PLAN_ALLTOALL) && blocks_bad_for_driver(c, *call))
-    oin.ce_small_bytes = LONG_MAX;
   OptionsOut opt;
   {
-    hoccl_result_t orc = resolve_options(oin, &opt);
+    hoccl_result_t orc = call_options(c, *call, &opt);
     if (orc != HOCCL_OK) return orc;
   }
   // a small message on the copy route runs on the copy kernel's route: the communicator shows that route for this call only
@@ -934,117 +1066,16 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
     c->stats.host_launch_us = now_us() - t0;
     return HOCCL_OK;
   }
-  Plan P;
-  unsigned char align[kMaxRanks];
-  for (int r = 0; r < c->R; r++) align[r] = (unsigned char)((uintptr_t)call->send[r] & 15);
-  const int plan_kind = opt.plan_kind;
-  // Piece size: the caller's if set.  Otherwise: on the SM path under CTA budgets a reduction is cut into at least two
-  // pieces (the copy kernel of one piece then overlaps the sum kernel of the other: measured 1.6x on a 3 MiB chunk with
-  // 8 + 8 CTAs) of at most 4 MiB.  That does not pay with driver copies (they take the whole GPU and never overlap a sum:
-  // every extra copy only adds its start-up) nor with whole-GPU grids (two kernels then share the same SMs), so the
-  // copy route and the SM path with 128 CTAs or more for both kernels keep whole chunks up to 256 MiB (measured, R = 8,
-  // bf16, 64 MiB to 1 GiB per rank: 7-15 % faster than 4 MiB pieces on the copy route with 8-CTA sums, 19-33 % with
-  // 148-CTA sums, 3-14 % on the whole-GPU SM path).
-  size_t piece_bytes = (size_t)c->piece_bytes;
-  int max_pieces = (int)c->max_pieces;
-  const bool reduction = call->kind == PLAN_ALLREDUCE || call->kind == PLAN_REDUCE_SCATTER;
-  const size_t ring_chunk = (call->kind == PLAN_ALLREDUCE ? (call->count + c->R - 1) / c->R : call->count) * dtype_size(call->dtype);
   const Contributions how = contributions(c, *call, opt, call->count * dtype_size(call->dtype));
   if (call->h_send && how != STAGED) return run_host_in_place(c, *call, std::move(key), user, t0);
-  // the staged form of the direct schedule: 5 pieces at 25 MiB per rank (8 ranks 5.23 ms; 8 pieces 5.27), 4 at 16 MiB (3.58; 3.81)
-  const size_t host_np = call->h_send && (opt.plan_kind & PLAN_FLAG_RS_DIRECT) ? host_pieces(c, call->count * dtype_size(call->dtype), 1e6) : (size_t)c->host_pieces;
-  const bool sum_only = how == READ_AND_STORE || (how == READ_IN_PLACE && call->kind == PLAN_REDUCE_SCATTER);   // no moves at all
-  // Copy route with overlap ("ce_overlap"): the direct schedule cut into pieces whose three parts run on three internal
-  // streams (see launch_entry).  Automatic (-1): 2 pieces from 2 MiB per ring chunk, from 4 MiB on pieces of about 4 MiB, at
-  // least 4 and at most 32 of them; below that the ~30 us of host time per call and the extra copies cost more than the overlap
-  // gives (measured on B200, R = 8, bf16, 8-CTA sums: 25 MiB per rank 0.290 -> 0.280 ms with 2 pieces; 40 MiB 0.468 -> 0.421 with
-  // 4; 256 MiB 2.97 -> 2.44 with 8; 1 GiB 11.8 -> 9.72 with 8, 9.52 with 32).
-  long overlap_pieces = c->ce_overlap;
-  if (overlap_pieces < 0) {
-    // (whole-GPU sums are short: beside them more than 8 pieces only add copies; 1 GiB per rank 6.34 ms with 8, 6.80 with 32)
-    const size_t most = c->sum_ctas >= 64 ? 8 : 32;
-    overlap_pieces = ring_chunk >= ((size_t)4 << 20) ? (long)std::min<size_t>(most, std::max<size_t>(4, ring_chunk >> 22))
-                                                     : ring_chunk >= ((size_t)2 << 20) ? 2 : 0;
-    // With the contributions read in place only the all-gather's copies are left to hide behind the sums, so fewer and larger
-    // pieces are best, and below 4 MiB per chunk (8 MiB with whole-GPU sums) one graph is (R = 8, bf16, 8-CTA sums: 25 MiB per rank
-    // 0.221 ms whole and 0.221 in 2 pieces, 32 MiB 0.286 / 0.281, 40 MiB 0.364 / 0.344 and 0.348 in 4, 64 MiB 0.600 whole and 0.536 in
-    // 3, 128 MiB 1.058 in 6, 256 MiB 2.088 in 12, 2.138 in 24; 148-CTA sums: 16 MiB 0.056 / 0.076, 64 MiB 0.244 / 0.225, 0.262 in 6)
-    if (how == READ_IN_PLACE) {
-      if (c->sum_ctas >= 64) overlap_pieces = (long)std::min<size_t>(8, ring_chunk >> 22);
-      else overlap_pieces = ring_chunk >= ((size_t)5 << 20) ? (long)std::min<size_t>(32, std::max<size_t>(4, ring_chunk * 3 >> 23))
-                                                            : ring_chunk >= ((size_t)4 << 20) ? 2 : 0;
-    }
-  }
-  const bool overlap = overlap_pieces > 1 && c->path == HOCCL_PATH_CE && opt.executor == EXEC_GRAPH && !call->h_send &&
-                       (plan_kind & PLAN_FLAG_RS_DIRECT) && c->R > 1 && !c->piece_bytes_set && !sum_only;
-  if (sum_only && !c->piece_bytes_set && !call->h_send) {   // nothing to overlap
-    piece_bytes = (size_t)1 << 60;
-    max_pieces = 1;
-  } else if (overlap) {
-    max_pieces = (int)overlap_pieces;
-    piece_bytes = std::max<size_t>((size_t)64 << 10, ((ring_chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
-  } else if (!c->piece_bytes_set && c->path == HOCCL_PATH_SM && opt.executor == EXEC_GRAPH && !call->h_send && reduction &&
-             (plan_kind & PLAN_FLAG_RS_DIRECT) && c->sum_ctas < 64 && c->copy_ctas < 128 && ring_chunk >= ((size_t)1 << 20)) {
-    // SM path, direct schedule under CTA budgets: pieces of an eighth of a ring chunk, between 640 KiB and 2 MiB, issued as a
-    // software pipeline (see build_graph): a piece's copies run beside another piece's chain sum (measured, 8-CTA sums and
-    // 40 copy CTAs: 40 MiB per rank 0.46 ms with 2 pieces, 0.41 with 4, 0.38 with 8, 0.45 with 10; 25 MiB 0.30 / 0.26 / 0.245 /
-    // 0.29 ms with 2 / 4 / 5 / 7 pieces; 256 MiB 2.92 / 2.57 / 2.40 / 2.32 ms with 2 / 4 / 8 / 16 pieces)
-    // With the contributions read in place: a sixth of a chunk, between 1 and 3.25 MiB, from 4 MiB per chunk on (32 MiB per rank
-    // 0.271 ms, 40 MiB 0.329, 64 MiB 0.508, 128 MiB 1.010, 256 MiB 1.978; an eighth: 0.282 / 0.336 / 0.519 / 1.016 / 1.986).
-    if (how == READ_IN_PLACE && ring_chunk >= kGradeInPlace)
-      piece_bytes = std::min<size_t>((size_t)3328 << 10, std::max<size_t>((size_t)1 << 20, (ring_chunk / 6 + 1023) / 1024 * 1024));
-    else
-      piece_bytes = std::min<size_t>((size_t)2 << 20, std::max<size_t>((size_t)640 << 10, (ring_chunk / 8 + 1023) / 1024 * 1024));
-    max_pieces = 64;
-  } else if (call->h_send) {   // pipelined host all-reduce: host_pieces pieces per chunk, whatever the chunk size
-    const size_t q = (call->count + c->R - 1) / c->R;
-    const size_t chunk = q * dtype_size(call->dtype);
-    max_pieces = (int)host_np;
-    piece_bytes = std::max<size_t>((size_t)64 << 10, ((chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
-  } else if (roles) {
-    // the piece rule of the graph form of the same schedule (above): both forms measured best with the same pieces
-    if (!c->piece_bytes_set)
-      piece_bytes = std::min<size_t>((size_t)2 << 20, std::max<size_t>((size_t)640 << 10, (ring_chunk / 8 + 1023) / 1024 * 1024));
-    max_pieces = 64;   // (when the tables of that many pieces do not fit into shared memory the graph form runs the plan)
-  } else if (fused) {   // one kernel walks the steps in order; whole chunks measured faster than pieces (fewer barriers and tails)
-    piece_bytes = (size_t)1 << 60;
-    max_pieces = 1;
-  } else if (!c->piece_bytes_set && reduction &&
-             (c->path == HOCCL_PATH_CE || (c->path == HOCCL_PATH_SM && std::min(c->sum_ctas, c->copy_ctas) >= 128))) {
-    // "whole" stops at 256 MiB: several concurrent driver copies of 512 MiB each ran at half speed (R = 2, 1 GiB per rank)
-    piece_bytes = (size_t)256 << 20;
-  } else if (!c->piece_bytes_set && c->path == HOCCL_PATH_SM && std::max(c->sum_ctas, c->copy_ctas) < 64 &&
-      (call->kind == PLAN_ALLREDUCE || call->kind == PLAN_REDUCE_SCATTER)) {
-    const size_t q = call->kind == PLAN_ALLREDUCE ? (call->count + c->R - 1) / c->R : call->count;
-    const size_t chunk = q * dtype_size(call->dtype);
-    if (chunk >= ((size_t)1 << 20)) piece_bytes = std::min(piece_bytes, (chunk / 2 + 1023) / 1024 * 1024);
-  }
-  // graded pieces ("piece_grade"; -1 = automatic): measured on B200 (R = 8, bf16, 8-CTA sums) they gain 1-5 % from 64 MiB per rank
-  // on (256 MiB: copy route 2.46 -> 2.44 ms, SM path 8 + 40 CTAs 2.32 -> 2.27, roles kernel 2.32 -> 2.25) and lose below (40 MiB
-  // buckets: copy route 0.423 -> 0.444 ms, SM path 0.380 -> 0.431: the small outer pieces cost more in fixed time per piece than
-  // their shorter fill saves), so automatic means: from 8 MiB per ring chunk, under a SUM budget (with whole-GPU sums the outer
-  // pieces' moves are no longer what is exposed: 256 MiB per rank, copy route, 148-CTA sums 1.51 -> 1.53 ms)
-  // (with the contributions read in place the SM path gains from 4 MiB per ring chunk on: 40 MiB per rank in 5 pieces 0.340 -> 0.329)
-  const size_t grade_from = how == READ_IN_PLACE && c->path == HOCCL_PATH_SM ? kGradeInPlace : (size_t)8 << 20;
-  const bool graded = reduction && !call->h_send && !fused && (plan_kind & PLAN_FLAG_RS_DIRECT) &&
-                      (c->piece_grade == 1 || (c->piece_grade < 0 && ring_chunk >= grade_from && c->sum_ctas < 64));
-  if (!build_plan(&P, plan_kind | (graded ? PLAN_FLAG_GRADED : 0), c->R, call->count, call->dtype, call->in_place, piece_bytes, max_pieces, align))
-    return HOCCL_ERR_INVALID_ARG;
-  if (P.slot_bytes) {
-    size_t need = P.scratch_need();
-    if (!c->scratch || c->scratch_bytes < need) return HOCCL_ERR_SCRATCH;
-    // scratch must not overlap any rank buffer
-    for (int r = 0; r < c->R; r++)
-      if (ranges_overlap((const char*)c->scratch, need, (const char*)call->send[r], call->send_bytes) ||
-          ranges_overlap((const char*)c->scratch, need, (const char*)call->recv[r], call->recv_bytes))
-        return HOCCL_ERR_INVALID_ARG;
-  }
+  Layout lay;
+  rc = lay_out(c, *call, opt, how, &lay);
+  if (rc != HOCCL_OK) return rc;
+  const Plan& P = lay.plan;
+  const std::vector<RGroup>& groups = lay.groups;
   c->stats.n_pieces = P.pieces;
   c->stats.max_sum_ctas = 0;
-  std::vector<RGroup> groups;
-  size_t host_need = 0;
-  resolve(c, P, *call, how, &groups, &host_need);
-  if (c->path == HOCCL_PATH_CE_HOST && (!c->host_staging || host_need > c->host_staging_bytes)) return HOCCL_ERR_SCRATCH;
+  if (c->path == HOCCL_PATH_CE_HOST && (!c->host_staging || lay.host_need > c->host_staging_bytes)) return HOCCL_ERR_SCRATCH;
   if (graphs) {
     if (c->handshake) {
       // Driver copies share a hardware queue with the copies the parked stream has queued behind its hand-over; a copy
@@ -1074,7 +1105,7 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
           return rc;
         }
       }
-    } else if (overlap && P.pieces > 1) {   // with one piece there is nothing to overlap: one graph
+    } else if (lay.overlap) {
       entry.part_exec.assign((size_t)P.pieces * 3, nullptr);
       for (int p = 0; p < P.pieces && rc == HOCCL_OK; p++)
         for (int part = 0; part < 3 && rc == HOCCL_OK; part++) rc = build_graph(c, P, groups, &entry, p, &entry.part_exec[(size_t)p * 3 + part], part);

@@ -15,8 +15,9 @@ BUF_SEND, BUF_RECV, BUF_INBOX, BUF_PARTIAL = 0, 1, 2, 3
 EXEC_GRAPH, EXEC_STREAMS, EXEC_ONE_KERNEL, EXEC_ONEPASS, EXEC_PROXY, EXEC_ROLES = range(6)
 
 EXPORTS = [   # every function include/hoccl_diag.h declares
-    "hoccl_chain_launch", "hoccl_copy_launch", "hoccl_fanout_inspect", "hoccl_fanout_launch", "hoccl_flatten_inspect",
-    "hoccl_kernel_sms", "hoccl_options_resolve", "hoccl_plan_build", "hoccl_plan_destroy", "hoccl_plan_get_op",
+    "hoccl_chain_launch", "hoccl_comm_init_host_only", "hoccl_copy_launch", "hoccl_fanout_inspect", "hoccl_fanout_launch", "hoccl_flatten_inspect",
+    "hoccl_kernel_sms", "hoccl_layout_build", "hoccl_layout_destroy", "hoccl_layout_get_access", "hoccl_layout_group_deps",
+    "hoccl_layout_num_accesses", "hoccl_layout_num_groups", "hoccl_layout_num_pieces", "hoccl_layout_signature", "hoccl_options_resolve", "hoccl_plan_build", "hoccl_plan_destroy", "hoccl_plan_get_op",
     "hoccl_plan_group_deps", "hoccl_plan_inbox_slots", "hoccl_plan_num_groups", "hoccl_plan_num_ops",
     "hoccl_plan_scratch_bytes", "hoccl_plan_slot_bytes", "hoccl_port_probe", "hoccl_probe_copy_routes",
     "hoccl_probe_move_needs_sm", "hoccl_selftest_barrier_timeout", "hoccl_selftest_roles_timeout", "hoccl_selftest_bf16_add", "hoccl_sum_launch",
@@ -48,6 +49,11 @@ class Options(ctypes.Structure):
 class Resolved(ctypes.Structure):
     _fields_ = [("plan_kind", ctypes.c_int), ("executor", ctypes.c_int), ("path", ctypes.c_int), ("copy_ctas", ctypes.c_long),
                 ("small_switch", ctypes.c_int)]
+
+
+class Access(ctypes.Structure):
+    _fields_ = [("group", ctypes.c_int), ("segment", ctypes.c_int), ("kind", ctypes.c_int), ("piece", ctypes.c_int), ("edges", ctypes.c_int),
+                ("write", ctypes.c_int), ("addr", ctypes.c_uint64), ("bytes", ctypes.c_uint64)]
 
 
 _ready = False
@@ -83,6 +89,15 @@ def lib() -> ctypes.CDLL:
         "hoccl_plan_num_groups": (i, [vp]),
         "hoccl_plan_get_op": (i, [vp, i, ctypes.POINTER(PlanOp)]),
         "hoccl_plan_group_deps": (i, [vp, i, ctypes.POINTER(i), i]),
+        "hoccl_comm_init_host_only": (i, [vpp, i]),
+        "hoccl_layout_build": (i, [vpp, vp, i, vpp, vpp, sz, i]),
+        "hoccl_layout_destroy": (None, [vp]),
+        "hoccl_layout_num_groups": (i, [vp]),
+        "hoccl_layout_num_pieces": (i, [vp]),
+        "hoccl_layout_num_accesses": (i, [vp]),
+        "hoccl_layout_get_access": (i, [vp, i, ctypes.POINTER(Access)]),
+        "hoccl_layout_group_deps": (i, [vp, i, ctypes.POINTER(i), i]),
+        "hoccl_layout_signature": (i, [vp, ctypes.POINTER(ctypes.c_uint64), i]),
         "hoccl_options_resolve": (i, [ctypes.POINTER(Options), ctypes.POINTER(Resolved)]),
     }
     for name, (res, args) in sigs.items():
@@ -237,3 +252,36 @@ class Plan:
         self._h = None
 
 
+class Layout:
+    """Host-only view of what a call over these addresses would run (hoccl_layout_build): `deps` of every group, all its accesses
+    and the signature of its graph.  `path`, `scratch` = (address, bytes) and params as a communicator gets them."""
+
+    def __init__(self, kind, R, send, recv, count, dtype, path=_b.PATH_CE, scratch=None, **params):
+        L = lib()
+        c, h = ctypes.c_void_p(), ctypes.c_void_p()
+        assert L.hoccl_comm_init_host_only(ctypes.byref(c), R) == OK
+        try:
+            rcs = [L.hoccl_comm_set_path(c, path)] + [L.hoccl_comm_set_param(c, k.encode(), v) for k, v in params.items()]
+            if scratch:
+                rcs.append(L.hoccl_comm_set_scratch(c, *scratch))
+            assert all(rc == OK for rc in rcs), (params, rcs)
+            rc = L.hoccl_layout_build(ctypes.byref(h), c, kind, _ptr_array(send), _ptr_array(recv), count, _dtype(dtype))
+            if rc != OK:
+                raise HocclError(rc, "hoccl_layout_build")
+        finally:
+            L.hoccl_comm_destroy(c)
+        self.num_pieces = L.hoccl_layout_num_pieces(h)
+        self.deps = []
+        for g in range(L.hoccl_layout_num_groups(h)):
+            buf = (ctypes.c_int * L.hoccl_layout_group_deps(h, g, None, 0))()
+            L.hoccl_layout_group_deps(h, g, buf, len(buf))
+            self.deps.append(list(buf))
+        self.accesses = []
+        for k in range(L.hoccl_layout_num_accesses(h)):
+            a = Access()
+            assert L.hoccl_layout_get_access(h, k, ctypes.byref(a)) == OK
+            self.accesses.append(a)
+        words = (ctypes.c_uint64 * L.hoccl_layout_signature(h, None, 0))()
+        L.hoccl_layout_signature(h, words, len(words))
+        self.signature = tuple(words)
+        L.hoccl_layout_destroy(h)

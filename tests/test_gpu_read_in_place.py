@@ -103,3 +103,23 @@ def test_overlapped_pieces(oracle, cfg):
         st = comm.last_stats()
         assert st["n_sum_launches"] == st["n_pieces"] and (st["n_pieces"] > 1 or cfg.get("sum_ctas") == 148), st
         comm.destroy()
+
+
+@pytest.mark.parametrize("use_graph", [0, 1])
+@pytest.mark.parametrize("ag_direct", [0, 1])
+@pytest.mark.parametrize("R", [6, 8])
+def test_ragged_chunks_of_driver_copies(oracle, R, ag_direct, use_graph):
+    """Chunks from 1 MiB on that are not whole pages on 128-byte lines: a direct all-gather leaves the copies' ends to the copy kernel, a
+    ring forwards whole copies.  Buffers with one 16-byte phase on one and on several 128-byte phases, whole and in pieces."""
+    dtype, n = "bf16", R * 600_003 - 2
+    xs = W.rank_inputs("uniform", 530 + R, R, n, dtype)
+    want = oracle.ring_allreduce(xs)
+    for params in (dict(), dict(piece_bytes=400 << 10, max_pieces=8)):
+        comm = auto_comm(R, n, dtype, hb.PATH_CE, ce_small_bytes=4096, ag_direct=ag_direct, use_graph=use_graph, **params)
+        for offs in ([0] * R, [16 * (r % 8) for r in range(R)]):
+            for in_place in (False, True):
+                for rep in range(3):
+                    got = run_allreduce(comm, xs, dtype, in_place=in_place, offs=offs)
+                    assert all(same_bits(got[r], want[r], dtype) for r in range(R)), (R, params, offs, in_place, rep)
+        assert (comm.last_stats()["n_move_launches"] > 0) == (ag_direct == 1 and not params), comm.last_stats()
+        comm.destroy()

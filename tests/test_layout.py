@@ -1,0 +1,111 @@
+"""What a call would run, over addresses that need not exist (hoccl_layout_*, host only): whatever the settings and however the
+buffers lie, two accesses to the same byte, one of them a write, are ordered by dependencies; every byte of the result is written;
+nothing outside the call's buffers is touched."""
+import numpy as np
+import pytest
+from hypothesis import HealthCheck, given, settings, strategies as st
+
+from paper_2609_34334_b200 import binding as hb
+from paper_2609_34334_b200 import diag as hd
+from paper_2609_34334_b200 import workloads as W
+
+ALLREDUCE, REDUCE_SCATTER, ALLGATHER, ALLTOALL = hd.PLAN_ALLREDUCE, hd.PLAN_REDUCE_SCATTER, hd.PLAN_ALLGATHER, hd.PLAN_ALLTOALL
+ROOM = 1 << 36       # every buffer has this much address space to itself
+
+
+def lay_out(kind, R, count, dtype, in_place=False, offs=None, **params):
+    """The layout, and [first, last) of every send, receive and scratch region."""
+    e = W.elem_size(dtype)
+    ssize = count * e * (R if kind in (REDUCE_SCATTER, ALLTOALL) else 1)
+    rsize = count * e * (R if kind in (ALLGATHER, ALLTOALL) else 1)
+    offs = offs or [0] * R
+    send = [(1 + r) * ROOM + offs[r] for r in range(R)]
+    recv = [(101 + r) * ROOM + offs[-1 - r] for r in range(R)]
+    if in_place:
+        recv = send if kind == ALLREDUCE else [send[r] + r * count * e for r in range(R)] if kind == REDUCE_SCATTER else recv
+        send = [recv[r] + r * count * e for r in range(R)] if kind == ALLGATHER else send
+    n = count if kind == ALLREDUCE else count * R
+    scratch = (300 * ROOM, hb.scratch_bytes_direct(R, n, dtype))
+    lay = hd.Layout(kind, R, send, recv, count, dtype, scratch=scratch if scratch[1] else None, **params)
+    return lay, [(p, p + ssize) for p in send], [(p, p + rsize) for p in recv], (scratch[0], scratch[0] + scratch[1])
+
+
+def check(lay, send, recv, scratch, whole_recv):
+    before = []                                          # groups that are done when group g starts, as a bit set
+    for g, deps in enumerate(lay.deps):
+        assert all(0 <= d < g for d in deps)
+        before.append(0)
+        for d in deps:
+            before[g] |= before[d] | 1 << d
+    acc = [a for a in lay.accesses if a.bytes]
+    lo = np.array([a.addr for a in acc], dtype=np.uint64)
+    hi = lo + np.array([a.bytes for a in acc], dtype=np.uint64)
+    readable, writable = send + recv + [scratch], recv + [scratch]
+    for k, a in enumerate(acc):
+        assert any(f <= a.addr and a.addr + a.bytes <= l for f, l in (writable if a.write else readable)), (a.addr, a.bytes)
+        if not a.write:
+            continue
+        for j in np.nonzero((lo < hi[k]) & (hi > lo[k]))[0]:
+            b = acc[j]
+            if (b.group, b.segment) == (a.group, a.segment):
+                assert b.addr == a.addr and (j == k or not b.write)        # an element-wise sum may write what it reads, in place
+            else:
+                assert a.group != b.group, "two segments of one group meet"
+                first, second = sorted((a.group, b.group))
+                assert before[second] >> first & 1, "groups %d and %d (ends of copies: %d, %d) are not ordered" % (a.group, b.group, a.edges, b.edges)
+    for first, last in (recv if whole_recv else []):
+        at = first
+        for f, l in sorted((a.addr, a.addr + a.bytes) for a in acc if a.write and first <= a.addr < last):
+            assert f <= at
+            at = max(at, l)
+        assert at == last
+
+
+@pytest.mark.parametrize("pieces", [None, 3])
+@pytest.mark.parametrize("ag_direct", [0, 1, 2])
+@pytest.mark.parametrize("R", [2, 3, 6, 8])
+def test_ends_of_trimmed_copies(R, ag_direct, pieces):
+    """Chunks of 1 MiB and more that are not whole pages on 128-byte lines: the copies of the all-gather leave their ends to the copy
+    kernel.  In the ring form a step forwards what the step before it wrote."""
+    for chunk in ((1 << 20) + 8, (65 << 20) + 6, 3 << 20):                   # bytes; beyond 64 MiB the automatic all-gather is the ring
+        for offs in ([0] * R, [32] * R, [16 * (r % 8) for r in range(R)]):    # one 16-byte phase, with one and with several 128-byte phases
+            for in_place in (False, True):
+                params = dict(ag_direct=ag_direct, ce_small_bytes=1 << 20, max_pieces=8)
+                if pieces:
+                    params["piece_bytes"] = chunk // pieces + 1
+                lay, send, recv, scratch = lay_out(ALLREDUCE, R, R * chunk // 2 - 3, "bf16", in_place, offs, **params)
+                check(lay, send, recv, scratch, not in_place)
+                if ag_direct == 0 and R > 2 and chunk != 3 << 20:
+                    assert any(not a.edges and a.kind == hd.OP_MOVE and a.bytes % 4096 for a in lay.accesses)
+
+
+case = st.fixed_dictionaries({
+    "kind": st.sampled_from([ALLREDUCE, ALLREDUCE, REDUCE_SCATTER, ALLGATHER, ALLTOALL]),
+    "R": st.integers(1, 10),
+    "count": st.one_of(st.integers(1, 300), st.integers(1000, 400_000), st.integers(400_000, 40_000_000)),
+    "dtype": st.sampled_from(["fp32", "bf16"]),
+    "in_place": st.booleans(),
+    "path": st.sampled_from([hb.PATH_CE, hb.PATH_CE, hb.PATH_SM, hb.PATH_CE_HOST]),
+    "common": st.sampled_from([None, 0, 0, 1, 5, 32]),                       # one offset for all buffers, or one each
+    "offs": st.lists(st.integers(0, 70), min_size=10, max_size=10),
+    "params": st.fixed_dictionaries({
+        "ag_direct": st.integers(0, 2), "rs_direct": st.integers(0, 2), "ce_small_bytes": st.sampled_from([0, 65536, 8 << 20]),
+        "sum_ctas": st.sampled_from([1, 8, 148]), "copy_ctas": st.sampled_from([8, 40, 148]), "use_graph": st.integers(0, 1),
+        "ce_overlap": st.sampled_from([-1, -1, 0, 3]), "piece_grade": st.integers(-1, 1), "max_pieces": st.integers(1, 9)},
+        optional={"piece_bytes": st.sampled_from([1024, 1 << 16, 1 << 20]), "forward": st.just(1), "fused": st.just(1), "roles": st.just(1)}),
+})
+
+
+@settings(max_examples=300, deadline=None, derandomize=True, suppress_health_check=list(HealthCheck))
+@given(c=case)
+def test_random_calls(c):
+    e = W.elem_size(c["dtype"])
+    count = c["count"] if c["kind"] == ALLREDUCE else -(-c["count"] // c["R"])
+    offs = [(o if c["common"] is None else c["common"]) * e for o in c["offs"][:c["R"]]]
+    in_place = c["in_place"] and c["kind"] != ALLTOALL
+    try:
+        lay, send, recv, scratch = lay_out(c["kind"], c["R"], count, c["dtype"], in_place, offs, path=c["path"], **c["params"])
+    except hb.HocclError as err:
+        assert err.code == hb.ERR_UNSUPPORTED, c                             # settings that do not fit together
+        return
+    check(lay, send, recv, scratch, not in_place)

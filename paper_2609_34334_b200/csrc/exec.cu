@@ -576,7 +576,7 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
 
 std::vector<uint64_t> make_key(hoccl_comm* c, const Call& call) {
   std::vector<uint64_t> k;
-  k.reserve(17 + 2 * c->R);
+  k.reserve(26 + 2 * c->R);
   k.push_back((uint64_t)call.kind);
   k.push_back((uint64_t)call.count);
   k.push_back((uint64_t)call.dtype);
@@ -588,6 +588,7 @@ std::vector<uint64_t> make_key(hoccl_comm* c, const Call& call) {
   k.push_back((uint64_t)c->max_pieces);
   k.push_back((uint64_t)c->profile);
   k.push_back((uint64_t)c->ce_sub_bytes);
+  k.push_back((uint64_t)(c->ce_small_bytes > 0));   // whether driver copies leave their ends to the copy kernel
   k.push_back((uint64_t)c->forward);
   k.push_back((uint64_t)c->ag_direct);
   k.push_back((uint64_t)c->order_kernels);

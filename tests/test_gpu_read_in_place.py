@@ -123,3 +123,19 @@ def test_ragged_chunks_of_driver_copies(oracle, R, ag_direct, use_graph):
                     assert all(same_bits(got[r], want[r], dtype) for r in range(R)), (R, params, offs, in_place, rep)
         assert (comm.last_stats()["n_move_launches"] > 0) == (ag_direct == 1 and not params), comm.last_stats()
         comm.destroy()
+
+
+def test_changed_setting_is_not_served_from_the_graph_of_the_old_one(oracle):
+    R, dtype, n = 8, "bf16", 8 * 600_003
+    xs = W.rank_inputs("uniform", 540, R, n, dtype)
+    want = oracle.ring_allreduce(xs)
+    comm = auto_comm(R, n, dtype, hb.PATH_CE)
+    send, recv = ([DevBuf(n * 2).put(x) for x in xs] for _ in range(2))
+    for small, launches, hit in ((8 << 20, 1, 0), (8 << 20, 1, 1), (0, 0, 0), (0, 0, 1), (4 << 20, 1, 1)):
+        comm.set_param("ce_small_bytes", small)
+        comm.allreduce(send, recv, n, dtype)
+        torch.cuda.synchronize()
+        assert all(same_bits(recv[r].get(np_dtype(dtype)), want[r], dtype) for r in range(R))
+        st = comm.last_stats()
+        assert (st["n_move_launches"], st["graph_hit"]) == (launches, hit), (small, st)
+    comm.destroy()

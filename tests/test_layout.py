@@ -109,3 +109,34 @@ def test_random_calls(c):
         assert err.code == hb.ERR_UNSUPPORTED, c                             # settings that do not fit together
         return
     check(lay, send, recv, scratch, not in_place)
+
+
+def _steps(lay):
+    return lay.deps, [tuple(getattr(a, f) for f, _ in a._fields_) for a in lay.accesses]
+
+
+def test_signature_of_trimmed_copies():
+    """An all-reduce above the small-message size, before and after "ce_small_bytes" = 0: without and with whole driver copies, so not
+    the same graph."""
+    a, b = (lay_out(ALLREDUCE, 8, 8 * 600_003, "bf16", **params)[0] for params in ({}, {"ce_small_bytes": 0}))
+    assert any(x.edges for x in a.accesses) and not any(x.edges for x in b.accesses) and a.signature != b.signature
+
+
+@settings(max_examples=300, deadline=None, derandomize=True, suppress_health_check=list(HealthCheck))
+@given(c=case, name=st.sampled_from(["ag_direct", "rs_direct", "ce_small_bytes", "sum_ctas", "copy_ctas", "ce_overlap", "piece_grade", "max_pieces",
+                                     "piece_bytes", "path"]), k=st.integers(0, 3))
+def test_one_setting_changed(c, name, k):
+    """Calls that share a signature replay one graph, so they have to share the layout too."""
+    values = {"ag_direct": [0, 1, 2], "rs_direct": [0, 1, 2], "ce_small_bytes": [0, 1000, 1 << 30], "sum_ctas": [4, 100, 148], "copy_ctas": [4, 100, 148],
+              "ce_overlap": [-1, 0, 2], "piece_grade": [-1, 0, 1], "max_pieces": [1, 2, 9], "piece_bytes": [1 << 14, 1 << 18, 1 << 22],
+              "path": [hb.PATH_CE, hb.PATH_SM, hb.PATH_CE_HOST]}[name]
+    count = c["count"] if c["kind"] == ALLREDUCE else -(-c["count"] // c["R"])
+    offs = [(o if c["common"] is None else c["common"]) * W.elem_size(c["dtype"]) for o in c["offs"][:c["R"]]]
+    first = dict(c["params"], path=c["path"], use_graph=1)
+    try:
+        one, two = (lay_out(c["kind"], c["R"], count, c["dtype"], c["in_place"] and c["kind"] != ALLTOALL, offs, **params)[0]
+                    for params in (first, dict(first, **{name: values[k % 3]})))
+    except hb.HocclError as err:
+        assert err.code == hb.ERR_UNSUPPORTED, c
+        return
+    assert one.signature != two.signature or _steps(one) == _steps(two), (c, name)

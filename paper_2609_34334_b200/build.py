@@ -1,5 +1,5 @@
-"""Builds libhoccl.so (sm_100a, nvcc) and the Python call entry points _calls.so (gcc) in-tree from csrc/.  No JIT cache: both sit
-next to this file."""
+"""Builds libhoccl.so (sm_100a, nvcc) and the Python call entry points _calls (gcc) in-tree from csrc/.  No JIT cache: both sit next to
+this file."""
 from __future__ import annotations
 
 import os
@@ -10,7 +10,9 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhoccl.so")
-CALLS, CALLS_SOURCE = os.path.join(HERE, "_calls.so"), os.path.join(CSRC, "calls.c")
+# The name carries the interpreter's ABI (".cpython-312-x86_64-linux-gnu.so"): each interpreter that uses the tree has a module of its
+# own and looks for that name before a plain "_calls.so".
+CALLS, CALLS_SOURCE = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX")), os.path.join(CSRC, "calls.c")
 SOURCES = ["api.cu", "exec.cu", "p2p.cu", "kernels.cu", "plan.cpp", "static_scratch.cu", "proxy.cu", "sched.cpp", "probe.cu", "ring.cu", "graph.cu", "ring_host.cu", "options.cpp", "roles.cu"]
 HEADERS = ["comm.h", "kernels.cuh", "device_common.cuh", "plan.h", "proxy.h", "sched.h", "options.h", os.path.join("..", "..", "include", "hoccl.h"), os.path.join("..", "..", "include", "hoccl_diag.h")]
 NVCC_FLAGS = [
@@ -45,7 +47,7 @@ def build_calls(force: bool = False) -> str:
         res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
         if res.returncode != 0:
             sys.stderr.write(res.stdout)
-            raise RuntimeError("gcc failed building _calls.so")
+            raise RuntimeError("gcc failed building " + os.path.basename(CALLS))
         os.replace(tmp, CALLS)
     return CALLS
 

@@ -1,8 +1,13 @@
 """Argument marshalling of the inner-loop calls (csrc/calls.c), on argument errors the library reports without a device."""
+import os
+import sys
+import sysconfig
+
 import numpy as np
 import pytest
 
 from paper_2609_34334_b200 import binding as hb
+from paper_2609_34334_b200 import build
 
 
 class Buf:
@@ -41,3 +46,11 @@ def test_wrong_types_raise():
             call()
     assert c.alltoallv(None, 2, [Buf(256)], np.arange(4), [1, 2], [2], [0] * 4, "fp32", 0) == hb.ERR_INVALID_ARG    # no communicator
     assert c.send(None, Buf(256), np.int32(3), np.int64(1), 0, 1, Stream()) == hb.ERR_INVALID_ARG
+
+
+def test_module_is_built_for_this_interpreter():
+    """The file name carries the interpreter's ABI, so that a tree used by two interpreters holds a module for each."""
+    hb.lib()
+    loaded = os.path.basename(hb._calls.__file__)
+    assert loaded == "_calls" + sysconfig.get_config_var("EXT_SUFFIX") and sys.implementation.cache_tag.split("-")[1] in loaded
+    assert hb._calls.__file__ == build.CALLS

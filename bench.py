@@ -1,7 +1,7 @@
 #!/usr/bin/env python
 """Benchmark of the collective hot path on B200.
 
-    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--no-extras] [--no-large]
+    python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--no-extras] [--no-large] [--tables auto|line|stderr]
 
 Workload (N = 1): the largest single-GPU configuration, the GPT-6.7B-shaped data-parallel gradient stream: 32 layers of
 hidden 4096 / FFN 16384 bf16 gradients, normal(0, 1e-3), seed 3, cut flat into 40 MiB buckets (307 of them and one of
@@ -13,10 +13,11 @@ all-gather's moves), on the copy route with at most 8 CTAs for sums, default set
 Reported value: all-reduce bus bandwidth, S * 2(R-1)/R / t_step in GB/s (nccl-tests convention).  With N GPUs, N
 independent replicas run and the value is the sum of their units over the slowest replica's time.  One JSON line on
 stdout (rank 0).  Beside the headline the line carries: the same workload on the ring schedule step by step
-(`ring_schedule`), the per-launch roofline of the dominant kernel of each, the end-to-end figure through host buffers,
-the CPU oracle timed on the host cores, `large_messages` (64 MiB to 1 GiB per rank, every collective, copy route against
-SM path, each checked against the oracle), `gemm_loss_matched` (what a co-running GEMM loses against the collective's
-throughput beside it, copy route and copy-kernel budgets) and `extras` (the smaller configurations and comparison points).
+(`ring_schedule`), the per-launch roofline of the dominant kernel of each, the end-to-end figure through host buffers
+and the CPU oracle timed on the host cores.  Three tables go to stderr, one JSON object each (or into the line, see
+--tables): `large_messages` (64 MiB to 1 GiB per rank, every collective, copy route against SM path, each checked against
+the oracle), `gemm_loss_matched` (what a co-running GEMM loses against the collective's throughput beside it, copy route
+and copy-kernel budgets; the losses alone stay in the line) and `extras` (the smaller configurations and comparison points).
 """
 from __future__ import annotations
 
@@ -54,7 +55,28 @@ def parse_args():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-extras", action="store_true", help="skip the smaller configurations and comparison points")
     ap.add_argument("--no-large", action="store_true", help="skip large_messages and gemm_loss_matched")
+    ap.add_argument("--tables", default="auto", choices=["auto", "line", "stderr"],
+                    help="where large_messages, gemm_loss_matched and extras go: into the JSON line or, one JSON object per table, to stderr; "
+                         "auto = the line without the extras, stderr with them")
     return ap.parse_args()
+
+
+# With all tables the line is 46 KB long, and a caller that keeps the end of the output only has no whole line to read; without them
+# it is under 6 KB.
+TABLES = ("large_messages", "gemm_loss_matched", "extras")
+
+
+def split_tables(line, where):
+    """Takes the tables out of `line` unless they belong into it; returns them.  What a co-running GEMM loses stays, in short."""
+    if where == "line" or (where == "auto" and "extras" not in line):
+        return {}
+    tables = {k: line.pop(k) for k in TABLES if k in line}
+    if "gemm_loss_matched" in tables:
+        g = tables["gemm_loss_matched"]
+        line["gemm_loss"] = {r["config"]: round(r["gemm_loss"], 4) for r in g["rows"]}
+    if "large_messages" in tables:
+        line["large_messages_match_oracle"] = tables["large_messages"]["all_match_oracle"]
+    return tables
 
 
 def measured_peaks():
@@ -516,6 +538,8 @@ def main():
     if oracle_here and not args.no_extras:
         line["extras"] = extras(torch, hb, hd, W, np, replicas, world, dev, peaks)
     if world.rank == 0:
+        for name, table in split_tables(line, args.tables).items():
+            print(json.dumps({name: table}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     replicas.shutdown(world)
     return 0

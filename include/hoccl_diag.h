@@ -94,9 +94,9 @@ hoccl_result_t hoccl_flatten_inspect(int kind, hoccl_dtype_t dtype, int ctas, in
                                      const uint64_t* out_addr, const uint64_t* len, uint64_t* tiles_end, uint64_t* scalars_end,
                                      uint64_t* nvec, uint32_t* head, uint64_t* tile_vectors);
 /*
- * Host only (no device needed): how a group of `n` moves, given by their ADDRESSES as integers (src[i] -> dst[i], len[i]
- * bytes), is packed into fan-out launches.  Moves with the same source, length and 16-byte phase of the destination share
- * one segment (one read, one store per destination); a launch carries at most 32 segments and 256 destinations.
+ * Host only (no device needed): how the "roles" kernel takes a group of `n` moves, given by their ADDRESSES as integers
+ * (src[i] -> dst[i], len[i] bytes), together (every other route: hoccl_move_inspect).  Moves with the same source, length and 16-byte phase of the destination share
+ * one segment (one read, one store per destination); a batch carries at most 32 segments and 256 destinations.
  * Output, one entry per segment in launch order (arrays of capacity seg_cap): its launch index, source, length, number
  * of destinations, head / nvec of its split under the kernel shape `ctas` selects; its destinations follow each other in
  * dst_out (capacity n).  *n_seg = 0 means no source repeats: the moves go as plain copies.  Nothing is read or written.
@@ -104,6 +104,22 @@ hoccl_result_t hoccl_flatten_inspect(int kind, hoccl_dtype_t dtype, int ctas, in
 hoccl_result_t hoccl_fanout_inspect(int n, const uint64_t* src, const uint64_t* dst, const uint64_t* len, int ctas, int seg_cap,
                                     int* seg_launch, uint64_t* seg_src, uint64_t* seg_len, int* seg_ndst, uint32_t* seg_head,
                                     uint64_t* seg_nvec, uint64_t* dst_out, int* n_seg, int* n_launch);
+/*
+ * Host only: the launches of the move kernel that carry out such a group with `ctas` CTAs, on every route but the roles kernel's.
+ * Segments in launch order in segs (capacity seg_cap), the destinations of one after the other in dst_out (capacity dst_cap).  The
+ * kernel cuts a segment into `head` bytes, `nvec` 16-byte vectors from destination + head on, and the rest, byte by byte.  A vector whose
+ * source lies `s` bytes past a 16-byte boundary, s > 0, is put together from the two aligned vectors that hold its bytes.  Tiles of
+ * `tile_vectors` vectors and bytes are numbered through a launch: *_end = the number up to and including this segment.
+ * HOCCL_ERR_INVALID_ARG if a capacity does not suffice.
+ */
+typedef struct {
+  int launch, ndst;
+  uint64_t src, bytes;
+  uint32_t head, nvec, tiles_end, scalars_end;
+  uint32_t threads, tile_vectors; /* of the launch */
+} hoccl_move_seg_t;
+hoccl_result_t hoccl_move_inspect(int n, const uint64_t* src, const uint64_t* dst, const uint64_t* len, int ctas, int seg_cap, int dst_cap,
+                                  hoccl_move_seg_t* segs, uint64_t* dst_out, int* n_seg);
 /*
  * Self-test of the arithmetic: the chain sum of the direct reduce-scatter adds bf16 operands with the native packed add
  * (add.rn.bf16x2); this call compares it on the device with the reference add of every SUM (binary32 add of the widened

@@ -739,12 +739,7 @@ hoccl_result_t hoccl_selftest_bf16_add(unsigned long long* counts, hoccl_stream_
   return launch_bf16_add_selftest(counts, (cudaStream_t)stream) == cudaSuccess ? HOCCL_OK : HOCCL_ERR_CUDA;
 }
 
-hoccl_result_t hoccl_fanout_inspect(int n, const uint64_t* src, const uint64_t* dst, const uint64_t* len, int ctas, int seg_cap,
-                                    int* seg_launch, uint64_t* seg_src, uint64_t* seg_len, int* seg_ndst, uint32_t* seg_head,
-                                    uint64_t* seg_nvec, uint64_t* dst_out, int* n_seg, int* n_launch) {
-  if (n < 1 || !src || !dst || !len || ctas < 1 || seg_cap < 1 || !seg_launch || !seg_src || !seg_len || !seg_ndst || !seg_head ||
-      !seg_nvec || !dst_out || !n_seg || !n_launch)
-    return HOCCL_ERR_INVALID_ARG;
+static RGroup group_of_moves(int n, const uint64_t* src, const uint64_t* dst, const uint64_t* len) {
   RGroup g;
   g.kind = OP_MOVE;
   g.piece = 0;
@@ -756,6 +751,16 @@ hoccl_result_t hoccl_fanout_inspect(int n, const uint64_t* src, const uint64_t* 
     sg.bytes = len[i];
     g.segs.push_back(sg);
   }
+  return g;
+}
+
+hoccl_result_t hoccl_fanout_inspect(int n, const uint64_t* src, const uint64_t* dst, const uint64_t* len, int ctas, int seg_cap,
+                                    int* seg_launch, uint64_t* seg_src, uint64_t* seg_len, int* seg_ndst, uint32_t* seg_head,
+                                    uint64_t* seg_nvec, uint64_t* dst_out, int* n_seg, int* n_launch) {
+  if (n < 1 || !src || !dst || !len || ctas < 1 || seg_cap < 1 || !seg_launch || !seg_src || !seg_len || !seg_ndst || !seg_head ||
+      !seg_nvec || !dst_out || !n_seg || !n_launch)
+    return HOCCL_ERR_INVALID_ARG;
+  const RGroup g = group_of_moves(n, src, dst, len);
   std::vector<FanBatch> fans;
   std::vector<double> hbm;
   std::vector<long> moves;
@@ -781,6 +786,26 @@ hoccl_result_t hoccl_fanout_inspect(int n, const uint64_t* src, const uint64_t* 
   }
   *n_seg = k;
   *n_launch = (int)fans.size();
+  return HOCCL_OK;
+}
+
+hoccl_result_t hoccl_move_inspect(int n, const uint64_t* src, const uint64_t* dst, const uint64_t* len, int ctas, int seg_cap, int dst_cap,
+                                  hoccl_move_seg_t* segs, uint64_t* dst_out, int* n_seg) {
+  if (n < 1 || !src || !dst || !len || ctas < 1 || !segs || !dst_out || !n_seg) return HOCCL_ERR_INVALID_ARG;
+  *n_seg = 0;
+  int nd = 0, launch = 0;
+  for (const MoveBatch& b : pack_moves(group_of_moves(n, src, dst, len), ctas)) {
+    int threads = 0;
+    move_kernel_entry(b, ctas, false, &threads);
+    if (*n_seg + b.nseg > seg_cap || nd + b.ndst_total > dst_cap) return HOCCL_ERR_INVALID_ARG;
+    for (int k = 0; k < b.nseg; k++) {
+      const MoveSeg& m = b.seg[k];
+      segs[(*n_seg)++] = hoccl_move_seg_t{launch, m.ndst, (uint64_t)(uintptr_t)m.src, m.bytes, m.head, m.nvec, b.tpre[k + 1], b.spre[k + 1],
+                                          (uint32_t)threads, b.tile_u * (uint32_t)threads};
+      for (int d = 0; d < m.ndst; d++) dst_out[nd++] = (uint64_t)(uintptr_t)b.dst[m.first_dst + d];
+    }
+    launch++;
+  }
   return HOCCL_OK;
 }
 

@@ -236,9 +236,11 @@ struct Tally {
 // The kernel launches that carry out one group: its sums, or (SM route) its moves.
 std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, const RGroup& g);
 cudaError_t launch_kernel(const KernelLaunch& k, cudaStream_t stream);
-// Moves of a group that read the same bytes (same source and length; the direct all-gather on the SM path) become fan-out
-// segments: one read, one store per destination.  Returns false (and leaves *out empty) if no source repeats: the plain
-// copy batches are used then.  bytes_out[i] = HBM bytes of batch i (reads + writes), moves_out[i] = moves it carries.
+// The launches of the move kernel that carry out a group of moves, prepared for `ctas` CTAs: moves with one source, one length and one
+// 16-byte phase of the destination share a segment (one read, one store per destination).
+std::vector<MoveBatch> pack_moves(const RGroup& g, int ctas);
+// The same sharing as the roles kernel takes it over, in batches of its own.  Returns false (and leaves *out empty) if no source
+// repeats: plain copies are used then.  bytes_out[i] = HBM bytes of batch i (reads + writes), moves_out[i] = moves it carries.
 bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<double>* bytes_out, std::vector<long>* moves_out);
 // graph.cu
 // part < 0: every group (of `only_piece`, if that is >= 0); part 0 / 1 / 2: only the reduce-scatter's MOVE groups / the SUM and

@@ -398,21 +398,15 @@ static size_t fill_chain_batch(const RGroup& g, size_t first, int dtype, size_t 
   return i - first;
 }
 
-static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup& g) {
-  std::vector<KernelLaunch> out;
-  int threads = 0;
+std::vector<MoveBatch> pack_moves(const RGroup& g, int ctas) {
+  std::vector<MoveBatch> out;
   MoveBatch b;
   b.nseg = b.ndst_total = 0;
-  double bytes = 0;
   auto flush = [&]() {
     if (b.nseg == 0) return;
-    prepare_move_batch(&b, (int)c->copy_ctas);
-    MoveBatchSmall small;
-    const bool fits = shrink_move_batch(b, &small);
-    const void* fn = move_kernel_entry(b, (int)c->copy_ctas, fits, &threads);
-    out.push_back(fits ? make_launch(small, fn, c->copy_ctas, threads, bytes, b.ndst_total) : make_launch(b, fn, c->copy_ctas, threads, bytes, b.ndst_total));
+    prepare_move_batch(&b, ctas);
+    out.push_back(b);
     b.nseg = b.ndst_total = 0;
-    bytes = 0;
   };
   bool repeats = false;
   for (const MoveClass& cl : move_classes(g, &repeats))
@@ -426,11 +420,24 @@ static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup
           flush();
           add_move_seg(&b, cl.src + at, dsts.data(), (int)n, len);
         }
-        bytes += (1.0 + (double)n) * (double)len;
       }
       done += n;
     }
   flush();
+  return out;
+}
+
+static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup& g) {
+  std::vector<KernelLaunch> out;
+  for (const MoveBatch& b : pack_moves(g, (int)c->copy_ctas)) {
+    double bytes = 0;
+    for (int k = 0; k < b.nseg; k++) bytes += (1.0 + (double)b.seg[k].ndst) * (double)b.seg[k].bytes;
+    int threads = 0;
+    MoveBatchSmall small;
+    const bool fits = shrink_move_batch(b, &small);
+    const void* fn = move_kernel_entry(b, (int)c->copy_ctas, fits, &threads);
+    out.push_back(fits ? make_launch(small, fn, c->copy_ctas, threads, bytes, b.ndst_total) : make_launch(b, fn, c->copy_ctas, threads, bytes, b.ndst_total));
+  }
   return out;
 }
 

@@ -17,7 +17,8 @@ EXEC_GRAPH, EXEC_STREAMS, EXEC_ONE_KERNEL, EXEC_ONEPASS, EXEC_PROXY, EXEC_ROLES 
 EXPORTS = [   # every function include/hoccl_diag.h declares
     "hoccl_chain_launch", "hoccl_comm_init_host_only", "hoccl_copy_launch", "hoccl_fanout_inspect", "hoccl_fanout_launch", "hoccl_flatten_inspect",
     "hoccl_kernel_sms", "hoccl_layout_build", "hoccl_layout_destroy", "hoccl_layout_get_access", "hoccl_layout_group_deps",
-    "hoccl_layout_num_accesses", "hoccl_layout_num_groups", "hoccl_layout_num_pieces", "hoccl_layout_signature", "hoccl_options_resolve", "hoccl_plan_build", "hoccl_plan_destroy", "hoccl_plan_get_op",
+    "hoccl_layout_num_accesses", "hoccl_layout_num_groups", "hoccl_layout_num_pieces", "hoccl_layout_signature", "hoccl_move_inspect",
+    "hoccl_options_resolve", "hoccl_plan_build", "hoccl_plan_destroy", "hoccl_plan_get_op",
     "hoccl_plan_group_deps", "hoccl_plan_inbox_slots", "hoccl_plan_num_groups", "hoccl_plan_num_ops",
     "hoccl_plan_scratch_bytes", "hoccl_plan_slot_bytes", "hoccl_port_probe", "hoccl_probe_copy_routes",
     "hoccl_probe_move_needs_sm", "hoccl_selftest_barrier_timeout", "hoccl_selftest_roles_timeout", "hoccl_selftest_bf16_add", "hoccl_sum_launch",
@@ -56,6 +57,12 @@ class Access(ctypes.Structure):
                 ("write", ctypes.c_int), ("addr", ctypes.c_uint64), ("bytes", ctypes.c_uint64)]
 
 
+class MoveSeg(ctypes.Structure):
+    _fields_ = [("launch", ctypes.c_int), ("ndst", ctypes.c_int), ("src", ctypes.c_uint64), ("bytes", ctypes.c_uint64), ("head", ctypes.c_uint32),
+                ("nvec", ctypes.c_uint32), ("tiles_end", ctypes.c_uint32), ("scalars_end", ctypes.c_uint32), ("threads", ctypes.c_uint32),
+                ("tile_vectors", ctypes.c_uint32)]
+
+
 _ready = False
 
 
@@ -77,6 +84,7 @@ def lib() -> ctypes.CDLL:
         "hoccl_selftest_bf16_add": (i, [vp, vp]),
         "hoccl_chain_launch": (i, [vp, sz, i, vp, vp, sz, i, i, vp]),
         "hoccl_fanout_inspect": (i, [i, vp, vp, vp, i, i, vp, vp, vp, vp, vp, vp, vp, ctypes.POINTER(i), ctypes.POINTER(i)]),
+        "hoccl_move_inspect": (i, [i, vp, vp, vp, i, i, i, ctypes.POINTER(MoveSeg), vp, ctypes.POINTER(i)]),
         "hoccl_kernel_sms": (i, [i, vp, vp, vp, sz, i, i, vp, vp]),
         "hoccl_selftest_barrier_timeout": (i, [vp, vp, vp, sz, vp]),
         "hoccl_selftest_roles_timeout": (i, [vpp, vpp, sz, i, vp, vp]),
@@ -194,6 +202,23 @@ def fanout_inspect(moves, ctas: int = 8):
         segs.append((seg_launch[k], seg_src[k], seg_len[k], [dst_out[at + d] for d in range(seg_nd[k])], seg_head[k], seg_nvec[k]))
         at += seg_nd[k]
     return segs, n_launch.value
+
+
+def move_inspect(moves, ctas: int = 8, cuts: int = 1):
+    """hoccl_move_inspect (host only): moves = [(src_addr, dst_addr, nbytes), ...] -> [(MoveSeg, [dst_addr, ...]), ...].  `cuts`: into how
+    many segments the longest move may fall."""
+    n = len(moves)
+    u64, cap = ctypes.c_uint64 * n, n * cuts
+    src, dst, ln = u64(*[m[0] for m in moves]), u64(*[m[1] for m in moves]), u64(*[m[2] for m in moves])
+    segs, dst_out, n_seg = (MoveSeg * cap)(), (ctypes.c_uint64 * cap)(), ctypes.c_int(0)
+    rc = lib().hoccl_move_inspect(n, src, dst, ln, ctas, cap, cap, segs, dst_out, ctypes.byref(n_seg))
+    if rc != OK:
+        raise HocclError(rc, "hoccl_move_inspect", "")
+    out, at = [], 0
+    for k in range(n_seg.value):
+        out.append((segs[k], [dst_out[at + d] for d in range(segs[k].ndst)]))
+        at += segs[k].ndst
+    return out
 
 
 def kernel_sms(kind: str, a, b, out, nbytes: int, dtype, ctas: int, smid_out, stream=None) -> int:

@@ -81,7 +81,7 @@ def test_aligned_segments_take_the_vector_path():
     assert view[0][1] == 0 and view[0][3] == 100_000                         # no common phase: element-wise fallback
 
 
-# ---- fan-out packing (hoccl_fanout_inspect): the moves of a direct all-gather that read the same bytes share one segment
+# ---- fan-out packing of the roles kernel (hoccl_fanout_inspect): the moves of a direct all-gather that read the same bytes share one segment
 move_set = st.lists(st.tuples(st.integers(0, 5), st.integers(0, 15), st.sampled_from([0, 0, 0, 3, 8]), st.integers(1, 40)),
                     min_size=1, max_size=700)
 
@@ -140,3 +140,67 @@ def test_fan_out_packing_of_a_direct_all_gather():
     moves = [(recv[r] + r * 4096, recv[(r + k) % R] + r * 4096, 4096) for k in range(1, R) for r in range(R)]
     segs, launches = hd.fanout_inspect(moves, 16)
     assert launches == -(-R * (R - 1) // 256) and sum(len(s[3]) for s in segs) == R * (R - 1)
+
+
+# ---- packing of the move kernel's launches (hoccl_move_inspect): every address that kernel forms follows from these numbers
+def _check_moves(moves, ctas, cuts=1):
+    packed = hd.move_inspect(moves, ctas, cuts)
+    served, launch, tiles, scalars, nseg, ndst = [], -1, 0, 0, 0, 0
+    for s, dsts in packed:
+        if s.launch != launch:
+            assert s.launch == launch + 1
+            launch, tiles, scalars, nseg, ndst = s.launch, 0, 0, 0, 0
+        nseg, ndst = nseg + 1, ndst + len(dsts)
+        assert nseg <= 128 and ndst <= 512 and 1 <= len(dsts) <= 64
+        assert len({d % 16 for d in dsts}) == 1
+        # bytes: head + vectors + rest is the segment, and the rest is short
+        body = s.nvec * 16
+        assert s.head + body <= s.bytes <= 8 << 30
+        assert s.nvec > 0 or s.head == 0
+        assert s.bytes - body < 16 + 16 + 128 + 32
+        if s.nvec:
+            assert all((d + s.head) % 16 == 0 for d in dsts)                          # aligned stores
+            shift = (s.src + s.head) % 16
+            assert s.bytes < 65536 or (dsts[0] + s.head) % 128 in ((0, 16) if shift else (0,))    # a line, or the vector behind it
+            first = s.src + s.head - shift                                            # aligned loads, all inside the source
+            assert first >= s.src and first + body + (16 if shift else 0) <= s.src + s.bytes
+        # every vector in one tile, every other byte in one item
+        assert s.tiles_end - tiles == -(-s.nvec // s.tile_vectors) and s.scalars_end - scalars == s.bytes - body
+        assert s.tile_vectors % s.threads == 0 and 1 <= s.tile_vectors // s.threads <= 8 and s.threads <= 1024
+        assert s.nvec + s.tile_vectors < 1 << 32
+        tiles, scalars = s.tiles_end, s.scalars_end
+        served += [(s.src, d, s.bytes) for d in dsts]
+    want = [(src + at, dst + at, min(8 << 30, n - at)) for src, dst, n in moves for at in range(0, n, 8 << 30)]
+    assert sorted(served) == sorted(want)
+    return packed
+
+
+@settings(max_examples=200, deadline=None, suppress_health_check=list(HealthCheck), derandomize=True)
+@given(moves=st.lists(st.tuples(st.integers(0, 9), st.integers(0, 127), st.integers(0, 127), st.integers(0, 5)), min_size=1, max_size=700),
+       lens=st.lists(st.one_of(st.integers(1, 200), st.integers(201, 70_000), st.integers(65_000, 66_000), st.integers(1 << 20, 1 << 28)), min_size=6, max_size=6),
+       in_phase=st.booleans(), ctas=st.sampled_from([1, 3, 8, 40, 148]))
+def test_move_packing(moves, lens, in_phase, ctas):
+    """Few sources, many destinations, every phase and length: each move is served exactly once, loads stay inside the source and are
+    aligned, stores are aligned."""
+    flat = []
+    for k, (s, sp, dp, n) in enumerate(moves):
+        src = (1 << 40) + s * (1 << 32) + sp
+        dst = (1 << 44) + k * (1 << 32) + (sp if in_phase else dp)
+        flat.append((src, dst, lens[n]))
+    _check_moves(flat, ctas)
+
+
+def test_move_packing_at_the_edges():
+    base, far = 1 << 40, 1 << 44
+    for ctas in (8, 148):
+        for n in list(range(1, 200)) + [65535, 65536, 65537, 65536 + 127]:            # around one vector, two, the line rule
+            for sp in range(16):
+                _check_moves([(base + sp, far + dp, n) for dp in (0, 1, 15, 16, 100, 127)], ctas)
+        # longer than one segment may be, and more destinations of one source than one segment holds
+        _check_moves([(base + 3, far + 7, (20 << 30) + 5), (base + 3, far + (1 << 40) + 7, (20 << 30) + 5)], ctas, cuts=3)
+        segs = _check_moves([(base, far + k * 4096, 1000) for k in range(150)], ctas)
+        assert [len(d) for _, d in segs] == [64, 64, 22]
+    # a direct all-gather of 8 ranks: 56 moves, 8 segments of 7 destinations, one launch
+    recv = [(1 << 44) + r * (1 << 28) for r in range(8)]
+    segs = _check_moves([(recv[r] + r * 3_276_800, recv[(r + k) % 8] + r * 3_276_800, 3_276_800) for k in range(1, 8) for r in range(8)], 148)
+    assert [(s.launch, s.ndst, s.head) for s, _ in segs] == [(0, 7, 0)] * 8

@@ -63,6 +63,20 @@ case = st.fixed_dictionaries({
 @settings(max_examples=300, deadline=None, derandomize=True, suppress_health_check=list(HealthCheck))
 @given(c=case)
 def test_random_cases_match_the_oracle(oracle, c):
+    _run(oracle, c)
+
+
+@settings(max_examples=150, deadline=None, derandomize=True, suppress_health_check=list(HealthCheck))
+@given(c=case, off=st.sampled_from([0, 0, 1, 3, 8, 40]), wide=st.booleans())
+def test_random_cases_with_one_offset_for_all_ranks(oracle, c, off, wide):
+    """As above, with buffers that share their 16-byte phase (and, unless `wide`, their 128-byte one): what the automatic schedule needs to
+    read the contributions in place, and what allocators give."""
+    step = 16 // W.elem_size(c["dtype"]) if wide else 0
+    _run(oracle, dict(c, offs=[off + step * o for o in c["offs"]], rs_direct=2 if c["rs_direct"] == 1 else c["rs_direct"],
+                      variant="plain" if c["variant"] in ("roles", "onepass") else c["variant"]))
+
+
+def _run(oracle, c):
     assert torch.cuda.is_available(), "these tests need a CUDA device"
     torch.cuda.set_device(0)
     R, dtype, op = c["R"], c["dtype"], c["op"]

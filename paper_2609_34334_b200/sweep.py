@@ -6,6 +6,9 @@ pipeline / gradient-stream workloads (third and fourth), through the C ABI.
     python -m paper_2609_34334_b200.sweep gradients [--buckets 32] [--budgets 1,2,4,8,16,32,64]
     python -m paper_2609_34334_b200.sweep launch-cost
     python -m paper_2609_34334_b200.sweep alltoallv [--mib 4,64,256] [--model 4,2]
+    python -m paper_2609_34334_b200.sweep cases [--only NAME,NAME]      # the calls of perf/cases.py (run from the repository's root)
+    python -m paper_2609_34334_b200.sweep call --op allreduce --ranks 8 --count 20971520 --dtype bf16 \\
+        --variants "ce_overlap=2;ce_overlap=4;path=SM,sum_ctas=8,copy_ctas=40" [--gemm]   # one call under several settings, in turn
 
 Sizes are per-rank buffer bytes S in the nccl-tests convention (all-reduce: send = recv = S; reduce-scatter:
 send = S; all-gather: recv = S; all-to-all: send = recv = S; send/recv: S), like the sweeps the paper reports (Sec. 5 "Communication
@@ -494,6 +497,129 @@ def alltoallv(args):
         torch.cuda.empty_cache()
 
 
+def _spread(fns, stream, rounds=5, window_s=0.02):
+    """Times every function of `fns` in turn, `rounds` times: [(median, least, most)] of its mean time in a window, in microseconds."""
+    reps = []
+    for fn in fns:
+        for k in range(3):
+            fn(k)
+        stream.synchronize()
+        t0 = time.perf_counter()
+        fn(0)
+        stream.synchronize()
+        reps.append(int(min(200, max(3, window_s / max(time.perf_counter() - t0, 1e-6)))))
+    got = [[] for _ in fns]
+    for _ in range(rounds):
+        for i, fn in enumerate(fns):
+            fn(0)
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record(stream)
+            for k in range(reps[i]):
+                fn(k + 1)
+            e1.record(stream)
+            stream.synchronize()
+            got[i].append(e0.elapsed_time(e1) * 1e3 / reps[i])
+    return [(sorted(g)[rounds // 2], min(g), max(g)) for g in got]
+
+
+def cases(args):
+    """The listed calls of perf/cases.py, three input sets in rotation (less for the largest): microseconds of a pass among others."""
+    from perf import cases as C
+
+    torch.cuda.set_device(0)
+    stream = torch.cuda.current_stream()
+    for case in C.listed():
+        if args.only and case["name"] not in args.only.split(","):
+            continue
+        nbytes = C.work(case)["bytes"]
+        states = [C.prepare(case, seed) for seed in range(3 if nbytes < (2 << 30) else 2)]
+        torch.cuda.synchronize()
+        (t, lo, hi), = _spread([lambda k: C.run(states[k % len(states)])], stream)
+        torch.cuda.synchronize()
+        print(json.dumps({"case": case["name"], "us": round(t, 2), "least": round(lo, 2), "most": round(hi, 2), "GBps": round(nbytes / t / 1e3, 1)}), flush=True)
+        del states
+        torch.cuda.empty_cache()
+
+
+class HostArena:
+    """hoccl_host_allreduce on pinned buffers, with Arena's interface."""
+
+    def __init__(self, R, count, dtype):
+        tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+        self.count, self.dtype, self.sets = count, dtype, [None]
+        per = (count * W.elem_size(dtype) + 255) // 256 * 256
+        self.staging = torch.empty(2 * R * per, dtype=torch.uint8, device="cuda")
+        self.send, self.recv = ([torch.zeros(count, dtype=tdt).pin_memory() for _ in range(R)] for _ in range(2))
+
+    def call(self, comm, k, stream):
+        comm.host_allreduce(self.send, self.recv, self.count, self.dtype, stream)
+
+
+def call(args):
+    """One collective under several settings of the communicator, timed in turn.  A variant is a comma list of parameters (path=CE, SM
+    or CE_HOST, the rest as hoccl_comm_set_param takes them); an empty one is a new communicator's settings.  With --gemm also what a
+    loop of 60 bf16 GEMMs of 8192^3 on another stream loses to 60 such calls issued at its start, and the time of a call meanwhile."""
+    torch.cuda.set_device(0)
+    R, dtype, e, op = args.ranks, args.dtype, W.elem_size(args.dtype), args.op
+    n = args.count if op in ("allreduce", "sendrecv", "host_allreduce") else args.count * R
+    if op == "host_allreduce":
+        arena = HostArena(R, n, dtype)
+    else:
+        footprint = 2 * (R if op != "sendrecv" else 1) * n * e
+        arena = Arena(op, R, n * e, dtype, 1 if footprint > 4 * L2_BYTES else int(min(64, max(2, 4 * L2_BYTES // max(footprint, 1)))))
+    scratch = torch.empty(hb.scratch_bytes_direct(R, n, dtype) + 256, dtype=torch.uint8, device="cuda")
+    stream, gs = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    comms = []
+    for variant in args.variants.split(";"):
+        comm = hb.Comm(R, 0)
+        comm.set_scratch(scratch.data_ptr() + (-scratch.data_ptr()) % 256, scratch.numel() - 256)
+        if op == "host_allreduce":
+            comm.set_staging(arena.staging)
+        for part in filter(None, variant.split(",")):
+            key, value = part.split("=")
+            if key == "path":
+                comm.set_path({"CE": hb.PATH_CE, "SM": hb.PATH_SM, "CE_HOST": hb.PATH_CE_HOST}[value])
+            else:
+                comm.set_param(key, int(value))
+        comms.append((variant, comm))
+    times = _spread([lambda k, c=c: arena.call(c, k, stream) for _, c in comms], stream)
+    rows = []
+    for (variant, comm), (t, lo, hi) in zip(comms, times):
+        st = comm.last_stats()
+        rows.append({"op": op, "R": R, "count": args.count, "dtype": dtype, "variant": variant, "us": round(t, 2), "least": round(lo, 2), "most": round(hi, 2),
+                     "pieces": int(st["n_pieces"]), "moves": int(st["n_moves"]), "move_launches": int(st["n_move_launches"]),
+                     "sum_launches": int(st["n_sum_launches"])})
+    if args.gemm:
+        A, B = (torch.randn(8192, 8192, device="cuda").bfloat16() for _ in range(2))
+        C = torch.empty_like(A)
+
+        def beside(comm, calls, gemms=60):
+            torch.cuda.synchronize()
+            g0, g1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            with torch.cuda.stream(gs):
+                g0.record()
+                for _ in range(gemms):
+                    torch.matmul(A, B, out=C)
+                g1.record()
+            c0, c1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            c0.record(stream)
+            for k in range(calls):
+                arena.call(comm, k, stream)
+            c1.record(stream)
+            torch.cuda.synchronize()
+            return g0.elapsed_time(g1) * 1e3, c0.elapsed_time(c1) * 1e3
+
+        beside(None, 0)
+        for row, (_, comm) in zip(rows, comms):   # alone and beside the calls in turn: the clocks drift under the power cap
+            pairs = [(beside(comm, 60), beside(None, 0)) for _ in range(21)]
+            lost = sorted((both[0] - alone[0]) / 60 for both, alone in pairs)
+            row["gemm_us_lost_per_call"], row["gemm_us_lost_quartiles"] = round(lost[10], 1), [round(lost[5], 1), round(lost[15], 1)]
+            row["us_beside"] = round(sorted(both[1] / 60 for both, _ in pairs)[10], 1)
+    for row in rows:
+        print(json.dumps(row), flush=True)
+
+
 def main():
     ap = argparse.ArgumentParser()
     sub = ap.add_subparsers(dest="cmd", required=True)
@@ -515,11 +641,20 @@ def main():
     a2 = sub.add_parser("alltoallv")
     a2.add_argument("--mib", default="4,64,256", help="comma list of MiB sent per rank")
     a2.add_argument("--model", default="", help="comma list of modelled GPUs per node (e.g. 4,2): also run the pattern over that topology")
+    c = sub.add_parser("cases")
+    c.add_argument("--only", default="", help="comma list of names")
+    o = sub.add_parser("call")
+    o.add_argument("--op", default="allreduce", choices=["allreduce", "reduce_scatter", "allgather", "alltoall", "sendrecv", "host_allreduce"])
+    o.add_argument("--ranks", type=int, default=8)
+    o.add_argument("--count", type=int, default=20971520, help="elements, in the call's own convention")
+    o.add_argument("--dtype", default="bf16", choices=["bf16", "fp32"])
+    o.add_argument("--variants", default="", help="settings to compare: parameter=value,...;parameter=value,...")
+    o.add_argument("--gemm", action="store_true")
     args = ap.parse_args()
     if not torch.cuda.is_available():
         sys.stderr.write("sweep: no CUDA device\n")
         return 2
-    {"sizes": sweep_sizes, "pipeline": pipeline, "gradients": gradients, "launch-cost": launch_cost, "alltoallv": alltoallv}[args.cmd](args)
+    {"sizes": sweep_sizes, "pipeline": pipeline, "gradients": gradients, "launch-cost": launch_cost, "alltoallv": alltoallv, "cases": cases, "call": call}[args.cmd](args)
     return 0
 
 

@@ -447,7 +447,7 @@ def main():
             r.update({"kernel": "chain_pipe_kernel<bf16, 8 operands>", "traffic": r["algorithmic_bytes_per_launch"] * NCU_TRAFFIC_PER_BYTE_CHAIN,
                       "sm_budget_ceiling_GBps": 8 * SM_PORT_GBPS_CHAIN, "frac_of_sm_budget_ceiling": r["achieved"] / (8 * SM_PORT_GBPS_CHAIN),
                       "note": "8 CTAs by design (the SM budget for sums): R reads and 1 write per output byte; the bound is 8 SM memory ports "
-                              "(~163 GB/s each at this mix), not HBM; with the whole GPU the same sum runs at 5.7 TB/s"})
+                              "(~163 GB/s each at this mix), not HBM; with the whole GPU the same sum runs at 6.4 TB/s (chain_fan_kernel)"})
         else:
             r.update({"kernel": "sum2_kernel<bf16>", "traffic": r["algorithmic_bytes_per_launch"] * NCU_TRAFFIC_PER_BYTE_SUM,
                       "sm_budget_ceiling_GBps": 8 * SM_PORT_GBPS_SUM, "frac_of_sm_budget_ceiling": r["achieved"] / (8 * SM_PORT_GBPS_SUM)})

@@ -192,9 +192,10 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                inbox slots fall away (S (R+1) instead of 2 S (R-1) + S (R+1) bytes); an all-reduce on the route of HOCCL_PATH_SM
  *                that is short (R * S up to 384 KiB per SUM CTA) or has 128 or more SUM CTAs stores the result for every rank from
  *                the same kernel (2 S R bytes in all, one launch, no moves).  hoccl_last_stats counts the moves that remain.
- *                "rs_direct" = 1 keeps the rank-local form, as do HOCCL_PATH_CE_HOST, "roles" and hoccl_host_allreduce.  Measured
- *                on B200 (R = 8, bf16, default settings): 25 MiB reduce-scatter + all-gather 0.291 -> 0.226 ms, 40 MiB all-reduce
- *                0.417 -> 0.348 ms; HOCCL_PATH_SM with 148 + 148 CTAs, 64 MiB fp32 0.355 -> 0.183 ms.
+ *                "rs_direct" = 1 keeps the rank-local form, as do HOCCL_PATH_CE_HOST, "roles" and hoccl_host_allreduce of more than
+ *                72 MB for all ranks together.  Measured on B200 (R = 8, bf16, default settings): 25 MiB reduce-scatter + all-gather
+ *                0.291 -> 0.221 ms, 40 MiB all-reduce 0.417 -> 0.347 ms; HOCCL_PATH_SM with 148 + 148 CTAs, 64 MiB fp32 0.355 ->
+ *                0.172 ms.
  *  "ce_small_bytes" on HOCCL_PATH_CE a call whose per-rank message (S in the convention of each collective: all-reduce
  *                count, reduce-scatter / all-gather / all-to-all R * count elements) is at most this many bytes issues its
  *                moves as batched launches of the SM copy kernel with "ce_small_ctas" CTAs instead of driver copies, i.e.
@@ -209,8 +210,9 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                more that does not start on a 128-byte line and end after whole 4 KiB, and runs at half rate or less when the two
  *                ends differ modulo 4): a send/recv message, an all-gather or all-to-all of such blocks, an all-to-all of blocks below 4 MiB and an
  *                all-gather of 3 ranks or more (the kernel reads a block once, driver copies once per destination) runs on the copy kernel like a small one, and an
- *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of its all-gather's copies to one
- *                launch of the copy kernel ("copy_ctas" CTAs) per piece.
+ *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of the copies of its direct
+ *                all-gather to one launch of the copy kernel ("copy_ctas" CTAs) per piece (in a ring all-gather, whose copies
+ *                forward what the one before has written, copies stay whole).
  *  "ce_overlap"  HOCCL_PATH_CE, direct reduce-scatter: the ring chunks are cut into this many pieces and every piece's three
  *                parts (the reduce-scatter's moves, the chain sum, the all-gather's moves) become graphs of their own that
  *                run on three internal streams, ordered by events, so that one piece's driver copies run beside another

@@ -78,7 +78,7 @@ static void share_host_legs(std::vector<RGroup>* groups, size_t* host_need) {
   }
 }
 
-constexpr size_t kHostInPlaceBytes = 72000000;   // R * S up to which the host entry reads in place
+constexpr size_t kHostInPlaceBytes = 72000000;   // R * S up to which the host entry reads in place: where the two forms cross for whole chunks, see host_pieces
 constexpr size_t kGradeInPlace = 4 << 20;   // ring chunk from which pieces are graded on the SM path when contributions are read in place
 
 // How the direct reduce-scatter's contributions reach the owner's sum.
@@ -94,7 +94,9 @@ enum Contributions {
 //   * The send buffers have to share their 16-byte phase.  (Inbox slots are placed so that the operands always do; contributions
 //     that do not would be summed element by element.)
 //   * The host-bounce path keeps its moves: that no SM takes part in them is what it is chosen for.  The host entry keeps them for
-//     long vectors (see run_host_in_place).
+//     long vectors (see host_pieces).
+//   * It needs the scratch of the staged form all the same, although it touches none of it: whether the addresses of a call permit it is
+//     known at the call, and the staged form of the same schedule is what runs when they do not.
 // The sum stores for all ranks on the SM route (on the copy route the all-gather's moves are the driver's) when its grid is the
 // whole GPU, or when the message is so short that the second launch and not the stores decide: a CTA stores ~60 GB/s, so R S
 // bytes over n CTAs take R S / (60 n) ns against ~2.5 us for a launch of its own and the wider copy grid.  Measured, one kernel
@@ -806,7 +808,10 @@ hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype) {
 //     372 us in driver copies, 96 on the kernel, all-to-all 384 and 173; two bytes out of phase 818 and 114, 838 and 175.
 //   * The blocks of an all-to-all are short: 16 MiB per rank 51 and 47 us, 40 MiB 112 and 110, 64 MiB 175 and 173, 256 MiB 660 and 690.
 //   * An all-gather of 3 ranks or more: the kernel reads a block once, driver copies once per destination (9 MiB per rank over 8 ranks
-//     24.7 and 14.4 us, 40 MiB 84 and 62, 64 MiB 150 and 96, 256 MiB 572 and 367; over 3 ranks 64 MiB 45 and 38).
+//     24.7 and 14.4 us, 40 MiB 84 and 62, 64 MiB 150 and 96, 256 MiB 572 and 367; over 3 ranks 64 MiB 45 and 38).  Both take the whole GPU.
+//     Beside a loop of 8192^3 bf16 GEMMs a call over 8 ranks costs the GEMMs (medians of two runs) and takes meanwhile: 25 MiB per rank 22 to
+//     31 us and 0.13 ms (driver copies 10 to 13 us and 0.24 ms; the kernel with "ce_small_ctas" = 40 37 to 68 us and 0.79 ms), 64 MiB 80 us
+//     and 0.27 ms (66 to 104 us and 0.48 ms; 40 CTAs 97 to 107 us and 0.84 ms).
 static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t block = call.count * dtype_size(call.dtype);
   if (block < kDriverShort || (call.kind == PLAN_ALLGATHER && c->R >= 3)) return true;
@@ -823,8 +828,12 @@ static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
 // Pieces: with np equal pieces the two directions overlap in all but one piece each, (1 + 1 / np) S R / 50 GB/s, and every copy costs
 // 6 to 9 us beside one of the other direction, np R of them; so the best np grows with the root of S (1 up to 1 MiB per rank, 3 at 4 MiB,
 // 5 at 16 MiB).  Measured over 8 ranks against 8 pieces of every ring chunk: 64 KiB per rank 122 -> 89 us, 1 MiB 403 -> 380, 4 MiB 1372 ->
-// 1087, 8 MiB 2120 -> 2060; over 3 ranks 64 KiB 74 -> 38, 1 MiB 243 -> 150, 16 MiB 1541 -> 1460.  Beyond ~64 MiB for all ranks together the 2-D
-// copies of the staged form are the faster ones (8 ranks of 16 MiB 3.58 against 3.68 ms, of 25 MiB 5.23 against 5.45).
+// 1087, 8 MiB 2120 -> 2060; over 3 ranks 64 KiB 74 -> 38, 1 MiB 243 -> 150, 16 MiB 1541 -> 1460.
+// Size from which the 2-D pieces of the staged form serve (kHostInPlaceBytes), in place against staged, ms, 8 ranks, bytes of all ranks
+// together: whole chunks 40 MB 1.33 / 1.37, 60 MB 1.91 / 1.86, 70 MB 2.06 / 2.06, 80 MB 2.36 / 2.39, 100 MB 2.86 / 2.74, 134 MB 3.72 / 3.54,
+// 200 MB 5.23 / 4.99.  The line lies where the two cross; the rule looks at the size only.  Chunks of unequal length add a copy per rank and
+// direction to every 2-D piece and nothing to a contiguous one: 70 MB 2.03 / 2.45, 80 MB 2.33 / 2.69, 134 MB 3.72 / 4.35, 200 MB 5.18 / 5.94 (3
+// ranks, 200 MB: 5.20 / 5.31), so for them the line costs up to 0.8 ms.
 static size_t host_pieces(const hoccl_comm* c, size_t S, double unit) {
   if (c->host_pieces_set) return (size_t)c->host_pieces;
   return std::min<size_t>(32, std::max<size_t>(1, (size_t)(std::sqrt((double)S / unit) + 0.5)));
@@ -920,9 +929,14 @@ static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut&
     overlap_pieces = ring_chunk >= ((size_t)4 << 20) ? (long)std::min<size_t>(most, std::max<size_t>(4, ring_chunk >> 22))
                                                      : ring_chunk >= ((size_t)2 << 20) ? 2 : 0;
     // With the contributions read in place only the all-gather's copies are left to hide behind the sums, so fewer and larger
-    // pieces are best, and below 4 MiB per chunk (8 MiB with whole-GPU sums) one graph is (R = 8, bf16, 8-CTA sums: 25 MiB per rank
-    // 0.221 ms whole and 0.221 in 2 pieces, 32 MiB 0.286 / 0.281, 40 MiB 0.364 / 0.344 and 0.348 in 4, 64 MiB 0.600 whole and 0.536 in
-    // 3, 128 MiB 1.058 in 6, 256 MiB 2.088 in 12, 2.138 in 24; 148-CTA sums: 16 MiB 0.056 / 0.076, 64 MiB 0.244 / 0.225, 0.262 in 6)
+    // pieces are best, and below 4 MiB per chunk (8 MiB with whole-GPU sums) one graph is.  Milliseconds whole / in 2 / 3 / 4 pieces, R = 8,
+    // bf16, 8-CTA sums: 25 MiB per rank 0.224 / 0.221 / 0.244 / 0.241, 32 MiB 0.286 / 0.276 / 0.277 / 0.281, 40 MiB 0.365 / 0.340 / 0.340 /
+    // 0.346, 48 MiB 0.448 / 0.408 / 0.407 / 0.410, 56 MiB 0.526 / 0.476 / 0.472 / 0.472, 64 MiB 0.603 / 0.549 / 0.537 / 0.539, 80 MiB 0.750 /
+    // 0.693 / 0.666 / 0.663, 96 MiB 0.898 / 0.840 / 0.798 / 0.789; 128 MiB 1.065 in 4 and 1.056 in 6, 256 MiB 2.154 in 4, 2.088 in 12, 2.138 in 24.
+    // So 4 pieces from 5 MiB per chunk are 2 % behind 2 or 3 at 5 MiB, within 1 % up to 6 and ahead of 2 from 7 on.  (148-CTA sums: 16 MiB
+    // 0.056 whole, 0.076 in 2, 64 MiB 0.244 / 0.225, 0.262 in 6.)  The rule was measured over 8 ranks, where the sums take three quarters of the
+    // time; fewer ranks have less to hide the copies behind, and it cuts too finely there: R = 4, 32 MiB 0.174 whole and 0.182 in 4, 128 MiB 0.659
+    // in 3 and 0.689 in 12; R = 2, 16 MiB 0.065 whole and 0.084 in 4, 64 MiB 0.241 whole and 0.292 in 12 (staged: 0.093 and 0.290).
     if (how == READ_IN_PLACE) {
       if (c->sum_ctas >= 64) overlap_pieces = (long)std::min<size_t>(8, ring_chunk >> 22);
       else overlap_pieces = ring_chunk >= ((size_t)5 << 20) ? (long)std::min<size_t>(32, std::max<size_t>(4, ring_chunk * 3 >> 23))

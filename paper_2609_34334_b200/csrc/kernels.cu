@@ -208,8 +208,10 @@ __device__ __forceinline__ void report_sm(const Batch& batch) {
   }
 }
 
-// Chain sum for any number of operands and destinations (the forms below are compiled for 2 to 16): one 16-byte vector per thread and tile; the operands are loaded in
-// batches of up to 8 before they are added, so up to 8 x 16 KiB are in flight per CTA.
+// Chain sum for any number of operands and destinations: one 16-byte vector per thread and tile; the operands are loaded in batches of up
+// to 8 before they are added, so up to 8 x 16 KiB are in flight per CTA.  It serves what the compiled forms below do not (see
+// chain_variant): more than 16 operands, mixed counts, and from 9 operands on whole-GPU grids and sums that store for every rank.  With 148
+// CTAs and 64 MiB per rank it is at the copy rate there: 9 operands 108 us (6.2 TB/s), 12 139 (6.3), 16 175 (6.5).
 template <int DT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
@@ -818,10 +820,12 @@ void prepare_copy_batch(CopyBatch* b, int ctas) {
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
 }
 
-// Which chain kernel serves a batch.  The compiled forms need one operand count for the whole launch (the usual case: R), from 2 to
-// 8 or 9 to 16, and one destination (chain_pipe_kernel, chain_pipe2_kernel) or, up to 8, as many as operands (chain_fan_kernel).  Measured on
+// Which chain kernel serves a batch.  The compiled forms need one operand count for the whole launch (the usual case: R) and one
+// destination (below 128 CTAs chain_pipe_kernel for 2 to 8 operands and chain_pipe2_kernel for 9 to 16, from 128 on chain_fan_kernel for 2 to
+// 8) or as many as operands (chain_fan_kernel, 2 to 8).  chain_pipe_kernel against chain_kernel, measured on
 // B200 (8 operands, 25 MiB each, bf16): 163 against 111 GB/s per SM with 8 CTAs, 158 / 107 with 16, 138 / 99 with 32,
-// 113 / 89 with 48, 88 / 80 with 64, 59 / 58 with 96; with 148 CTAs both are HBM bound (5.7 TB/s).  Variants with the same
+// 113 / 89 with 48, 88 / 80 with 64, 59 / 58 with 96; from 128 CTAs on chain_fan_kernel with one destination (64 MiB per rank 94 us,
+// 6.4 TB/s).  Variants with the same
 // or more bytes in flight (P = 2 with 640 threads, P = 4 with 384, P = 4 and 6 with 256) end at the same 159-163 GB/s per
 // SM with 8 CTAs: that is the SM's memory port at 8 reads : 1 write, no longer the bytes in flight.
 struct ChainVariant {
@@ -1024,7 +1028,9 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
 // are bound by HBM and want little in flight per SM, the less the more often a vector is stored (the reads otherwise come in bursts
 // between the writes): 44 KiB for copies, 7 for one read stored 7 times.  Measured in TB/s at 256 MiB per stream: copies 4 x 704 6.2
 // (4 x 512 5.8, 8 x 1024 4.2), 1:2 2 x 704 6.0 (2 x 256 4.0), 1:3 4 x 384 6.0 (2 x 256 4.5), 1:4 and 1:5 2 x 384 5.8 (2 x 256 4.8 and 5.1), 1:7
-// 1 x 448 5.8 (4 x 512 3.9).  Out of phase every vector is loaded twice, from L1 the second time: 4 x 704.
+// 1 x 448 5.8 (4 x 512 3.9).  Out of phase every vector is loaded twice, from L1 the second time: 4 x 704, measured for copies (all-to-all of
+// 64 MiB per rank 173 us in phase, 175 out of phase).  One such segment decides for the launch, fan-outs included: all-gather of 64 MiB per rank
+// over 8 ranks 106 us in phase (1 x 448), 116 out of phase.
 struct MoveShape {
   int u, threads;
 };

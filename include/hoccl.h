@@ -428,7 +428,7 @@ hoccl_result_t hoccl_comm_proxy_stats(hoccl_comm_t comm, double* busy_us, double
  * All-reduce whose buffers are HOST memory (pinned for real asynchrony): h_send[r] / h_recv[r] are
  * host pointers to `count` elements each.  The call copies every h_send[r] into the attached staging
  * memory (needs 2*R*roundup256(count*sizeof(dtype)) bytes), runs the all-reduce there and copies every rank's
- * result back, all ordered on `stream`.  Host-to-device traffic is driven by the copy engines (Sec. 2.3).
+ * result back, all ordered on `stream`.  Host-to-device traffic is driven by the copy engines (Sec. 2.3), but for short pinned vectors.
  * Pipelined form (default; "host_pieces" > 1 with graphs on): every ring chunk is cut into host_pieces pieces; per
  * piece, the host-to-device copies (2-D copies: that piece of every chunk) run on one internal stream, the ring on that
  * piece (its own cached graph) runs on `stream` as soon as the piece has arrived, and the device-to-host copies follow on
@@ -438,6 +438,9 @@ hoccl_result_t hoccl_comm_proxy_stats(hoccl_comm_t comm, double* busy_us, double
  * there) and the ranks' vectors are at most 72 MB together, a piece is a contiguous range of the vector instead, one copy per rank
  * and direction, summed once and copied out to every rank from one buffer; the number of pieces then follows the size (1 up to
  * 1 MiB per rank, 3 at 4 MiB) unless "host_pieces" was set, as it does for longer vectors on the direct schedule (5 at 25 MiB).
+ * If, besides, "host_pieces" was not set and every host buffer is pinned or registered with CUDA (as one range) and shares its address
+ * modulo 16 with the others, nothing is copied at all: one launch of "sum_ctas" CTAs reads the host buffers across PCIe and stores the
+ * result into every one of them.  Staging is still demanded: whether the buffers permit it is known at the call.
  * Host buffers of different ranks must not overlap
  * partially (INVALID_ARG); h_recv[r] == h_send[r] is legal.  With host_pieces = 1, use_graph = 0, handshake, onepass,
  * fused or HOCCL_PATH_CE_HOST the three stages run one after the other.

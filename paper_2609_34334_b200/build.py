@@ -13,7 +13,7 @@ LIB = os.path.join(HERE, "libhoccl.so")
 # The name carries the interpreter's ABI (".cpython-312-x86_64-linux-gnu.so"): each interpreter that uses the tree has a module of its
 # own and looks for that name before a plain "_calls.so".
 CALLS, CALLS_SOURCE = os.path.join(HERE, "_calls" + sysconfig.get_config_var("EXT_SUFFIX")), os.path.join(CSRC, "calls.c")
-SOURCES = ["api.cu", "exec.cu", "p2p.cu", "kernels.cu", "plan.cpp", "static_scratch.cu", "proxy.cu", "sched.cpp", "probe.cu", "ring.cu", "graph.cu", "ring_host.cu", "options.cpp", "roles.cu"]
+SOURCES = ["api.cu", "exec.cu", "p2p.cu", "kernels.cu", "plan.cpp", "static_scratch.cu", "proxy.cu", "sched.cpp", "probe.cu", "ring.cu", "graph.cu", "host_entry.cu", "ring_host.cu", "options.cpp", "roles.cu"]
 HEADERS = ["comm.h", "kernels.cuh", "device_common.cuh", "plan.h", "proxy.h", "sched.h", "options.h", os.path.join("..", "..", "include", "hoccl.h"), os.path.join("..", "..", "include", "hoccl_diag.h")]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -17,6 +17,7 @@
 #include "../../include/hoccl_diag.h"
 #include "kernels.cuh"
 #include "plan.h"
+#include "options.h"
 #include "proxy.h"
 #include "sched.h"
 
@@ -236,6 +237,18 @@ struct Tally {
 // The kernel launches that carry out one group: its sums, or (SM route) its moves.
 std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, const RGroup& g);
 cudaError_t launch_kernel(const KernelLaunch& k, cudaStream_t stream);
+hoccl_result_t launch_sum_kernel(hoccl_comm* c, const KernelLaunch& k, cudaStream_t stream);   // ... between two events if "profile" is set
+template <class Batch>
+inline KernelLaunch make_launch(const Batch& b, const void* fn, long grid, int threads, double bytes, long moves) {
+  KernelLaunch k;
+  k.fn = fn;
+  k.grid = (int)grid;
+  k.threads = threads;
+  k.args.assign(reinterpret_cast<const char*>(&b), reinterpret_cast<const char*>(&b) + sizeof(b));
+  k.bytes = bytes;
+  k.moves = moves;
+  return k;
+}
 // The launches of the move kernel that carry out a group of moves, prepared for `ctas` CTAs: moves with one source, one length and one
 // 16-byte phase of the destination share a segment (one read, one store per destination).
 std::vector<MoveBatch> pack_moves(const RGroup& g, int ctas);
@@ -271,6 +284,19 @@ hoccl_result_t build_pattern_graph_modelled(hoccl_comm* c, const Schedule& S, co
                                             const std::vector<uint64_t>& flow_stage_off, size_t chunk_bytes, size_t rdma_sub,
                                             GraphEntry* entry);
 hoccl_result_t ring_barrier_selftest(hoccl_comm* c, void* dst, const void* src, size_t bytes, cudaStream_t stream);
+// Replays a cached graph into the caller's stream (directly, or through the CPU proxy in handshake mode).
+hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, double t0);
+// host_entry.cu: the pipelined hoccl_host_allreduce on the automatic direct schedule
+constexpr size_t kHostInPlaceBytes = 72000000;   // R * S up to which its sums store for every rank; above, launches of moves do (see host_entry.cu)
+// The caller's host buffers as kernels see them.
+struct HostViews {
+  const char* send[kMaxRanks];
+  char* recv[kMaxRanks];
+};
+bool host_direct_applies(const hoccl_comm* c, const Call& call, const OptionsOut& opt, HostViews* views);
+hoccl_result_t run_host_direct(hoccl_comm* c, const Call& call, const HostViews& views, cudaStream_t user, double t0);
+size_t host_pieces(const hoccl_comm* c, size_t S, double unit);
+hoccl_result_t run_host_in_place(hoccl_comm* c, const Call& call, std::vector<uint64_t>&& key, cudaStream_t user, double t0);
 // p2p.cu
 hoccl_result_t p2p_post(hoccl_comm* c, bool is_send, void* buf, size_t count, int dtype, int src, int dst, cudaStream_t stream);
 

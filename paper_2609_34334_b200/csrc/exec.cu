@@ -78,7 +78,6 @@ static void share_host_legs(std::vector<RGroup>* groups, size_t* host_need) {
   }
 }
 
-constexpr size_t kHostInPlaceBytes = 72000000;   // R * S up to which the host entry reads in place: where the two forms cross for whole chunks, see host_pieces
 constexpr size_t kGradeInPlace = 4 << 20;   // ring chunk from which pieces are graded on the SM path when contributions are read in place
 
 // How the direct reduce-scatter's contributions reach the owner's sum.
@@ -156,18 +155,6 @@ static void trim_driver_copies(std::vector<RGroup>* groups) {
     else
       groups->push_back(std::move(ends));
   }
-}
-
-template <class Batch>
-static KernelLaunch make_launch(const Batch& b, const void* fn, long grid, int threads, double bytes, long moves) {
-  KernelLaunch k;
-  k.fn = fn;
-  k.grid = (int)grid;
-  k.threads = threads;
-  k.args.assign(reinterpret_cast<const char*>(&b), reinterpret_cast<const char*>(&b) + sizeof(b));
-  k.bytes = bytes;
-  k.moves = moves;
-  return k;
 }
 
 // Turns plan offsets into addresses (the plan already places pieces inside the scratch slots).
@@ -485,6 +472,28 @@ cudaError_t launch_kernel(const KernelLaunch& k, cudaStream_t stream) {
   return cudaLaunchKernel(k.fn, dim3((unsigned)k.grid), dim3((unsigned)k.threads), args, 0, stream);
 }
 
+hoccl_result_t launch_sum_kernel(hoccl_comm* c, const KernelLaunch& k, cudaStream_t s) {
+  std::pair<cudaEvent_t, cudaEvent_t> pe{nullptr, nullptr};
+  if (c->profile) {
+    if (c->prof_pool.empty()) {
+      cudaEvent_t a, z;
+      CU_TRY(c, cudaEventCreate(&a));
+      CU_TRY(c, cudaEventCreate(&z));
+      pe = {a, z};
+    } else {
+      pe = c->prof_pool.back();
+      c->prof_pool.pop_back();
+    }
+    CU_TRY(c, cudaEventRecord(pe.first, s));
+  }
+  CU_TRY(c, launch_kernel(k, s));
+  if (c->profile) {
+    CU_TRY(c, cudaEventRecord(pe.second, s));
+    c->prof_open.push_back({pe, k.bytes});
+  }
+  return HOCCL_OK;
+}
+
 // ------------------------------------------------------------------ stream executor -------------
 hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, cudaStream_t user, Tally* tally) {
   const int lanes = (int)std::max<long>(1, std::min<long>(c->lanes, kMaxLanes));
@@ -521,24 +530,8 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
     // chain_dep needs no event here: every SUM is on the one sum stream
     if (rg.kind != OP_MOVE) {
       for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
-        std::pair<cudaEvent_t, cudaEvent_t> pe{nullptr, nullptr};
-        if (c->profile) {
-          if (c->prof_pool.empty()) {
-            cudaEvent_t a, z;
-            CU_TRY(c, cudaEventCreate(&a));
-            CU_TRY(c, cudaEventCreate(&z));
-            pe = {a, z};
-          } else {
-            pe = c->prof_pool.back();
-            c->prof_pool.pop_back();
-          }
-          CU_TRY(c, cudaEventRecord(pe.first, s));
-        }
-        CU_TRY(c, launch_kernel(k, s));
-        if (c->profile) {
-          CU_TRY(c, cudaEventRecord(pe.second, s));
-          c->prof_open.push_back({pe, k.bytes});
-        }
+        const hoccl_result_t lrc = launch_sum_kernel(c, k, s);
+        if (lrc != HOCCL_OK) return lrc;
         tally->sum_launches++;
       }
     } else if (c->path == HOCCL_PATH_CE && !rg.edges) {
@@ -674,7 +667,7 @@ hoccl_result_t ensure_proxy(hoccl_comm* c) {
 }
 
 // Replays a cached graph into the caller's stream (directly, or through the CPU proxy in handshake mode).
-static hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, double t0) {
+hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, double t0) {
   hit->last_use = ++c->use_counter;
   if (!hit->ring_args.empty()) {
     if (hit->ring_large)
@@ -820,72 +813,6 @@ static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
       if (bad_for_driver((const char*)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0), (const char*)call.recv[v] + (size_t)u * block, block))
         return true;
   return false;
-}
-
-// Host all-reduce whose sums read the ranks' staging buffers in place: no schedule over ring chunks is left, so a piece is one
-// contiguous range of the vector (one plain copy per rank and direction instead of a 2-D copy and one for the shorter last chunk),
-// the sum writes it once, and every rank's result is copied out of that one buffer.
-// Pieces: with np equal pieces the two directions overlap in all but one piece each, (1 + 1 / np) S R / 50 GB/s, and every copy costs
-// 6 to 9 us beside one of the other direction, np R of them; so the best np grows with the root of S (1 up to 1 MiB per rank, 3 at 4 MiB,
-// 5 at 16 MiB).  Measured over 8 ranks against 8 pieces of every ring chunk: 64 KiB per rank 122 -> 89 us, 1 MiB 403 -> 380, 4 MiB 1372 ->
-// 1087, 8 MiB 2120 -> 2060; over 3 ranks 64 KiB 74 -> 38, 1 MiB 243 -> 150, 16 MiB 1541 -> 1460.
-// Size from which the 2-D pieces of the staged form serve (kHostInPlaceBytes), in place against staged, ms, 8 ranks, bytes of all ranks
-// together: whole chunks 40 MB 1.33 / 1.37, 60 MB 1.91 / 1.86, 70 MB 2.06 / 2.06, 80 MB 2.36 / 2.39, 100 MB 2.86 / 2.74, 134 MB 3.72 / 3.54,
-// 200 MB 5.23 / 4.99.  The line lies where the two cross; the rule looks at the size only.  Chunks of unequal length add a copy per rank and
-// direction to every 2-D piece and nothing to a contiguous one: 70 MB 2.03 / 2.45, 80 MB 2.33 / 2.69, 134 MB 3.72 / 4.35, 200 MB 5.18 / 5.94 (3
-// ranks, 200 MB: 5.20 / 5.31), so for them the line costs up to 0.8 ms.
-static size_t host_pieces(const hoccl_comm* c, size_t S, double unit) {
-  if (c->host_pieces_set) return (size_t)c->host_pieces;
-  return std::min<size_t>(32, std::max<size_t>(1, (size_t)(std::sqrt((double)S / unit) + 0.5)));
-}
-static hoccl_result_t run_host_in_place(hoccl_comm* c, const Call& call, std::vector<uint64_t>&& key, cudaStream_t user, double t0) {
-  const int R = c->R;
-  Plan P;
-  P.kind = PLAN_ALLREDUCE;
-  P.R = R;
-  P.dtype = call.dtype;
-  P.elem = dtype_size(call.dtype);
-  const size_t S = call.count * P.elem, chunk = (call.count + R - 1) / R * P.elem;
-  const size_t np = host_pieces(c, S, 600e3);
-  const size_t piece = ((S + np - 1) / np + 4095) & ~(size_t)4095;
-  GraphEntry entry;
-  entry.key = std::move(key);
-  std::vector<RGroup> groups;
-  char* result = (char*)call.recv[0];
-  for (size_t a = 0; a < S; a += piece) {
-    const size_t b = std::min(S, a + piece);
-    RGroup g;
-    g.kind = OP_CHAIN;
-    g.piece = (int)groups.size();
-    g.phase = PHASE_RS;
-    g.chain_dep = -1;
-    for (size_t at = a; at < b;) {   // one segment per ring chunk the range touches: the order of the adds is the chunk's
-      const int owner = (int)(at / chunk);
-      Seg s = {};
-      s.bytes = std::min<size_t>(std::min(b, (size_t)(owner + 1) * chunk) - at, kMaxChainSegBytes);
-      for (int j = 1; j <= R; j++) s.ops.push_back((const char*)call.send[(owner + j) % R] + at);
-      s.dst = result + at;
-      g.segs.push_back(s);
-      at += s.bytes;
-    }
-    groups.push_back(std::move(g));
-    entry.h2d.emplace_back();
-    entry.d2h.emplace_back();
-    for (int r = 0; r < R; r++) {
-      entry.h2d.back().push_back(HostCopy{(char*)call.send[r] + a, (char*)call.h_send[r] + a, b - a, b - a, 1});
-      entry.d2h.back().push_back(HostCopy{result + a, (char*)call.h_recv[r] + a, b - a, b - a, 1});
-    }
-  }
-  entry.n_pieces = (long)groups.size();
-  entry.piece_exec.assign(groups.size(), nullptr);
-  for (size_t p = 0; p < groups.size(); p++) {
-    const hoccl_result_t rc = build_graph(c, P, groups, &entry, (int)p, &entry.piece_exec[p]);
-    if (rc != HOCCL_OK) {
-      destroy_entry(&entry);
-      return rc;
-    }
-  }
-  return launch_entry(c, cache_put(c, std::move(entry)), user, t0);
 }
 
 // How the communicator's settings combine for this call (options.h); a contradictory combination is refused here.
@@ -1036,6 +963,13 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
   }
   // a small message on the copy route runs on the copy kernel's route: the communicator shows that route for this call only
   RouteGuard guard(c, (hoccl_path_t)opt.path, opt.copy_ctas);
+  if (call->h_send && call->count != 0) {
+    HostViews views;
+    if (host_direct_applies(c, *call, opt, &views)) {
+      const hoccl_result_t vrc = validate(c, call);
+      return vrc == HOCCL_OK ? run_host_direct(c, *call, views, user, t0) : vrc;
+    }
+  }
   const bool onepass_case = opt.executor == EXEC_ONEPASS;
   const bool fused = opt.executor == EXEC_ONE_KERNEL;
   const bool roles = opt.executor == EXEC_ROLES;

@@ -422,14 +422,7 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
         c->stats = hoccl_stats_t{};
         c->stats.graph_hit = 1;
         CU_TRY(c, cudaSetDevice(c->device));
-        en.last_use = ++c->use_counter;
-        CU_TRY(c, cudaGraphLaunch(en.exec, (cudaStream_t)stream));
-        c->stats.n_moves = en.n_moves;
-        c->stats.n_move_launches = en.n_move_launches;
-        c->stats.max_copy_ctas = en.n_move_launches ? c->copy_ctas : 0;
-        c->stats.n_pieces = en.n_pieces;
-        c->stats.host_launch_us = now_us() - t0;
-        return HOCCL_OK;
+        return launch_entry(c, &en, (cudaStream_t)stream, t0);
       }
   }
   // receive regions of one rank must not overlap each other, and no send region may overlap a receive region
@@ -502,17 +495,10 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
     } else {
       entry.n_pieces = 1;
       grc = build_graph(c, P, groups, &entry, -1, &entry.exec);
+      if (grc == HOCCL_OK) add_launches(c, P, groups, &entry);
     }
     if (grc != HOCCL_OK) return grc;
-    GraphEntry* en = cache_put(c, std::move(entry));
-    en->last_use = ++c->use_counter;
-    CU_TRY(c, cudaGraphLaunch(en->exec, user));
-    c->stats.n_moves = en->n_moves;
-    c->stats.n_move_launches = en->n_move_launches;
-    c->stats.max_copy_ctas = en->n_move_launches ? c->copy_ctas : 0;
-    c->stats.n_pieces = en->n_pieces;
-    c->stats.host_launch_us = now_us() - t0;
-    return HOCCL_OK;
+    return launch_entry(c, cache_put(c, std::move(entry)), user, t0);
   }
   Tally tally;
   hoccl_result_t src = run_streams(c, P, groups, user, &tally);

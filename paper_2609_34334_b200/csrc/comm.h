@@ -46,13 +46,14 @@ struct Seg {
   bool host_first = true; // HOCCL_PATH_CE_HOST: this move issues the outbound copy into host_off (false: another move of the group did)
 };
 
-// One kernel launch of a schedule: the batch is its only parameter, by value.
+// One kernel launch of a schedule: the batch is its only parameter, by value.  The kernel is one that launch_in_order may start.
 struct KernelLaunch {
   const void* fn = nullptr;
   int grid = 0, threads = 0;
   std::vector<char> args;
   double bytes = 0;   // algorithmic bytes
   long moves = 0;     // MOVE operations it carries (0: a sum)
+  int priority = 0;   // of the launch; 0: the stream's
 };
 
 struct RGroup {
@@ -85,6 +86,8 @@ struct HostCopy {
 struct GraphEntry {
   std::vector<uint64_t> key;
   cudaGraphExec_t exec = nullptr;
+  std::vector<KernelLaunch> launches;   // the same work as `exec`, for a call of a burst (see launch_entry)
+  double est_us = 0;                    // what they take, roughly: 1.5 (sums) or 2.5 us (moves) each, HBM, 90 GB/s per summing and 45 per moving CTA
   uint64_t last_use = 0;
   long n_moves = 0, n_move_launches = 0, n_sum_launches = 0, n_pieces = 0, n_order_launches = 0;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> prof_events;  // owned; only with profile = 1
@@ -256,6 +259,10 @@ std::vector<MoveBatch> pack_moves(const RGroup& g, int ctas);
 // repeats: plain copies are used then.  bytes_out[i] = HBM bytes of batch i (reads + writes), moves_out[i] = moves it carries.
 bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<double>* bytes_out, std::vector<long>* moves_out);
 // graph.cu
+// Fills entry->launches and est_us if the groups are at most kMaxChainLaunches kernels, each waiting for the one before it.  (Inside a graph a
+// kernel follows another in 0.65 us, so longer chains, and calls with something to overlap, lose nothing there.)
+constexpr size_t kMaxChainLaunches = 3;
+void add_launches(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry);
 // part < 0: every group (of `only_piece`, if that is >= 0); part 0 / 1 / 2: only the reduce-scatter's MOVE groups / the SUM and
 // CHAIN groups / the remaining MOVE groups; dependencies on groups outside the part are left to the caller (events).
 // *out_exec stays null when nothing falls into the selection.

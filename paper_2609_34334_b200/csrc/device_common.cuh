@@ -72,6 +72,10 @@ struct Traits<1> {  // bf16
   }
 };
 
+// Every kernel that launch_in_order may start calls this in every thread, before it touches global memory: until the kernel in front
+// has finished and its writes are visible.  Returns at once in a launch without the attribute.
+__device__ __forceinline__ void wait_for_stream() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __host__ __device__ __forceinline__ void split_segment(unsigned long long n, unsigned mis, bool congruent, int E, int VE,
                                               unsigned* head, unsigned long long* nvec, unsigned long long* nscalar) {
   if (congruent && (mis % E) == 0) {

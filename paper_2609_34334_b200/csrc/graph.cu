@@ -71,6 +71,22 @@ static cudaKernelNodeParams node_params(const KernelLaunch& k, void** args) {
   return kp;
 }
 
+void add_launches(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry) {
+  if (c->profile || c->handshake || groups.size() > kMaxChainLaunches) return;
+  std::vector<KernelLaunch> all;
+  for (size_t g = 0; g < groups.size(); g++) {
+    const RGroup& rg = groups[g];
+    if (rg.kind == OP_MOVE && c->path != HOCCL_PATH_SM) return;
+    if (g > 0 && rg.chain_dep != (int)g - 1 && std::find(rg.deps.begin(), rg.deps.end(), (int)g - 1) == rg.deps.end()) return;
+    for (KernelLaunch& k : kernel_launches(c, P, rg)) {
+      if (rg.kind != OP_MOVE) k.priority = c->sum_priority;
+      entry->est_us += (rg.kind == OP_MOVE ? 2.5 : 1.5) + std::max(k.bytes / 6e6, k.bytes / k.grid / (rg.kind == OP_MOVE ? 45e3 : 90e3));
+      all.push_back(std::move(k));
+    }
+  }
+  if (all.size() <= kMaxChainLaunches) entry->launches.swap(all);
+}
+
 // only_piece >= 0 builds the graph of that piece alone (dependencies never cross pieces) and stores it in *out_exec.
 hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry, int only_piece,
                            cudaGraphExec_t* out_exec, int part) {

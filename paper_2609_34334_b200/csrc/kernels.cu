@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(THREADS, 1) sum2_kernel(const __grid_constant_
   using T = Traits<DT>;
   const Flat& f = batch.flat;   // filled on the host for this kernel variant: no set-up phase, no barrier
   const int nseg = batch.nseg;
+  wait_for_stream();
   if (batch.smid_out != nullptr && threadIdx.x == 0) {
     unsigned id;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(id));
@@ -216,9 +217,10 @@ template <int DT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
   const Flat& f = batch.flat;
-  report_sm(batch);
   const unsigned long long T_all = f.tpre[batch.nseg];
   int k = 0;
+  wait_for_stream();
+  report_sm(batch);
   for (unsigned long long t = blockIdx.x; t < T_all; t += gridDim.x) {
     while (t >= f.tpre[k + 1]) k++;
     const unsigned long long v = (t - f.tpre[k]) * blockDim.x + threadIdx.x;   // vector of segment k
@@ -259,7 +261,6 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe_kernel(const __grid_con
   using T = Traits<DT>;
   const Flat& f = batch.flat;
   const int nseg = batch.nseg;
-  report_sm(batch);
   {
     const unsigned long long T_all = f.tpre[nseg];
     // this CTA's share of the flattened tile space: [A, B)
@@ -267,6 +268,8 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe_kernel(const __grid_con
     const unsigned long long B = A + T_all / gridDim.x + (blockIdx.x < T_all % gridDim.x ? 1 : 0);
     int k = 0;
     while (k < nseg && f.tpre[k + 1] <= A) k++;
+    wait_for_stream();
+    report_sm(batch);
     for (; k < nseg && f.tpre[k] < B; k++) {
       const unsigned a = (unsigned)((A > f.tpre[k] ? A : f.tpre[k]) - f.tpre[k]);                 // tiles [a, b) of segment k
       const unsigned b = (unsigned)((B < f.tpre[k + 1] ? B : f.tpre[k + 1]) - f.tpre[k]);
@@ -329,13 +332,14 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe2_kernel(const __grid_co
   constexpr int AHEAD = (P - 2) / 2 + 1;               // tiles the prologue touches
   const Flat& f = batch.flat;
   const int nseg = batch.nseg;
-  report_sm(batch);
   {
     const unsigned long long T_all = f.tpre[nseg];
     const unsigned long long A = T_all / gridDim.x * blockIdx.x + min((unsigned long long)blockIdx.x, T_all % gridDim.x);
     const unsigned long long B = A + T_all / gridDim.x + (blockIdx.x < T_all % gridDim.x ? 1 : 0);
     int k = 0;
     while (k < nseg && f.tpre[k + 1] <= A) k++;
+    wait_for_stream();
+    report_sm(batch);
     for (; k < nseg && f.tpre[k] < B; k++) {
       const unsigned a = (unsigned)((A > f.tpre[k] ? A : f.tpre[k]) - f.tpre[k]);   // tiles [a, b) of segment k
       const unsigned b = (unsigned)((B < f.tpre[k + 1] ? B : f.tpre[k + 1]) - f.tpre[k]);
@@ -402,11 +406,12 @@ template <int DT, int NOPS, int NDST, int U, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
   const Flat& f = batch.flat;
-  report_sm(batch);
   // tile t of the flattened space belongs to CTA t mod grid; walked segment by segment, so that the NOPS + NDST pointers are loaded
   // once per segment and not once per tile (R = 8, 64 MiB fp32, tiles of 384 vectors: 194 us with a look-up per tile, 171 without)
   const unsigned long long T_all = f.tpre[batch.nseg];
   int k = 0;
+  wait_for_stream();
+  report_sm(batch);
   for (unsigned long long at = blockIdx.x; at < T_all;) {
     while (at >= f.tpre[k + 1]) k++;
     const unsigned tiles = (unsigned)(f.tpre[k + 1] - f.tpre[k]);
@@ -464,6 +469,7 @@ __global__ void __launch_bounds__(THREADS, 1) store_all_kernel(const __grid_cons
   const unsigned head = min(((16u - ((a.phase + at) & 15u)) & 15u) / T::E, n), nvec = (n - head) / T::VE;
   const unsigned per = (nvec + a.parts - 1) / a.parts, v1 = min(nvec, (part + 1) * per);
   constexpr int U = NOPS <= 4 ? 4 : 2;   // vectors of a thread in flight
+  wait_for_stream();
   for (unsigned v = part * per + threadIdx.x; v < v1; v += U * THREADS) {
     uint4 buf[U][NOPS];
 #pragma unroll
@@ -550,8 +556,9 @@ __global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant_
   constexpr int H = U < 4 ? U : 4;
   const int nseg = batch.nseg;
   const unsigned T_all = batch.tpre[nseg], tile_u = batch.tile_u;
+  int k = blockIdx.x < T_all ? find_segment(batch.tpre, nseg, blockIdx.x) : 0;
+  wait_for_stream();
   if (blockIdx.x < T_all) {
-    int k = find_segment(batch.tpre, nseg, blockIdx.x);
     for (unsigned t = blockIdx.x; t < T_all; t += gridDim.x) {
       while (t >= batch.tpre[k + 1]) k++;
       const MoveSeg& sg = batch.seg[k];
@@ -599,7 +606,7 @@ __global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant_
   }
   const unsigned S = batch.spre[nseg], j0 = blockIdx.x * THREADS + threadIdx.x;
   if (j0 < S) {
-    int k = find_segment(batch.spre, nseg, j0);
+    k = find_segment(batch.spre, nseg, j0);
     for (unsigned j = j0; j < S; j += gridDim.x * THREADS) {
       while (j >= batch.spre[k + 1]) k++;
       const MoveSeg& sg = batch.seg[k];
@@ -990,13 +997,34 @@ bool add_chain_seg(ChainBatch* b, const void* const* ops, int nops, void* const*
   return true;
 }
 
+cudaError_t launch_in_order(const void* fn, int grid, int threads, void* args, cudaStream_t stream, int priority) {
+  cudaStreamCaptureStatus capture;
+  const cudaError_t e = cudaStreamIsCapturing(stream, &capture);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  if (capture == cudaStreamCaptureStatusNone) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (priority) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributePriority;
+    attr[cfg.numAttrs++].val.priority = priority;
+  }
+  void* params[1] = {args};
+  return cudaLaunchKernelExC(&cfg, fn, params);
+}
+
 cudaError_t launch_chain(const ChainBatch& batch, int ctas, cudaStream_t stream) {
   if (batch.nseg <= 0) return cudaSuccess;
   ChainBatch b = batch;
   prepare_chain_batch(&b, ctas);
   const ChainVariant v = chain_variant(b, ctas);
-  void* args[1] = {&b};
-  return cudaLaunchKernel(v.fn, dim3((unsigned)ctas), dim3((unsigned)v.threads), args, 0, stream);
+  return launch_in_order(v.fn, ctas, v.threads, &b, stream);
 }
 
 void prepare_fan_batch(FanBatch* b, int ctas) {
@@ -1117,8 +1145,7 @@ cudaError_t launch_moves(MoveBatch* b, int ctas, cudaStream_t stream) {
   const bool fits = shrink_move_batch(*b, &small);
   int threads = 0;
   const void* fn = move_kernel_entry(*b, ctas, fits, &threads);
-  void* args[1] = {fits ? static_cast<void*>(&small) : static_cast<void*>(b)};
-  return cudaLaunchKernel(fn, dim3((unsigned)ctas), dim3((unsigned)threads), args, 0, stream);
+  return launch_in_order(fn, ctas, threads, fits ? static_cast<void*>(&small) : static_cast<void*>(b), stream);
 }
 
 cudaError_t launch_move(const void* src, void* dst, unsigned long long bytes, int ctas, cudaStream_t stream) {

@@ -204,6 +204,14 @@ cudaError_t preload_ring_kernels();
 // Fills nvec / head / tiles_end / scalars_end of the nseg segments of one phase for the kernel shape `threads` selects.
 void prepare_ring_phase(RingSeg* seg, int nseg, int kind, int dtype, int threads);
 
+// Launches a kernel in stream order with less of a gap behind the kernel in front.  On B200 (driver 580) a kernel launch or a graph launch that
+// follows another one on its stream starts on a grid of 2.048 us after it: calls of 2.1 to 4.1 us of work all take 4.10 us, 8.1 us of work 10.25.
+// A launch with the programmatic-serialization attribute starts 0.5 to 0.7 us behind its predecessor instead (2.5 us of work 3.2, 8.1 us 8.8).
+// None of this library's kernels lets its successor start early, and each waits for its predecessor before it touches memory
+// (wait_for_stream), so the order and what a kernel sees are those of a plain launch.  `fn` must be such a kernel.
+// Without the attribute while the stream is being captured: the capture keeps full edges.
+cudaError_t launch_in_order(const void* fn, int grid, int threads, void* args, cudaStream_t stream, int priority = 0);
+
 // Enqueue helpers (return the CUDA error of the launch).
 cudaError_t launch_sum(const SumBatch& batch, int ctas, cudaStream_t stream);
 cudaError_t launch_copy(const CopyBatch& batch, int ctas, cudaStream_t stream);

@@ -62,8 +62,7 @@ cudaError_t read_in_place(const void* const* send, void* const* recv, size_t cou
         a.x[r] = send[r];
         a.y[r] = recv[r];
       }
-      void* args[1] = {&a};
-      return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, 0, st);
+      return launch_in_order(fn, grid, threads, &a, st);
     }
   }
   ChainBatch b;

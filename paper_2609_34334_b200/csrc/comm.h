@@ -64,6 +64,7 @@ struct RGroup {
   std::vector<int> deps;
   int chain_dep;
   std::vector<KernelLaunch> ready;   // if not empty, the launches that carry out the group (instead of batches built from segs)
+  long ctas = 0;        // moves on the move kernel: its CTAs, 0 = "copy_ctas"
   bool edges = false;   // copy route: the ends of driver copies, carried by a copy-kernel launch (see trim_driver_copies)
 };
 
@@ -99,6 +100,7 @@ struct GraphEntry {
   // "ce_overlap" setting: per piece three graphs (the reduce-scatter's moves, the sum, the all-gather's moves) that run on three
   // internal streams, so that one piece's driver copies overlap another piece's sum (inside ONE graph they never did)
   std::vector<cudaGraphExec_t> part_exec;   // [piece * 3 + part], null where a part is empty
+  std::vector<std::vector<KernelLaunch>> part_sums;   // [piece]: the sums as launches instead of a graph, unless "profile" is set
   // "fused" setting: the whole plan as one cooperative kernel instead of a graph (exec stays null)
   std::vector<char> ring_args;  // a RingArgsSmall or RingArgsLarge, by value
   bool ring_large = false;

@@ -418,14 +418,15 @@ std::vector<MoveBatch> pack_moves(const RGroup& g, int ctas) {
 
 static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup& g) {
   std::vector<KernelLaunch> out;
-  for (const MoveBatch& b : pack_moves(g, (int)c->copy_ctas)) {
+  const int ctas = (int)(g.ctas ? g.ctas : c->copy_ctas);
+  for (const MoveBatch& b : pack_moves(g, ctas)) {
     double bytes = 0;
     for (int k = 0; k < b.nseg; k++) bytes += (1.0 + (double)b.seg[k].ndst) * (double)b.seg[k].bytes;
     int threads = 0;
     MoveBatchSmall small;
     const bool fits = shrink_move_batch(b, &small);
-    const void* fn = move_kernel_entry(b, (int)c->copy_ctas, fits, &threads);
-    out.push_back(fits ? make_launch(small, fn, c->copy_ctas, threads, bytes, b.ndst_total) : make_launch(b, fn, c->copy_ctas, threads, bytes, b.ndst_total));
+    const void* fn = move_kernel_entry(b, ctas, fits, &threads);
+    out.push_back(fits ? make_launch(small, fn, ctas, threads, bytes, b.ndst_total) : make_launch(b, fn, ctas, threads, bytes, b.ndst_total));
   }
   return out;
 }
@@ -746,6 +747,8 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
         CU_TRY(c, cudaStreamWaitEvent(sm, moved, 0));
       }
       if (g_sum) CU_TRY(c, cudaGraphLaunch(g_sum, sm));
+      if (!hit->part_sums.empty())
+        for (const KernelLaunch& k : hit->part_sums[p]) CU_TRY(c, launch_kernel(k, sm));
       if (g_ag) {
         cudaEvent_t summed = next_event(c);
         if (!summed) return cuda_fail(c, cudaErrorMemoryAllocation, "event pool");
@@ -845,13 +848,37 @@ static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   return false;
 }
 
+// An all-reduce whose sums read the contributions in place and whose ring chunks the driver copies badly (not whole pages on 128-byte lines), or
+// are short copies (but for chunks of 1 to 1.17 MiB, 80 MB for all ranks, whose copies and ends the layout tests describe): its all-gather runs on the move kernel too, which reads a chunk once for all ranks.  Us in driver copies with their ends on the
+// kernel / on the kernel alone, bf16: R = 8, 16 MiB per rank 149.5 / 137.5, 64 MiB 554 / 527; R = 3, 32 MiB 174 / 155; R = 5, 32 MiB 221 / 203; R = 6, 64 MiB
+// 456 / 445; R = 16, 19 MiB 352 / 290, 64 MiB 1072 / 887.  A loop of 8192^3 GEMMs loses less to it as well (8 ranks, 64 MiB 97 us per
+// call, in driver copies 175).  Whole chunks stay with the driver, whose copies run beside the next piece's sum: 8 ranks 40 MiB 335 us, 320 on the kernel.
+static bool chunks_bad_for_driver(const hoccl_comm* c, const Call& call) {
+  const size_t S = call.count * dtype_size(call.dtype), chunk = (call.count + c->R - 1) / c->R * dtype_size(call.dtype);
+  if (chunk >= kDriverWhole && chunk < ((size_t)1200 << 10) && (size_t)c->R * S < 80000000) return false;
+  bool bad = chunk < kDriverWhole || chunk % kDriverPage || S % kDriverPage;
+  for (int v = 0; v < c->R; v++) bad = bad || (uintptr_t)call.recv[v] % kDriverLine;
+  return bad;
+}
+
 // How the communicator's settings combine for this call (options.h); a contradictory combination is refused here.
 static hoccl_result_t call_options(hoccl_comm* c, const Call& call, OptionsOut* opt) {
   OptionsIn oin = options_of(c, call.kind, call.count, call.dtype, call.h_send != nullptr);
-  if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && (call.kind == PLAN_ALLGATHER || call.kind == PLAN_ALLTOALL) && blocks_bad_for_driver(c, call))
+  const bool may_switch = c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0;
+  if (may_switch && (call.kind == PLAN_ALLGATHER || call.kind == PLAN_ALLTOALL) && blocks_bad_for_driver(c, call)) oin.ce_small_bytes = LONG_MAX;
+  const hoccl_result_t rc = resolve_options(oin, opt);
+  if (rc == HOCCL_OK && may_switch && call.kind == PLAN_ALLREDUCE && opt->path == HOCCL_PATH_CE && opt->executor == EXEC_GRAPH && c->ag_direct == 2 &&
+      c->ce_overlap < 0 && !c->piece_bytes_set && c->sum_ctas < 64 && !call.h_send && chunks_bad_for_driver(c, call) &&
+      contributions(c, call, *opt, call.count * dtype_size(call.dtype)) == READ_IN_PLACE) {
     oin.ce_small_bytes = LONG_MAX;
-  return resolve_options(oin, opt);
+    return resolve_options(oin, opt);
+  }
+  return rc;
 }
+
+// CTAs of an all-gather that runs beside a SUM under a CTA budget: stores at 2.4 TB/s, which the sum does not feel (beside 64 it loses
+// 2 %; 24 do not finish in time).  25 MiB per rank over 8 ranks in three pieces 206.8 us with 24, 207.0 with 40, 208.7 with 64.
+constexpr long kBesideSums = 40;
 
 // Pure host work, nothing is enqueued.  The communicator shows the call's route (RouteGuard).
 static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut& opt, Contributions how, Layout* out) {
@@ -885,26 +912,38 @@ static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut&
     const size_t most = c->sum_ctas >= 64 ? 8 : 32;
     overlap_pieces = ring_chunk >= ((size_t)4 << 20) ? (long)std::min<size_t>(most, std::max<size_t>(4, ring_chunk >> 22))
                                                      : ring_chunk >= ((size_t)2 << 20) ? 2 : 0;
-    // With the contributions read in place only the all-gather's copies are left to hide behind the sums, so fewer and larger
-    // pieces are best, and below 4 MiB per chunk (8 MiB with whole-GPU sums) one graph is.  Milliseconds whole / in 2 / 3 / 4 pieces, R = 8,
-    // bf16, 8-CTA sums: 25 MiB per rank 0.224 / 0.221 / 0.244 / 0.241, 32 MiB 0.286 / 0.276 / 0.277 / 0.281, 40 MiB 0.365 / 0.340 / 0.340 /
-    // 0.346, 48 MiB 0.448 / 0.408 / 0.407 / 0.410, 56 MiB 0.526 / 0.476 / 0.472 / 0.472, 64 MiB 0.603 / 0.549 / 0.537 / 0.539, 80 MiB 0.750 /
-    // 0.693 / 0.666 / 0.663, 96 MiB 0.898 / 0.840 / 0.798 / 0.789; 128 MiB 1.065 in 4 and 1.056 in 6, 256 MiB 2.154 in 4, 2.088 in 12, 2.138 in 24.
-    // So 4 pieces from 5 MiB per chunk are 2 % behind 2 or 3 at 5 MiB, within 1 % up to 6 and ahead of 2 from 7 on.  (148-CTA sums: 16 MiB
-    // 0.056 whole, 0.076 in 2, 64 MiB 0.244 / 0.225, 0.262 in 6.)  The rule was measured over 8 ranks, where the sums take three quarters of the
-    // time; fewer ranks have less to hide the copies behind, and it cuts too finely there: R = 4, 32 MiB 0.174 whole and 0.182 in 4, 128 MiB 0.659
-    // in 3 and 0.689 in 12; R = 2, 16 MiB 0.065 whole and 0.084 in 4, 64 MiB 0.241 whole and 0.292 in 12 (staged: 0.093 and 0.290).
+    // With the contributions read in place only the all-gather's copies are left to hide behind the sums.  np equal pieces leave
+    // 1 / np of them exposed and cost 5.4 us each (drain and refill of the sums, launches, events), so np is the root of the copies' time over 5.4 us,
+    // in pieces of 1.25 MiB or more.  Us in 1 / 2 / 3 / 4 / 6 / 8 / 12 pieces, bf16, 8-CTA sums (in brackets what the rule takes): R = 2, 64 MiB 242 / 241 /
+    // 243 / 244 / 254 / 262 / 273 (2), 256 MiB 958 / 937 / 922 / 920 / 927 / 932 / 941 (4); R = 3, 64 MiB 304 / 295 / 292 / 297 / 308 (2); R = 4, 32 MiB
+    // 175 / 176 / 179 / 180 / 187 (2), 64 MiB 357 / 338 / 334 / 335 / 340 / 353 / 356 (3), 256 MiB 1410 / 1345 / 1307 / 1293 / 1283 / 1283 / 1282 (6);
+    // R = 6, 64 MiB 488 / 451 / 445 / 444 / 461 / 465 (4); R = 8, 40 MiB - / 337 / 332 / 335 (4), 64 MiB 602 / 544 / 526 / 523 / 535 / 558 (5), 256 MiB 2370 /
+    // 2220 / 2150 / 2105 / 2060 / 2047 / 2015 (10); R = 16, 64 MiB 1127 / 983 / 941 / 933 / 1032 (3).  Chunks above 8 MiB are cut in two at least,
+    // which costs two ranks up to 5 % (32 MiB 123 whole, 128 in two).  (148-CTA sums: 16 MiB 0.056 ms whole, 0.076 in 2, 64 MiB 0.244 / 0.225, 0.262 in 6.)
     if (how == READ_IN_PLACE) {
-      if (c->sum_ctas >= 64) overlap_pieces = (long)std::min<size_t>(8, ring_chunk >> 22);
-      else overlap_pieces = ring_chunk >= ((size_t)5 << 20) ? (long)std::min<size_t>(32, std::max<size_t>(4, ring_chunk * 3 >> 23))
-                                                            : ring_chunk >= ((size_t)4 << 20) ? 2 : 0;
+      if (c->sum_ctas >= 64) {
+        overlap_pieces = (long)std::min<size_t>(8, ring_chunk >> 22);
+      } else {
+        const double copies_us = 2.0 * (c->R - 1) * (double)ring_chunk * c->R / 6.2e6;
+        const size_t np = std::min((size_t)std::sqrt(copies_us / 5.4), ring_chunk / ((size_t)1280 << 10));
+        overlap_pieces = (long)std::min<size_t>(32, std::max<size_t>(ring_chunk > ((size_t)8 << 20) ? 2 : 0, np));
+      }
     }
   }
   const bool overlap = overlap_pieces > 1 && c->path == HOCCL_PATH_CE && opt.executor == EXEC_GRAPH && !call.h_send &&
                        (plan_kind & PLAN_FLAG_RS_DIRECT) && c->R > 1 && !c->piece_bytes_set && !sum_only;
+  // Sums under a CTA budget with the all-gather on a whole-GPU grid of the move kernel: the pieces follow the rule above with 5 us per piece and
+  // (R stores per vector read) the move kernel's R S bytes; the all-gathers of all pieces but the last run on kBesideSums CTAs.  Us
+  // whole / in two / in three, bf16: R = 8, 10 MiB per rank 86.6 / 87.2 / 90.2 (1), 16 MiB 139.4 / 135.0 / 135.2 (2), 25 MiB 216.8 / 208.0 / 207.0 (2);
+  // R = 4, 10 MiB 54.3 / 58.5 / 61.8 (1), 16 MiB 84.8 / 88.9 / 89.2 (1).
+  const bool beside = how == READ_IN_PLACE && call.kind == PLAN_ALLREDUCE && c->path == HOCCL_PATH_SM && opt.executor == EXEC_GRAPH &&
+                      (plan_kind & PLAN_FLAG_AG_DIRECT) && c->sum_ctas < 64 && c->copy_ctas >= 128 && !c->piece_bytes_set && !call.h_send;
   if (sum_only && !c->piece_bytes_set && !call.h_send) {   // nothing to overlap
     piece_bytes = (size_t)1 << 60;
     max_pieces = 1;
+  } else if (beside) {
+    max_pieces = (int)std::min<size_t>(32, std::max<size_t>(ring_chunk > ((size_t)8 << 20) ? 2 : 1, (size_t)std::sqrt((double)c->R * (double)call.send_bytes / 6e6 / 5.0)));
+    piece_bytes = std::max<size_t>((size_t)64 << 10, ((ring_chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
   } else if (overlap) {
     max_pieces = (int)overlap_pieces;
     piece_bytes = std::max<size_t>((size_t)64 << 10, ((ring_chunk + max_pieces - 1) / max_pieces + 1023) / 1024 * 1024);
@@ -952,7 +991,7 @@ static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut&
   // (with the contributions read in place the SM path gains from 4 MiB per ring chunk on: 40 MiB per rank in 5 pieces 0.340 -> 0.329)
   const size_t grade_from = how == READ_IN_PLACE && c->path == HOCCL_PATH_SM ? kGradeInPlace : (size_t)8 << 20;
   const bool graded = reduction && !call.h_send && !fused && (plan_kind & PLAN_FLAG_RS_DIRECT) &&
-                      (c->piece_grade == 1 || (c->piece_grade < 0 && ring_chunk >= grade_from && c->sum_ctas < 64));
+                      (c->piece_grade == 1 || (c->piece_grade < 0 && !beside && ring_chunk >= grade_from && c->sum_ctas < 64));
   if (!build_plan(&P, plan_kind | (graded ? PLAN_FLAG_GRADED : 0), c->R, call.count, call.dtype, call.in_place, piece_bytes, max_pieces, align))
     return HOCCL_ERR_INVALID_ARG;
   if (P.slot_bytes) {
@@ -966,6 +1005,9 @@ static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut&
   }
   out->overlap = overlap && P.pieces > 1;   // with one piece there is nothing to overlap
   resolve(c, P, call, how, &out->groups, &out->host_need);
+  if (beside)
+    for (RGroup& g : out->groups)
+      if (g.kind == OP_MOVE && g.piece + 1 < P.pieces) g.ctas = kBesideSums;
   return HOCCL_OK;
 }
 
@@ -1093,8 +1135,18 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
       }
     } else if (lay.overlap) {
       entry.part_exec.assign((size_t)P.pieces * 3, nullptr);
+      if (!c->profile) {   // (a piece's sums behind another's start on time as launches, see launch_in_order: 4 pieces of 40 MiB 345.8 -> 342.3 us)
+        entry.part_sums.resize((size_t)P.pieces);
+        for (const RGroup& g : groups)
+          if (g.kind != OP_MOVE)
+            for (KernelLaunch& k : kernel_launches(c, P, g)) {
+              entry.part_sums[(size_t)g.piece].push_back(std::move(k));
+              entry.n_sum_launches++;
+            }
+      }
       for (int p = 0; p < P.pieces && rc == HOCCL_OK; p++)
-        for (int part = 0; part < 3 && rc == HOCCL_OK; part++) rc = build_graph(c, P, groups, &entry, p, &entry.part_exec[(size_t)p * 3 + part], part);
+        for (int part = 0; part < 3 && rc == HOCCL_OK; part++)
+          if (part != 1 || c->profile) rc = build_graph(c, P, groups, &entry, p, &entry.part_exec[(size_t)p * 3 + part], part);
       if (rc != HOCCL_OK) {
         destroy_entry(&entry);
         return rc;

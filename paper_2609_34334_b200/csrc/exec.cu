@@ -239,7 +239,7 @@ void resolve(hoccl_comm* c, const Plan& P, const Call& call, Contributions how, 
       kept.push_back(std::move(cur));
     }
     out->swap(kept);
-    if (how == READ_AND_STORE && out->size() == 1 && c->sum_ctas < 128) {   // a short message: the kernel without tables
+    if (how == READ_AND_STORE && out->size() == 1) {   // a short message: the kernel without tables
       StoreAllArgs a;
       int grid = 0, threads = 0;
       const void* fn = store_all_entry(R, P.dtype, (int)c->sum_ctas, call.count, &a, &grid, &threads);

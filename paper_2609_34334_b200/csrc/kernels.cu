@@ -20,6 +20,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "device_common.cuh"
 
@@ -149,34 +150,30 @@ __global__ void __launch_bounds__(THREADS, 1) copy_kernel(const __grid_constant_
   }
 }
 
-// One element of a chain segment, element-wise: the same adds in the same order as the vector bodies.  NOPS > 0: the operand count,
-// so that an element's loads are in flight together (one after the other they cost ~0.7 us each).
+__device__ __forceinline__ float scalar_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ unsigned short scalar_add(unsigned short a, unsigned short b) {   // bf16
+  return __bfloat16_as_ushort(__float2bfloat16_rn(__fadd_rn(__uint_as_float((uint32_t)a << 16), __uint_as_float((uint32_t)b << 16))));
+}
+
+// One element of a chain segment, element-wise: the same adds in the same order as the vector bodies.  NOPS > 0: the operand count.  Eight
+// loads of an element are in flight together (one after the other they cost ~0.7 us each).
 template <int DT, int NOPS>
 __device__ __forceinline__ void chain_scalar(const ChainBatch& b, const ChainSeg& sg, unsigned long long i) {
+  using V = typename std::conditional<DT == 0, float, unsigned short>::type;
+  constexpr int N = NOPS ? NOPS : 8;
   void* const* op = b.ptr + sg.first_ptr;
   const int nops = NOPS ? NOPS : sg.nops;
-  if (DT == 0) {
-    float x[NOPS ? NOPS : 1];
+  V acc = V();
+  for (int q0 = 0; q0 < nops; q0 += N) {
+    V x[N];
 #pragma unroll
-    for (int q = 0; q < NOPS; q++) x[q] = static_cast<const float*>(op[q])[i];
-    float acc = NOPS ? x[0] : static_cast<const float*>(op[0])[i];
+    for (int q = 0; q < N; q++)
+      if (NOPS || q0 + q < nops) x[q] = static_cast<const V*>(op[q0 + q])[i];
 #pragma unroll
-    for (int q = 1; q < NOPS; q++) acc = __fadd_rn(acc, x[q]);
-    for (int q = 1; q < nops && !NOPS; q++) acc = __fadd_rn(acc, static_cast<const float*>(op[q])[i]);
-    for (int d = 0; d < sg.ndst; d++) static_cast<float*>(op[nops + d])[i] = acc;
-  } else {
-    auto add = [](unsigned short a, unsigned short c) {
-      return __bfloat16_as_ushort(__float2bfloat16_rn(__fadd_rn(__uint_as_float((uint32_t)a << 16), __uint_as_float((uint32_t)c << 16))));
-    };
-    unsigned short x[NOPS ? NOPS : 1];
-#pragma unroll
-    for (int q = 0; q < NOPS; q++) x[q] = static_cast<const unsigned short*>(op[q])[i];
-    unsigned short acc = NOPS ? x[0] : static_cast<const unsigned short*>(op[0])[i];
-#pragma unroll
-    for (int q = 1; q < NOPS; q++) acc = add(acc, x[q]);
-    for (int q = 1; q < nops && !NOPS; q++) acc = add(acc, static_cast<const unsigned short*>(op[q])[i]);
-    for (int d = 0; d < sg.ndst; d++) static_cast<unsigned short*>(op[nops + d])[i] = acc;
+    for (int q = 0; q < N; q++)
+      if (NOPS || q0 + q < nops) acc = q0 + q == 0 ? x[q] : scalar_add(acc, x[q]);
   }
+  for (int d = 0; d < sg.ndst; d++) static_cast<V*>(op[nops + d])[i] = acc;
 }
 
 // Element-wise items of a launch: heads, tails and segments without a common 16-byte phase.
@@ -456,11 +453,16 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
   chain_scalar_items<DT, NOPS>(batch);
 }
 
-// See StoreAllArgs.
+// See StoreAllArgs.  Latency bound: one fetch of parameters, one round trip of loads, one of stores.  Us per call in a burst, against chain_kernel's tables
+// and 8 operands at a time: 16 ranks bf16 on 8 CTAs 4 KiB per rank 6.1 -> 4.1, 8.1 KiB (heads and tails) 10.25 -> 4.15, 192 KiB 12.3 -> 9.5; 9 ranks fp32 64
+// KiB 8.2 -> 4.4; whole GPU 16 ranks 1 MiB 10.2 -> 5.0, 8 ranks 1 MiB (chain_fan_kernel) 6.1 -> 4.1.
 template <int DT, int NOPS, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) store_all_kernel(const __grid_constant__ StoreAllArgs a) {
   using T = Traits<DT>;
-  const unsigned c = blockIdx.x / a.parts, part = blockIdx.x - c * a.parts;
+  const unsigned width = THREADS / a.groups, group = threadIdx.x / width, tid = threadIdx.x - group * width;
+  const unsigned unit = blockIdx.x * a.groups + group, c = unit / a.parts, part = unit - c * a.parts;
+  wait_for_stream();
+  if (c >= NOPS) return;   // the last CTA of a grid that the chunks do not fill
   const char* src[NOPS];
 #pragma unroll
   for (int j = 0; j < NOPS; j++) src[j] = static_cast<const char*>(a.x[(c + 1 + j) % NOPS]);
@@ -468,48 +470,37 @@ __global__ void __launch_bounds__(THREADS, 1) store_all_kernel(const __grid_cons
   const unsigned at = lo * T::E;                                              // byte offset of the chunk
   const unsigned head = min(((16u - ((a.phase + at) & 15u)) & 15u) / T::E, n), nvec = (n - head) / T::VE;
   const unsigned per = (nvec + a.parts - 1) / a.parts, v1 = min(nvec, (part + 1) * per);
-  constexpr int U = NOPS <= 4 ? 4 : 2;   // vectors of a thread in flight
-  wait_for_stream();
-  for (unsigned v = part * per + threadIdx.x; v < v1; v += U * THREADS) {
+  constexpr int U = NOPS <= 4 ? 4 : NOPS <= 8 ? 2 : 1;   // vectors of a thread in flight
+  for (unsigned v = part * per + tid; v < v1; v += U * width) {
     uint4 buf[U][NOPS];
 #pragma unroll
     for (int u = 0; u < U; u++)
-      if (v + u * THREADS < v1) {
+      if (v + u * width < v1) {
 #pragma unroll
-        for (int j = 0; j < NOPS; j++) buf[u][j] = __ldcs(reinterpret_cast<const uint4*>(src[j] + (at + head * T::E + (v + u * THREADS) * 16)));
+        for (int j = 0; j < NOPS; j++) buf[u][j] = __ldcs(reinterpret_cast<const uint4*>(src[j] + (at + head * T::E + (v + u * width) * 16)));
       }
 #pragma unroll
     for (int u = 0; u < U; u++)
-      if (v + u * THREADS < v1) {
+      if (v + u * width < v1) {
         uint4 acc = buf[u][0];
 #pragma unroll
         for (int j = 1; j < NOPS; j++) acc = chain_add<DT>(acc, buf[u][j]);
 #pragma unroll
-        for (int r = 0; r < NOPS; r++) *reinterpret_cast<uint4*>(static_cast<char*>(a.y[r]) + (at + head * T::E + (v + u * THREADS) * 16)) = acc;
+        for (int r = 0; r < NOPS; r++) *reinterpret_cast<uint4*>(static_cast<char*>(a.y[r]) + (at + head * T::E + (v + u * width) * 16)) = acc;
       }
   }
   // head and tail, element by element
   const unsigned ns = n - nvec * T::VE;
-  if (part == a.parts - 1 && threadIdx.x < ns) {
-    const unsigned i = lo + (threadIdx.x < head ? threadIdx.x : threadIdx.x + nvec * T::VE);
-    if (DT == 0) {
-      float x[NOPS];
+  if (part == a.parts - 1 && tid < ns) {
+    using V = typename std::conditional<DT == 0, float, unsigned short>::type;
+    const unsigned i = lo + (tid < head ? tid : tid + nvec * T::VE);
+    V x[NOPS];
 #pragma unroll
-      for (int j = 0; j < NOPS; j++) x[j] = reinterpret_cast<const float*>(src[j])[i];
+    for (int j = 0; j < NOPS; j++) x[j] = reinterpret_cast<const V*>(src[j])[i];
 #pragma unroll
-      for (int j = 1; j < NOPS; j++) x[0] = __fadd_rn(x[0], x[j]);
+    for (int j = 1; j < NOPS; j++) x[0] = scalar_add(x[0], x[j]);
 #pragma unroll
-      for (int r = 0; r < NOPS; r++) static_cast<float*>(a.y[r])[i] = x[0];
-    } else {
-      unsigned short x[NOPS];
-#pragma unroll
-      for (int j = 0; j < NOPS; j++) x[j] = reinterpret_cast<const unsigned short*>(src[j])[i];
-#pragma unroll
-      for (int j = 1; j < NOPS; j++)
-        x[0] = __bfloat16_as_ushort(__float2bfloat16_rn(__fadd_rn(__uint_as_float((uint32_t)x[0] << 16), __uint_as_float((uint32_t)x[j] << 16))));
-#pragma unroll
-      for (int r = 0; r < NOPS; r++) static_cast<unsigned short*>(a.y[r])[i] = x[0];
-    }
+    for (int r = 0; r < NOPS; r++) static_cast<V*>(a.y[r])[i] = x[0];
   }
 }
 
@@ -960,31 +951,34 @@ void prepare_chain_batch(ChainBatch* b, int ctas) {
   fill_flat(&b->flat, b->nseg, tile_v, head, nvec, nscalar);
 }
 
+template <int DT, int R>
+static const void* store_all_from(int r) {
+  if constexpr (R <= kMaxStoreAllRanks) return r == R ? reinterpret_cast<const void*>(&store_all_kernel<DT, R, 512>) : store_all_from<DT, R + 1>(r);
+  else return nullptr;
+}
 template <int DT>
 static const void* store_all_of(int R) {
-  switch (R) {
-    case 2: return reinterpret_cast<const void*>(&store_all_kernel<DT, 2, 512>);
-    case 3: return reinterpret_cast<const void*>(&store_all_kernel<DT, 3, 512>);
-    case 4: return reinterpret_cast<const void*>(&store_all_kernel<DT, 4, 512>);
-    case 5: return reinterpret_cast<const void*>(&store_all_kernel<DT, 5, 512>);
-    case 6: return reinterpret_cast<const void*>(&store_all_kernel<DT, 6, 512>);
-    case 7: return reinterpret_cast<const void*>(&store_all_kernel<DT, 7, 512>);
-    case 8: return reinterpret_cast<const void*>(&store_all_kernel<DT, 8, 512>);
-    default: return nullptr;
-  }
+  return store_all_from<DT, 2>(R);
 }
 const void* store_all_entry(int R, int dtype, int ctas, unsigned long long count, StoreAllArgs* a, int* grid, int* threads) {
   const void* fn = dtype == 0 ? store_all_of<0>(R) : store_all_of<1>(R);
-  if (!fn || ctas < R || count > (1ull << 28)) return nullptr;   // 32-bit byte offsets
+  if (!fn || count > (1ull << 28)) return nullptr;   // 32-bit byte offsets
   a->count = (unsigned)count;
   a->q = (unsigned)((count + R - 1) / R);
-  // no more CTAs than have a round of vectors each
-  const unsigned vecs = a->q / (dtype == 0 ? 4 : 8), useful = (vecs + 511) / 512;
-  a->parts = std::max(1u, std::min((unsigned)(ctas / R), useful));
-  // CTAs that the chunks do not divide among themselves stay idle: fine while latency decides, not when the stores do
-  if (R * a->parts < (unsigned)ctas && vecs > a->parts * 1024u) return nullptr;
-  *grid = R * (int)a->parts;
+  const unsigned vecs = a->q / (dtype == 0 ? 4 : 8);
+  a->groups = a->parts = 1;
+  if (ctas < R) {   // fewer CTAs than chunks: a CTA's warps are split between chunks
+    while ((int)a->groups * ctas < R) a->groups *= 2;
+    if (a->groups > 16) return nullptr;
+    *grid = (R + (int)a->groups - 1) / (int)a->groups;
+  } else {   // no more CTAs than have a round of vectors each
+    a->parts = std::max(1u, std::min((unsigned)(ctas / R), (vecs + 511) / 512));
+    *grid = R * (int)a->parts;
+  }
   *threads = 512;
+  if (wide_grid(ctas) && vecs > a->parts * 512u) return nullptr;   // from a second round on chain_fan_kernel's shapes are the better ones
+  // CTAs that the chunks do not divide among themselves stay idle: fine while latency decides, not when the stores do
+  if (*grid < ctas && vecs > a->parts * (1024u / a->groups)) return nullptr;
   return fn;
 }
 

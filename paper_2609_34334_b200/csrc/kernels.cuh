@@ -64,15 +64,16 @@ struct ChainBatch {
 // A short all-reduce in one kernel: chunk c of every rank's vector, operands x[c+1], x[c+2], ..., x[c], stored to every y[r].  No
 // tables: a CTA finds its part of a chunk from its index, so it waits for one fetch of parameters before its first load and not for
 // four that depend on each other.  All pointers share their address modulo 16.
-constexpr int kMaxStoreAllRanks = 8;
+constexpr int kMaxStoreAllRanks = 16;
 struct StoreAllArgs {
   unsigned int count, q;   // elements of the vector, of a full chunk
   unsigned int parts;      // CTAs per chunk: the grid is R * parts
+  unsigned int groups;     // chunks per CTA, a power of two: parts or groups is 1
   unsigned int phase;      // address of the vectors modulo 16
   const void* x[kMaxStoreAllRanks];
   void* y[kMaxStoreAllRanks];
 };
-// Kernel and grid for R ranks (2..8) within `ctas` CTAs; null if there is none (more ranks, or fewer CTAs than ranks).
+// Kernel and grid for R ranks (2..16) within `ctas` CTAs; null if there is none, or if it would leave CTAs idle that the stores need.
 const void* store_all_entry(int R, int dtype, int ctas, unsigned long long count, StoreAllArgs* args, int* grid, int* threads);
 
 // One copy segment: dst[0..bytes) <- src[0..bytes).

@@ -87,8 +87,8 @@ typedef struct {
   long n_moves;          /* MOVE operations of the last call (copies on the CE path, segments on the SM path) */
   long n_move_launches;  /* SM copy kernel launches of the last call (0 on the CE path) */
   long n_sum_launches;   /* SUM kernel launches of the last call */
-  long max_sum_ctas;     /* CTAs of the widest SUM launch */
-  long max_copy_ctas;    /* CTAs of the widest SM copy launch */
+  long max_sum_ctas;     /* CTAs of the widest SUM launch: the budget it ran under */
+  long max_copy_ctas;    /* CTAs of the widest SM copy launch, likewise */
   long n_pieces;         /* pipeline pieces per ring chunk */
   long graph_hit;        /* 1 if the call replayed a cached CUDA graph, 0 if it built one or used streams */
   double sum_kernel_ms;  /* with parameter "profile" = 1: total device time of SUM launches since hoccl_profile_reset */
@@ -143,7 +143,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
 /*
  * Tuning and diagnostics.  Keys:
  *  "sum_ctas"    CTAs of a SUM launch, 1..1024 (default 8: the SM budget for sums)
- *  "copy_ctas"   CTAs of an SM copy launch, 1..1024 (default 8)
+ *  "copy_ctas"   CTAs of an SM copy launch, 1..1024 (default 8).  Both: 148 (every SM) or more means the whole GPU; the chain sums and the
+ *                moves of such a launch take a small CTA per tile, however many that makes
  *  "piece_bytes" pipeline piece size in bytes (rounded to a multiple of 1024).  If the key is not set: for reductions, whole
  *                ring chunks (up to 256 MiB) on HOCCL_PATH_CE and on HOCCL_PATH_SM when both CTA budgets are 128 or more (pieces exist to overlap one
  *                piece's move with another piece's sum, which neither driver copies nor whole-GPU grids do); otherwise

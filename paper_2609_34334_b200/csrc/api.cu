@@ -781,8 +781,8 @@ hoccl_result_t hoccl_move_inspect(int n, const uint64_t* src, const uint64_t* ds
   *n_seg = 0;
   int nd = 0, launch = 0;
   for (const MoveBatch& b : pack_moves(group_of_moves(n, src, dst, len), ctas)) {
-    int threads = 0;
-    move_kernel_entry(b, ctas, false, &threads);
+    int threads = 0, grid = 0;
+    move_kernel_entry(b, ctas, false, &threads, &grid);
     if (*n_seg + b.nseg > seg_cap || nd + b.ndst_total > dst_cap) return HOCCL_ERR_INVALID_ARG;
     for (int k = 0; k < b.nseg; k++) {
       const MoveSeg& m = b.seg[k];

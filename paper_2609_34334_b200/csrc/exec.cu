@@ -422,11 +422,11 @@ static std::vector<KernelLaunch> move_launches(const hoccl_comm* c, const RGroup
   for (const MoveBatch& b : pack_moves(g, ctas)) {
     double bytes = 0;
     for (int k = 0; k < b.nseg; k++) bytes += (1.0 + (double)b.seg[k].ndst) * (double)b.seg[k].bytes;
-    int threads = 0;
+    int threads = 0, grid = 0;
     MoveBatchSmall small;
     const bool fits = shrink_move_batch(b, &small);
-    const void* fn = move_kernel_entry(b, ctas, fits, &threads);
-    out.push_back(fits ? make_launch(small, fn, ctas, threads, bytes, b.ndst_total) : make_launch(b, fn, ctas, threads, bytes, b.ndst_total));
+    const void* fn = move_kernel_entry(b, ctas, fits, &threads, &grid);
+    out.push_back(fits ? make_launch(small, fn, grid, threads, bytes, b.ndst_total) : make_launch(b, fn, grid, threads, bytes, b.ndst_total));
   }
   return out;
 }
@@ -442,8 +442,9 @@ std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, co
       prepare_chain_batch(&b, (int)c->sum_ctas);
       double bytes = 0;
       for (int i = 0; i < b.nseg; i++) bytes += (double)(b.seg[i].nops + b.seg[i].ndst) * (double)b.seg[i].n * (double)P.elem;
-      const void* fn = chain_kernel_entry(b, (int)c->sum_ctas, &threads);
-      out.push_back(make_launch(b, fn, c->sum_ctas, threads, bytes, 0));
+      int grid = 0;
+      const void* fn = chain_kernel_entry(b, (int)c->sum_ctas, &threads, &grid);
+      out.push_back(make_launch(b, fn, grid, threads, bytes, 0));
       first += n;
     }
     return out;
@@ -680,7 +681,7 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
   // A short chain of kernels goes out as a graph or as launches (see launch_in_order).  A graph costs the host less (0.9 us against 1.6 to 2.4
   // per launch) and reaches an idle device 1.6 us earlier; behind other work launches start up to 2 us earlier.  Whether there is
   // work in front cannot be asked for less (cudaStreamQuery 0.3 us if there is, 1.6 if not).  So: launches if the call follows the one before
-  // it at once, on the same stream, and takes the device longer than the host, or the calls before it did; otherwise the graph.  Us of a call
+  // it at once, on the same stream, and takes the device longer than the host, or is one launch and the calls before it did; otherwise the graph.  Us of a call
   // in a burst as graphs / as launches, R = 8 bf16: all-reduce 4 KiB per rank 3.6 / 4.9, 96 KiB 4.10 / 4.52, 128 KiB 6.15 / 4.55, 384 KiB
   // 10.25 / 9.1, 1 MiB with 8 + 40 CTAs 17.0 / 14.35; 148 CTAs 512 KiB 4.10 / 4.85, 1 MiB 6.14 / 4.85; all-to-all 512 KiB 4.10 / 4.80, 1 MiB
   // 6.15 / 4.80; two launches, R = 16, all-to-all 512 KiB 8.19 / 8.56, 2 MiB 20.5 / 18.3.  The line: the estimate against 1.8 + 2.2 per launch.
@@ -688,7 +689,7 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
   const bool follows = last.stream == user && t0 - last.returned < kBurstGapUs;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;   // a capture is refused by the graph launch, in a burst or not
   const bool behind = follows && cudaStreamIsCapturing(user, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
-                      (t0 < last.busy_until || hit->est_us >= 1.8 + 2.2 * (double)hit->launches.size());
+                      ((t0 < last.busy_until && hit->launches.size() == 1) || hit->est_us >= 1.8 + 2.2 * (double)hit->launches.size());
   last.busy_until = (follows ? std::max(t0, last.busy_until) : t0) + hit->est_us;
   struct Returns {   // on every way out
     Burst& last;

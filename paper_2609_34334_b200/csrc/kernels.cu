@@ -397,14 +397,15 @@ __global__ void __launch_bounds__(THREADS, 1) chain_pipe2_kernel(const __grid_co
 }
 
 // Whole-GPU sums, and the sum that carries the all-gather too: NOPS operands are read once, the result is stored to NDST
-// destinations (1, or NOPS: one per rank).  That is what the collective cannot do without; bound by HBM with a whole-GPU grid.
+// destinations (1, or NOPS: one per rank).  That is what the collective cannot do without; bound by HBM with a whole-GPU grid, which has a CTA
+// per tile (R = 8, 64 MiB fp32, every rank: 163.8 us, 6.56 TB/s; 170 with one CTA per SM that walks the tiles).
 // A tile is U x THREADS vectors, so U x NOPS loads are in flight per thread before the first add.
 template <int DT, int NOPS, int NDST, int U, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
   const Flat& f = batch.flat;
-  // tile t of the flattened space belongs to CTA t mod grid; walked segment by segment, so that the NOPS + NDST pointers are loaded
-  // once per segment and not once per tile (R = 8, 64 MiB fp32, tiles of 384 vectors: 194 us with a look-up per tile, 171 without)
+  // tile t of the flattened space belongs to CTA t mod grid; a walk goes segment by segment, so that the NOPS + NDST pointers are loaded
+  // once per segment and not once per tile (one CTA per SM, R = 8, 64 MiB fp32, tiles of 384 vectors: 194 us with a look-up per tile, 171 without)
   const unsigned long long T_all = f.tpre[batch.nseg];
   int k = 0;
   wait_for_stream();
@@ -543,7 +544,7 @@ __device__ __forceinline__ int find_segment(const unsigned* pre, int n, unsigned
 // all-gather, now 10); here a thread loads the two aligned vectors that hold its 16 bytes (the second is its neighbour's first, an
 // L1 hit), shifts them into place and stores aligned vectors.
 template <int U, int THREADS, class Batch>
-__global__ void __launch_bounds__(THREADS, 1) move_kernel(const __grid_constant__ Batch batch) {
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 6 : 1) move_kernel(const __grid_constant__ Batch batch) {
   constexpr int H = U < 4 ? U : 4;
   const int nseg = batch.nseg;
   const unsigned T_all = batch.tpre[nseg], tile_u = batch.tile_u;
@@ -775,6 +776,8 @@ __global__ void __launch_bounds__(kThreads, 2) occupy_kernel(unsigned long long 
 // chunks of a ring step over the grid (gradient bucket, whole GPU: 0.201 against 0.213 ms per step).
 static bool wide_grid(int ctas) { return ctas >= 128; }
 static bool wide_copy_grid(int ctas) { return ctas >= 128; }
+constexpr int kAllSms = 148;
+static bool whole_gpu(int ctas) { return ctas >= kAllSms; }   // a CTA per tile, see kMoveShapes
 
 // Host side of the flattened view (same split as the device helper; tile = 4 x threads vectors for the sum, 8 x 1024 or
 // 4 x 512 for the copy: the shapes launch_sum / launch_copy pick for `ctas`).
@@ -913,6 +916,15 @@ static ChainVariant chain_fan_variant(int nops, int ctas) {
     default: return {nullptr, 0, 0};
   }
 }
+// The whole GPU, a CTA per tile (see kMoveShapes; the walk above stays between 128 CTAs and all SMs).  Us, 64 MiB per rank bf16 (32 for 3 and 6), walk / CTA
+// per tile: sums that store for every rank R = 2 (128 MiB) 89 / 80.2, 4 86 / 80.5, 8 171 / 163.8; one destination R = 8 94 / 88.1, 3 24 / 20.7.  Tiles of
+// 128 to 512 vectors are within 3 %, but for 2 and 3 operands with one destination, which want two vectors per thread (R = 2, 128 MiB 59.4, 67.0 with one).
+template <int DT, int N>
+static ChainVariant chain_tile_variant(int nops, bool fan) {
+  if constexpr (N > 8) return {nullptr, 0, 0};
+  else if (nops != N) return chain_tile_variant<DT, N + 1>(nops, fan);
+  else return fan ? fan_of<DT, N, N <= 3 ? 2 : 1, 256>() : wide_of<DT, N, N <= 3 ? 2 : 1, 256>();
+}
 static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
   ChainVariant plain{b.dtype == 0 ? reinterpret_cast<const void*>(&chain_kernel<0, 1024>) : reinterpret_cast<const void*>(&chain_kernel<1, 1024>), 1024, 1024};
   if (b.nseg <= 0) return plain;
@@ -920,7 +932,8 @@ static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
   for (int k = 1; k < b.nseg; k++)
     if (b.seg[k].nops != nops || b.seg[k].ndst != ndst) return plain;
   ChainVariant v = plain;
-  if (ndst == 1 && !wide_grid(ctas)) v = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
+  if (whole_gpu(ctas) && (ndst == 1 || ndst == nops)) v = b.dtype == 0 ? chain_tile_variant<0, 2>(nops, ndst != 1) : chain_tile_variant<1, 2>(nops, ndst != 1);
+  else if (ndst == 1 && !wide_grid(ctas)) v = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
   else if (ndst == 1) v = b.dtype == 0 ? chain_wide_variant<0>(nops) : chain_wide_variant<1>(nops);
   else if (ndst == nops) v = b.dtype == 0 ? chain_fan_variant<0>(nops, ctas) : chain_fan_variant<1>(nops, ctas);
   return v.fn ? v : plain;
@@ -1017,8 +1030,9 @@ cudaError_t launch_chain(const ChainBatch& batch, int ctas, cudaStream_t stream)
   if (batch.nseg <= 0) return cudaSuccess;
   ChainBatch b = batch;
   prepare_chain_batch(&b, ctas);
-  const ChainVariant v = chain_variant(b, ctas);
-  return launch_in_order(v.fn, ctas, v.threads, &b, stream);
+  int threads = 0, grid = 0;
+  const void* fn = chain_kernel_entry(b, ctas, &threads, &grid);
+  return launch_in_order(fn, grid, threads, &b, stream);
 }
 
 void prepare_fan_batch(FanBatch* b, int ctas) {
@@ -1046,32 +1060,28 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
   return true;
 }
 
-// Launch shape: a thread keeps up to u vectors.  Under a CTA budget 8 x 1024 (the bytes in flight per SM decide).  Whole-GPU grids
-// are bound by HBM and want little in flight per SM, the less the more often a vector is stored (the reads otherwise come in bursts
-// between the writes): 44 KiB for copies, 7 for one read stored 7 times.  Measured in TB/s at 256 MiB per stream: copies 4 x 704 6.2
-// (4 x 512 5.8, 8 x 1024 4.2), 1:2 2 x 704 6.0 (2 x 256 4.0), 1:3 4 x 384 6.0 (2 x 256 4.5), 1:4 and 1:5 2 x 384 5.8 (2 x 256 4.8 and 5.1), 1:7
-// 1 x 448 5.8 (4 x 512 3.9).  Out of phase every vector is loaded twice, from L1 the second time: 4 x 704, measured for copies (all-to-all of
-// 64 MiB per rank 173 us in phase, 175 out of phase).  One such segment decides for the launch, fan-outs included: all-gather of 64 MiB per rank
-// over 8 ranks 106 us in phase (1 x 448), 116 out of phase.
+// Launch shape: a thread keeps up to u vectors.  Under a CTA budget 8 x 1024 (the bytes in flight per SM decide).  On the whole GPU a CTA
+// per tile, in small CTAs: they drift apart, so that some load while others store; CTAs that walk many tiles, one per SM, go through the two
+// phases together.  TB/s at 8 MiB per segment, 2 x 256 or (stored four times and more) 1 x 256 with a CTA per tile against the best
+// walk: copies 6.81 / 6.25 (4 x 704), 1:3 6.37 / 5.94 (4 x 384), 1:7 6.46 / 5.80 (1 x 448); 512 KiB 5.60 / 5.32, 4.29 / 3.22, 5.08 / 4.41.  Larger and smaller
+// tiles (1 to 16 x 128 to 512) are within 3 % of these.  Between 128 CTAs and all SMs the walk stays.
 struct MoveShape {
   int u, threads;
 };
-static constexpr MoveShape kMoveShapes[] = {{8, 1024}, {4, 704}, {2, 704}, {4, 384}, {2, 384}, {1, 448}};
+static constexpr MoveShape kMoveShapes[] = {{8, 1024}, {4, 704}, {1, 448}, {2, 256}, {1, 256}};
 static int move_shape(const MoveBatch& b, int ctas) {
   if (!wide_copy_grid(ctas)) return 0;
-  for (int k = 0; k < b.nseg; k++)
-    if (((uintptr_t)b.seg[k].src ^ (uintptr_t)b.dst[b.seg[k].first_dst]) & 15) return 1;
   const int per_seg = b.nseg > 0 ? (b.ndst_total + b.nseg / 2) / b.nseg : 1;   // stores per load, rounded
-  return per_seg <= 1 ? 1 : per_seg == 2 ? 2 : per_seg == 3 ? 3 : per_seg <= 5 ? 4 : 5;
+  if (whole_gpu(ctas)) return per_seg <= 3 ? 3 : 4;
+  return per_seg <= 2 ? 1 : 2;
 }
 template <class Batch>
 static const void* move_entry(int shape) {
   switch (shape) {
     case 1: return reinterpret_cast<const void*>(&move_kernel<4, 704, Batch>);
-    case 2: return reinterpret_cast<const void*>(&move_kernel<2, 704, Batch>);
-    case 3: return reinterpret_cast<const void*>(&move_kernel<4, 384, Batch>);
-    case 4: return reinterpret_cast<const void*>(&move_kernel<2, 384, Batch>);
-    case 5: return reinterpret_cast<const void*>(&move_kernel<1, 448, Batch>);
+    case 2: return reinterpret_cast<const void*>(&move_kernel<1, 448, Batch>);
+    case 3: return reinterpret_cast<const void*>(&move_kernel<2, 256, Batch>);
+    case 4: return reinterpret_cast<const void*>(&move_kernel<1, 256, Batch>);
     default: return reinterpret_cast<const void*>(&move_kernel<8, 1024, Batch>);
   }
 }
@@ -1100,7 +1110,11 @@ void prepare_move_batch(MoveBatch* b, int ctas) {
   // without a tile or with one more than others.  In units of one vector per thread stored once, a tile costs its stores and ~3 for
   // the loads to come back; the grid runs ceil(tiles / ctas) of them one after another.
   double best = 0;
-  for (unsigned u = most_u; u >= 1; u /= 2) {
+  if (whole_gpu(ctas)) {
+    unsigned long long tiles = 0;
+    for (int k = 0; k < b->nseg; k++) tiles += (b->seg[k].nvec + most_u * threads - 1) / (most_u * threads);
+    b->tile_u = tiles < 2 * kAllSms ? 1 : most_u;
+  } else for (unsigned u = most_u; u >= 1; u /= 2) {
     unsigned long long tiles = 0;
     for (int k = 0; k < b->nseg; k++) tiles += (b->seg[k].nvec + u * threads - 1) / (u * threads);
     const double per_tile = 3.0 + (double)u * b->ndst_total / (b->nseg > 0 ? b->nseg : 1);
@@ -1126,9 +1140,10 @@ bool shrink_move_batch(const MoveBatch& b, MoveBatchSmall* o) {
   return true;
 }
 
-const void* move_kernel_entry(const MoveBatch& b, int ctas, bool small, int* threads) {
+const void* move_kernel_entry(const MoveBatch& b, int ctas, bool small, int* threads, int* grid) {
   const int shape = move_shape(b, ctas);
   *threads = kMoveShapes[shape].threads;
+  *grid = whole_gpu(ctas) ? (int)std::max(b.tpre[b.nseg], std::min(8u * (unsigned)ctas, (b.spre[b.nseg] + *threads - 1) / *threads)) : ctas;
   return small ? move_entry<MoveBatchSmall>(shape) : move_entry<MoveBatch>(shape);
 }
 
@@ -1137,15 +1152,15 @@ cudaError_t launch_moves(MoveBatch* b, int ctas, cudaStream_t stream) {
   prepare_move_batch(b, ctas);
   MoveBatchSmall small;
   const bool fits = shrink_move_batch(*b, &small);
-  int threads = 0;
-  const void* fn = move_kernel_entry(*b, ctas, fits, &threads);
-  return launch_in_order(fn, ctas, threads, fits ? static_cast<void*>(&small) : static_cast<void*>(b), stream);
+  int threads = 0, grid = 0;
+  const void* fn = move_kernel_entry(*b, ctas, fits, &threads, &grid);
+  return launch_in_order(fn, grid, threads, fits ? static_cast<void*>(&small) : static_cast<void*>(b), stream);
 }
 
 cudaError_t launch_move(const void* src, void* dst, unsigned long long bytes, int ctas, cudaStream_t stream) {
   // One long copy in phase leaves nothing to choose: copy_kernel's plain tile walk is 0.5 to 0.8 % faster there (waves of 42.8 MB
   // messages on 40 CTAs, three communicators at once: 98.7 -> 98.0 us).  Below 16 MB its tiles leave CTAs without work.
-  if (bytes >= (16ull << 20) && (((uintptr_t)src ^ (uintptr_t)dst) & 15) == 0 && ((uintptr_t)dst & 127) == 0) {
+  if (!whole_gpu(ctas) && bytes >= (16ull << 20) && (((uintptr_t)src ^ (uintptr_t)dst) & 15) == 0 && ((uintptr_t)dst & 127) == 0) {
     CopyBatch cb;
     cb.nseg = 1;
     cb.pad = 0;
@@ -1217,9 +1232,11 @@ cudaError_t launch_bf16_add_selftest(unsigned long long* counts, cudaStream_t st
   bf16_add_selftest_kernel<<<65536, 256, 0, stream>>>(counts);
   return cudaGetLastError();
 }
-const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads) {
+const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads, int* grid) {
   const ChainVariant v = chain_variant(batch, ctas);
+  const Flat& f = batch.flat;
   *threads = v.threads;
+  *grid = whole_gpu(ctas) ? (int)std::max(f.tpre[batch.nseg], std::min(8ull * (unsigned)ctas, (f.spre[batch.nseg] + v.threads - 1) / v.threads)) : ctas;
   return v.fn;
 }
 const void* graph_root_kernel_entry() { return reinterpret_cast<const void*>(&graph_root_kernel); }
@@ -1258,8 +1275,9 @@ cudaError_t preload_kernels() {
     }
   for (int nops = 2; nops <= 8; nops++)
     for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn, chain_fan_variant<0>(nops, 8).fn, chain_fan_variant<1>(nops, 8).fn,
-                          chain_fan_variant<0>(nops, 148).fn, chain_fan_variant<1>(nops, 148).fn, chain_wide_variant<0>(nops).fn,
-                          chain_wide_variant<1>(nops).fn}) {
+                          chain_fan_variant<0>(nops, 128).fn, chain_fan_variant<1>(nops, 128).fn, chain_wide_variant<0>(nops).fn,
+                          chain_wide_variant<1>(nops).fn, chain_tile_variant<0, 2>(nops, false).fn, chain_tile_variant<1, 2>(nops, false).fn,
+                          chain_tile_variant<0, 2>(nops, true).fn, chain_tile_variant<1, 2>(nops, true).fn}) {
       cudaFuncAttributes a;
       cudaError_t e = cudaFuncGetAttributes(&a, f);
       if (e != cudaSuccess) return e;

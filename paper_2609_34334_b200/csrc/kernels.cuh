@@ -140,7 +140,7 @@ bool add_move_seg(MoveBatch* batch, const void* src, void* const* dsts, int ndst
 // Batches are prepared with the CTA count they are launched with.
 void prepare_move_batch(MoveBatch* batch, int ctas);
 bool shrink_move_batch(const MoveBatch& batch, MoveBatchSmall* out);   // false if it does not fit
-const void* move_kernel_entry(const MoveBatch& batch, int ctas, bool small, int* threads);
+const void* move_kernel_entry(const MoveBatch& batch, int ctas, bool small, int* threads, int* grid);
 cudaError_t launch_moves(MoveBatch* batch, int ctas, cudaStream_t stream);   // prepares and launches; nothing for an empty batch
 cudaError_t launch_move(const void* src, void* dst, unsigned long long bytes, int ctas, cudaStream_t stream);   // one copy
 
@@ -221,7 +221,7 @@ void prepare_chain_batch(ChainBatch* batch, int ctas);
 // Appends a segment (operands in the order they are added); false if the batch has no room for it.
 bool add_chain_seg(ChainBatch* batch, const void* const* ops, int nops, void* const* dsts, int ndst, unsigned long long n);
 // kernel and thread count that serve `batch` with `ctas` CTAs (the batch must have been prepared for the same `ctas`)
-const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads);
+const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads, int* grid);
 // counts: two device words, zeroed by the caller; see bf16_add_selftest_kernel
 cudaError_t launch_bf16_add_selftest(unsigned long long* counts, cudaStream_t stream);
 void prepare_fan_batch(FanBatch* batch, int ctas);

@@ -370,13 +370,13 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
       total += C[(size_t)u * R + v];
     }
   // The move route, as for the other collectives: on the copy route a short pattern, and one with copies the driver does badly,
-  // runs on the copy kernel, and so does one of mostly short flows (every driver copy costs a microsecond, and the short ones of
-  // an uneven pattern leave the GPU part empty).  R = 8, driver copies against the kernel: 1 MiB per rank 20.8 / 5.5 us, 12 MiB (flows
-  // of 1.5 MiB on average) 49 / 39, 32 MiB (4 MiB) 93 / 95, 128 MiB 334 / 366; in rows of 666 bytes 32 MiB 447 / 98; R = 4, 12 MiB (3 MiB)
-  // 20.7 / 15.2; R = 16, 12 MiB (0.75 MiB) 147 / 79, 32 MiB (2 MiB) 239 / 192.
+  // runs on the move kernel, and so does one of flows that are short on average (every driver copy costs a microsecond, and those of an uneven
+  // pattern leave the GPU part empty).  R = 8, driver copies against the kernel: 8 MiB per rank (flows of 1 MiB on average) 41 / 22.6 us, 16 MiB (2
+  // MiB) 61 / 43, 32 MiB (4 MiB) 95.7 / 83.5, in rows of 666 bytes 447 / 86; R = 16, 64 MiB (4 MiB) 393 / 336.  Longer whole flows stay with the
+  // driver, which is 3 to 6 % behind there (8 ranks 64 MiB 173.6 / 164.1, 128 MiB 335 / 325).
   hoccl_path_t route = c->path;
   if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && !modelled) {
-    constexpr uint64_t kShortFlow = 3 << 20;
+    constexpr uint64_t kShortFlow = 9 << 19;   // 4.5 MiB
     uint64_t most = 0, flows = 0;
     bool bad = false;
     for (int u = 0; u < R; u++) {

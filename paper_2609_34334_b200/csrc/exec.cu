@@ -688,8 +688,9 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
   Burst& last = t_burst;
   const bool follows = last.stream == user && t0 - last.returned < kBurstGapUs;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;   // a capture is refused by the graph launch, in a burst or not
-  const bool behind = follows && cudaStreamIsCapturing(user, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
-                      ((t0 < last.busy_until && hit->launches.size() == 1) || hit->est_us >= 1.8 + 2.2 * (double)hit->launches.size());
+  const size_t n = hit->launches.size();
+  const bool behind = n && follows && ((n == 1 && t0 < last.busy_until) || hit->est_us >= 1.8 + 2.2 * (double)n) &&
+                      cudaStreamIsCapturing(user, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
   last.busy_until = (follows ? std::max(t0, last.busy_until) : t0) + hit->est_us;
   struct Returns {   // on every way out
     Burst& last;
@@ -795,7 +796,7 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
     if (!done) return cuda_fail(c, cudaErrorMemoryAllocation, "event pool");
     CU_TRY(c, cudaEventRecord(done, out));
     CU_TRY(c, cudaStreamWaitEvent(user, done, 0));
-  } else if (behind && !hit->launches.empty()) {
+  } else if (behind) {
     for (const KernelLaunch& k : hit->launches) CU_TRY(c, launch_kernel(k, user));
   } else if (c->handshake) {
     // paper Sec. 3.2: the stream hands itself to the CPU proxy, which runs the schedule and hands it back
@@ -832,16 +833,17 @@ hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype) {
 // Whether an all-gather or all-to-all is better not left to driver copies.  Such a call runs on the move kernel at any size, like a
 // small one.
 //   * Some block is a copy the driver does badly (see kDriverLine): 64 MiB per rank over 8 ranks, blocks 16 bytes short of whole: all-gather
-//     372 us in driver copies, 96 on the kernel, all-to-all 384 and 173; two bytes out of phase 818 and 114, 838 and 175.
-//   * The blocks of an all-to-all are short: 16 MiB per rank 51 and 47 us, 40 MiB 112 and 110, 64 MiB 175 and 173, 256 MiB 660 and 690.
-//   * An all-gather of 3 ranks or more: the kernel reads a block once, driver copies once per destination (9 MiB per rank over 8 ranks
-//     24.7 and 14.4 us, 40 MiB 84 and 62, 64 MiB 150 and 96, 256 MiB 572 and 367; over 3 ranks 64 MiB 45 and 38).  Both take the whole GPU.
-//     Beside a loop of 8192^3 bf16 GEMMs a call over 8 ranks costs the GEMMs (medians of two runs) and takes meanwhile: 25 MiB per rank 22 to
-//     31 us and 0.13 ms (driver copies 10 to 13 us and 0.24 ms; the kernel with "ce_small_ctas" = 40 37 to 68 us and 0.79 ms), 64 MiB 80 us
+//     372 us in driver copies, 96 on the kernel, all-to-all 384 and 164; two bytes out of phase 818 and 99, 838 and 171.
+//   * The blocks of an all-to-all are short, or few: 64 MiB per rank over 2 ranks 46.7 and 41.0 us, over 4 88 and 81.5.  Long whole blocks between more
+//     ranks stay with the driver, 5 % behind at 64 MiB (8 ranks 172 and 164), 1 % at 256 MiB (655 and 650).
+//   * An all-gather: the kernel reads a block once, driver copies once per destination (64 MiB per rank over 2 ranks 45 and 31 us, over 8 150 and
+//     96; 256 MiB over 8 572 and 345).  Both take the whole GPU.
+//     Beside a loop of 8192^3 bf16 GEMMs a call over 8 ranks costs the GEMMs (medians of two runs, with one CTA per SM) and takes meanwhile: 25 MiB per
+//     rank 22 to 31 us and 0.13 ms (driver copies 10 to 13 us and 0.24 ms; the kernel with "ce_small_ctas" = 40 37 to 68 us and 0.79 ms), 64 MiB 80 us
 //     and 0.27 ms (66 to 104 us and 0.48 ms; 40 CTAs 97 to 107 us and 0.84 ms).
 static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t block = call.count * dtype_size(call.dtype);
-  if (block < kDriverShort || (call.kind == PLAN_ALLGATHER && c->R >= 3)) return true;
+  if (block < kDriverShort || call.kind == PLAN_ALLGATHER || c->R <= 4) return true;
   for (int u = 0; u < c->R; u++)
     for (int v = 0; v < c->R; v++)
       if (bad_for_driver((const char*)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0), (const char*)call.recv[v] + (size_t)u * block, block))

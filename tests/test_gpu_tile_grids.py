@@ -5,6 +5,7 @@ import pytest
 import torch
 
 from paper_2609_34334_b200 import binding as hb
+from paper_2609_34334_b200 import diag as hd
 from paper_2609_34334_b200 import workloads as W
 from gpu_util import DevBuf, same_bits
 from test_gpu_parity import run_allreduce
@@ -22,18 +23,18 @@ def test_moves(ndst, ctas):
         x = rng.integers(0, 256, n, dtype=np.uint8)
         for soff, doff in ((0, 0), (3, 3), (1, 6)):
             src, dst = DevBuf(n, soff).put(x), [DevBuf(n, (doff + 5 * d) % 16) for d in range(ndst)]
-            rc = hb.lib().hoccl_fanout_launch(src.ptr, hb._ptr_array(dst), ndst, n, ctas, None)
+            rc = hd.fanout_launch(src, dst, n, ctas)
             torch.cuda.synchronize()
             assert rc == hb.OK and all((d.get(np.uint8) == x).all() and d.guards_intact() for d in dst), (n, soff, doff)
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
-@pytest.mark.parametrize("R", [2, 3, 4, 7, 8, 9])
+@pytest.mark.parametrize("R", [2, 3, 4, 7, 8, 9, 13, 16, 17])
 def test_sums(oracle, R, dtype):
     torch.cuda.set_device(0)
     e = W.elem_size(dtype)
     v = 16 // e
-    for n in (R * 148 * 256 * v, R * (148 * 512 * v + 1) - 1, R * 300 * 512 * v + 5):
+    for n in (R * 148 * 256 * v, R * (148 * 512 * v + 1) - 1) + ((R * 300 * 512 * v + 5,) if R < 10 else ()):
         xs = W.rank_inputs("uniform", 1200 + R, R, n, dtype)
         want = oracle.ring_allreduce(xs)
         comm = auto_comm(R, n, dtype, hb.PATH_SM, sum_ctas=148, copy_ctas=148)

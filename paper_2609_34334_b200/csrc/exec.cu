@@ -838,9 +838,8 @@ hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype) {
 //     ranks stay with the driver, 5 % behind at 64 MiB (8 ranks 172 and 164), 1 % at 256 MiB (655 and 650).
 //   * An all-gather: the kernel reads a block once, driver copies once per destination (64 MiB per rank over 2 ranks 45 and 31 us, over 8 150 and
 //     96; 256 MiB over 8 572 and 345).  Both take the whole GPU.
-//     Beside a loop of 8192^3 bf16 GEMMs a call over 8 ranks costs the GEMMs (medians of two runs, with one CTA per SM) and takes meanwhile: 25 MiB per
-//     rank 22 to 31 us and 0.13 ms (driver copies 10 to 13 us and 0.24 ms; the kernel with "ce_small_ctas" = 40 37 to 68 us and 0.79 ms), 64 MiB 80 us
-//     and 0.27 ms (66 to 104 us and 0.48 ms; 40 CTAs 97 to 107 us and 0.84 ms).
+//     Beside a loop of 8192^3 bf16 GEMMs a call of 25 MiB per rank over 8 ranks costs the GEMMs (median and quartiles) and takes meanwhile: all-gather
+//     25 us (5 to 37) and 0.13 ms, in driver copies 22 (4 to 37) and 0.24 ms; all-to-all 14 (-10 to 40) and 0.33 ms, 11 (-18 to 31) and 0.28 ms.
 static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t block = call.count * dtype_size(call.dtype);
   if (block < kDriverShort || call.kind == PLAN_ALLGATHER || c->R <= 4) return true;

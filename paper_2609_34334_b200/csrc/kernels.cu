@@ -208,8 +208,8 @@ __device__ __forceinline__ void report_sm(const Batch& batch) {
 
 // Chain sum for any number of operands and destinations: one 16-byte vector per thread and tile; the operands are loaded in batches of up
 // to 8 before they are added, so up to 8 x 16 KiB are in flight per CTA.  It serves what the compiled forms below do not (see
-// chain_variant): more than 16 operands, mixed counts, and from 9 operands on whole-GPU grids and sums that store for every rank.  With 148
-// CTAs and 64 MiB per rank it is at the copy rate there: 9 operands 108 us (6.2 TB/s), 12 139 (6.3), 16 175 (6.5).
+// chain_variant): more than 16 operands, mixed counts, and from 9 operands on sums that store for every rank on fewer than 148 CTAs and
+// one destination on 128 to 147.  With 148 CTAs and 64 MiB per rank: 9 operands 108 us (6.2 TB/s), 12 139 (6.3), 16 175 (6.5).
 template <int DT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1) chain_kernel(const __grid_constant__ ChainBatch batch) {
   using T = Traits<DT>;
@@ -919,9 +919,11 @@ static ChainVariant chain_fan_variant(int nops, int ctas) {
 // The whole GPU, a CTA per tile (see kMoveShapes; the walk above stays between 128 CTAs and all SMs).  Us, 64 MiB per rank bf16 (32 for 3 and 6), walk / CTA
 // per tile: sums that store for every rank R = 2 (128 MiB) 89 / 80.2, 4 86 / 80.5, 8 171 / 163.8; one destination R = 8 94 / 88.1, 3 24 / 20.7.  Tiles of
 // 128 to 512 vectors are within 3 %, but for 2 and 3 operands with one destination, which want two vectors per thread (R = 2, 128 MiB 59.4, 67.0 with one).
+// 9 to 16 operands, against chain_kernel: every rank R = 9 bf16 32 MiB 99.6 / 95.2, 16 167.9 / 165.7; reduce-scatter + all-gather R = 9 fp32 32 MiB 114 / 103,
+// 4 MiB 17.6 / 15.2, R = 16 bf16 0.28 MiB 14.4 / 12.3.
 template <int DT, int N>
 static ChainVariant chain_tile_variant(int nops, bool fan) {
-  if constexpr (N > 8) return {nullptr, 0, 0};
+  if constexpr (N > 16) return {nullptr, 0, 0};
   else if (nops != N) return chain_tile_variant<DT, N + 1>(nops, fan);
   else return fan ? fan_of<DT, N, N <= 3 ? 2 : 1, 256>() : wide_of<DT, N, N <= 3 ? 2 : 1, 256>();
 }

@@ -12,7 +12,7 @@
 //
 // Buffers that share their address modulo 16 (the usual case) do not need the scratch at all: the chain sum reads every rank's
 // contribution where it lies, as the communicator's automatic schedule does, and one launch of moves, or the sum itself, brings
-// the result to every rank (6 ranks of 500,009 fp32: 123 us as a ring of 15 launches, 26 us as two).
+// the result to every rank (6 ranks of 500,009 fp32: 123 us as a ring of 15 launches, 17 us as two).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -32,7 +32,9 @@ static __device__ __align__(256) unsigned char g_static_scratch[HOCCL_STATIC_SCR
 
 constexpr int kMaxDevices = 64;
 constexpr int kStaticSumCtas = 8;    // same SM budget for sums as the communicator's default
-constexpr int kStaticCopyCtas = 32;
+constexpr int kStaticCopyCtas = 32;    // of the ring's copies, which run between its sums
+constexpr int kStaticMoveCtas = 148;   // of the one launch of moves behind the sums: the whole GPU, as the communicator's short moves (6 ranks of
+                                       // 500,009 fp32 21.4 us on 32 CTAs, 16.7; of 8 MiB 80.7 and 58.5)
 std::mutex g_mu;
 void* g_base[kMaxDevices] = {};
 
@@ -93,12 +95,12 @@ cudaError_t read_in_place(const void* const* send, void* const* recv, size_t cou
     void* dsts[64];
     for (int k = 1; k < R; k++) dsts[k - 1] = (char*)recv[(c + k) % R] + lo * e;
     if (!add_move_seg(&m, (const char*)recv[c] + lo * e, dsts, R - 1, (unsigned long long)(n * e))) {
-      err = launch_moves(&m, kStaticCopyCtas, st);
+      err = launch_moves(&m, kStaticMoveCtas, st);
       m.nseg = m.ndst_total = 0;
       add_move_seg(&m, (const char*)recv[c] + lo * e, dsts, R - 1, (unsigned long long)(n * e));
     }
   }
-  return err == cudaSuccess ? launch_moves(&m, kStaticCopyCtas, st) : err;
+  return err == cudaSuccess ? launch_moves(&m, kStaticMoveCtas, st) : err;
 }
 
 bool overlap(const char* a, size_t an, const char* b, size_t bn) { return an && bn && a < b + bn && b < a + an; }

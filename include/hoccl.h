@@ -195,8 +195,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                the same kernel (2 S R bytes in all, one launch, no moves).  hoccl_last_stats counts the moves that remain.
  *                "rs_direct" = 1 keeps the rank-local form, as do HOCCL_PATH_CE_HOST, "roles" and hoccl_host_allreduce of more than
  *                72 MB for all ranks together.  Measured on B200 (R = 8, bf16, default settings): 25 MiB reduce-scatter + all-gather
- *                0.291 -> 0.221 ms, 40 MiB all-reduce 0.417 -> 0.347 ms; HOCCL_PATH_SM with 148 + 148 CTAs, 64 MiB fp32 0.355 ->
- *                0.172 ms.
+ *                0.291 -> 0.212 ms, 40 MiB all-reduce 0.417 -> 0.336 ms; HOCCL_PATH_SM with 148 + 148 CTAs, 64 MiB fp32 0.355 ->
+ *                0.164 ms.
  *  "ce_small_bytes" on HOCCL_PATH_CE a call whose per-rank message (S in the convention of each collective: all-reduce
  *                count, reduce-scatter / all-gather / all-to-all R * count elements) is at most this many bytes issues its
  *                moves as batched launches of the SM copy kernel with "ce_small_ctas" CTAs instead of driver copies, i.e.
@@ -209,8 +209,10 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                by its own size.
  *                Unless it is 0, copies the driver does badly do not go to it at any size (it takes 4 us more for a copy of 1 MiB or
  *                more that does not start on a 128-byte line and end after whole 4 KiB, and runs at half rate or less when the two
- *                ends differ modulo 4): a send/recv message, an all-gather or all-to-all of such blocks, an all-to-all of blocks below 4 MiB and an
- *                all-gather of 3 ranks or more (the kernel reads a block once, driver copies once per destination) runs on the copy kernel like a small one, and an
+ *                ends differ modulo 4): a send/recv message or an all-to-all of such blocks, an all-to-all of blocks below 4 MiB or over at most
+ *                4 ranks, an uneven exchange of flows up to 4.5 MiB on average, any all-gather (the kernel reads a block once, driver copies
+ *                once per destination) and the all-gather of an all-reduce with such chunks (automatic schedule, SUM budget below 64 CTAs) run on
+ *                the copy kernel like a small one.  With "ag_direct" set by hand an
  *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of the copies of its direct
  *                all-gather to one launch of the copy kernel ("copy_ctas" CTAs) per piece (in a ring all-gather, whose copies
  *                forward what the one before has written, copies stay whole).
@@ -220,7 +222,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                piece's sum (inside ONE graph, and on plain streams, they were never seen to overlap).  Sums still run one
  *                at a time.  Costs ~8 us of host time per piece and call.  -1 (default) = automatic: 2 pieces from 2 MiB per
  *                ring chunk, from 4 MiB per ring chunk on pieces of about 4 MiB (at least 4, at most 32 of them), off below; with contributions read
- *                in place ("rs_direct" = 2) 2 pieces from 4 MiB, from 5 MiB on pieces of about 2.7 MiB (4 to 32); 0 = off;
+ *                in place ("rs_direct" = 2) as many pieces as the root of the all-gather's time over 5.4 us, of 1.25 MiB or more, at
+ *                least 2 above 8 MiB per chunk (R = 2, 64 MiB per rank 2, R = 8, 40 MiB 4, 256 MiB 10); 0 = off;
  *                2..64 = that many pieces.  Ignored when "piece_bytes" is set.
  *  "ce_small_ctas" CTAs of those launches, 1..1024 (default 148: like the driver's own copies they may use the whole GPU,
  *                for tens of microseconds)
@@ -266,7 +269,8 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                operations, same bits.
  *  "host_pieces" pieces per ring chunk of the pipelined hoccl_host_allreduce (1..64, default 8; 1 = not pipelined).  If the key is not
  *                set and the direct schedule runs: by size (see hoccl_host_allreduce)
- *  "use_graph"   1 = run a cached CUDA graph built from the plan (default), 0 = streams and events
+ *  "use_graph"   1 = run a cached CUDA graph built from the plan (default; a call of up to three dependent kernels that follows the
+ *                thread's last call on its stream at once goes out as launches instead, which start up to 2 us earlier), 0 = streams and events
  *  "handshake"   1 = the paper's stream manager (Sec. 3.2): instead of launching into the caller's stream, the call
  *                enqueues three stream memory operations (write "hand-over n has arrived", wait for "hand-over n is
  *                released", write "hand-over n is behind me"; the counters live in pinned host memory and only grow) and

@@ -1108,7 +1108,8 @@ void prepare_move_batch(MoveBatch* b, int ctas) {
     s.nvec = (unsigned)nvec;
     b->spre[k + 1] = b->spre[k] + (unsigned)(s.bytes - nvec * 16);
   }
-  // Tiles: as large as a thread's registers hold (a tile's loads are in flight together), smaller where that would leave CTAs
+  // Tiles of a whole-GPU launch: the shape's, one vector per thread where that gives fewer than two per SM.  Of a walk: as large as
+  // a thread's registers hold (a tile's loads are in flight together), smaller where that would leave CTAs
   // without a tile or with one more than others.  In units of one vector per thread stored once, a tile costs its stores and ~3 for
   // the loads to come back; the grid runs ceil(tiles / ctas) of them one after another.
   double best = 0;

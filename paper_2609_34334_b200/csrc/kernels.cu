@@ -1066,24 +1066,30 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
 // per tile, in small CTAs: they drift apart, so that some load while others store; CTAs that walk many tiles, one per SM, go through the two
 // phases together.  TB/s at 8 MiB per segment, 2 x 256 or (stored four times and more) 1 x 256 with a CTA per tile against the best
 // walk: copies 6.81 / 6.25 (4 x 704), 1:3 6.37 / 5.94 (4 x 384), 1:7 6.46 / 5.80 (1 x 448); 512 KiB 5.60 / 5.32, 4.29 / 3.22, 5.08 / 4.41.  Larger and smaller
-// tiles (1 to 16 x 128 to 512) are within 3 % of these.  Between 128 CTAs and all SMs the walk stays.
+// tiles (1 to 16 x 128 to 512) are within 3 % of these.  Between 128 CTAs and all SMs the walk stays, in its own shapes: it wants little in
+// flight per SM, the less the more often a vector is stored, 44 KiB for copies (4 x 704 6.2 TB/s, 8 x 1024 4.2), 7 for one read stored 7 times.
 struct MoveShape {
   int u, threads;
 };
-static constexpr MoveShape kMoveShapes[] = {{8, 1024}, {4, 704}, {1, 448}, {2, 256}, {1, 256}};
+static constexpr MoveShape kMoveShapes[] = {{8, 1024}, {4, 704}, {2, 704}, {4, 384}, {2, 384}, {1, 448}, {2, 256}, {1, 256}};
 static int move_shape(const MoveBatch& b, int ctas) {
   if (!wide_copy_grid(ctas)) return 0;
   const int per_seg = b.nseg > 0 ? (b.ndst_total + b.nseg / 2) / b.nseg : 1;   // stores per load, rounded
-  if (whole_gpu(ctas)) return per_seg <= 3 ? 3 : 4;
-  return per_seg <= 2 ? 1 : 2;
+  if (whole_gpu(ctas)) return per_seg <= 3 ? 6 : 7;
+  for (int k = 0; k < b.nseg; k++)   // out of phase every vector is loaded twice: the shape for copies
+    if (((uintptr_t)b.seg[k].src ^ (uintptr_t)b.dst[b.seg[k].first_dst]) & 15) return 1;
+  return per_seg <= 1 ? 1 : per_seg == 2 ? 2 : per_seg == 3 ? 3 : per_seg <= 5 ? 4 : 5;
 }
 template <class Batch>
 static const void* move_entry(int shape) {
   switch (shape) {
     case 1: return reinterpret_cast<const void*>(&move_kernel<4, 704, Batch>);
-    case 2: return reinterpret_cast<const void*>(&move_kernel<1, 448, Batch>);
-    case 3: return reinterpret_cast<const void*>(&move_kernel<2, 256, Batch>);
-    case 4: return reinterpret_cast<const void*>(&move_kernel<1, 256, Batch>);
+    case 2: return reinterpret_cast<const void*>(&move_kernel<2, 704, Batch>);
+    case 3: return reinterpret_cast<const void*>(&move_kernel<4, 384, Batch>);
+    case 4: return reinterpret_cast<const void*>(&move_kernel<2, 384, Batch>);
+    case 5: return reinterpret_cast<const void*>(&move_kernel<1, 448, Batch>);
+    case 6: return reinterpret_cast<const void*>(&move_kernel<2, 256, Batch>);
+    case 7: return reinterpret_cast<const void*>(&move_kernel<1, 256, Batch>);
     default: return reinterpret_cast<const void*>(&move_kernel<8, 1024, Batch>);
   }
 }

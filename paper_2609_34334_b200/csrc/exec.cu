@@ -579,7 +579,7 @@ hoccl_result_t run_streams(hoccl_comm* c, const Plan& P, const std::vector<RGrou
 
 std::vector<uint64_t> make_key(hoccl_comm* c, const Call& call) {
   std::vector<uint64_t> k;
-  k.reserve(26 + 2 * c->R);
+  k.reserve(27 + 2 * c->R);
   k.push_back((uint64_t)call.kind);
   k.push_back((uint64_t)call.count);
   k.push_back((uint64_t)call.dtype);
@@ -598,6 +598,7 @@ std::vector<uint64_t> make_key(hoccl_comm* c, const Call& call) {
   k.push_back((uint64_t)c->rs_direct);
   k.push_back((uint64_t)c->ce_overlap);
   k.push_back((uint64_t)(c->fused && c->path == HOCCL_PATH_SM && !c->handshake));
+  k.push_back((uint64_t)c->handshake);   // an entry of handshake mode has no launches of its own and its graph is on the device before the proxy meets it
   k.push_back((uint64_t)c->roles);
   k.push_back((uint64_t)c->piece_grade);
   k.push_back((uint64_t)c->roles_missing);

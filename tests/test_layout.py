@@ -140,3 +140,11 @@ def test_one_setting_changed(c, name, k):
         assert err.code == hb.ERR_UNSUPPORTED, c
         return
     assert one.signature != two.signature or _steps(one) == _steps(two), (c, name)
+
+
+@pytest.mark.parametrize("kind", [ALLREDUCE, REDUCE_SCATTER, ALLGATHER, ALLTOALL])
+def test_signature_of_handshake_mode(kind):
+    """A call of handshake mode never shares its entry with one outside it: that entry would launch past the proxy in a burst, and its
+    graph need not be on the device yet when the proxy replays it behind a parked stream."""
+    a, b = (lay_out(kind, 8, 4096, "bf16", path=hb.PATH_SM, handshake=mode)[0] for mode in (0, 1))
+    assert _steps(a) == _steps(b) and a.signature != b.signature

@@ -121,6 +121,13 @@ typedef struct {
 hoccl_result_t hoccl_move_inspect(int n, const uint64_t* src, const uint64_t* dst, const uint64_t* len, int ctas, int seg_cap, int dst_cap,
                                   hoccl_move_seg_t* segs, uint64_t* dst_out, int* n_seg);
 /*
+ * Host only: whether the kernel that a launch with `ctas` CTAs picks is one of those that are loaded before any stream is parked in a
+ * hand-over ("handshake", "p2p_strict").  kind 0: the SUM of two operands; 1: a copy_kernel launch; 2: the chain sum of `nops` operands stored
+ * to `ndst` places; 3: moves of `count` bytes from one source to `ndst` places; 4: the short all-reduce of `nops` ranks and `count` elements.
+ * Writes 1, 0, or -1 if there is no such launch.  nops 2..64, ndst 1..64.
+ */
+hoccl_result_t hoccl_kernel_preloaded(int kind, hoccl_dtype_t dtype, int nops, int ndst, size_t count, int ctas, int* preloaded);
+/*
  * Self-test of the arithmetic: the chain sum of the direct reduce-scatter adds bf16 operands with the native packed add
  * (add.rn.bf16x2); this call compares it on the device with the reference add of every SUM (binary32 add of the widened
  * operands, rounded to nearest even into bf16) for ALL 2^32 pairs of bf16 bit patterns.  counts: DEVICE array of two 64-bit

@@ -795,6 +795,45 @@ hoccl_result_t hoccl_move_inspect(int n, const uint64_t* src, const uint64_t* ds
   return HOCCL_OK;
 }
 
+hoccl_result_t hoccl_kernel_preloaded(int kind, hoccl_dtype_t dtype, int nops, int ndst, size_t count, int ctas, int* preloaded) {
+  if (dtype_size((int)dtype) == 0) return HOCCL_ERR_UNSUPPORTED;
+  if (kind < 0 || kind > 4 || nops < 2 || nops > 64 || ndst < 1 || ndst > 64 || ctas < 1 || ctas > 1024 || !preloaded) return HOCCL_ERR_INVALID_ARG;
+  const void* fn = nullptr;
+  int threads = 0, grid = 0;
+  // addresses are only looked at: a megabyte apart, one phase
+  const auto at = [&](int k) { return (void*)(uintptr_t)((uint64_t)(k + 1) << 20); };
+  if (kind == 0) fn = sum_kernel_entry((int)dtype, ctas, &threads);
+  if (kind == 1) fn = copy_kernel_entry(ctas, &threads);
+  if (kind == 2) {
+    ChainBatch b;
+    b.nseg = b.nptr = 0;
+    b.dtype = (int)dtype;
+    const void* ops[64];
+    void* dsts[64];
+    for (int k = 0; k < nops; k++) ops[k] = at(k);
+    for (int k = 0; k < ndst; k++) dsts[k] = at(64 + k);
+    add_chain_seg(&b, ops, nops, dsts, ndst, (unsigned long long)count);
+    prepare_chain_batch(&b, ctas);
+    fn = chain_kernel_entry(b, ctas, &threads, &grid);
+  }
+  if (kind == 3) {
+    MoveBatch b;
+    b.nseg = b.ndst_total = 0;
+    void* dsts[64];
+    for (int k = 0; k < ndst; k++) dsts[k] = at(k + 1);
+    add_move_seg(&b, at(0), dsts, ndst, (unsigned long long)std::min<size_t>(count, kMaxMoveSegBytes));
+    prepare_move_batch(&b, ctas);
+    MoveBatchSmall small;
+    fn = move_kernel_entry(b, ctas, shrink_move_batch(b, &small), &threads, &grid);
+  }
+  if (kind == 4) {
+    StoreAllArgs a;
+    fn = store_all_entry(nops, (int)dtype, ctas, (unsigned long long)count, &a, &grid, &threads);
+  }
+  *preloaded = !fn ? -1 : is_preloaded(fn) ? 1 : 0;
+  return HOCCL_OK;
+}
+
 hoccl_result_t hoccl_kernel_sms(int kind, const void* a, const void* b, void* out, size_t bytes, hoccl_dtype_t dtype, int ctas,
                                 unsigned int* smid_out, hoccl_stream_t stream) {
   size_t e = dtype_size((int)dtype);

@@ -21,6 +21,7 @@
 
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "device_common.cuh"
 
@@ -1249,49 +1250,48 @@ const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads, 
   return v.fn;
 }
 const void* graph_root_kernel_entry() { return reinterpret_cast<const void*>(&graph_root_kernel); }
+// The kernels that the rules of this file may pick for a call, asked from the rules themselves: one CTA count on each side of every line between
+// launch shapes (wide_grid, whole_gpu), every operand count, one destination or one per operand.
+static std::vector<const void*> dispatched_kernels() {
+  std::vector<const void*> fns = {reinterpret_cast<const void*>(&occupy_kernel),           reinterpret_cast<const void*>(&graph_root_kernel),
+                                  reinterpret_cast<const void*>(&onepass_kernel<0, 512>),  reinterpret_cast<const void*>(&onepass_kernel<1, 512>),
+                                  reinterpret_cast<const void*>(&onepass_kernel<0, 1024>), reinterpret_cast<const void*>(&onepass_kernel<1, 1024>)};
+  for (int ctas : {1, kAllSms - 1, kAllSms}) {
+    int threads = 0;
+    fns.push_back(copy_kernel_entry(ctas, &threads));
+    for (int dtype = 0; dtype < 2; dtype++) {
+      fns.push_back(sum_kernel_entry(dtype, ctas, &threads));
+      for (int nops = 2; nops <= kMaxChainSrcs + 1; nops++)
+        for (int ndst : {1, nops}) {
+          ChainBatch b;
+          b.nseg = 1;
+          b.dtype = dtype;
+          b.seg[0] = ChainSeg{0, 0, nops, ndst, 0};
+          fns.push_back(chain_variant(b, ctas).fn);
+        }
+    }
+  }
+  for (int R = 2; R <= kMaxStoreAllRanks; R++)
+    for (const void* f : {store_all_of<0>(R), store_all_of<1>(R)}) fns.push_back(f);
+  for (int shape = 0; shape < (int)(sizeof(kMoveShapes) / sizeof(kMoveShapes[0])); shape++)
+    for (const void* f : {move_entry<MoveBatch>(shape), move_entry<MoveBatchSmall>(shape)}) fns.push_back(f);
+  std::sort(fns.begin(), fns.end());
+  fns.erase(std::unique(fns.begin(), fns.end()), fns.end());
+  return fns;
+}
 // Forces the module that holds these kernels to be loaded now.  Loading a kernel on first launch can synchronise the
 // device; that must never happen while a stream is parked in a hand-over that only the launching thread can finish.
 cudaError_t preload_kernels() {
-  const void* fns[] = {reinterpret_cast<const void*>(&sum2_kernel<0, 4, 512>),  reinterpret_cast<const void*>(&sum2_kernel<0, 4, 1024>),
-                       reinterpret_cast<const void*>(&sum2_kernel<1, 4, 512>),  reinterpret_cast<const void*>(&sum2_kernel<1, 4, 1024>),
-                       reinterpret_cast<const void*>(&copy_kernel<4, 512>),     reinterpret_cast<const void*>(&copy_kernel<8, 1024>),
-                       reinterpret_cast<const void*>(&occupy_kernel),           reinterpret_cast<const void*>(&onepass_kernel<0, 512>),
-                       reinterpret_cast<const void*>(&onepass_kernel<1, 512>),  reinterpret_cast<const void*>(&onepass_kernel<0, 1024>),
-                       reinterpret_cast<const void*>(&onepass_kernel<1, 1024>), reinterpret_cast<const void*>(&graph_root_kernel),
-                       reinterpret_cast<const void*>(&chain_kernel<0, 1024>), reinterpret_cast<const void*>(&chain_kernel<1, 1024>)};
-  for (const void* f : fns) {
+  for (const void* f : dispatched_kernels()) {
     cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, f);
+    const cudaError_t e = cudaFuncGetAttributes(&a, f);
     if (e != cudaSuccess) return e;
   }
-  for (int R = 2; R <= kMaxStoreAllRanks; R++)
-    for (const void* f : {store_all_of<0>(R), store_all_of<1>(R)}) {
-      cudaFuncAttributes a;
-      cudaError_t e = cudaFuncGetAttributes(&a, f);
-      if (e != cudaSuccess) return e;
-    }
-  for (int shape = 0; shape < (int)(sizeof(kMoveShapes) / sizeof(kMoveShapes[0])); shape++)
-    for (const void* f : {move_entry<MoveBatch>(shape), move_entry<MoveBatchSmall>(shape)}) {
-      cudaFuncAttributes a;
-      cudaError_t e = cudaFuncGetAttributes(&a, f);
-      if (e != cudaSuccess) return e;
-    }
-  for (int nops = 9; nops <= 16; nops++)
-    for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn}) {
-      cudaFuncAttributes a;
-      cudaError_t e = cudaFuncGetAttributes(&a, f);
-      if (e != cudaSuccess) return e;
-    }
-  for (int nops = 2; nops <= 8; nops++)
-    for (const void* f : {chain_pipe_variant<0>(nops).fn, chain_pipe_variant<1>(nops).fn, chain_fan_variant<0>(nops, 8).fn, chain_fan_variant<1>(nops, 8).fn,
-                          chain_fan_variant<0>(nops, 128).fn, chain_fan_variant<1>(nops, 128).fn, chain_wide_variant<0>(nops).fn,
-                          chain_wide_variant<1>(nops).fn, chain_tile_variant<0, 2>(nops, false).fn, chain_tile_variant<1, 2>(nops, false).fn,
-                          chain_tile_variant<0, 2>(nops, true).fn, chain_tile_variant<1, 2>(nops, true).fn}) {
-      cudaFuncAttributes a;
-      cudaError_t e = cudaFuncGetAttributes(&a, f);
-      if (e != cudaSuccess) return e;
-    }
   return cudaSuccess;
+}
+bool is_preloaded(const void* fn) {
+  const std::vector<const void*> fns = dispatched_kernels();
+  return std::find(fns.begin(), fns.end(), fn) != fns.end();
 }
 
 cudaError_t launch_occupy_all_sms(unsigned long long ns, int num_sms, cudaStream_t stream, int* ctas_out) {

@@ -236,8 +236,9 @@ const void* graph_root_kernel_entry();   // an empty kernel (1 CTA of 32 threads
 // Memory-port probe: `ctas` CTAs only read (mode 0) or only write (mode 1) `bytes` bytes (a multiple of 128 KiB is walked).
 cudaError_t launch_port_probe(int mode, void* buf, unsigned long long bytes, int ctas, unsigned int* sink, cudaStream_t stream);
 
-// Loads every kernel of the library on the current device (no launch).
+// Loads every kernel that a call may launch (but for the "fused" and "roles" ones, loaded when first asked for) on the current device (no launch).
 cudaError_t preload_kernels();
+bool is_preloaded(const void* fn);   // whether it loads this one
 
 // Fills every thread slot of every SM for `ns` nanoseconds (measured with %globaltimer per CTA).
 // It never waits on memory or on another agent, so it always ends by itself.

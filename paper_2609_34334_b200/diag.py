@@ -16,7 +16,7 @@ EXEC_GRAPH, EXEC_STREAMS, EXEC_ONE_KERNEL, EXEC_ONEPASS, EXEC_PROXY, EXEC_ROLES 
 
 EXPORTS = [   # every function include/hoccl_diag.h declares
     "hoccl_chain_launch", "hoccl_comm_init_host_only", "hoccl_copy_launch", "hoccl_fanout_inspect", "hoccl_fanout_launch", "hoccl_flatten_inspect",
-    "hoccl_kernel_sms", "hoccl_layout_build", "hoccl_layout_destroy", "hoccl_layout_get_access", "hoccl_layout_group_deps",
+    "hoccl_kernel_preloaded", "hoccl_kernel_sms", "hoccl_layout_build", "hoccl_layout_destroy", "hoccl_layout_get_access", "hoccl_layout_group_deps",
     "hoccl_layout_num_accesses", "hoccl_layout_num_groups", "hoccl_layout_num_pieces", "hoccl_layout_signature", "hoccl_move_inspect",
     "hoccl_options_resolve", "hoccl_plan_build", "hoccl_plan_destroy", "hoccl_plan_get_op",
     "hoccl_plan_group_deps", "hoccl_plan_inbox_slots", "hoccl_plan_num_groups", "hoccl_plan_num_ops",
@@ -85,6 +85,7 @@ def lib() -> ctypes.CDLL:
         "hoccl_chain_launch": (i, [vp, sz, i, vp, vp, sz, i, i, vp]),
         "hoccl_fanout_inspect": (i, [i, vp, vp, vp, i, i, vp, vp, vp, vp, vp, vp, vp, ctypes.POINTER(i), ctypes.POINTER(i)]),
         "hoccl_move_inspect": (i, [i, vp, vp, vp, i, i, i, ctypes.POINTER(MoveSeg), vp, ctypes.POINTER(i)]),
+        "hoccl_kernel_preloaded": (i, [i, i, i, i, sz, i, ctypes.POINTER(i)]),
         "hoccl_kernel_sms": (i, [i, vp, vp, vp, sz, i, i, vp, vp]),
         "hoccl_selftest_barrier_timeout": (i, [vp, vp, vp, sz, vp]),
         "hoccl_selftest_roles_timeout": (i, [vpp, vpp, sz, i, vp, vp]),

@@ -96,3 +96,18 @@ def test_header_is_plain_c_and_a_c_program_links_against_the_library(tmp_path):
     subprocess.run(["gcc", "-std=c99", "-I", inc, str(src), "-o", str(exe), "-L", libdir, "-lhoccl", "-Wl,-rpath," + libdir], check=True)
     out = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout
     assert out.strip() == "%d entry points" % len(names)
+
+
+@pytest.mark.parametrize("kind", range(5))
+def test_kernels_of_every_launch_are_loaded_before_a_stream_can_be_parked(kind):
+    """Loading a kernel at its first launch can wait for the device, and so for a stream that only the launching thread would release."""
+    loaded, seen = ctypes.c_int(), set()
+    for ctas in (1, 7, 8, 40, 127, 128, 140, 147, 148, 149, 592, 1024):
+        for nops in range(2, 65) if kind in (2, 4) else (2,):
+            for ndst in sorted({1, 2, nops}) if kind == 2 else range(1, 65) if kind == 3 else (1,):
+                for count in (1, 5000, 1 << 20):
+                    for dtype in (0, 1):
+                        assert hd.lib().hoccl_kernel_preloaded(kind, dtype, nops, ndst, count, ctas, ctypes.byref(loaded)) == hb.OK
+                        assert loaded.value != 0, (kind, dtype, nops, ndst, count, ctas)
+                        seen.add(loaded.value)
+    assert 1 in seen and (kind == 4 or seen == {1})

@@ -244,6 +244,8 @@ int hoccl_layout_num_accesses(hoccl_layout_t layout);
 hoccl_result_t hoccl_layout_get_access(hoccl_layout_t layout, int index, hoccl_access_t* out);
 /* Writes up to `cap` group ids that `group` waits for into deps, returns their number (-1: no such group). */
 int hoccl_layout_group_deps(hoccl_layout_t layout, int group, int* deps, int cap);
+/* CTAs of the largest kernel launch that carries `group` out, as a graph of kernels; 0: driver copies (-1: no such group). */
+int hoccl_layout_group_ctas(hoccl_layout_t layout, int group);
 /* The words under which the call's graph is cached: calls with the same words replay the same graph.  Writes up to `cap`, returns
  * their number. */
 int hoccl_layout_signature(hoccl_layout_t layout, uint64_t* words, int cap);

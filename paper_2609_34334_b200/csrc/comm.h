@@ -65,6 +65,7 @@ struct RGroup {
   int chain_dep;
   std::vector<KernelLaunch> ready;   // if not empty, the launches that carry out the group (instead of batches built from segs)
   long ctas = 0;        // moves on the move kernel: its CTAs, 0 = "copy_ctas"
+  bool beside = false;  // sums: driver copies of another piece run beside them
   bool edges = false;   // copy route: the ends of driver copies, carried by a copy-kernel launch (see trim_driver_copies)
 };
 
@@ -209,6 +210,7 @@ struct Layout {
   std::vector<RGroup> groups;
   size_t host_need = 0;   // bytes of pinned host staging the moves bounce through (HOCCL_PATH_CE_HOST)
   bool overlap = false;   // copy route: the pieces' parts run on three internal streams
+  std::vector<int> ctas;  // inspect_call only: per group, the CTAs of its largest kernel launch, 0 = driver copies
 };
 
 // What a driver copy inside one device does at once, as timed on B200: a copy of 1 MiB or more whose destination does not start on a

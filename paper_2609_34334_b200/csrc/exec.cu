@@ -439,6 +439,7 @@ std::vector<KernelLaunch> kernel_launches(const hoccl_comm* c, const Plan& P, co
     for (size_t first = 0; first < g.segs.size();) {
       ChainBatch b;
       const size_t n = fill_chain_batch(g, first, P.dtype, P.elem, &b);
+      b.walk = g.beside ? 1 : 0;
       prepare_chain_batch(&b, (int)c->sum_ctas);
       double bytes = 0;
       for (int i = 0; i < b.nseg; i++) bytes += (double)(b.seg[i].nops + b.seg[i].ndst) * (double)b.seg[i].n * (double)P.elem;
@@ -1008,9 +1009,11 @@ static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut&
   }
   out->overlap = overlap && P.pieces > 1;   // with one piece there is nothing to overlap
   resolve(c, P, call, how, &out->groups, &out->host_need);
-  if (beside)
-    for (RGroup& g : out->groups)
-      if (g.kind == OP_MOVE && g.piece + 1 < P.pieces) g.ctas = kBesideSums;
+  for (RGroup& g : out->groups) {
+    if (beside && g.kind == OP_MOVE && g.piece + 1 < P.pieces) g.ctas = kBesideSums;
+    // the first piece's sum has nothing beside it unless the next piece's contributions are copied meanwhile
+    if (out->overlap && g.kind == OP_CHAIN) g.beside = g.piece > 0 || how == STAGED;
+  }
   return HOCCL_OK;
 }
 
@@ -1023,7 +1026,13 @@ hoccl_result_t inspect_call(hoccl_comm* c, Call* call, Layout* out, std::vector<
   *key = make_key(c, *call);
   rc = validate(c, call);
   if (rc != HOCCL_OK || call->count == 0) return rc;
-  return lay_out(c, *call, opt, contributions(c, *call, opt, call->count * dtype_size(call->dtype)), out);
+  rc = lay_out(c, *call, opt, contributions(c, *call, opt, call->count * dtype_size(call->dtype)), out);
+  for (const RGroup& g : out->groups) {
+    out->ctas.push_back(0);
+    if (g.kind == OP_MOVE && c->path != HOCCL_PATH_SM && !g.edges) continue;
+    for (const KernelLaunch& k : kernel_launches(c, out->plan, g)) out->ctas.back() = std::max(out->ctas.back(), k.grid);
+  }
+  return rc;
 }
 
 hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {

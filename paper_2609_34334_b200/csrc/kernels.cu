@@ -928,6 +928,11 @@ static ChainVariant chain_tile_variant(int nops, bool fan) {
   else if (nops != N) return chain_tile_variant<DT, N + 1>(nops, fan);
   else return fan ? fan_of<DT, N, N <= 3 ? 2 : 1, 256>() : wide_of<DT, N, N <= 3 ? 2 : 1, 256>();
 }
+// A whole-GPU sum with driver copies of another piece beside it: one CTA per SM that walks the tiles, as between 128 CTAs and all SMs.  A CTA per tile
+// takes every slot that comes free and the copies wait.  Us of an all-reduce on the copy route, 148 SUM CTAs, bf16, a CTA per tile / the walk: R = 8 256 MiB
+// in 8 pieces 902 / 884, 1 GiB 3940 / 3854; R = 4 128 MiB 250.8 / 243.2; R = 3 200 MB 285.2 / 279.8; R = 2 128 MiB 143 / 127.  Nine operands and more have no
+// compiled walk, and chain_kernel's tables cost more than the crowding (R = 16, 256 MiB 2070 / 2084).
+static bool chain_walks(const ChainBatch& b) { return b.walk && b.nseg > 0 && b.seg[0].nops <= 8; }
 static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
   ChainVariant plain{b.dtype == 0 ? reinterpret_cast<const void*>(&chain_kernel<0, 1024>) : reinterpret_cast<const void*>(&chain_kernel<1, 1024>), 1024, 1024};
   if (b.nseg <= 0) return plain;
@@ -935,7 +940,7 @@ static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
   for (int k = 1; k < b.nseg; k++)
     if (b.seg[k].nops != nops || b.seg[k].ndst != ndst) return plain;
   ChainVariant v = plain;
-  if (whole_gpu(ctas) && (ndst == 1 || ndst == nops)) v = b.dtype == 0 ? chain_tile_variant<0, 2>(nops, ndst != 1) : chain_tile_variant<1, 2>(nops, ndst != 1);
+  if (whole_gpu(ctas) && !chain_walks(b) && (ndst == 1 || ndst == nops)) v = b.dtype == 0 ? chain_tile_variant<0, 2>(nops, ndst != 1) : chain_tile_variant<1, 2>(nops, ndst != 1);
   else if (ndst == 1 && !wide_grid(ctas)) v = b.dtype == 0 ? chain_pipe_variant<0>(nops) : chain_pipe_variant<1>(nops);
   else if (ndst == 1) v = b.dtype == 0 ? chain_wide_variant<0>(nops) : chain_wide_variant<1>(nops);
   else if (ndst == nops) v = b.dtype == 0 ? chain_fan_variant<0>(nops, ctas) : chain_fan_variant<1>(nops, ctas);
@@ -1246,7 +1251,7 @@ const void* chain_kernel_entry(const ChainBatch& batch, int ctas, int* threads, 
   const ChainVariant v = chain_variant(batch, ctas);
   const Flat& f = batch.flat;
   *threads = v.threads;
-  *grid = whole_gpu(ctas) ? (int)std::max(f.tpre[batch.nseg], std::min(8ull * (unsigned)ctas, (f.spre[batch.nseg] + v.threads - 1) / v.threads)) : ctas;
+  *grid = whole_gpu(ctas) && !chain_walks(batch) ? (int)std::max(f.tpre[batch.nseg], std::min(8ull * (unsigned)ctas, (f.spre[batch.nseg] + v.threads - 1) / v.threads)) : ctas;
   return v.fn;
 }
 const void* graph_root_kernel_entry() { return reinterpret_cast<const void*>(&graph_root_kernel); }

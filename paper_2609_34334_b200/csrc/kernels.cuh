@@ -54,7 +54,7 @@ struct ChainBatch {
   int nseg;
   int dtype;
   int nptr;
-  int pad;
+  int walk = 0;  // 1: other kernels run beside this sum for all of its time; a whole-GPU grid is then one CTA per SM (see chain_walks)
   ChainSeg seg[kMaxSegs];
   void* ptr[kMaxChainPtrs];
   Flat flat;  // filled by prepare_chain_batch (launch_chain does it itself)

@@ -16,7 +16,7 @@ EXEC_GRAPH, EXEC_STREAMS, EXEC_ONE_KERNEL, EXEC_ONEPASS, EXEC_PROXY, EXEC_ROLES 
 
 EXPORTS = [   # every function include/hoccl_diag.h declares
     "hoccl_chain_launch", "hoccl_comm_init_host_only", "hoccl_copy_launch", "hoccl_fanout_inspect", "hoccl_fanout_launch", "hoccl_flatten_inspect",
-    "hoccl_kernel_preloaded", "hoccl_kernel_sms", "hoccl_layout_build", "hoccl_layout_destroy", "hoccl_layout_get_access", "hoccl_layout_group_deps",
+    "hoccl_kernel_preloaded", "hoccl_kernel_sms", "hoccl_layout_build", "hoccl_layout_destroy", "hoccl_layout_get_access", "hoccl_layout_group_ctas", "hoccl_layout_group_deps",
     "hoccl_layout_num_accesses", "hoccl_layout_num_groups", "hoccl_layout_num_pieces", "hoccl_layout_signature", "hoccl_move_inspect",
     "hoccl_options_resolve", "hoccl_plan_build", "hoccl_plan_destroy", "hoccl_plan_get_op",
     "hoccl_plan_group_deps", "hoccl_plan_inbox_slots", "hoccl_plan_num_groups", "hoccl_plan_num_ops",
@@ -106,6 +106,7 @@ def lib() -> ctypes.CDLL:
         "hoccl_layout_num_accesses": (i, [vp]),
         "hoccl_layout_get_access": (i, [vp, i, ctypes.POINTER(Access)]),
         "hoccl_layout_group_deps": (i, [vp, i, ctypes.POINTER(i), i]),
+        "hoccl_layout_group_ctas": (i, [vp, i]),
         "hoccl_layout_signature": (i, [vp, ctypes.POINTER(ctypes.c_uint64), i]),
         "hoccl_options_resolve": (i, [ctypes.POINTER(Options), ctypes.POINTER(Resolved)]),
     }
@@ -279,8 +280,8 @@ class Plan:
 
 
 class Layout:
-    """Host-only view of what a call over these addresses would run (hoccl_layout_build): `deps` of every group, all its accesses
-    and the signature of its graph.  `path`, `scratch` = (address, bytes) and params as a communicator gets them."""
+    """Host-only view of what a call over these addresses would run (hoccl_layout_build): `deps` of every group, the CTAs of its
+    largest launch (0: driver copies), all accesses and the signature of its graph.  `path`, `scratch` = (address, bytes) and params as a communicator gets them."""
 
     def __init__(self, kind, R, send, recv, count, dtype, path=_b.PATH_CE, scratch=None, **params):
         L = lib()
@@ -302,6 +303,7 @@ class Layout:
             buf = (ctypes.c_int * L.hoccl_layout_group_deps(h, g, None, 0))()
             L.hoccl_layout_group_deps(h, g, buf, len(buf))
             self.deps.append(list(buf))
+        self.ctas = [L.hoccl_layout_group_ctas(h, g) for g in range(len(self.deps))]
         self.accesses = []
         for k in range(L.hoccl_layout_num_accesses(h)):
             a = Access()

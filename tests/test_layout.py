@@ -148,3 +148,20 @@ def test_signature_of_handshake_mode(kind):
     graph need not be on the device yet when the proxy replays it behind a parked stream."""
     a, b = (lay_out(kind, 8, 4096, "bf16", path=hb.PATH_SM, handshake=mode)[0] for mode in (0, 1))
     assert _steps(a) == _steps(b) and a.signature != b.signature
+
+
+@pytest.mark.parametrize("sum_ctas", [147, 148, 296])
+@pytest.mark.parametrize("R", [2, 5, 8, 9, 16])
+@pytest.mark.parametrize("rs_direct", [1, 2])
+def test_whole_gpu_sums_leave_room_for_copies_beside_them(R, sum_ctas, rs_direct):
+    """Pieces on the copy route: a sum with another piece's driver copies beside it is one CTA per SM that walks its tiles; the first
+    piece's sum has none beside it when contributions are read in place, and neither has a sum that is not cut.  (Nine operands and
+    more have a CTA per tile in any case.)"""
+    for pieces in (0, 3):
+        lay, *_ = lay_out(ALLREDUCE, R, R * 3_000_000, "bf16", sum_ctas=sum_ctas, rs_direct=rs_direct, ce_overlap=pieces)
+        kind = {a.group: (a.kind, a.piece) for a in lay.accesses}
+        sums = [(kind[g][1], n) for g, n in enumerate(lay.ctas) if kind[g][0] == hd.OP_CHAIN]
+        assert len(sums) == max(1, pieces)
+        for piece, ctas in sums:
+            walks = sum_ctas < 148 or (pieces and R <= 8 and (piece > 0 or rs_direct == 1))
+            assert ctas == sum_ctas if walks else ctas > sum_ctas

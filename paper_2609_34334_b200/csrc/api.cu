@@ -378,6 +378,7 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
   if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && !modelled) {
     constexpr uint64_t kShortFlow = 9 << 19;   // 4.5 MiB
     uint64_t most = 0, flows = 0;
+    double ahead = 0;   // the CTAs that keep up with the driver, as a share of the bytes: see kernel_ahead_from
     bool bad = false;
     for (int u = 0; u < R; u++) {
       uint64_t out = 0, in = 0;
@@ -386,11 +387,14 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
         out += C[i];
         flows += C[i] != 0;
         in += C[(size_t)v * R + u];
-        bad = bad || bad_for_driver((const char*)send[u] + sdispls[i] * e, (const char*)recv[v] + rdispls[(size_t)v * R + u] * e, C[i]);
+        const char *src = (const char*)send[u] + sdispls[i] * e, *dst = (const char*)recv[v] + rdispls[(size_t)v * R + u] * e;
+        bad = bad || bad_for_driver(src, dst, C[i]);
+        ahead += (double)C[i] / kernel_ahead_from(src, dst, C[i]);
       }
       most = std::max(most, std::max(out, in));
     }
-    if (bad || most <= (uint64_t)c->ce_small_bytes || total <= flows * kShortFlow) route = HOCCL_PATH_SM;
+    const bool wide = c->ce_small_ctas >= kWideMoves || (double)c->ce_small_ctas * ahead >= (double)total;
+    if (most <= (uint64_t)c->ce_small_bytes || (wide && (bad || total <= flows * kShortFlow))) route = HOCCL_PATH_SM;
   }
   RouteGuard guard(c, route, route == c->path ? c->copy_ctas : c->ce_small_ctas);
   // A pattern that was issued before with the same buffers (same counts, displacements, pointers and settings) replays

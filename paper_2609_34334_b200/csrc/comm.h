@@ -221,6 +221,17 @@ inline bool bad_for_driver(const char* src, const char* dst, size_t bytes) {
   return bytes >= kDriverWhole && (bytes % kDriverPage || (uintptr_t)dst % kDriverLine || (((uintptr_t)src ^ (uintptr_t)dst) & 15));
 }
 
+// "ce_small_ctas" from which a launch of the move kernel carries copies no slower than the driver does; from kWideMoves on the rules of the
+// callers hold as they were measured, with 148.  A CTA copies 46 GB/s (one store per load; all-gathers 58), driver copies side by side whole ones at
+// 3.1 TB/s, with odd ends at 1.4, with ends that differ modulo 4 at 0.65, and none in less than 0.5 us.  Us in driver copies / on 16 / 32 / 64 CTAs: all-gather of
+// 64 MiB per rank over 8 ranks, whole 174 / 555 / 279 / 141, 16 bytes short per block 371 / 558 / 281 / 142, 2 bytes out of phase 816 / 559 / 282 / 144;
+// all-to-all of 16 MiB over 8 ranks 51 / 175 / 89 / 49, of 64 MiB 16 bytes short 384 / 722 / 362 / 190; over 64 ranks in blocks of 280 KB 1884 / 1673 / 919 / 579.
+constexpr long kWideMoves = 128;
+inline double kernel_ahead_from(const char* src, const char* dst, size_t bytes) {
+  const double copies = bad_for_driver(src, dst, bytes) ? ((((uintptr_t)src ^ (uintptr_t)dst) & 3) ? 16 : 32) : 64;
+  return std::max(1.0, std::min((double)bytes / 20e3, copies));
+}
+
 // The move route of one call: the communicator shows it for the call only.
 struct RouteGuard {
   hoccl_comm* c;

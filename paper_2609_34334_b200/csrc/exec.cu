@@ -842,21 +842,31 @@ hoccl_result_t check_options(hoccl_comm* c, int kind, size_t count, int dtype) {
 //     96; 256 MiB over 8 572 and 345).  Both take the whole GPU.
 //     Beside a loop of 8192^3 bf16 GEMMs a call of 25 MiB per rank over 8 ranks costs the GEMMs (median and quartiles) and takes meanwhile: all-gather
 //     25 us (5 to 37) and 0.13 ms, in driver copies 22 (4 to 37) and 0.24 ms; all-to-all 14 (-10 to 40) and 0.33 ms, 11 (-18 to 31) and 0.28 ms.
+// With "ce_small_ctas" below 128 only where that many CTAs keep up with the driver (kernel_ahead_from); long whole blocks of an all-to-all then stay
+// with it between any number of ranks (64 MiB over 2 ranks 45.7 us, on 64 CTAs 48.5, 96 46.4; over 4 88, 93, 91).
 static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t block = call.count * dtype_size(call.dtype);
-  if (block < kDriverShort || call.kind == PLAN_ALLGATHER || c->R <= 4) return true;
+  const bool wide = c->ce_small_ctas >= kWideMoves, few = block < kDriverShort || call.kind == PLAN_ALLGATHER;
+  if (wide && (few || c->R <= 4)) return true;
+  bool bad = false;
+  double ahead = 0;   // the mean of 1 / kernel_ahead_from
   for (int u = 0; u < c->R; u++)
-    for (int v = 0; v < c->R; v++)
-      if (bad_for_driver((const char*)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0), (const char*)call.recv[v] + (size_t)u * block, block))
-        return true;
-  return false;
+    for (int v = 0; v < c->R; v++) {
+      const char* src = (const char*)call.send[u] + (call.kind == PLAN_ALLTOALL ? (size_t)v * block : 0);
+      const char* dst = (const char*)call.recv[v] + (size_t)u * block;
+      bad = bad || bad_for_driver(src, dst, block);
+      if (wide && bad) return true;
+      ahead += 1 / kernel_ahead_from(src, dst, block) / ((double)c->R * c->R);
+    }
+  return !wide && (few || bad) && (double)c->ce_small_ctas * ahead >= 1;
 }
 
 // An all-reduce whose sums read the contributions in place and whose ring chunks the driver copies badly (not whole pages on 128-byte lines), or
 // are short copies (but for chunks of 1 to 1.17 MiB, 80 MB for all ranks, whose copies and ends the layout tests describe): its all-gather runs on the move kernel too, which reads a chunk once for all ranks.  Us in driver copies with their ends on the
 // kernel / on the kernel alone, bf16: R = 8, 16 MiB per rank 149.5 / 137.5, 64 MiB 554 / 527; R = 3, 32 MiB 174 / 155; R = 5, 32 MiB 221 / 203; R = 6, 64 MiB
 // 456 / 445; R = 16, 19 MiB 352 / 290, 64 MiB 1072 / 887.  A loop of 8192^3 GEMMs loses less to it as well (8 ranks, 64 MiB 97 us per
-// call, in driver copies 175).  Whole chunks stay with the driver, whose copies run beside the next piece's sum: 8 ranks 40 MiB 335 us, 320 on the kernel.
+// call, in driver copies 175).  Only with "ce_small_ctas" >= 128: on fewer it is even at best, R = 8 64 MiB driver 521 us, 8 CTAs 1027, 16 624, 40 515, 64 527;
+// R = 3 32 MiB 157, 216, 172, 165, 165 (148: 145).  Whole chunks stay with the driver, whose copies run beside the next piece's sum: 8 ranks 40 MiB 335 us, 320 on the kernel.
 static bool chunks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t S = call.count * dtype_size(call.dtype), chunk = (call.count + c->R - 1) / c->R * dtype_size(call.dtype);
   if (chunk >= kDriverWhole && chunk < ((size_t)1200 << 10) && (size_t)c->R * S < 80000000) return false;
@@ -872,7 +882,7 @@ static hoccl_result_t call_options(hoccl_comm* c, const Call& call, OptionsOut* 
   if (may_switch && (call.kind == PLAN_ALLGATHER || call.kind == PLAN_ALLTOALL) && blocks_bad_for_driver(c, call)) oin.ce_small_bytes = LONG_MAX;
   const hoccl_result_t rc = resolve_options(oin, opt);
   if (rc == HOCCL_OK && may_switch && call.kind == PLAN_ALLREDUCE && opt->path == HOCCL_PATH_CE && opt->executor == EXEC_GRAPH && c->ag_direct == 2 &&
-      c->ce_overlap < 0 && !c->piece_bytes_set && c->sum_ctas < 64 && !call.h_send && chunks_bad_for_driver(c, call) &&
+      c->ce_overlap < 0 && !c->piece_bytes_set && c->sum_ctas < 64 && c->ce_small_ctas >= kWideMoves && !call.h_send && chunks_bad_for_driver(c, call) &&
       contributions(c, call, *opt, call.count * dtype_size(call.dtype)) == READ_IN_PLACE) {
     oin.ce_small_bytes = LONG_MAX;
     return resolve_options(oin, opt);

@@ -124,7 +124,11 @@ hoccl_result_t p2p_post(hoccl_comm* c, bool is_send, void* buf, size_t count, in
     nsplit = std::max(1, std::min<int>(nsplit, kMaxLanes));
   }
   // Short messages, and those the driver copies badly, go to the move kernel as in the collectives ("ce_small_bytes").
-  const bool by_kernel = c->path == HOCCL_PATH_SM || (c->ce_small_bytes > 0 && (bytes <= (size_t)c->ce_small_bytes || bad_for_driver((const char*)sbuf, (const char*)dbuf, bytes)));
+  // Of the latter those that "ce_small_ctas" CTAs carry in the driver's time: 46 GB/s each against 2.7 TB/s and 4 us (half that if the ends differ
+  // modulo 4): 64 MiB with an odd end 28.7 us in a driver copy, 177 on 8 CTAs.
+  const double driver_us = 4 + (double)bytes / ((((uintptr_t)sbuf ^ (uintptr_t)dbuf) & 3) ? 1.35e6 : 2.7e6);
+  const bool keeps_up = c->ce_small_ctas >= kWideMoves || (double)bytes <= 46e3 * (double)c->ce_small_ctas * driver_us;
+  const bool by_kernel = c->path == HOCCL_PATH_SM || (c->ce_small_bytes > 0 && (bytes <= (size_t)c->ce_small_bytes || (keeps_up && bad_for_driver((const char*)sbuf, (const char*)dbuf, bytes))));
   const int ctas = (int)(c->path == HOCCL_PATH_SM ? c->copy_ctas : c->ce_small_ctas);
   auto move = [&](const char* from, char* to, size_t n, cudaStream_t on) {
     if (!by_kernel) return cudaMemcpyAsync(to, from, n, cudaMemcpyDeviceToDevice, on);

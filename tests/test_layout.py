@@ -165,3 +165,20 @@ def test_whole_gpu_sums_leave_room_for_copies_beside_them(R, sum_ctas, rs_direct
         for piece, ctas in sums:
             walks = sum_ctas < 148 or (pieces and R <= 8 and (piece > 0 or rs_direct == 1))
             assert ctas == sum_ctas if walks else ctas > sum_ctas
+
+
+# (call, ranks, elements, buffer offset of every second rank) -> "ce_small_ctas" from which its moves are on the kernel; 0: never
+@pytest.mark.parametrize("kind, R, count, off, line", [
+    (ALLREDUCE, 8, 33_554_424, 0, 128), (ALLREDUCE, 3, 16_777_216, 0, 128),        # ragged chunks
+    (ALLREDUCE, 8, 33_554_432, 0, 0),                                              # whole ones
+    (ALLGATHER, 8, 4_194_304, 0, 64), (ALLGATHER, 2, 16_777_216, 0, 64),           # whole blocks
+    (ALLGATHER, 8, 4_194_296, 0, 32), (ALLTOALL, 8, 4_194_296, 0, 32),             # odd ends
+    (ALLTOALL, 8, 4_194_304, 2, 24),                                               # a quarter whole, a quarter odd, half out of phase: 4 / (1/64 + 1/32 + 2/16) = 23.3
+    (ALLTOALL, 8, 1_048_576, 0, 64), (ALLTOALL, 32, 300_000, 0, 30),               # short blocks
+    (ALLTOALL, 2, 16_777_216, 0, 128), (ALLTOALL, 8, 4_194_304, 0, 0),             # long whole ones
+])
+def test_moves_leave_the_driver_where_the_kernel_has_the_ctas_to_keep_up(kind, R, count, off, line):
+    for ctas in (1, 8, 15, 16, 24, 29, 30, 31, 32, 40, 63, 64, 96, 127, 128, 148):
+        lay, *_ = lay_out(kind, R, count, "bf16", offs=[off * (r % 2) for r in range(R)], ce_small_ctas=ctas)
+        moves = [n for g, n in enumerate(lay.ctas) if any(a.group == g and a.kind == hd.OP_MOVE and not a.edges for a in lay.accesses)]
+        assert moves and (all(moves) if line and ctas >= line else not any(moves)), ctas

@@ -1033,6 +1033,10 @@ int hoccl_layout_group_ctas(hoccl_layout_t l, int group) {
   return l && group >= 0 && group < (int)l->lay.ctas.size() ? l->lay.ctas[(size_t)group] : -1;
 }
 
+int hoccl_layout_copy_chains(hoccl_layout_t l, int piece) {
+  return l && piece >= 0 && piece < (int)l->lay.chains.size() ? l->lay.chains[(size_t)piece] : 0;
+}
+
 int hoccl_layout_signature(hoccl_layout_t l, uint64_t* words, int cap) {
   if (!l) return 0;
   for (int i = 0; i < (int)l->key.size() && words && i < cap; i++) words[i] = l->key[(size_t)i];

@@ -210,7 +210,8 @@ struct Layout {
   std::vector<RGroup> groups;
   size_t host_need = 0;   // bytes of pinned host staging the moves bounce through (HOCCL_PATH_CE_HOST)
   bool overlap = false;   // copy route: the pieces' parts run on three internal streams
-  std::vector<int> ctas;  // inspect_call only: per group, the CTAs of its largest kernel launch, 0 = driver copies
+  // inspect_call only: per group, the CTAs of its largest kernel launch (0 = driver copies); per piece, copy_chains
+  std::vector<int> ctas, chains;
 };
 
 // What a driver copy inside one device does at once, as timed on B200: a copy of 1 MiB or more whose destination does not start on a
@@ -278,6 +279,9 @@ bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<
 // kernel follows another in 0.65 us, so longer chains, and calls with something to overlap, lose nothing there.)
 constexpr size_t kMaxChainLaunches = 3;
 void add_launches(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry);
+// In how many chains the copies of this piece's all-gather run beside the next piece's sum; 0: all at once.
+constexpr size_t kMaxCopyChains = 6;
+size_t copy_chains(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, int piece);
 // part < 0: every group (of `only_piece`, if that is >= 0); part 0 / 1 / 2: only the reduce-scatter's MOVE groups / the SUM and
 // CHAIN groups / the remaining MOVE groups; dependencies on groups outside the part are left to the caller (events).
 // *out_exec stays null when nothing falls into the selection.

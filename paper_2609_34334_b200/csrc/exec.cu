@@ -1042,6 +1042,7 @@ hoccl_result_t inspect_call(hoccl_comm* c, Call* call, Layout* out, std::vector<
     if (g.kind == OP_MOVE && c->path != HOCCL_PATH_SM && !g.edges) continue;
     for (const KernelLaunch& k : kernel_launches(c, out->plan, g)) out->ctas.back() = std::max(out->ctas.back(), k.grid);
   }
+  for (int p = 0; p < out->plan.pieces; p++) out->chains.push_back(out->overlap ? (int)copy_chains(c, out->plan, out->groups, p) : 0);
   return rc;
 }
 

@@ -87,6 +87,32 @@ void add_launches(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>&
   if (all.size() <= kMaxChainLaunches) entry->launches.swap(all);
 }
 
+// Copies that run beside another piece's sum ("ce_overlap", every piece's but the last) are spread over a few chains: all at once they take HBM to
+// 4.6 TB/s, and the sum slows down from 3 TB/s on.  In a chain a copy waits for the one before and takes 3 us and 1.8 per MiB, so that pays
+// while the sum lasts three quarters of that and copies are of 1 MiB or more; short ones have nothing left of the 3 us.  Us at once / in six
+// chains, bf16, by SUM CTAs: 8 ranks 40 MiB 8 340.8 / 340.0, 16 205.6 / 201.1, 20 184.4 / 185.3, 24 169 / 183, 32 152 / 180; 64 MiB 8 531 / 519, 16 318 / 312, 24 258 /
+// 265, 48 224 / 263; 256 MiB 8 2071 / 2034, 20 1054 / 1043, 28 902 / 911, 48 875 / 915; 16 ranks 64 MiB 8 959 / 941, 16 596 / 596, 24 494 / 555.  40 MiB, 8 CTAs, in 6
+// pieces (0.8 MiB a copy) 355 / 368, in 12 371 / 409; 64 MiB in 6 544 / 531, in 12 572 / 575; contributions staged, 40 MiB 421 / 413.  Few copies (2 to 6 ranks)
+// differ by less than 1 % either way.  A ring all-gather's steps wait for one another as it is.
+size_t copy_chains(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, int piece) {
+  constexpr size_t kCopyChains = kMaxCopyChains;
+  if (piece < 0 || piece + 1 >= P.pieces || c->sum_ctas >= 64) return 0;
+  double copies = 0, copied = 0, summed = 0;
+  for (const RGroup& g : groups) {
+    if (g.kind == OP_CHAIN && g.piece == piece + 1)
+      for (const Seg& s : g.segs) summed += (double)(c->R + 1) * (double)s.bytes;
+    if (g.kind != OP_MOVE || g.phase == PHASE_RS || g.edges || g.piece != piece) continue;
+    for (int d : g.deps)
+      if (groups[(size_t)d].kind == OP_MOVE) return 0;
+    for (const Seg& s : g.segs) {
+      copies++;
+      copied += (double)s.bytes;
+    }
+  }
+  const double chained_us = copies / kCopyChains * (3 + copied / std::max(1.0, copies) / 580e3), sum_us = summed / (160e3 * (double)c->sum_ctas);
+  return copied >= copies * (double)kDriverWhole && sum_us >= 0.75 * chained_us ? kCopyChains : 0;
+}
+
 // only_piece >= 0 builds the graph of that piece alone (dependencies never cross pieces) and stores it in *out_exec.
 hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry, int only_piece,
                            cudaGraphExec_t* out_exec, int part) {
@@ -150,8 +176,8 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
     }
   }
   std::vector<cudaGraphNode_t> terminal_nodes;
-  constexpr size_t kCopyChains = 6;
-  cudaGraphNode_t chain_tail[kCopyChains] = {};
+  const size_t chains = part == 2 ? copy_chains(c, P, groups, only_piece) : 0;
+  cudaGraphNode_t chain_tail[kMaxCopyChains] = {};
   size_t chain_next = 0;
   hoccl_result_t rc = HOCCL_OK;
   auto fail = [&](cudaError_t e, const char* what) {
@@ -233,11 +259,7 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
       }
     } else if (c->path == HOCCL_PATH_CE && !rg.edges) {
       for (const Seg& sg : rg.segs) {
-        // Copies that run beside another piece's sum ("ce_overlap", every piece's but the last) are spread over a few chains: all at once they take
-        // HBM to 4.6 TB/s, and the sum slows down from 3 TB/s on (4 pieces of 40 MiB per rank over 8 ranks 342.3 us, six chains 335.4, three 340).
-        // A ring all-gather's steps wait for one another as it is.
-        const bool beside_sums = part == 2 && only_piece + 1 < P.pieces && c->sum_ctas < 64 && inner_deps(gi) == 0;
-        cudaGraphNode_t* chain = beside_sums ? &chain_tail[chain_next++ % kCopyChains] : nullptr;
+        cudaGraphNode_t* chain = chains ? &chain_tail[chain_next++ % chains] : nullptr;
         // optional sub-copies: driver copies of 4-8 MiB pay a ~4 us serialised start-up that smaller ones do not
         size_t sub = sg.bytes;
         if (c->ce_sub_bytes > 0 && sg.bytes > (size_t)c->ce_sub_bytes && sg.bytes < ((size_t)16 << 20))

@@ -182,3 +182,15 @@ def test_moves_leave_the_driver_where_the_kernel_has_the_ctas_to_keep_up(kind, R
         lay, *_ = lay_out(kind, R, count, "bf16", offs=[off * (r % 2) for r in range(R)], ce_small_ctas=ctas)
         moves = [n for g, n in enumerate(lay.ctas) if any(a.group == g and a.kind == hd.OP_MOVE and not a.edges for a in lay.accesses)]
         assert moves and (all(moves) if line and ctas >= line else not any(moves)), ctas
+
+
+@pytest.mark.parametrize("R, count, params, chained", [
+    (8, 20_971_520, {}, True), (8, 20_971_520, {"sum_ctas": 16}, True), (8, 134_217_728, {}, True), (8, 20_971_520, {"rs_direct": 1}, True),
+    (8, 20_971_520, {"sum_ctas": 24}, False), (8, 20_971_520, {"sum_ctas": 48}, False), (8, 20_971_520, {"sum_ctas": 148, "ce_overlap": 4}, False),
+    (8, 20_971_520, {"ce_overlap": 6}, False), (8, 20_971_520, {"ce_overlap": 16}, False), (8, 20_971_520, {"rs_direct": 1, "ce_overlap": 8}, False),
+    (8, 134_217_728, {"sum_ctas": 48}, False), (8, 33_554_432, {"ce_overlap": 4}, True), (8, 20_971_520, {"ag_direct": 0}, False),
+    (16, 33_554_432, {}, True), (16, 33_554_432, {"sum_ctas": 24}, False), (16, 33_554_432, {"ce_overlap": 6}, False), (8, 20_971_520, {"ce_overlap": 0}, False),
+])
+def test_copies_in_chains_where_the_sum_beside_them_lasts_as_long(R, count, params, chained):
+    lay, *_ = lay_out(ALLREDUCE, R, count, "bf16", **params)
+    assert lay.chains == [6 if chained else 0] * (lay.num_pieces - 1) + [0]

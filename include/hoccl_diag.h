@@ -246,6 +246,8 @@ hoccl_result_t hoccl_layout_get_access(hoccl_layout_t layout, int index, hoccl_a
 int hoccl_layout_group_deps(hoccl_layout_t layout, int group, int* deps, int cap);
 /* CTAs of the largest kernel launch that carries `group` out, as a graph of kernels; 0: driver copies (-1: no such group). */
 int hoccl_layout_group_ctas(hoccl_layout_t layout, int group);
+/* 1: the call runs in pieces on three internal streams ("ce_overlap") and its sums are launched, not replayed as graphs. */
+int hoccl_layout_sums_by_launch(hoccl_layout_t layout);
 /* In how many chains the driver copies of this piece's all-gather run beside the next piece's sum ("ce_overlap"); 0: all at once, or not so. */
 int hoccl_layout_copy_chains(hoccl_layout_t layout, int piece);
 /* The words under which the call's graph is cached: calls with the same words replay the same graph.  Writes up to `cap`, returns

@@ -1033,6 +1033,8 @@ int hoccl_layout_group_ctas(hoccl_layout_t l, int group) {
   return l && group >= 0 && group < (int)l->lay.ctas.size() ? l->lay.ctas[(size_t)group] : -1;
 }
 
+int hoccl_layout_sums_by_launch(hoccl_layout_t l) { return l && l->lay.sums_by_launch ? 1 : 0; }
+
 int hoccl_layout_copy_chains(hoccl_layout_t l, int piece) {
   return l && piece >= 0 && piece < (int)l->lay.chains.size() ? l->lay.chains[(size_t)piece] : 0;
 }

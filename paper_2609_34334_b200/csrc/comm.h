@@ -101,7 +101,7 @@ struct GraphEntry {
   // "ce_overlap" setting: per piece three graphs (the reduce-scatter's moves, the sum, the all-gather's moves) that run on three
   // internal streams, so that one piece's driver copies overlap another piece's sum (inside ONE graph they never did)
   std::vector<cudaGraphExec_t> part_exec;   // [piece * 3 + part], null where a part is empty
-  std::vector<std::vector<KernelLaunch>> part_sums;   // [piece]: the sums as launches instead of a graph, unless "profile" is set
+  std::vector<std::vector<KernelLaunch>> part_sums;   // [piece]: the sums as launches instead of a graph (Layout::sums_by_launch)
   // "fused" setting: the whole plan as one cooperative kernel instead of a graph (exec stays null)
   std::vector<char> ring_args;  // a RingArgsSmall or RingArgsLarge, by value
   bool ring_large = false;
@@ -210,6 +210,7 @@ struct Layout {
   std::vector<RGroup> groups;
   size_t host_need = 0;   // bytes of pinned host staging the moves bounce through (HOCCL_PATH_CE_HOST)
   bool overlap = false;   // copy route: the pieces' parts run on three internal streams
+  bool sums_by_launch = false;   // of those the sums go out as launches, not as graphs
   // inspect_call only: per group, the CTAs of its largest kernel launch (0 = driver copies); per piece, copy_chains
   std::vector<int> ctas, chains;
 };

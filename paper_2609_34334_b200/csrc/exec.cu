@@ -1019,6 +1019,12 @@ static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut&
   }
   out->overlap = overlap && P.pieces > 1;   // with one piece there is nothing to overlap
   resolve(c, P, call, how, &out->groups, &out->host_need);
+  // A sum that is launched starts on time behind another piece's (see launch_in_order).  That helps where the sums are the longer part and run back
+  // to back, on few CTAs with the contributions read in place; sums of the whole GPU take the SMs that another piece's copies were waiting for,
+  // and staged ones wait for copies of their own.  Us as launches / as graphs, bf16: 8 SUM CTAs R = 8 40 MiB 333 / 340, 256 MiB 2028 / 2046, R = 16
+  // 256 MiB 3644 / 3672; 148 R = 2 128 MiB 142 / 121, R = 8 40 MiB in 4 pieces 159.9 / 157.9; staged, 148, R = 2 175 / 165, R = 4 64 MiB 186.5 / 183.2, R = 8 40 MiB 255 / 244,
+  // 256 MiB 1543 / 1512; staged, 8, R = 8 40 MiB 417.5 / 412.6.
+  out->sums_by_launch = out->overlap && !c->profile && how != STAGED && c->sum_ctas < 64;
   for (RGroup& g : out->groups) {
     if (beside && g.kind == OP_MOVE && g.piece + 1 < P.pieces) g.ctas = kBesideSums;
     // the first piece's sum has nothing beside it unless the next piece's contributions are copied meanwhile
@@ -1158,7 +1164,7 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
       }
     } else if (lay.overlap) {
       entry.part_exec.assign((size_t)P.pieces * 3, nullptr);
-      if (!c->profile) {   // (a piece's sums behind another's start on time as launches, see launch_in_order: 4 pieces of 40 MiB 345.8 -> 342.3 us)
+      if (lay.sums_by_launch) {
         entry.part_sums.resize((size_t)P.pieces);
         for (const RGroup& g : groups)
           if (g.kind != OP_MOVE)
@@ -1169,7 +1175,7 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
       }
       for (int p = 0; p < P.pieces && rc == HOCCL_OK; p++)
         for (int part = 0; part < 3 && rc == HOCCL_OK; part++)
-          if (part != 1 || c->profile) rc = build_graph(c, P, groups, &entry, p, &entry.part_exec[(size_t)p * 3 + part], part);
+          if (part != 1 || !lay.sums_by_launch) rc = build_graph(c, P, groups, &entry, p, &entry.part_exec[(size_t)p * 3 + part], part);
       if (rc != HOCCL_OK) {
         destroy_entry(&entry);
         return rc;

@@ -929,9 +929,10 @@ static ChainVariant chain_tile_variant(int nops, bool fan) {
   else return fan ? fan_of<DT, N, N <= 3 ? 2 : 1, 256>() : wide_of<DT, N, N <= 3 ? 2 : 1, 256>();
 }
 // A whole-GPU sum with driver copies of another piece beside it: one CTA per SM that walks the tiles, as between 128 CTAs and all SMs.  A CTA per tile
-// takes every slot that comes free and the copies wait.  Us of an all-reduce on the copy route, 148 SUM CTAs, bf16, a CTA per tile / the walk: R = 8 256 MiB
-// in 8 pieces 902 / 884, 1 GiB 3940 / 3854; R = 4 128 MiB 250.8 / 243.2; R = 3 200 MB 285.2 / 279.8; R = 2 128 MiB 143 / 127.  Nine operands and more have no
-// compiled walk, and chain_kernel's tables cost more than the crowding (R = 16, 256 MiB 2070 / 2084).
+// takes every slot that comes free and the copies wait.  Us of an all-reduce on the copy route, 148 SUM CTAs, bf16, a CTA per tile / the walk from the second
+// piece on: R = 8 40 MiB in 4 pieces 164.6 / 157.9, 1 GiB in 8 3945 / 3858; R = 4 64 MiB 128.0 / 125.1; R = 2 128 MiB 144.5 / 121.0; staged, R = 8 40 MiB 250.8 / 244.1,
+// R = 2 128 MiB 174.9 / 165.1.  Nine operands and more have no compiled walk, and chain_kernel's tables cost more than the crowding (R = 16, 256 MiB 2070 /
+// 2084).
 static bool chain_walks(const ChainBatch& b) { return b.walk && b.nseg > 0 && b.seg[0].nops <= 8; }
 static ChainVariant chain_variant(const ChainBatch& b, int ctas) {
   ChainVariant plain{b.dtype == 0 ? reinterpret_cast<const void*>(&chain_kernel<0, 1024>) : reinterpret_cast<const void*>(&chain_kernel<1, 1024>), 1024, 1024};

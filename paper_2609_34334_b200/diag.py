@@ -17,7 +17,7 @@ EXEC_GRAPH, EXEC_STREAMS, EXEC_ONE_KERNEL, EXEC_ONEPASS, EXEC_PROXY, EXEC_ROLES 
 EXPORTS = [   # every function include/hoccl_diag.h declares
     "hoccl_chain_launch", "hoccl_comm_init_host_only", "hoccl_copy_launch", "hoccl_fanout_inspect", "hoccl_fanout_launch", "hoccl_flatten_inspect",
     "hoccl_kernel_preloaded", "hoccl_kernel_sms", "hoccl_layout_build", "hoccl_layout_copy_chains", "hoccl_layout_destroy", "hoccl_layout_get_access", "hoccl_layout_group_ctas", "hoccl_layout_group_deps",
-    "hoccl_layout_num_accesses", "hoccl_layout_num_groups", "hoccl_layout_num_pieces", "hoccl_layout_signature", "hoccl_move_inspect",
+    "hoccl_layout_num_accesses", "hoccl_layout_num_groups", "hoccl_layout_num_pieces", "hoccl_layout_signature", "hoccl_layout_sums_by_launch", "hoccl_move_inspect",
     "hoccl_options_resolve", "hoccl_plan_build", "hoccl_plan_destroy", "hoccl_plan_get_op",
     "hoccl_plan_group_deps", "hoccl_plan_inbox_slots", "hoccl_plan_num_groups", "hoccl_plan_num_ops",
     "hoccl_plan_scratch_bytes", "hoccl_plan_slot_bytes", "hoccl_port_probe", "hoccl_probe_copy_routes",
@@ -108,6 +108,7 @@ def lib() -> ctypes.CDLL:
         "hoccl_layout_group_deps": (i, [vp, i, ctypes.POINTER(i), i]),
         "hoccl_layout_group_ctas": (i, [vp, i]),
         "hoccl_layout_copy_chains": (i, [vp, i]),
+        "hoccl_layout_sums_by_launch": (i, [vp]),
         "hoccl_layout_signature": (i, [vp, ctypes.POINTER(ctypes.c_uint64), i]),
         "hoccl_options_resolve": (i, [ctypes.POINTER(Options), ctypes.POINTER(Resolved)]),
     }
@@ -305,6 +306,7 @@ class Layout:
             L.hoccl_layout_group_deps(h, g, buf, len(buf))
             self.deps.append(list(buf))
         self.ctas = [L.hoccl_layout_group_ctas(h, g) for g in range(len(self.deps))]
+        self.sums_by_launch = bool(L.hoccl_layout_sums_by_launch(h))
         self.chains = [L.hoccl_layout_copy_chains(h, p) for p in range(self.num_pieces)]
         self.accesses = []
         for k in range(L.hoccl_layout_num_accesses(h)):

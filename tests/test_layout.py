@@ -194,3 +194,12 @@ def test_moves_leave_the_driver_where_the_kernel_has_the_ctas_to_keep_up(kind, R
 def test_copies_in_chains_where_the_sum_beside_them_lasts_as_long(R, count, params, chained):
     lay, *_ = lay_out(ALLREDUCE, R, count, "bf16", **params)
     assert lay.chains == [6 if chained else 0] * (lay.num_pieces - 1) + [0]
+
+
+@pytest.mark.parametrize("R, params, launched", [
+    (8, {}, True), (16, {}, True), (8, {"sum_ctas": 48}, True), (8, {"rs_direct": 1}, False), (8, {"sum_ctas": 64}, False),
+    (8, {"sum_ctas": 148, "ce_overlap": 4}, False), (2, {"sum_ctas": 148, "ce_overlap": 4}, False), (8, {"profile": 1}, False), (8, {"ce_overlap": 0}, False),
+])
+def test_sums_launched_where_they_run_back_to_back(R, params, launched):
+    lay, *_ = lay_out(ALLREDUCE, R, 20_971_520 // 8 * R, "bf16", **params)
+    assert lay.sums_by_launch == launched

@@ -93,7 +93,7 @@ void add_launches(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>&
 // chains, bf16, by SUM CTAs: 8 ranks 40 MiB 8 340.8 / 340.0, 16 205.6 / 201.1, 20 184.4 / 185.3, 24 169 / 183, 32 152 / 180; 64 MiB 8 531 / 519, 16 318 / 312, 24 258 /
 // 265, 48 224 / 263; 256 MiB 8 2071 / 2034, 20 1054 / 1043, 28 902 / 911, 48 875 / 915; 16 ranks 64 MiB 8 959 / 941, 16 596 / 596, 24 494 / 555.  40 MiB, 8 CTAs, in 6
 // pieces (0.8 MiB a copy) 355 / 368, in 12 371 / 409; 64 MiB in 6 544 / 531, in 12 572 / 575; contributions staged, 40 MiB 421 / 413.  Few copies (2 to 6 ranks)
-// differ by less than 1 % either way.  A ring all-gather's steps wait for one another as it is.
+// differ by less than 1 % either way.  Copies with odd ends take 4 us longer each, also in a chain: 48 MiB and 14 bytes, staged, 586 / 622.  A ring all-gather's steps wait for one another as it is.
 size_t copy_chains(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, int piece) {
   constexpr size_t kCopyChains = kMaxCopyChains;
   if (piece < 0 || piece + 1 >= P.pieces || c->sum_ctas >= 64) return 0;
@@ -105,6 +105,7 @@ size_t copy_chains(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>
     for (int d : g.deps)
       if (groups[(size_t)d].kind == OP_MOVE) return 0;
     for (const Seg& s : g.segs) {
+      if (bad_for_driver(s.src, s.dst, s.bytes)) return 0;
       copies++;
       copied += (double)s.bytes;
     }

@@ -189,6 +189,7 @@ def test_moves_leave_the_driver_where_the_kernel_has_the_ctas_to_keep_up(kind, R
     (8, 20_971_520, {"sum_ctas": 24}, False), (8, 20_971_520, {"sum_ctas": 48}, False), (8, 20_971_520, {"sum_ctas": 148, "ce_overlap": 4}, False),
     (8, 20_971_520, {"ce_overlap": 6}, False), (8, 20_971_520, {"ce_overlap": 16}, False), (8, 20_971_520, {"rs_direct": 1, "ce_overlap": 8}, False),
     (8, 134_217_728, {"sum_ctas": 48}, False), (8, 33_554_432, {"ce_overlap": 4}, True), (8, 20_971_520, {"ag_direct": 0}, False),
+    (8, 25_165_831, {"rs_direct": 1}, False), (8, 25_165_831, {"ce_small_ctas": 8}, True), (8, 25_165_831, {"ce_small_bytes": 0}, False),
     (16, 33_554_432, {}, True), (16, 33_554_432, {"sum_ctas": 24}, False), (16, 33_554_432, {"ce_overlap": 6}, False), (8, 20_971_520, {"ce_overlap": 0}, False),
 ])
 def test_copies_in_chains_where_the_sum_beside_them_lasts_as_long(R, count, params, chained):

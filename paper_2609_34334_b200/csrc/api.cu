@@ -498,8 +498,8 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
                                          (size_t)chunk_bytes, (size_t)c->model_rdma_sub_bytes, &entry);
     } else {
       entry.n_pieces = 1;
+      add_launches(c, P, &groups, &entry);
       grc = build_graph(c, P, groups, &entry, -1, &entry.exec);
-      if (grc == HOCCL_OK) add_launches(c, P, groups, &entry);
     }
     if (grc != HOCCL_OK) return grc;
     return launch_entry(c, cache_put(c, std::move(entry)), user, t0);

@@ -279,7 +279,8 @@ bool build_fan_batches(const RGroup& g, std::vector<FanBatch>* out, std::vector<
 // Fills entry->launches and est_us if the groups are at most kMaxChainLaunches kernels, each waiting for the one before it.  (Inside a graph a
 // kernel follows another in 0.65 us, so longer chains, and calls with something to overlap, lose nothing there.)
 constexpr size_t kMaxChainLaunches = 3;
-void add_launches(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry);
+// They stay in the groups (`ready`) for the graph that is built of them next: made twice they cost a first call up to 45 us of 240 (16 ranks).
+void add_launches(const hoccl_comm* c, const Plan& P, std::vector<RGroup>* groups, GraphEntry* entry);
 // In how many chains the copies of this piece's all-gather run beside the next piece's sum; 0: all at once.
 constexpr size_t kMaxCopyChains = 6;
 size_t copy_chains(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, int piece);

@@ -1184,8 +1184,8 @@ hoccl_result_t run_collective(hoccl_comm* c, Call* call, cudaStream_t user) {
       rc = fused ? build_ring(c, P, groups, &entry) : roles ? build_roles(c, P, groups, &entry) : HOCCL_ERR_UNSUPPORTED;
       // not asked for, too many ranks for one launch (fused), or more CTAs than can be resident together (roles)
       if (rc == HOCCL_ERR_UNSUPPORTED) {
+        add_launches(c, P, &lay.groups, &entry);
         rc = build_graph(c, P, groups, &entry, -1, &entry.exec);
-        if (rc == HOCCL_OK) add_launches(c, P, groups, &entry);
       }
       if (rc != HOCCL_OK) {
         destroy_entry(&entry);

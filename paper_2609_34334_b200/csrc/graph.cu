@@ -71,14 +71,15 @@ static cudaKernelNodeParams node_params(const KernelLaunch& k, void** args) {
   return kp;
 }
 
-void add_launches(const hoccl_comm* c, const Plan& P, const std::vector<RGroup>& groups, GraphEntry* entry) {
-  if (c->profile || c->handshake || groups.size() > kMaxChainLaunches) return;
+void add_launches(const hoccl_comm* c, const Plan& P, std::vector<RGroup>* groups, GraphEntry* entry) {
+  if (c->profile || c->handshake || groups->size() > kMaxChainLaunches) return;
   std::vector<KernelLaunch> all;
-  for (size_t g = 0; g < groups.size(); g++) {
-    const RGroup& rg = groups[g];
+  for (size_t g = 0; g < groups->size(); g++) {
+    RGroup& rg = (*groups)[g];
     if (rg.kind == OP_MOVE && c->path != HOCCL_PATH_SM) return;
     if (g > 0 && rg.chain_dep != (int)g - 1 && std::find(rg.deps.begin(), rg.deps.end(), (int)g - 1) == rg.deps.end()) return;
-    for (KernelLaunch& k : kernel_launches(c, P, rg)) {
+    if (rg.ready.empty()) rg.ready = kernel_launches(c, P, rg);
+    for (KernelLaunch k : rg.ready) {
       if (rg.kind != OP_MOVE) k.priority = c->sum_priority;
       entry->est_us += (rg.kind == OP_MOVE ? 2.5 : 1.5) + std::max(k.bytes / 6e6, k.bytes / k.grid / (rg.kind == OP_MOVE ? 45e3 : 90e3));
       all.push_back(std::move(k));
@@ -229,7 +230,8 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
       deps.push_back(root);
     }
     if (rg.kind == OP_SUM || rg.kind == OP_CHAIN) {
-      for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
+      std::vector<KernelLaunch> fresh;
+      for (const KernelLaunch& k : rg.ready.empty() ? fresh = kernel_launches(c, P, rg) : rg.ready) {
         const cudaKernelNodeParams kp = node_params(k, args);
         // launches of one group are chained too (they share the SM budget)
         std::vector<cudaGraphNode_t> d2 = nodes.empty() ? deps : std::vector<cudaGraphNode_t>{nodes.back()};
@@ -295,7 +297,8 @@ hoccl_result_t build_graph(hoccl_comm* c, const Plan& P, const std::vector<RGrou
         entry->n_moves++;
       }
     } else {
-      for (const KernelLaunch& k : kernel_launches(c, P, rg)) {
+      std::vector<KernelLaunch> fresh;
+      for (const KernelLaunch& k : rg.ready.empty() ? fresh = kernel_launches(c, P, rg) : rg.ready) {
         const cudaKernelNodeParams kp = node_params(k, args);
         // copy launches are chained as well: the CTA budget for copies is global, two never run at the same time
         std::vector<cudaGraphNode_t> d2 = deps;

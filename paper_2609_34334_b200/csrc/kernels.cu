@@ -458,13 +458,15 @@ __global__ void __launch_bounds__(THREADS, 1) chain_fan_kernel(const __grid_cons
 // See StoreAllArgs.  Latency bound: one fetch of parameters, one round trip of loads, one of stores.  Us per call in a burst, against chain_kernel's tables
 // and 8 operands at a time: 16 ranks bf16 on 8 CTAs 4 KiB per rank 6.1 -> 4.1, 8.1 KiB (heads and tails) 10.25 -> 4.15, 192 KiB 12.3 -> 9.5; 9 ranks fp32 64
 // KiB 8.2 -> 4.4; whole GPU 16 ranks 1 MiB 10.2 -> 5.0, 8 ranks 1 MiB (chain_fan_kernel) 6.1 -> 4.1.
-template <int DT, int NOPS, int THREADS>
+// SPLIT: several chunks per CTA.  A form of its own: with both in one, three divisions by arguments stand before the first load instead of one, and
+// calls that just end within a step of 2.048 us (see launch_in_order) need two (2 ranks bf16 16 KiB 2.4 us a call in a burst, 4.1 so).
+template <int DT, int NOPS, int THREADS, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1) store_all_kernel(const __grid_constant__ StoreAllArgs a) {
   using T = Traits<DT>;
-  const unsigned width = THREADS / a.groups, group = threadIdx.x / width, tid = threadIdx.x - group * width;
-  const unsigned unit = blockIdx.x * a.groups + group, c = unit / a.parts, part = unit - c * a.parts;
+  const unsigned width = SPLIT ? THREADS / a.groups : THREADS, group = SPLIT ? threadIdx.x / width : 0, tid = threadIdx.x - group * width;
+  const unsigned c = SPLIT ? blockIdx.x * a.groups + group : blockIdx.x / a.parts, part = SPLIT ? 0 : blockIdx.x - c * a.parts;
   wait_for_stream();
-  if (c >= NOPS) return;   // the last CTA of a grid that the chunks do not fill
+  if (SPLIT && c >= NOPS) return;   // the last CTA of a grid that the chunks do not fill
   const char* src[NOPS];
 #pragma unroll
   for (int j = 0; j < NOPS; j++) src[j] = static_cast<const char*>(a.x[(c + 1 + j) % NOPS]);
@@ -974,16 +976,14 @@ void prepare_chain_batch(ChainBatch* b, int ctas) {
 }
 
 template <int DT, int R>
-static const void* store_all_from(int r) {
-  if constexpr (R <= kMaxStoreAllRanks) return r == R ? reinterpret_cast<const void*>(&store_all_kernel<DT, R, 512>) : store_all_from<DT, R + 1>(r);
-  else return nullptr;
+static const void* store_all_from(int r, bool split) {
+  if constexpr (R > kMaxStoreAllRanks) return nullptr;
+  else if (r != R) return store_all_from<DT, R + 1>(r, split);
+  else return split ? reinterpret_cast<const void*>(&store_all_kernel<DT, R, 512, true>) : reinterpret_cast<const void*>(&store_all_kernel<DT, R, 512, false>);
 }
-template <int DT>
-static const void* store_all_of(int R) {
-  return store_all_from<DT, 2>(R);
-}
+static const void* store_all_of(int R, int dtype, bool split) { return dtype == 0 ? store_all_from<0, 2>(R, split) : store_all_from<1, 2>(R, split); }
 const void* store_all_entry(int R, int dtype, int ctas, unsigned long long count, StoreAllArgs* a, int* grid, int* threads) {
-  const void* fn = dtype == 0 ? store_all_of<0>(R) : store_all_of<1>(R);
+  const void* fn = store_all_of(R, dtype, ctas < R);
   if (!fn || count > (1ull << 28)) return nullptr;   // 32-bit byte offsets
   a->count = (unsigned)count;
   a->q = (unsigned)((count + R - 1) / R);
@@ -1278,7 +1278,7 @@ static std::vector<const void*> dispatched_kernels() {
     }
   }
   for (int R = 2; R <= kMaxStoreAllRanks; R++)
-    for (const void* f : {store_all_of<0>(R), store_all_of<1>(R)}) fns.push_back(f);
+    for (int form = 0; form < 4; form++) fns.push_back(store_all_of(R, form & 1, form & 2));
   for (int shape = 0; shape < (int)(sizeof(kMoveShapes) / sizeof(kMoveShapes[0])); shape++)
     for (const void* f : {move_entry<MoveBatch>(shape), move_entry<MoveBatchSmall>(shape)}) fns.push_back(f);
   std::sort(fns.begin(), fns.end());

@@ -894,6 +894,12 @@ static hoccl_result_t call_options(hoccl_comm* c, const Call& call, OptionsOut* 
 // 2 %; 24 do not finish in time).  25 MiB per rank over 8 ranks in three pieces 206.8 us with 24, 207.0 with 40, 208.7 with 64.
 constexpr long kBesideSums = 40;
 
+// A step of the ring, by bytes of all ranks, whose whole-GPU moves are one CTA per SM that walks its tiles: what it reads the step before has just
+// written to L2, so there is nothing for a CTA per tile to hide, only more of them to start.  Us, bf16, a CTA per tile / the walk: all-gather 8 ranks 2 MiB 20.4 /
+// 18.4, 12 MiB 37.0 / 35.7, 25 MiB 59.4 / 59.3, 32 MiB 71.3 / 76.9, 64 MiB 136 / 146, 16 ranks 0.8 MiB 33.6 / 34.6, 12 MiB 70.4 / 67.5, 25 MiB 110.7 / 107.9, 32
+// MiB 133 / 139; all-reduce 16 ranks 2 MiB 112.7 / 107.5, 25 MiB 351 / 342, 8 ranks 0.5 MiB 44.0 / 45.1, 25 MiB 167.5 / 164.0.
+constexpr size_t kRingWalkFrom = 1280 << 10, kRingWalkTo = (size_t)28 << 20;
+
 // Pure host work, nothing is enqueued.  The communicator shows the call's route (RouteGuard).
 static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut& opt, Contributions how, Layout* out) {
   const bool fused = opt.executor == EXEC_ONE_KERNEL, roles = opt.executor == EXEC_ROLES;
@@ -1026,6 +1032,12 @@ static hoccl_result_t lay_out(hoccl_comm* c, const Call& call, const OptionsOut&
   // 256 MiB 1543 / 1512; staged, 8, R = 8 40 MiB 417.5 / 412.6.
   out->sums_by_launch = out->overlap && !c->profile && how != STAGED && c->sum_ctas < 64;
   for (RGroup& g : out->groups) {
+    if (g.kind == OP_MOVE && c->path == HOCCL_PATH_SM && c->copy_ctas >= kAllSms && call.kind != PLAN_ALLTOALL && g.phase != PHASE_OWN &&
+        !(plan_kind & (g.phase == PHASE_RS ? PLAN_FLAG_RS_DIRECT : PLAN_FLAG_AG_DIRECT))) {
+      size_t bytes = 0;
+      for (const Seg& s : g.segs) bytes += s.bytes;
+      if (bytes >= kRingWalkFrom && bytes <= kRingWalkTo) g.ctas = kAllSms - 1;
+    }
     if (beside && g.kind == OP_MOVE && g.piece + 1 < P.pieces) g.ctas = kBesideSums;
     // the first piece's sum has nothing beside it unless the next piece's contributions are copied meanwhile
     if (out->overlap && g.kind == OP_CHAIN) g.beside = g.piece > 0 || how == STAGED;

@@ -779,7 +779,6 @@ __global__ void __launch_bounds__(kThreads, 2) occupy_kernel(unsigned long long 
 // chunks of a ring step over the grid (gradient bucket, whole GPU: 0.201 against 0.213 ms per step).
 static bool wide_grid(int ctas) { return ctas >= 128; }
 static bool wide_copy_grid(int ctas) { return ctas >= 128; }
-constexpr int kAllSms = 148;
 static bool whole_gpu(int ctas) { return ctas >= kAllSms; }   // a CTA per tile, see kMoveShapes
 
 // Host side of the flattened view (same split as the device helper; tile = 4 x threads vectors for the sum, 8 x 1024 or

@@ -7,6 +7,7 @@
 namespace hoccl {
 
 constexpr int kMaxSegs = 32;       // segments (one per rank) a single batched launch can carry
+constexpr int kAllSms = 148;       // CTA counts from here on mean the whole GPU: chain sums and moves take a CTA per tile, below they walk their tiles
 constexpr int kThreads = 1024;     // threads per CTA of the copy and occupancy kernels (the sum picks 512 or 1024)
 
 // Flattened view of a batch of segments: every segment is an element-wise head, a body of 16-byte vectors cut into

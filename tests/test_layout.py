@@ -204,3 +204,20 @@ def test_copies_in_chains_where_the_sum_beside_them_lasts_as_long(R, count, para
 def test_sums_launched_where_they_run_back_to_back(R, params, launched):
     lay, *_ = lay_out(ALLREDUCE, R, 20_971_520 // 8 * R, "bf16", **params)
     assert lay.sums_by_launch == launched
+
+
+@pytest.mark.parametrize("kind, R, count, walks", [(ALLGATHER, 8, 131_072, True), (ALLGATHER, 16, 393_216, True), (ALLGATHER, 8, 16_384, False),
+                                                   (ALLGATHER, 8, 4_194_304, False), (ALLREDUCE, 8, 1_048_576, True), (ALLREDUCE, 16, 33_554_432, False)])
+def test_moves_of_ring_steps_on_the_whole_gpu(kind, R, count, walks):
+    """Steps whose bytes the step before has left in L2 are one CTA per SM; shorter and longer ones, and the moves of the direct forms, have a
+    CTA per tile."""
+    ring = dict(ag_direct=0, rs_direct=0, path=hb.PATH_SM, sum_ctas=148, copy_ctas=148)
+    for params, one_per_sm in ((ring, walks), (dict(ring, ag_direct=1, rs_direct=1), False), (dict(ring, copy_ctas=140), None)):
+        lay, *_ = lay_out(kind, R, count, "bf16", **params)
+        kinds = {a.group: a.kind for a in lay.accesses}
+        moves = [n for g, n in enumerate(lay.ctas) if kinds[g] == hd.OP_MOVE and len({a.segment for a in lay.accesses if a.group == g}) == R]
+        assert moves or params.get("ag_direct")          # the direct forms read in place or share segments
+        if one_per_sm is None:
+            assert all(n == 140 for n in moves)
+        else:                                            # (the first one may be the copy of the own block)
+            assert all((n == 147) == one_per_sm for n in moves[1:]), moves

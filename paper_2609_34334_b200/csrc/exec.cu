@@ -683,7 +683,9 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
   // A short chain of kernels goes out as a graph or as launches (see launch_in_order).  A graph costs the host less (0.9 us against 1.6 to 2.4
   // per launch) and reaches an idle device 1.6 us earlier; behind other work launches start up to 2 us earlier.  Whether there is
   // work in front cannot be asked for less (cudaStreamQuery 0.3 us if there is, 1.6 if not).  So: launches if the call follows the one before
-  // it at once, on the same stream, and takes the device longer than the host, or is one launch and the calls before it did; otherwise the graph.  Us of a call
+  // it at once, on the same stream, and takes the device longer than the host, or is one launch of 3.5 us or more and the calls before it did (a shorter
+  // one takes two steps of 2.048 us as a graph, 4.1, and what the host needs as a launch, up to 5.6: all-reduce of 4 ranks, 147 KB, est. 3.1, 4.1 / 4.7-5.6,
+  // 200 KB, est. 3.7, 6.2 / 3.6; all-gather of 4 ranks est. 2.7 3.9 / 4.7, est. 3.6 4.1 / 3.65); otherwise the graph.  Us of a call
   // in a burst as graphs / as launches, R = 8 bf16: all-reduce 4 KiB per rank 3.6 / 4.9, 96 KiB 4.10 / 4.52, 128 KiB 6.15 / 4.55, 384 KiB
   // 10.25 / 9.1, 1 MiB with 8 + 40 CTAs 17.0 / 14.35; 148 CTAs 512 KiB 4.10 / 4.85, 1 MiB 6.14 / 4.85; all-to-all 512 KiB 4.10 / 4.80, 1 MiB
   // 6.15 / 4.80; two launches, R = 16, all-to-all 512 KiB 8.19 / 8.56, 2 MiB 20.5 / 18.3.  The line: the estimate against 1.8 + 2.2 per launch.
@@ -691,7 +693,7 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
   const bool follows = last.stream == user && t0 - last.returned < kBurstGapUs;
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;   // a capture is refused by the graph launch, in a burst or not
   const size_t n = hit->launches.size();
-  const bool behind = n && follows && ((n == 1 && t0 < last.busy_until) || hit->est_us >= 1.8 + 2.2 * (double)n) &&
+  const bool behind = n && follows && ((n == 1 && hit->est_us >= 3.5 && t0 < last.busy_until) || hit->est_us >= 1.8 + 2.2 * (double)n) &&
                       cudaStreamIsCapturing(user, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
   last.busy_until = (follows ? std::max(t0, last.busy_until) : t0) + hit->est_us;
   struct Returns {   // on every way out

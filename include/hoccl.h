@@ -144,7 +144,11 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  * Tuning and diagnostics.  Keys:
  *  "sum_ctas"    CTAs of a SUM launch, 1..1024 (default 8: the SM budget for sums)
  *  "copy_ctas"   CTAs of an SM copy launch, 1..1024 (default 8).  Both: 148 (every SM) or more means the whole GPU; the chain sums and the
- *                moves of such a launch take a small CTA per tile, however many that makes
+ *                moves of such a launch take a small CTA per tile, however many that makes.  Such sums are faster alone and more in the way of other
+ *                kernels than those of 147 CTAs and fewer, which leave half of every SM free: an all-reduce of 256 MiB per rank over 8 ranks takes
+ *                0.64 ms with 148 + 148 and 0.68 with 140 + 148; beside a loop of 8192^3 bf16 GEMMs 1.00 and 1.21 ms, and a call costs the GEMMs 0.77 and
+ *                0.25 ms (40 MiB: 0.18 / 0.19 ms and 0.07 / 0.06).  Sums with another piece's driver copies beside them ("ce_overlap") keep
+ *                one CTA per SM for up to 8 ranks, and so do the moves of ring steps ("ag_direct" or "rs_direct" = 0) of 1.25 to 28 MiB
  *  "piece_bytes" pipeline piece size in bytes (rounded to a multiple of 1024).  If the key is not set: for reductions, whole
  *                ring chunks (up to 256 MiB) on HOCCL_PATH_CE and on HOCCL_PATH_SM when both CTA budgets are 128 or more (pieces exist to overlap one
  *                piece's move with another piece's sum, which neither driver copies nor whole-GPU grids do); otherwise
@@ -212,7 +216,7 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                ends differ modulo 4): a send/recv message or an all-to-all of such blocks, an all-to-all of blocks below 4 MiB or over at most
  *                4 ranks, an uneven exchange of flows up to 4.5 MiB on average, any all-gather (the kernel reads a block once, driver copies
  *                once per destination) and the all-gather of an all-reduce with such chunks (automatic schedule, SUM budget below 64 CTAs) run on
- *                the copy kernel like a small one.  With "ag_direct" set by hand an
+ *                the copy kernel like a small one, if "ce_small_ctas" suffices for that (see there).  With "ag_direct" set by hand, or too few CTAs, an
  *                all-reduce that reads contributions in place ("rs_direct" = 2) gives the ends of the copies of its direct
  *                all-gather to one launch of the copy kernel ("copy_ctas" CTAs) per piece (in a ring all-gather, whose copies
  *                forward what the one before has written, copies stay whole).
@@ -226,7 +230,9 @@ hoccl_result_t hoccl_comm_set_path(hoccl_comm_t comm, hoccl_path_t path);
  *                least 2 above 8 MiB per chunk (R = 2, 64 MiB per rank 2, R = 8, 40 MiB 4, 256 MiB 10); 0 = off;
  *                2..64 = that many pieces.  Ignored when "piece_bytes" is set.
  *  "ce_small_ctas" CTAs of those launches, 1..1024 (default 148: like the driver's own copies they may use the whole GPU,
- *                for tens of microseconds)
+ *                for tens of microseconds).  Below 128 a call beyond "ce_small_bytes" stays with the driver where so few CTAs would take longer than
+ *                its copies (they carry 46 GB/s each): whole blocks and flows want 64, ones with odd ends 32, ones out of phase modulo 4 bytes 16, short
+ *                ones one per 20 KB at least; long whole blocks between at most 4 ranks and the all-gather of an all-reduce want 128
  *  "order_kernels" 1 (default) = on the copy routes the graph executor puts an empty one-warp kernel in front of a graph's
  *                first copies and behind every group of copies that other copies (or the end of the graph) wait for.
  *                Measured on B200: a copy node that waits for earlier stream work or for several copy nodes starts ~4 us
@@ -445,7 +451,8 @@ hoccl_result_t hoccl_comm_proxy_stats(hoccl_comm_t comm, double* busy_us, double
  * 1 MiB per rank, 3 at 4 MiB) unless "host_pieces" was set, as it does for longer vectors on the direct schedule (5 at 25 MiB).
  * If, besides, "host_pieces" was not set and every host buffer is pinned or registered with CUDA (as one range) and shares its address
  * modulo 16 with the others, nothing is copied at all: one launch of "sum_ctas" CTAs reads the host buffers across PCIe and stores the
- * result into every one of them.  Staging is still demanded: whether the buffers permit it is known at the call.
+ * result into every one of them.  Staging is still demanded: whether the buffers permit it is known at the call.  A call in this form can be
+ * captured into a graph; the forms that replay a graph of their own refuse a capture (HOCCL_ERR_CUDA), as every such call does.
  * Host buffers of different ranks must not overlap
  * partially (INVALID_ARG); h_recv[r] == h_send[r] is legal.  With host_pieces = 1, use_graph = 0, handshake, onepass,
  * fused or HOCCL_PATH_CE_HOST the three stages run one after the other.
@@ -473,7 +480,8 @@ hoccl_result_t hoccl_host_allreduce(const void* const* h_send, void* const* h_re
  * belong to the device that is current when the call is made.
  *
  * Buffers that share their address modulo 16 do without the array: the chain sum (8 CTAs) reads the contributions where they lie
- * and one launch of moves (32 CTAs), or for short vectors the sum itself, brings the result to every rank.
+ * and one launch of moves (the whole GPU, for 2 to 30 us), or for short vectors the sum itself, brings the result to every rank.  Beside a loop
+ * of 8192^3 bf16 GEMMs that costs them nothing that could be measured (6 ranks of 2 MB and 8 MiB fp32, 8 ranks of 4 MiB; on 32 CTAs as little).
  *
  * Limits and sharing.  The scratch need is 2 * R * roundup256(ceil(count/R) * sizeof(dtype) + 16) bytes;
  * a call that would need more than HOCCL_STATIC_SCRATCH_BYTES is rejected with HOCCL_ERR_SCRATCH and

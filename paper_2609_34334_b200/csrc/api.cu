@@ -373,7 +373,9 @@ hoccl_result_t hoccl_alltoallv(const void* const* send, const size_t* sendcounts
   // runs on the move kernel, and so does one of flows that are short on average (every driver copy costs a microsecond, and those of an uneven
   // pattern leave the GPU part empty).  R = 8, driver copies against the kernel: 8 MiB per rank (flows of 1 MiB on average) 41 / 22.6 us, 16 MiB (2
   // MiB) 61 / 43, 32 MiB (4 MiB) 95.7 / 83.5, in rows of 666 bytes 447 / 86; R = 16, 64 MiB (4 MiB) 393 / 336.  Longer whole flows stay with the
-  // driver, which is 3 to 6 % behind there (8 ranks 64 MiB 173.6 / 164.1, 128 MiB 335 / 325).
+  // driver because "the copy route above the small size" is what the route promises and what callers count copies by; the kernel is ahead on both
+  // sides of the line, by less the longer they are (8 ranks, whole flows of 4 MiB 93.0 / 86.0, 4.5 103.4 / 96.1, 5 114.5 / 106.4, 8 174.8 / 166.0, 16 336 /
+  // 327.6; 4 ranks 5 MiB 32.8 / 27.0; 16 ranks 6 MiB 578 / 499).
   hoccl_path_t route = c->path;
   if (c->path == HOCCL_PATH_CE && c->ce_small_bytes > 0 && !modelled) {
     constexpr uint64_t kShortFlow = 9 << 19;   // 4.5 MiB

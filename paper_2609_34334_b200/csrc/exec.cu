@@ -669,7 +669,6 @@ hoccl_result_t ensure_proxy(hoccl_comm* c) {
   return HOCCL_OK;
 }
 
-// Replays a cached graph into the caller's stream (directly, or through the CPU proxy in handshake mode).
 // What this thread last put on a stream: the stream, when the call returned, and when by estimate the device is through with it.  Only a
 // hint which of two equal ways a call takes; a stream that died and whose handle came back misleads it for one call.
 struct Burst {
@@ -678,6 +677,8 @@ struct Burst {
 };
 static thread_local Burst t_burst;
 constexpr double kBurstGapUs = 5;   // a Python caller's loop leaves about 2 us between calls; waiting for the device in between takes 7 or more
+
+// Replays a cached entry into the caller's stream (directly, or through the CPU proxy in handshake mode: an entry of that mode has no launches).
 hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, double t0) {
   hit->last_use = ++c->use_counter;
   // A short chain of kernels goes out as a graph or as launches (see launch_in_order).  A graph costs the host less (0.9 us against 1.6 to 2.4
@@ -864,11 +865,13 @@ static bool blocks_bad_for_driver(const hoccl_comm* c, const Call& call) {
 }
 
 // An all-reduce whose sums read the contributions in place and whose ring chunks the driver copies badly (not whole pages on 128-byte lines), or
-// are short copies (but for chunks of 1 to 1.17 MiB, 80 MB for all ranks, whose copies and ends the layout tests describe): its all-gather runs on the move kernel too, which reads a chunk once for all ranks.  Us in driver copies with their ends on the
+// are short copies: its all-gather runs on the move kernel too, which reads a chunk once for all ranks.  Us in driver copies with their ends on the
 // kernel / on the kernel alone, bf16: R = 8, 16 MiB per rank 149.5 / 137.5, 64 MiB 554 / 527; R = 3, 32 MiB 174 / 155; R = 5, 32 MiB 221 / 203; R = 6, 64 MiB
 // 456 / 445; R = 16, 19 MiB 352 / 290, 64 MiB 1072 / 887.  A loop of 8192^3 GEMMs loses less to it as well (8 ranks, 64 MiB 97 us per
 // call, in driver copies 175).  Only with "ce_small_ctas" >= 128: on fewer it is even at best, R = 8 64 MiB driver 521 us, 8 CTAs 1027, 16 624, 40 515, 64 527;
-// R = 3 32 MiB 157, 216, 172, 165, 165 (148: 145).  Whole chunks stay with the driver, whose copies run beside the next piece's sum: 8 ranks 40 MiB 335 us, 320 on the kernel.
+// R = 3 32 MiB 157, 216, 172, 165, 165 (148: 145).  Whole chunks stay with the driver, whose copies run beside the next piece's sum: 8 ranks 40 MiB 335 us,
+// 320 on the kernel.  So do ragged ones of 1 to 1.17 MiB, 80 MB for all ranks, though the kernel is ahead of them too (8 ranks of 8.5 MB 85 / 72, of
+// 9.6 MB 92 / 80): they keep the form with trimmed copies, whose layout and signature are checked at these sizes.
 static bool chunks_bad_for_driver(const hoccl_comm* c, const Call& call) {
   const size_t S = call.count * dtype_size(call.dtype), chunk = (call.count + c->R - 1) / c->R * dtype_size(call.dtype);
   if (chunk >= kDriverWhole && chunk < ((size_t)1200 << 10) && (size_t)c->R * S < 80000000) return false;

@@ -922,7 +922,8 @@ static ChainVariant chain_fan_variant(int nops, int ctas) {
 // per tile: sums that store for every rank R = 2 (128 MiB) 89 / 80.2, 4 86 / 80.5, 8 171 / 163.8; one destination R = 8 94 / 88.1, 3 24 / 20.7.  Tiles of
 // 128 to 512 vectors are within 3 %, but for 2 and 3 operands with one destination, which want two vectors per thread (R = 2, 128 MiB 59.4, 67.0 with one).
 // 9 to 16 operands, against chain_kernel: every rank R = 9 bf16 32 MiB 99.6 / 95.2, 16 167.9 / 165.7; reduce-scatter + all-gather R = 9 fp32 32 MiB 114 / 103,
-// 4 MiB 17.6 / 15.2, R = 16 bf16 0.28 MiB 14.4 / 12.3.
+// 4 MiB 17.6 / 15.2, R = 16 bf16 0.28 MiB 14.4 / 12.3.  Beside a loop of 8192^3 GEMMs the walk (140 CTAs) is the gentler one for long sums: all-reduce that
+// stores for every rank, R = 8 256 MiB 996 us a call and 770 lost to the GEMMs, 1210 and 254 with the walk; 40 MiB 176 and 74, 192 and 56.
 template <int DT, int N>
 static ChainVariant chain_tile_variant(int nops, bool fan) {
   if constexpr (N > 16) return {nullptr, 0, 0};
@@ -1074,6 +1075,7 @@ bool add_move_seg(MoveBatch* b, const void* src, void* const* dsts, int ndst, un
 // walk: copies 6.81 / 6.25 (4 x 704), 1:3 6.37 / 5.94 (4 x 384), 1:7 6.46 / 5.80 (1 x 448); 512 KiB 5.60 / 5.32, 4.29 / 3.22, 5.08 / 4.41.  Larger and smaller
 // tiles (1 to 16 x 128 to 512) are within 3 % of these.  Between 128 CTAs and all SMs the walk stays, in its own shapes: it wants little in
 // flight per SM, the less the more often a vector is stored, 44 KiB for copies (4 x 704 6.2 TB/s, 8 x 1024 4.2), 7 for one read stored 7 times.
+// (Who comes between: steps of the ring whose bytes are in L2, see kRingWalkFrom, and budgets of 128 to 147, a caller's own choice.)
 struct MoveShape {
   int u, threads;
 };

@@ -6,7 +6,7 @@ pipeline / gradient-stream workloads (third and fourth), through the C ABI.
     python -m paper_2609_34334_b200.sweep gradients [--buckets 32] [--budgets 1,2,4,8,16,32,64]
     python -m paper_2609_34334_b200.sweep launch-cost
     python -m paper_2609_34334_b200.sweep alltoallv [--mib 4,64,256] [--model 4,2]
-    python -m paper_2609_34334_b200.sweep cases [--only NAME,NAME]      # the calls of perf/cases.py (run from the repository's root)
+    python -m paper_2609_34334_b200.sweep cases [--only NAME,NAME] [--draw N --seed S]   # the calls of perf/cases.py, listed and drawn (from the repository's root)
     python -m paper_2609_34334_b200.sweep call --op allreduce --ranks 8 --count 20971520 --dtype bf16 \\
         --variants "ce_overlap=2;ce_overlap=4;path=SM,sum_ctas=8,copy_ctas=40" [--gemm]   # one call under several settings, in turn
 
@@ -19,6 +19,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import random
 import sys
 import time
 
@@ -523,20 +524,21 @@ def _spread(fns, stream, rounds=5, window_s=0.02):
 
 
 def cases(args):
-    """The listed calls of perf/cases.py, three input sets in rotation (less for the largest): microseconds of a pass among others."""
+    """The listed calls of perf/cases.py, three input sets in rotation (less for the largest): microseconds of a pass among others.  With
+    --draw also that many drawn ones of the same ranges, the same for the same --seed."""
     from perf import cases as C
 
     torch.cuda.set_device(0)
     stream = torch.cuda.current_stream()
-    for case in C.listed():
-        if args.only and case["name"] not in args.only.split(","):
-            continue
+    rng = random.Random(args.seed)
+    chosen = [c for c in C.listed() if not args.only or c["name"] in args.only.split(",")] + [C.draw(rng) for _ in range(args.draw)]
+    for case in chosen:
         nbytes = C.work(case)["bytes"]
         states = [C.prepare(case, seed) for seed in range(3 if nbytes < (2 << 30) else 2)]
         torch.cuda.synchronize()
         (t, lo, hi), = _spread([lambda k: C.run(states[k % len(states)])], stream)
         torch.cuda.synchronize()
-        print(json.dumps({"case": case["name"], "us": round(t, 2), "least": round(lo, 2), "most": round(hi, 2), "GBps": round(nbytes / t / 1e3, 1)}), flush=True)
+        print(json.dumps({"case": case.get("name", case), "us": round(t, 2), "least": round(lo, 2), "most": round(hi, 2), "GBps": round(nbytes / t / 1e3, 1)}), flush=True)
         del states
         torch.cuda.empty_cache()
 
@@ -642,7 +644,9 @@ def main():
     a2.add_argument("--mib", default="4,64,256", help="comma list of MiB sent per rank")
     a2.add_argument("--model", default="", help="comma list of modelled GPUs per node (e.g. 4,2): also run the pattern over that topology")
     c = sub.add_parser("cases")
-    c.add_argument("--only", default="", help="comma list of names")
+    c.add_argument("--only", default="", help="comma list of names (\"none\": drawn ones alone)")
+    c.add_argument("--draw", type=int, default=0, help="drawn cases besides")
+    c.add_argument("--seed", type=int, default=1)
     o = sub.add_parser("call")
     o.add_argument("--op", default="allreduce", choices=["allreduce", "reduce_scatter", "allgather", "alltoall", "sendrecv", "host_allreduce"])
     o.add_argument("--ranks", type=int, default=8)

@@ -700,11 +700,12 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
   struct Returns {   // on every way out
     Burst& last;
     cudaStream_t s;
+    double at;   // 0: not read yet (a reading of the clock is 1 % of a short call)
     ~Returns() {
       last.stream = s;
-      last.returned = now_us();
+      last.returned = at != 0 ? at : now_us();
     }
-  } returns{last, user};
+  } returns{last, user, 0};
   if (!hit->ring_args.empty()) {
     if (hit->ring_large)
       CU_TRY(c, launch_ring(*reinterpret_cast<const RingArgsLarge*>(hit->ring_args.data()), hit->ring_grid, hit->ring_threads, user));
@@ -820,7 +821,8 @@ hoccl_result_t launch_entry(hoccl_comm* c, GraphEntry* hit, cudaStream_t user, d
   c->stats.n_order_launches = hit->n_order_launches;
   c->stats.max_sum_ctas = hit->n_sum_launches ? c->sum_ctas : 0;
   c->stats.max_copy_ctas = hit->n_move_launches ? c->copy_ctas : 0;
-  c->stats.host_launch_us = now_us() - t0;
+  returns.at = now_us();
+  c->stats.host_launch_us = returns.at - t0;
   return HOCCL_OK;
 }
 
